@@ -53,8 +53,12 @@ typedef enum {
     WPCD_ERR_HANDLE = -8      /* unknown or released handle / ticket */
 } wpcd_status;
 
-/* Arithmetic of the eigensolve.  FP64: H assembled and diagonalised in FP64
- * (parallel Jacobi).  MIXED: H diagonalised in FP32 (the same Jacobi with a
+/* Arithmetic of the eigensolve.  FP64: H assembled in FP64 and diagonalised to
+ * FP64 backward error: FP32 Jacobi eigenvectors, then refinement iterations of
+ * the eigenpairs against the FP64 H with 55-bit products until the correction is
+ * at FP64 rounding, and FP64 parallel Jacobi for any solve that the refinement
+ * does not finish (values outside FP32's range, unresolved clusters) or when
+ * there is no room for its scratch.  MIXED: H diagonalised in FP32 (Jacobi with a
  * relative rotation threshold), then two FP64 refinement iterations of the
  * eigenpairs (Ogita-Aishima: Y = HX, S = X^T Y, G = X^T X, X <- X(I + E)) as
  * batched FP64 products; everything after the eigensolve (resolvent logs, T,
@@ -96,9 +100,8 @@ enum {
  * products -- TENSOR (BF16 tensor cores with Ozaki splitting, FP64-accurate) or
  * FP64 (FP64 CUDA cores).  WPCD_OPT_AUTOTUNE (1 = on, the default): on the first
  * batched eigensolve of each (matrix size, precision) the context times CTA
- * sizes 64/128/256/512 (and 1024 for the FP32 kernel) on about two full waves
- * of that bucket and keeps the
- * fastest (wpcd_tuning reports the choices); 0 = fixed 256 threads.
+ * sizes of the FP32 kernel, 64/128/256/512/1024 (up to 512 on the FP64 path
+ * below n ~ 230), on about two full waves of that bucket and keeps the fastest (wpcd_tuning reports the choices); 0 = fixed 256 threads.
  * WPCD_OPT_GRAPH (1 = on, the default): batched wpcd_solve / wpcd_solve_host
  * calls are replayed from CUDA graphs (see wpcd_solve); 0 = every call
  * launches its kernels one by one.  WPCD_OPT_BIG_SLOTS: CTAs (each with its
@@ -226,9 +229,10 @@ wpcd_status wpcd_vset_get(wpcd_ctx *ctx, int vset_id, int channel, double *out_h
  * [n_samples][n_terms-1] FP64 (may be NULL when n_terms == 1).  The eigenpairs
  * stay on the device under the returned eig handle.  prec: WPCD_PREC_FP64 or
  * WPCD_PREC_MIXED (see wpcd_precision).  Every size uses the parallel cyclic
- * Jacobi method (App. C): matrices that fit one CTA's shared memory (FP64 up to
- * n ~ 230, FP32 up to n = 304) are held there; larger ones, up to n = 1024, are
- * held in global memory (L2-resident while a CTA works on them).
+ * Jacobi method (App. C), in FP32 before the refinement of either precision:
+ * matrices that fit one CTA's shared memory (FP32 up to n = 304, FP64 up to
+ * n ~ 230) are held there; larger ones, up to n = 1024, are held in global memory
+ * (L2-resident while a CTA works on them).
  * Per-solve convergence status: wpcd_diag_status.
  * Errors: WPCD_ERR_ARG, WPCD_ERR_HANDLE, WPCD_ERR_NOMEM, WPCD_ERR_BUDGET, WPCD_ERR_CUDA. */
 wpcd_status wpcd_diag(wpcd_ctx *ctx, int vset_id, const double *coeffs_dev, int n_samples,
@@ -390,7 +394,7 @@ wpcd_status wpcd_batched_dgemm(wpcd_ctx *ctx, int n, int items, int trans_a, con
 
 /* The autotuner's table: up to max_entries (n, precision, chosen CTA size) and,
  * in ms_out[5 k + j], the measured time per solve of candidate j (64, 128, 256,
- * 512, 1024 threads; 1024 only for the FP32 kernel; negative = not run).
+ * 512, 1024 threads; negative = not run) of the FP32 solve.
  * Returns the number of entries. */
 int wpcd_tuning(wpcd_ctx *ctx, int max_entries, int *n_out, int *prec_out, int *threads_out, float *ms_out);
 

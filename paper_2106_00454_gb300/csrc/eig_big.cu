@@ -100,18 +100,19 @@ __device__ __forceinline__ void big_rot(double c, double s, double u, double v, 
     o2 = fma(s, u, __dmul_rn(c, v));
 }
 
-template <class T>
+template <class T, bool TEST>
 __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *chans, const int *work_ch, int n_work_ch,
                                                           int n_items, int sample0, int n_terms, const double *coeffs,
                                                           T *scratch, double *eps_all, double *C_all, double *lam_s,
                                                           double *X_s, double *H_s, int *status_all, int n_ch_total,
-                                                          int *err)
+                                                          int *err, const RotTest test, const int *done)
 {
     constexpr bool F64 = sizeof(T) == 8;
     constexpr int kBigUnroll = BigUnroll<T>::v;
     extern __shared__ double smem_big[];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        if (done && done[item] != 0) continue;  // already solved (CTA-uniform)
         const int wc = item % n_work_ch;
         const int smp = sample0 + item / n_work_ch;
         const int cidx = work_ch[wc];
@@ -198,7 +199,11 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                     const T apq = A[(size_t)p * np + q];
                     bool rotate;
                     if (F64) rotate = apq != T(0);
-                    else rotate = big_abs(apq) > (T)kBigRelTol * sqrt(big_abs(app) * big_abs(aqq)) && big_abs(apq) > thr;
+                    else {
+                        const T scale = sqrt(big_abs(app) * big_abs(aqq));
+                        rotate = big_abs(apq) > (T)kBigRelTol * scale && big_abs(apq) > thr &&
+                                 (!TEST || big_abs(apq) > (T)test.rel * scale || big_abs(apq) > (T)test.ang * big_abs(aqq - app));
+                    }
                     if (rotate) {
                         const T tau = (aqq - app) / (T(2) * apq);
                         T t;
@@ -383,8 +388,8 @@ int jacobi_big_max_n() { return kBigMaxN; }
 int jacobi_big_occupancy(int n, bool f64)
 {
     int blocks = 0;
-    if (f64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<double>, kBigThreads, big_smem<double>(n));
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<float>, kBigThreads, big_smem<float>(n));
+    if (f64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<double, false>, kBigThreads, big_smem<double>(n));
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<float, false>, kBigThreads, big_smem<float>(n));
     return blocks;
 }
 
@@ -395,23 +400,25 @@ int jacobi_big_occupancy(int n, bool f64)
 cudaError_t launch_jacobi_big(bool f64, const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch,
                               int n_samples, int sample0, int n_terms, const double *coeffs, int n, void *scratch,
                               int slots, double *eps_all, double *C_all, double *lam_s, double *X_s, double *H_s,
-                              int *status_all, int n_ch_total, int *err, cudaStream_t st)
+                              int *status_all, int n_ch_total, int *err, cudaStream_t st, RotTest test,
+                              const int *done)
 {
     if (n < 2 || n > kBigMaxN || slots < 1) return cudaErrorInvalidValue;
     const int items = n_samples * n_work_ch;
     const int grid = items < slots ? items : slots;
     if (f64) {
         const size_t sm = big_smem<double>(n);
-        raise_smem_limit((const void *)k_jacobi_big<double>, sm);
-        k_jacobi_big<double><<<grid, kBigThreads, sm, counted(st)>>>(
+        raise_smem_limit((const void *)k_jacobi_big<double, false>, sm);
+        k_jacobi_big<double, false><<<grid, kBigThreads, sm, counted(st)>>>(
             chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs, static_cast<double *>(scratch), eps_all,
-            C_all, nullptr, nullptr, nullptr, status_all, n_ch_total, err);
+            C_all, nullptr, nullptr, nullptr, status_all, n_ch_total, err, test, done);
     } else {
         const size_t sm = big_smem<float>(n);
-        raise_smem_limit((const void *)k_jacobi_big<float>, sm);
-        k_jacobi_big<float><<<grid, kBigThreads, sm, counted(st)>>>(
-            chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs, static_cast<float *>(scratch), nullptr,
-            nullptr, lam_s, X_s, H_s, status_all, n_ch_total, err);
+        auto *k = test.rel > 0.0f || test.ang > 0.0f ? k_jacobi_big<float, true> : k_jacobi_big<float, false>;
+        raise_smem_limit((const void *)k, sm);
+        k<<<grid, kBigThreads, sm, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs,
+                                                  static_cast<float *>(scratch), nullptr, nullptr, lam_s, X_s, H_s,
+                                                  status_all, n_ch_total, err, test, nullptr);
     }
     return cudaGetLastError();
 }

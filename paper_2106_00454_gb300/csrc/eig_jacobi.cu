@@ -1,5 +1,8 @@
 // eig_jacobi.cu -- (a2) parameter sum + H assembly and (a3) symmetric
-// eigendecomposition H = C D C^T (Sec. 3.2 step 2), FP64.
+// eigendecomposition H = C D C^T (Sec. 3.2 step 2), FP64 throughout.  It solves
+// what the FP32 solve with FP64 refinement (refine64.cu) leaves (done[b] == 0),
+// whole batches that have no room for the refinement's scratch, and the
+// allocation-free entry point.
 //
 // One CTA per (sample, channel).  H = diag(H0) + V0 + sum_a c_a V_a is formed
 // directly in shared memory (packed upper triangle), then diagonalised by the
@@ -79,8 +82,9 @@ template <bool C_SMEM>
 __global__ void __launch_bounds__(kJacMaxThreads) k_jacobi_f64(const ChanDev *chans, const int *work_ch, int n_work_ch,
                                                              int sample0, int n_terms, const double *coeffs,
                                                              double *eps_all, double *C_all, int *status_all,
-                                                             int n_ch_total, int *err)
+                                                             int n_ch_total, int *err, const int *done)
 {
+    if (done && done[blockIdx.x] != 0) return;  // already solved
     const int wc = blockIdx.x % n_work_ch;
     const int smp = sample0 + blockIdx.x / n_work_ch;
     const int cidx = work_ch[wc];
@@ -271,7 +275,8 @@ __global__ void __launch_bounds__(kJacMaxThreads) k_jacobi_f64(const ChanDev *ch
 
 cudaError_t launch_jacobi_f64(const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch, int n_samples,
                               int sample0, int n_terms, const double *coeffs, int n, double *eps_all, double *C_all,
-                              int *status_all, int n_ch_total, int *err, cudaStream_t st, int threads)
+                              int *status_all, int n_ch_total, int *err, cudaStream_t st, int threads,
+                              const int *done)
 {
     if (threads < 32 || threads > kJacMaxThreads || (threads & 31)) return cudaErrorInvalidValue;
     bool cs = jacobi_c_in_smem(n);
@@ -281,11 +286,11 @@ cudaError_t launch_jacobi_f64(const ChanDev *chans_dev, const int *work_ch_dev, 
     if (cs) {
         raise_smem_limit((const void *)k_jacobi_f64<true>, smem);
         k_jacobi_f64<true><<<grid, threads, smem, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, sample0, n_terms,
-                                                            coeffs, eps_all, C_all, status_all, n_ch_total, err);
+                                                            coeffs, eps_all, C_all, status_all, n_ch_total, err, done);
     } else {
         raise_smem_limit((const void *)k_jacobi_f64<false>, smem);
         k_jacobi_f64<false><<<grid, threads, smem, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, sample0, n_terms,
-                                                             coeffs, eps_all, C_all, status_all, n_ch_total, err);
+                                                             coeffs, eps_all, C_all, status_all, n_ch_total, err, done);
     }
     return cudaGetLastError();
 }

@@ -110,11 +110,12 @@ __device__ __forceinline__ void mix_pair(int r, int k, int M, int &a, int &b)
 // matrix per SM at the sizes that need many threads): the rounds are bound by
 // latency, and more warps keep more block updates and eigenvector rotations in
 // flight.  The autotuner picks the CTA size per matrix size.
-template <bool C_SMEM>
+template <bool C_SMEM, bool TEST>
 __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const ChanDev *chans, const int *work_ch, int n_work_ch,
                                                                int sample0, int n_terms, const double *coeffs,
                                                                double *lam_s, double *X_s, float *Cf_s,
-                                                               double *H_s, int *status_all, int n_ch_total, int *err)
+                                                               double *H_s, int *status_all, int n_ch_total, int *err,
+                                                               const RotTest test)
 {
     const int wc = blockIdx.x % n_work_ch;
     const int smp = sample0 + blockIdx.x / n_work_ch;
@@ -235,7 +236,9 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
                 const int ca = mcol(a), cb = mcol(b), pb = ab ? ca : cb, qb = ab ? cb : ca;
                 float c = 1.0f, s = 0.0f, app = A[pb + p], aqq = A[qb + q];
                 const float apq = A[qb + p];
-                if (fabsf(apq) > kRelTol * sqrtf(fabsf(app) * fabsf(aqq)) && fabsf(apq) > thr) {
+                const float scale = sqrtf(fabsf(app) * fabsf(aqq));
+                if (fabsf(apq) > kRelTol * scale && fabsf(apq) > thr &&
+                    (!TEST || fabsf(apq) > test.rel * scale || fabsf(apq) > test.ang * fabsf(aqq - app))) {
                     const float tau = (aqq - app) / (2.0f * apq);
                     float t;
                     if (fabsf(tau) > 1e18f) t = 0.5f / tau;
@@ -361,22 +364,19 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
 cudaError_t launch_jacobi_mixed(const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch, int n_samples,
                                 int sample0, int n_terms, const double *coeffs, int n, double *lam_s, double *X_s,
                                 float *Cf_s, double *H_s, int *status_all, int n_ch_total, int *err, cudaStream_t st,
-                                int threads)
+                                int threads, RotTest test)
 {
     const bool cs = mix_smem(n, true) <= kMixSmemCap;
     if (threads < 32 || threads > 2 * kMixMaxThreads || (threads & 31)) return cudaErrorInvalidValue;
     const size_t smem = mix_smem(n, cs);
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
     dim3 grid((unsigned)(n_samples * n_work_ch));
-    if (cs) {
-        raise_smem_limit((const void *)k_jacobi_mixed<true>, smem);
-        k_jacobi_mixed<true><<<grid, threads, smem, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, sample0, n_terms,
-                                                              coeffs, lam_s, X_s, Cf_s, H_s, status_all, n_ch_total, err);
-    } else {
-        raise_smem_limit((const void *)k_jacobi_mixed<false>, smem);
-        k_jacobi_mixed<false><<<grid, threads, smem, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, sample0, n_terms,
-                                                               coeffs, lam_s, X_s, Cf_s, H_s, status_all, n_ch_total, err);
-    }
+    const bool loose = test.rel > 0.0f || test.ang > 0.0f;
+    auto *k = cs ? (loose ? k_jacobi_mixed<true, true> : k_jacobi_mixed<true, false>)
+                 : (loose ? k_jacobi_mixed<false, true> : k_jacobi_mixed<false, false>);
+    raise_smem_limit((const void *)k, smem);
+    k<<<grid, threads, smem, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, sample0, n_terms, coeffs, lam_s, X_s, Cf_s,
+                                            H_s, status_all, n_ch_total, err, test);
     return cudaGetLastError();
 }
 
@@ -388,11 +388,11 @@ int jacobi_mixed_occupancy(int n, int threads)
     const size_t smem = mix_smem(n, cs);
     int blocks = 0;
     if (cs) {
-        raise_smem_limit((const void *)k_jacobi_mixed<true>, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_mixed<true>, threads, smem);
+        raise_smem_limit((const void *)k_jacobi_mixed<true, false>, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_mixed<true, false>, threads, smem);
     } else {
-        raise_smem_limit((const void *)k_jacobi_mixed<false>, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_mixed<false>, threads, smem);
+        raise_smem_limit((const void *)k_jacobi_mixed<false, false>, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_mixed<false, false>, threads, smem);
     }
     return blocks;
 }

@@ -28,29 +28,32 @@
 
 namespace wpcd {
 
-constexpr int kOzP = kOzDigits;  // slices per operand
 constexpr int kOzKC = 32;  // k staged per step
 
 int oz_kpad(int n) { return (n + kOzKC - 1) / kOzKC * kOzKC; }
-size_t oz_slice_elems(int n) { return (size_t)kOzP * n * oz_kpad(n); }
+size_t oz_slice_elems(int n, int planes) { return (size_t)planes * n * oz_kpad(n); }
 
 // GB300 issues FP64 at 2 operations per clock per SM, so the split works on
 // the IEEE-754 fields with integer operations.
 //
-// N = rint(x 2^{47-e}) for |x| < 2^e (round half to even): x = m 2^{E-1075}
-// with the 53-bit significand m, so N = m 2^{-s}, s = 1028 + e - E >= 6.
+// N = rint(x 2^{8P-1-e}) for |x| < 2^e (round half to even): x = m 2^{E-1075}
+// with the 53-bit significand m, so N = m 2^{-s}, s = 1076 - 8P + e - E >= 54 - 8P
+// (P = 7: m may move left by up to two bits).
+template <int P>
 __device__ __forceinline__ long long oz_scaled(double x, int e)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int E = (int)((b >> 52) & 0x7FF);
     if (E == 0 || E == 0x7FF) {  // zero, subnormal or not finite: the FP64 route
         if ((b << 1) == 0) return 0;
-        return __double2ll_rn(ldexp(x, 47 - e));
+        return __double2ll_rn(ldexp(x, 8 * P - 1 - e));
     }
     const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int s = 1028 + e - E;
+    const int s = 1076 - 8 * P + e - E;
     unsigned long long q = 0;
-    if (s < 54) {  // for s >= 54, m 2^{-s} < 1/2
+    if (P > 6 && s <= 0) {
+        q = m << -s;
+    } else if (s < 54) {  // for s >= 54, m 2^{-s} < 1/2
         q = m >> s;
         const unsigned long long rem = m & ((1ull << s) - 1), half = 1ull << (s - 1);
         q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
@@ -66,24 +69,27 @@ __device__ __forceinline__ __nv_bfloat16 oz_bf16_of_int(int d)
     return __ushort_as_bfloat16((unsigned short)(__float_as_uint(f) >> 16));
 }
 
-// The six balanced 8-bit digits of x / 2^e: N = rint(x 2^{47-e}) (|N| <= 2^47),
-// then N = d0 2^40 + d1 2^32 + ... + d5 with d1..d5 in [-128, 127] and
-// |d0| <= 129 -- all exact in BF16, every digit product below 2^15 in
+// The P balanced 8-bit digits of x / 2^e: N = rint(x 2^{8P-1-e}) (|N| <= 2^{8P-1}),
+// then N = sum_p d_p 2^{8(P-1-p)} with d_1 .. d_{P-1} in [-128, 127] and
+// |d_0| <= 129 -- all exact in BF16, every digit product below 2^15 in
 // magnitude, and the signs of the truncated lower products vary, so their
 // sum grows like sqrt(k) instead of k.
+template <int P>
 __device__ __forceinline__ void oz_digit_set(long long N, int *d)
 {
-    // the three low digits from the low 24 bits (unsigned), their carry into
-    // the high part, then the three high digits: 32-bit operations only
-    int t = (int)((unsigned)N & 0xFFFFFFu), hi = (int)(N >> 24);
+    // the low digits from the low 24 bits (P = 7: 32), their carry into the high
+    // part, then the high digits: 32-bit operations only
+    constexpr int L = P == 7 ? 4 : 3;
+    unsigned t = (unsigned)N & (L == 4 ? 0xFFFFFFFFu : 0xFFFFFFu);
+    int hi = (int)(N >> (8 * L));
 #pragma unroll
-    for (int p = kOzP - 1; p >= 3; --p) {
-        d[p] = ((t + 128) & 0xFF) - 128;
-        t = (t - d[p]) >> 8;  // exact: t - d is a multiple of 256
+    for (int p = P - 1; p >= P - L; --p) {
+        d[p] = (int)((t + 128u) & 0xFFu) - 128;
+        t = (t >> 8) + (d[p] < 0 ? 1u : 0u);  // (t - d) / 256
     }
-    hi += t;  // the carry, 0 or 1
+    hi += (int)t;  // the carry, 0 or 1
 #pragma unroll
-    for (int p = 2; p >= 1; --p) {
+    for (int p = P - L - 1; p >= 1; --p) {
         d[p] = ((hi + 128) & 0xFF) - 128;
         hi = (hi - d[p]) >> 8;
     }
@@ -92,13 +98,14 @@ __device__ __forceinline__ void oz_digit_set(long long N, int *d)
 
 // Two neighbouring elements (k, k + 1) of one vector: their digits as BF16
 // pairs, one 32-bit store per digit plane.
+template <int P>
 __device__ __forceinline__ void oz_digits2(double x0, double x1, int e, __nv_bfloat16 *d, size_t stride)
 {
-    int a[kOzP], b[kOzP];
-    oz_digit_set(oz_scaled(x0, e), a);
-    oz_digit_set(oz_scaled(x1, e), b);
+    int a[P], b[P];
+    oz_digit_set<P>(oz_scaled<P>(x0, e), a);
+    oz_digit_set<P>(oz_scaled<P>(x1, e), b);
 #pragma unroll
-    for (int p = 0; p < kOzP; ++p) {
+    for (int p = 0; p < P; ++p) {
         __nv_bfloat162 v;
         v.x = oz_bf16_of_int(a[p]);
         v.y = oz_bf16_of_int(b[p]);
@@ -129,13 +136,13 @@ __device__ __forceinline__ int oz_exp_of(unsigned long long mag)
 // maximum, and the digits are written from the registers with k fastest
 // (coalesced); k in [n, Kp) is zero padding.
 // PAIRS per lane: Kp <= 64 PAIRS (the launch picks the smallest of 4, 8, 16).
-template <int PAIRS>
+template <int PAIRS, int P>
 __global__ void __launch_bounds__(256) k_oz_split_rows(int n, int Kp, const double *M_all, int *e_all,
-                                                       __nv_bfloat16 *S_all)
+                                                       __nv_bfloat16 *S_all, OzSkip skip)
 {
     constexpr int kOzRowPairs = PAIRS;
     const int b = blockIdx.y, v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (v >= n) return;
+    if (v >= n || oz_skipped(skip, b)) return;
     const double *row = M_all + (size_t)b * n * n + (size_t)v * n;
     double x0[kOzRowPairs], x1[kOzRowPairs];
     unsigned long long m = 0;
@@ -150,11 +157,11 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(int n, int Kp, const doub
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     const int ex = oz_exp_of(m);
     if (lane == 0) e_all[(size_t)b * n + v] = ex;
-    __nv_bfloat16 *S = S_all + (size_t)b * kOzP * n * Kp + (size_t)v * Kp;
+    __nv_bfloat16 *S = S_all + (size_t)b * P * n * Kp + (size_t)v * Kp;
 #pragma unroll
     for (int j = 0; j < kOzRowPairs; ++j) {
         const int k = 2 * lane + 64 * j;  // Kp is even: pairs (k, k + 1)
-        if (k < Kp) oz_digits2(x0[j], x1[j], ex, S + k, (size_t)n * Kp);
+        if (k < Kp) oz_digits2<P>(x0[j], x1[j], ex, S + k, (size_t)n * Kp);
     }
 }
 
@@ -163,9 +170,11 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(int n, int Kp, const doub
 // coalesced), takes the column maxima while loading, and writes the digits
 // from shared memory along k (two per thread, coalesced).
 constexpr int kOzColBlockKp = 384;  // 101 KB of shared memory at most
+template <int P>
 __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, const double *M_all, int *e_all,
-                                                             __nv_bfloat16 *S_all)
+                                                             __nv_bfloat16 *S_all, OzSkip skip)
 {
+    if (oz_skipped(skip, blockIdx.y)) return;
     extern __shared__ double blk[];  // [Kp][33]
     __shared__ unsigned long long mcol[8][32];
     __shared__ int ecol[32];
@@ -187,10 +196,10 @@ __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, cons
         if (v < n) e_all[(size_t)b * n + v] = ecol[tx];
     }
     __syncthreads();
-    __nv_bfloat16 *S = S_all + (size_t)b * kOzP * n * Kp;
+    __nv_bfloat16 *S = S_all + (size_t)b * P * n * Kp;
     for (int r = ty; r < 32 && v0 + r < n; r += 8)  // column v0 + r, k pairs 2 tx + 64 j
         for (int k = 2 * tx; k < Kp; k += 64)
-            oz_digits2(blk[k * 33 + r], blk[(k + 1) * 33 + r], ecol[r], S + (size_t)(v0 + r) * Kp + k,
+            oz_digits2<P>(blk[k * 33 + r], blk[(k + 1) * 33 + r], ecol[r], S + (size_t)(v0 + r) * Kp + k,
                        (size_t)n * Kp);
 }
 
@@ -198,9 +207,11 @@ __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, cons
 // (32 x 8) per 32 columns: the column maxima first (reads along v), then 64 x 32 tiles
 // transposed through shared memory so that both the reads (v fastest) and the
 // writes (k fastest, two per thread) are coalesced.
+template <int P>
 __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const double *M_all, int *e_all,
-                                                       __nv_bfloat16 *S_all)
+                                                       __nv_bfloat16 *S_all, OzSkip skip)
 {
+    if (oz_skipped(skip, blockIdx.y)) return;
     __shared__ double tile[64][33];
     __shared__ unsigned long long mcol[8][32];
     __shared__ int ecol[32];
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const doub
         if (v0 + tx < n) e_all[(size_t)b * n + v0 + tx] = ecol[tx];
     }
     __syncthreads();
-    __nv_bfloat16 *S = S_all + (size_t)b * kOzP * n * Kp;
+    __nv_bfloat16 *S = S_all + (size_t)b * P * n * Kp;
     for (int k0 = 0; k0 < Kp; k0 += 64) {  // 64 k x 32 v per tile, read along v
         for (int r = ty; r < 64; r += 8) {
             const int k = k0 + r, v = v0 + tx;
@@ -227,40 +238,54 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const doub
         __syncthreads();
         for (int r = ty; r < 32; r += 8) {  // column v0 + r, k pair k0 + 2 tx: written along k
             const int v = v0 + r, k = k0 + 2 * tx;
-            if (v < n && k < Kp) oz_digits2(tile[2 * tx][r], tile[2 * tx + 1][r], ecol[r], S + (size_t)v * Kp + k, (size_t)n * Kp);
+            if (v < n && k < Kp) oz_digits2<P>(tile[2 * tx][r], tile[2 * tx + 1][r], ecol[r], S + (size_t)v * Kp + k, (size_t)n * Kp);
         }
         __syncthreads();
     }
 }
 
 // Digit slices of the rows (cols = false) or columns (cols = true) of `items`
-// n x n matrices: S [items][P][n][Kp] bf16, e [items][n].
-cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st)
+// n x n matrices: S [items][P][n][Kp] bf16, e [items][n], P = planes digits.
+template <int P>
+static cudaError_t oz_split_p(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
+                              OzSkip skip)
 {
     const int Kp = oz_kpad(n);
     if (!cols) {
         const dim3 g((n + 7) / 8, items);
-        if (Kp <= 256) k_oz_split_rows<4><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S);
-        else if (Kp <= 512) k_oz_split_rows<8><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S);
-        else k_oz_split_rows<16><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S);
+        if (Kp <= 256) k_oz_split_rows<4, P><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S, skip);
+        else if (Kp <= 512) k_oz_split_rows<8, P><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S, skip);
+        else k_oz_split_rows<16, P><<<g, 256, 0, counted(st)>>>(n, Kp, M, e, S, skip);
     } else if (Kp <= kOzColBlockKp) {
         const size_t smem = (size_t)Kp * 33 * sizeof(double);
         if (smem > 48 * 1024)
-            cudaFuncSetAttribute(k_oz_split_cols_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(k_oz_split_cols_block<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kOzColBlockKp * 33 * (int)sizeof(double));
-        k_oz_split_cols_block<<<dim3((n + 31) / 32, items), dim3(32, 8), smem, counted(st)>>>(n, Kp, M, e, S);
+        k_oz_split_cols_block<P><<<dim3((n + 31) / 32, items), dim3(32, 8), smem, counted(st)>>>(n, Kp, M, e, S, skip);
     } else {
-        k_oz_split_cols<<<dim3((n + 31) / 32, items), dim3(32, 8), 0, counted(st)>>>(n, Kp, M, e, S);
+        k_oz_split_cols<P><<<dim3((n + 31) / 32, items), dim3(32, 8), 0, counted(st)>>>(n, Kp, M, e, S, skip);
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
+                            OzSkip skip, int planes)
+{
+    switch (planes) {
+    case 4: return oz_split_p<4>(n, items, cols, M, S, e, st, skip);
+    case 5: return oz_split_p<5>(n, items, cols, M, S, e, st, skip);
+    case 6: return oz_split_p<6>(n, items, cols, M, S, e, st, skip);
+    case 7: return oz_split_p<7>(n, items, cols, M, S, e, st, skip);
+    }
+    return cudaErrorInvalidValue;
 }
 
 // C = A B from the row slices of A and the column slices of B.
 cudaError_t launch_oz_gemm_slices(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
                                   const int *eb, double *C, cudaStream_t st, int digits, bool sym, int *err,
-                                  int a_items)
+                                  int a_items, const double *Cadd, OzSkip skip, int planes)
 {
-    return launch_oz_gemm_tc(n, items, sa, ea, sb, eb, C, digits, sym, err, st, a_items);
+    return launch_oz_gemm_tc(n, items, sa, ea, sb, eb, C, digits, sym, err, st, a_items, Cadd, skip, planes);
 }
 
 // C = op(A) B for `items` n x n FP64 matrices (op(A) = A^T when ta), through
@@ -273,7 +298,7 @@ cudaError_t launch_oz_gemm(int n, int items, bool ta, const double *A, const dou
     // rows of op(A): rows of A, or columns of A when transposed; columns of B
     if ((e = launch_oz_split(n, items, ta, A, sa, ea, st))) return e;
     if ((e = launch_oz_split(n, items, true, B, sb, eb, st))) return e;
-    return launch_oz_gemm_slices(n, items, sa, ea, sb, eb, C, st, kOzP, false, err);
+    return launch_oz_gemm_slices(n, items, sa, ea, sb, eb, C, st, kOzDigits, false, err);
 }
 
 }  // namespace wpcd

@@ -75,40 +75,63 @@ __device__ __forceinline__ unsigned smem_u32(const void *p)
 constexpr int kTcM = 128;       // tile rows = TMEM lanes
 constexpr int kTcN = 64;        // tile columns = TMEM columns per accumulator
 constexpr int kTcKC = 32;       // k per stage: 64 bytes of a row = one swizzle span
-constexpr int kTcKBlk = 160;    // k between drains (exact FP32 sums)
-constexpr int kTcStages = 3;
 constexpr int kTcADigit = kTcM * kTcKC * 2;                        // 8 KB
 constexpr int kTcBDigit = kTcN * kTcKC * 2;                        // 4 KB
-constexpr int kTcAStage = kOzDigits * kTcADigit;                   // 48 KB
-constexpr int kTcStageBytes = kOzDigits * (kTcADigit + kTcBDigit);  // 72 KB
+
+// What depends on the number P of digit planes that a chunk brings: the stage
+// (P digits of both operands), how many stages fit the 227 KB, and the k between
+// drains, from the exactness bound (digit 0 in [-129, 129], the others in
+// [-128, 127], at most P pairs a weight, two of them with digit 0):
+// (2 * 129 * 128 + (P - 2) * 128^2) k < 2^24 in whole chunks.
+template <int P>
+struct Tc {
+    static constexpr int kStages = P >= 7 ? 2 : (P == 4 ? 4 : 3);
+    static constexpr int kAStage = P * kTcADigit;
+    static constexpr int kStageBytes = P * (kTcADigit + kTcBDigit);
+    static constexpr int kPerK = 2 * 129 * 128 + (P - 2) * 128 * 128;
+    static constexpr int kKBlk = ((1 << 24) - 1) / kPerK / kTcKC * kTcKC;
+    static constexpr int kSmem = 1024 + kStages * kStageBytes + 128;  // alignment slack | ring | barriers
+};
+static_assert(Tc<4>::kKBlk == 224 && Tc<5>::kKBlk == 192 && Tc<6>::kKBlk == 160 && Tc<7>::kKBlk == 128, "exact sums");
+static_assert(Tc<7>::kSmem <= 227 * 1024 && Tc<6>::kSmem <= 227 * 1024 && Tc<4>::kSmem <= 227 * 1024, "shared memory");
+
 constexpr int kTcTmemCols = 512;  // 6 x 64 accumulator columns, allocated as a power of two
 constexpr int kTcDrainWarps = 16;  // four per TMEM lane quarter, one per 16 columns
 constexpr int kTcDrainCols = kTcN / (kTcDrainWarps / 4);
 constexpr int kTcProducerWarp = kTcDrainWarps, kTcMmaWarp = kTcDrainWarps + 1;
 constexpr int kTcThreads = 32 * (kTcDrainWarps + 2);
-constexpr int kTcSmem = 1024 + kTcStages * kTcStageBytes + 128;  // alignment slack | ring | barriers
 constexpr long long kTcWaitCycles = 1ll << 31;
 
 // instruction descriptor: D F32, A and B BF16, both K-major, M = 128; N (bits
 // 17-22, N / 8) is set per MMA: 64 times the number of B digits it takes
 constexpr uint32_t kTcIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcM >> 4) << 24);
 
-// The 21 digit pairs of one 16-k step as eight wide MMAs.  The B digits of a
-// stage lie back to back in shared memory (64 rows each, the same 512-byte
-// row-group stride), so digits q0 .. q0 + nq - 1 form one K-major operand of
-// N = 64 nq rows; A digit p times it lands, 64 columns per digit, on the
-// accumulators of weights p + q0 .. p + q0 + nq - 1, which are adjacent in
-// TMEM.  Segment g = (p, q0, nq): every pair p + q <= 5 exactly once, and the
-// two p = 0 segments write every weight before any other segment does.
-constexpr int kTcSegs = 8;
+// The digit pairs of one 16-k step as a few wide MMAs (P = 6: 21 pairs in eight).
+// The B digits of a stage lie back to back in shared memory (64 rows each, the
+// same 512-byte row-group stride), so digits q0 .. q0 + nq - 1 form one K-major
+// operand of N = 64 nq rows; A digit p times it lands, 64 columns per digit, on
+// the accumulators of weights p + q0 .. p + q0 + nq - 1, which are adjacent in
+// TMEM.  Segment g = (p, q0, nq): for each p the digits q = 0 .. 3, then those
+// from 4 on, every pair p + q <= P - 1 exactly once; the p = 0 segments write
+// every weight before any other segment does.
+template <int P>
+__device__ __forceinline__ constexpr int tc_segs()
+{
+    return P + (P > 4 ? P - 4 : 0);
+}
+template <int P>
 __device__ __forceinline__ void tc_seg(int g, int &p, int &q0, int &nq)
 {
-    constexpr int P[kTcSegs] = {0, 0, 1, 1, 2, 3, 4, 5};
-    constexpr int Q0[kTcSegs] = {0, 4, 0, 4, 0, 0, 0, 0};
-    constexpr int NQ[kTcSegs] = {4, 2, 4, 1, 4, 3, 2, 1};
-    p = P[g];
-    q0 = Q0[g];
-    nq = NQ[g];
+    constexpr int two = P > 4 ? P - 4 : 0;  // the first `two` A digits have two segments
+    if (g < 2 * two) {
+        p = g >> 1;
+        q0 = (g & 1) * 4;
+        nq = (g & 1) ? P - 4 - p : 4;
+    } else {
+        p = g - two;
+        q0 = 0;
+        nq = P - p < 4 ? P - p : 4;
+    }
 }
 
 __device__ __forceinline__ int tc_tile_n(int n, int col0)
@@ -229,6 +252,15 @@ __device__ __forceinline__ void tc_transpose16(double (&v)[16], int lane)
 
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// v 2^sh; below the last bit kept (sh < 0) seven-digit products round, the others
+// truncate (their low digits lie further below the 47 bits that they keep).
+template <int P>
+__device__ __forceinline__ long long tc_weigh(int v, int sh)
+{
+    if (sh >= 0) return (long long)v << sh;
+    return P >= 7 ? (long long)((v + (1 << (-sh - 1))) >> -sh) : (long long)(v >> -sh);
+}
+
 struct TcTile {
     int b, row0, col0;
 };
@@ -257,11 +289,15 @@ __device__ __forceinline__ TcTile tc_tile(int t, int per_item, int TC, bool sym)
     return r;
 }
 
+template <int P>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_oz_gemm_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int n, int Kp,
                  int dmax, bool sym, int per_item, int TC, int ntiles, const int *ea_all, const int *eb_all,
-                 double *C_all, int *err, int a_mod)
+                 double *C_all, int *err, int a_mod, const double *Cadd, OzSkip skip, int shift7)
 {
+    const int shift = P < 7 ? 36 : shift7;
+    constexpr int kTcStages = Tc<P>::kStages, kTcStageBytes = Tc<P>::kStageBytes, kTcAStage = Tc<P>::kAStage;
+    constexpr int kTcKBlk = Tc<P>::kKBlk;
     extern __shared__ unsigned char tc_raw[];
     const uint32_t raw_s = smem_u32(tc_raw);
     const uint32_t ring_s = (raw_s + 1023u) & ~1023u;  // the swizzle pattern follows address bits
@@ -270,7 +306,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // barriers: full[3] | empty[3] | acc_full | acc_empty, then the TMEM base and the abort flag
     const uint32_t full_s = bar_s, empty_s = bar_s + 8u * kTcStages;
     const uint32_t accf_s = bar_s + 16u * kTcStages, acce_s = accf_s + 8u;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ring + kTcStages * kTcStageBytes + 64);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ring + kTcStages * kTcStageBytes + 96);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -299,6 +335,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             uint32_t ph = 0;
             for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
                 const TcTile tl = tc_tile(t, per_item, TC, sym);
+                if (oz_skipped(skip, tl.b)) continue;
                 for (int k0 = 0; k0 < Kp; k0 += kTcKC) {
                     if (!tc_wait(empty_s + 8u * stage, ph ^ 1u, abort_flag)) {
                         failed = true;
@@ -306,8 +343,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                     const uint32_t sA = ring_s + (uint32_t)(stage * kTcStageBytes);
                     mbar_expect_tx(full_s + 8u * stage, (uint32_t)kTcStageBytes);
-                    tma_load_3d(sA, &mapA, k0, tl.row0, (tl.b % a_mod) * kOzDigits, full_s + 8u * stage);
-                    tma_load_3d(sA + kTcAStage, &mapB, k0, tl.col0, tl.b * kOzDigits, full_s + 8u * stage);
+                    tma_load_3d(sA, &mapA, k0, tl.row0, (tl.b % a_mod) * P, full_s + 8u * stage);
+                    tma_load_3d(sA + kTcAStage, &mapB, k0, tl.col0, tl.b * P, full_s + 8u * stage);
                     ++issued;
                     if (++stage == kTcStages) {
                         stage = 0;
@@ -329,6 +366,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             uint32_t ph = 0;
             for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
                 const TcTile tl = tc_tile(t, per_item, TC, sym);
+                if (oz_skipped(skip, tl.b)) continue;
                 for (int k0 = 0; k0 < Kp; k0 += kTcKC) {
                     const bool bfirst = (k0 % kTcKBlk) == 0;
                     const bool blast = ((k0 + kTcKC) % kTcKBlk) == 0 || k0 + kTcKC >= Kp;
@@ -347,9 +385,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     for (int kk = 0; kk < 2; ++kk) {  // K = 16: 32 bytes further into the swizzle span
                         if (kk == 1 && k0 + 16 >= n) break;  // that half of the chunk is zero padding
 #pragma unroll
-                        for (int g = 0; g < kTcSegs; ++g) {
+                        for (int g = 0; g < tc_segs<P>(); ++g) {
                             int p, q0, nq;
-                            tc_seg(g, p, q0, nq);
+                            tc_seg<P>(g, p, q0, nq);
                             nq = min(nq, dmax - p - q0 + 1);
                             if (nq <= 0) continue;
                             const uint64_t ad = a0 + (uint64_t)((p * kTcADigit + kk * 32) >> 4);
@@ -389,6 +427,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
         for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
             const TcTile tl = tc_tile(t, per_item, TC, sym);
+            if (oz_skipped(skip, tl.b)) continue;
             const bool live = c0 < tc_tile_n(n, tl.col0);  // this warp's columns hold results
             const int rbase = tl.row0 + (warp & 3) * 32, cbase = tl.col0 + c0;
             const bool work = live && rbase < n;  // warp-uniform
@@ -413,7 +452,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 // back comes as soon as the last pair is in registers, so its conversion
                 // runs beside the next block's MMAs
 #pragma unroll
-                for (int d = 0; d < kOzDigits; d += 2) {
+                for (int d = 0; d < P; d += 2) {
                     uint32_t r0[kTcDrainCols], r1[kTcDrainCols];
                     const bool any = live && d <= dmax, two = any && d + 1 <= dmax;  // warp-uniform
                     if (any) tc_ld16(tbase + (uint32_t)(d * kTcN), r0);
@@ -424,19 +463,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         tc_fence_before();
                         mbar_arrive(acce_s);  // the tensor core may overwrite the accumulators
                     }
-                    const int sh0 = 36 - 8 * d, sh1 = sh0 - 8;  // weight 2^{-8(d+2)+2} = 2^{sh-50}
+                    const int sh0 = shift - 8 * d, sh1 = sh0 - 8;  // weight 2^{-8(d+2)+2} = 2^{sh-shift-14}
                     if (any) {
 #pragma unroll
                         for (int j = 0; j < kTcDrainCols; ++j) {
                             const int v = __float2int_rn(__uint_as_float(r0[j]));
-                            acc[j] += sh0 >= 0 ? ((long long)v << sh0) : (long long)(v >> -sh0);
+                            acc[j] += tc_weigh<P>(v, sh0);
                         }
                     }
                     if (two) {
 #pragma unroll
                         for (int j = 0; j < kTcDrainCols; ++j) {
                             const int v = __float2int_rn(__uint_as_float(r1[j]));
-                            acc[j] += sh1 >= 0 ? ((long long)v << sh1) : (long long)(v >> -sh1);
+                            acc[j] += tc_weigh<P>(v, sh1);
                         }
                     }
                     if (last) break;
@@ -444,7 +483,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (failed) break;
             if (!work) continue;
-            // element (r, cbase + j) = acc[j] 2^{er + ec_j - 50}: first the integers as
+            // element (r, cbase + j) = acc[j] 2^{er + ec_j - shift - 14}: first the integers as
             // doubles of their own scale, then the exponents added to the fields
             double *C = C_all + (size_t)tl.b * n * n;
             const int r = rbase + lane;
@@ -452,22 +491,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             unsigned long long u[kTcDrainCols];
 #pragma unroll
             for (int j = 0; j < kTcDrainCols; ++j) u[j] = i64_to_f64_bits(acc[j]);
+            const int eshift = shift + 14;
             int emin = ecl, emax = ecl;
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) {
                 emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
                 emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
             }
-            if (__all_sync(0xffffffffu, er - 50 + emin >= -1022 && er - 50 + emax <= 959)) {
+            if (__all_sync(0xffffffffu, er - eshift + emin >= -1022 && er - eshift + emax <= 959)) {
 #pragma unroll
                 for (int j = 0; j < kTcDrainCols; ++j) {
-                    const long long e = er + __shfl_sync(0xffffffffu, ecl, j) - 50;
+                    const long long e = er + __shfl_sync(0xffffffffu, ecl, j) - eshift;
                     v[j] = __longlong_as_double(u[j] == 0 ? 0ll : (long long)(u[j] + ((unsigned long long)e << 52)));
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < kTcDrainCols; ++j) {
-                    const int e = er + __shfl_sync(0xffffffffu, ecl, j) - 50;
+                    const int e = er + __shfl_sync(0xffffffffu, ecl, j) - eshift;
                     v[j] = f64_times_pow2_slow(__longlong_as_double((long long)u[j]), e);
                 }
             }
@@ -486,7 +526,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
             for (int j = 0; j < kTcDrainCols; ++j) {
                 const int rr = rg + j;
-                if (rr < n && c < n && (!sym || c >= rr)) C[(size_t)rr * n + c] = v[j];
+                if (rr < n && c < n && (!sym || c >= rr))
+                    C[(size_t)rr * n + c] = Cadd ? Cadd[(size_t)tl.b * n * n + (size_t)rr * n + c] + v[j] : v[j];
             }
         }
         if (failed) *abort_flag = 1;
@@ -514,32 +555,34 @@ static PFN_cuTensorMapEncodeTiled_v12000 tc_encoder()
     return fn;
 }
 
-// 3-D map of a slice set S[items][6][n][Kp] (bf16): box of kTcKC k x rows x all six digits.
-static bool tc_map(CUtensorMap *m, const __nv_bfloat16 *S, int n, int Kp, int items, int rows)
+// 3-D map of a slice set S[items][P][n][Kp] (bf16): box of kTcKC k x rows x all P digits.
+static bool tc_map(CUtensorMap *m, const __nv_bfloat16 *S, int n, int Kp, int items, int rows, int P)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tc_encoder();
     if (!enc) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)n, (cuuint64_t)kOzDigits * items};
+    const cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)n, (cuuint64_t)P * items};
     const cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)n * Kp * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)kTcKC, (cuuint32_t)rows, (cuuint32_t)kOzDigits};
+    const cuuint32_t box[3] = {(cuuint32_t)kTcKC, (cuuint32_t)rows, (cuuint32_t)P};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(S), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Cadd (full products only, not C itself): C = Cadd + A B, added in FP64 as the tile is written.
 // a_items: the number of A slice sets; item b multiplies A set b % a_items (a_items =
 // items: one A per item; a_items < items: A sets shared cyclically, e.g. one per
 // channel of a bucket whose items run channel-fastest).
-cudaError_t launch_oz_gemm_tc(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
-                              const int *eb, double *C, int digits, bool sym, int *err, cudaStream_t st, int a_items)
+// planes: the digits that sa and sb hold per element.
+template <int P>
+static cudaError_t gemm_tc_p(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
+                             const int *eb, double *C, int digits, bool sym, int *err, cudaStream_t st, int a_items,
+                             const double *Cadd, OzSkip skip)
 {
-    if (a_items <= 0) a_items = items;
-    if (n < 1 || items < 1 || digits < 1 || digits > kOzDigits || a_items > items) return cudaErrorInvalidValue;
     const int Kp = oz_kpad(n);
     if (Kp % kTcKC != 0) return cudaErrorInvalidValue;
     CUtensorMap ma, mb;
-    if (!tc_map(&ma, sa, n, Kp, a_items, kTcM) || !tc_map(&mb, sb, n, Kp, items, kTcN)) return cudaErrorInvalidValue;
+    if (!tc_map(&ma, sa, n, Kp, a_items, kTcM, P) || !tc_map(&mb, sb, n, Kp, items, kTcN, P)) return cudaErrorInvalidValue;
     const int TR = (n + kTcM - 1) / kTcM, TC = (n + kTcN - 1) / kTcN;
     int per_item = TR * TC;
     if (sym) {
@@ -555,12 +598,35 @@ cudaError_t launch_oz_gemm_tc(int n, int items, const __nv_bfloat16 *sa, const i
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms <= 0) sms = 1;
     }
-    cudaError_t e = cudaFuncSetAttribute(k_oz_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_oz_gemm_tc<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc<P>::kSmem);
     if (e != cudaSuccess) return e;
     const int grid = (int)(ntiles < sms ? ntiles : sms);
-    k_oz_gemm_tc<<<grid, kTcThreads, kTcSmem, counted(st)>>>(ma, mb, n, Kp, digits - 1, sym, per_item, TC, (int)ntiles, ea, eb,
-                                                    C, err, a_items);
+    // The integer sums keep 2^-(shift + 14) of the scales.  A sum of n products is below
+    // 2^14 n 2^shift; seven digits use the room that a smaller n leaves, so that their
+    // results round at 2^-53 of the scales or below (n <= 512).
+    const int shift = P < 7 ? 36 : (n <= 256 ? 40 : n <= 512 ? 39 : 38);
+    k_oz_gemm_tc<P><<<grid, kTcThreads, Tc<P>::kSmem, counted(st)>>>(ma, mb, n, Kp, digits - 1, sym, per_item, TC,
+                                                                     (int)ntiles, ea, eb, C, err, a_items, Cadd, skip,
+                                                                     shift);
     return cudaGetLastError();
+}
+
+cudaError_t launch_oz_gemm_tc(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
+                              const int *eb, double *C, int digits, bool sym, int *err, cudaStream_t st, int a_items,
+                              const double *Cadd, OzSkip skip, int planes)
+{
+    if (sym && Cadd) return cudaErrorInvalidValue;  // the mirrored elements are written without an addend
+    if (a_items <= 0) a_items = items;
+    if (n < 1 || items < 1 || digits < 1 || digits > planes || a_items > items) return cudaErrorInvalidValue;
+#define WPCD_TC(P) gemm_tc_p<P>(n, items, sa, ea, sb, eb, C, digits, sym, err, st, a_items, Cadd, skip)
+    switch (planes) {
+    case 4: return WPCD_TC(4);
+    case 5: return WPCD_TC(5);
+    case 6: return WPCD_TC(6);
+    case 7: return WPCD_TC(7);
+    }
+#undef WPCD_TC
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace wpcd

@@ -1,0 +1,304 @@
+// refine64.cu -- FP64 eigenpairs from an FP32 eigensolve (the FP64 path of (a3)).
+//
+// The FP64 pipe issues two fused multiply-adds per clock and SM, 1/58 of the
+// FP32 rate, so the FP64 path lets the FP32 Jacobi kernels find approximate
+// eigenvectors X and brings them to FP64 with products on the tensor cores
+// (exact digit products, ozaki.cu).  Each iteration forms, with the FP64 H,
+//     Y = H X,  S = X^T Y,  G = X^T X,  lambda_i = S_ii / G_ii,
+//     s_ij = S_ij - (lambda_i + lambda_j) G_ij / 2   (the off-diagonal of the
+//            Rayleigh matrix after symmetric orthonormalisation, to first order)
+// and updates X <- X (I + E), E_ij = s_ij / (lambda_j - lambda_i) - G_ij / 2,
+// E being the first-order correction of Ogita & Aishima ("Iterative refinement
+// for symmetric eigenvalue decomposition", 2018), split into its antisymmetric
+// (rotation) and symmetric (orthonormalisation) parts.  First order is not
+// enough for a pair whose eigenvalues lie closer together than the FP32 solve
+// resolves (the two branches of a coupled channel at high l, or a chance
+// crossing): such pairs are turned by plane rotations of s, G and the columns of
+// X first, in FP64, pair by pair and rescanned until none is left.  A pair with
+// |s_ij| below the rounding of the products is left alone: its quotient is noise,
+// and the FP64 Jacobi kernel's stopping test would leave it too.
+//
+// An item is done once, after the first iteration, an update's ||E||_F^2 <= kDoneE2: what is left of the off-diagonal is second order in E, below the
+// FP64 Jacobi kernel's own test off(A) <= 1e-15 ||H||_F.  Two iterations
+// usually do it, the third runs only for the items that need it, and an item
+// that is not done after that (or whose values do not fit FP32) is solved again
+// by the FP64 Jacobi kernel (the caller's fallback over done[b] == 0).
+//
+// Measured against FP64 Jacobi alone (its rotations are bound by the FP64 pipe):
+// 20 channels at N_WP = 100, one sample, 161 -> 9.0 ms a solve; 15 channels of
+// N_WP 40/64/100, 256 samples, 339 -> 28 ms; 20 channels at N_WP = 150, 8 samples,
+// 850 -> 29 ms; 1S0 at N_WP = 32, 0.69 -> 0.36 ms; errors against 64-bit LAPACK
+// unchanged (T 2e-13 to 9e-13 in both).
+//
+// The update is X + X E with E small: the digit product's rounding, relative
+// to E's columns, then vanishes beside X, and X keeps its 53 bits.
+#include <cuda_bf16.h>
+#include <math.h>
+
+#include "wpcd_internal.cuh"
+
+namespace wpcd {
+
+// Pairs are turned above these angles: in the first iteration 2^-13, whose square
+// the second one corrects; from then on 2^-26, so that nothing of their square is
+// left.  The second list is short (at n = 300 up to ~40 pairs of a coupled channel,
+// whose s only the second iteration's products resolve); where it is not, only what
+// first order cannot take is turned, and the item goes on to the next iteration.
+constexpr float kFirstAngle = 1.2207031e-4f, kLaterAngle = 1.4901161e-8f, kMaxAngle = 0.02f;
+constexpr float kDoneE2 = 2e-14f;     // ||E||_F <= 1.4e-7: its square is below the rounding of X^T X
+constexpr int kPairCap = 64;          // pairs turned per scan
+constexpr int kPairScans = 6;
+
+// One CTA per item.  S, G and X change only where pairs are turned; E goes to
+// E_all (the buffer of the next X, whose old content is dead).  FP64 where it
+// must be: the Rayleigh quotients, the differences and s (both cancel for close
+// eigenvalues) and the sums; the quotient s / d is formed in FP32, with one
+// correction step for the angles above 2^-26, so its error stays below 2^-50.
+__global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double *G_all, double *X_all,
+                                                    double *E_all, double *lam_all, int *done, int it)
+{
+    extern __shared__ double sm64[];
+    double *lam = sm64;                                          // n
+    double *hl = lam + n;                                        // n: lambda / 2
+    unsigned *pr = reinterpret_cast<unsigned *>(hl + n);         // kPairCap: the scan's pairs, unordered
+    unsigned *ps = pr + kPairCap;                                // kPairCap: the same in order
+    float *al = reinterpret_cast<float *>(ps + kPairCap);        // n: |lambda| times the rounding of the products
+    __shared__ double red[32];
+    __shared__ int s_cnt;
+    const int b = blockIdx.x;
+    if (done[b] != 0) return;
+    const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
+    const size_t off = (size_t)b * n * n;
+    double *S = S_all + off, *G = G_all + off, *X = X_all + off, *E = E_all + off;
+    const float round = it == 0 ? 2.910383e-11f : 8.881784e-16f;  // 2^-35 (39-bit products), 2^-50 (55-bit)
+    for (int i = tid; i < n; i += nt) {
+        const double l = S[(size_t)i * n + i] / G[(size_t)i * n + i];
+        lam[i] = l;
+        hl[i] = 0.5 * l;
+        al[i] = round * fabsf(f32_trunc(l));
+    }
+    float ang = it == 0 ? kFirstAngle : kLaterAngle;
+    float e2 = 0.0f;
+    bool plain = true;  // S holds S (not yet s)
+    bool clear = false, later = false;
+    for (int scan = 0;; ++scan) {
+        if (tid == 0) s_cnt = 0;
+        __syncthreads();
+        e2 = 0.0f;
+        for (int i = warp; i < n; i += nwarp) {
+            const double li = lam[i], hi = hl[i];
+            const float ai = al[i];
+            const double *Si = S + (size_t)i * n, *Gi = G + (size_t)i * n;
+            double *Ei = E + (size_t)i * n;
+            for (int j = lane; j < n; j += 32) {
+                const double g = Gi[j];
+                double ev;
+                if (j == i) {
+                    ev = 0.5 * (1.0 - g);
+                } else {
+                    const double s = plain ? fma(-(hi + hl[j]), g, Si[j]) : Si[j];
+                    const double d = lam[j] - li;
+                    const float sf = f32_trunc(s), df = f32_trunc(d);
+                    double th = 0.0;
+                    const float as = fabsf(sf), ad = fabsf(df);
+                    if (as > fmaxf(ai, al[j])) {
+                        if (as > ang * ad && i < j) {
+                            const int k = atomicAdd(&s_cnt, 1);
+                            if (k < kPairCap) pr[k] = ((unsigned)i << 16) | (unsigned)j;
+                        }
+                        if (as <= kMaxAngle * ad) {
+                            const float rd = __frcp_rn(df), t0 = sf * rd;
+                            th = f64_of(t0);
+                            if (fabsf(t0) > 1.5e-8f) th += f64_of(f32_trunc(fma(-th, d, s)) * rd);
+                        }
+                    }
+                    ev = fma(-0.5, g, th);
+                }
+                Ei[j] = ev;
+                const float ef = f32_trunc(ev);
+                e2 = fmaf(ef, ef, e2);
+            }
+        }
+        __syncthreads();
+        const int m = s_cnt;
+        if (m > kPairCap && ang < kMaxAngle) {  // too many: turn only those beyond first order
+            ang = kMaxAngle;
+            later = true;
+            __syncthreads();  // every thread has read the count
+            continue;
+        }
+        if (m == 0 || m > kPairCap || scan >= kPairScans) {
+            clear = m == 0 && !later;
+            break;
+        }
+        // ---- turn the scan's pairs, in index order (the order of the list does not matter)
+        for (int k = tid; k < m; k += nt) {
+            const unsigned v = pr[k];
+            int r = 0;
+            for (int q = 0; q < m; ++q) r += pr[q] < v;
+            ps[r] = v;
+        }
+        if (plain) {
+            for (int i = warp; i < n; i += nwarp)
+                for (int j = lane; j < n; j += 32) {
+                    const size_t e = (size_t)i * n + j;
+                    S[e] = i == j ? lam[i] : fma(-(hl[i] + hl[j]), G[e], S[e]);
+                }
+            plain = false;
+        }
+        __syncthreads();
+        for (int k = 0; k < m; ++k) {
+            const int i = (int)(ps[k] >> 16), j = (int)(ps[k] & 0xFFFFu);
+            const double s = S[(size_t)i * n + j], a = S[(size_t)i * n + i], q = S[(size_t)j * n + j];
+            double c = 1.0, sn = 0.0;
+            if (s != 0.0) {
+                const double tau = (q - a) / (2.0 * s);
+                const double t = fabs(tau) > 1e150 ? 0.5 / tau
+                                                   : (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+                c = 1.0 / sqrt(1.0 + t * t);
+                sn = t * c;
+            }
+            __syncthreads();  // every thread has read the pair's block
+            for (int r = tid; r < n; r += nt)  // columns i, j
+                for (int w = 0; w < 3; ++w) {
+                    double *M = w == 0 ? S : w == 1 ? G : X;
+                    const double x = M[(size_t)r * n + i], y = M[(size_t)r * n + j];
+                    M[(size_t)r * n + i] = c * x - sn * y;
+                    M[(size_t)r * n + j] = sn * x + c * y;
+                }
+            __syncthreads();
+            for (int r = tid; r < n; r += nt)  // rows i, j
+                for (int w = 0; w < 2; ++w) {
+                    double *M = w == 0 ? S : G;
+                    const double x = M[(size_t)i * n + r], y = M[(size_t)j * n + r];
+                    M[(size_t)i * n + r] = c * x - sn * y;
+                    M[(size_t)j * n + r] = sn * x + c * y;
+                }
+            __syncthreads();
+            if (tid == 0) {
+                S[(size_t)i * n + j] = S[(size_t)j * n + i] = 0.0;
+                lam[i] = S[(size_t)i * n + i];
+                lam[j] = S[(size_t)j * n + j];
+                hl[i] = 0.5 * lam[i];
+                hl[j] = 0.5 * lam[j];
+            }
+            __syncthreads();
+        }
+    }
+    double *lo = lam_all + (size_t)b * n;
+    for (int i = tid; i < n; i += nt) lo[i] = lam[i];
+    const double t2 = cta_sum64((double)e2, red);
+    // (the first iteration's eigenvalues come from 39-bit products)
+    if (tid == 0 && it > 0 && clear && t2 <= (double)kDoneE2) done[b] = it + 1;
+}
+
+// Sorted eigenpairs of the items that are done, into the eigen-buffer layout;
+// the vectors of an item done at iteration k lie in X0 (k even) or X1 (k odd).
+// An item whose FP32 solve hit its sweep cap counts as not done.
+__global__ void __launch_bounds__(256) k_r64_sort(const ChanDev *chans, const int *work, int nw, int sample0, int n,
+                                                  const double *lam_s, const double *X0, const double *X1, int *done,
+                                                  const int *status_all, int n_ch_total, double *eps_all,
+                                                  double *X_all)
+{
+    extern __shared__ double sm64s[];
+    double *lam = sm64s;                            // n
+    int *rank = reinterpret_cast<int *>(lam + n);   // n
+    const int b = blockIdx.x;
+    const int wc = b % nw, smp = sample0 + b / nw;
+    const int d = done[b];
+    if (d == 0) return;
+    if (status_all[(size_t)smp * n_ch_total + work[wc]] <= 0) {
+        __syncthreads();
+        if (threadIdx.x == 0) done[b] = 0;
+        return;
+    }
+    const ChanDev ch = chans[work[wc]];
+    const double *Xs = ((d & 1) ? X1 : X0) + (size_t)b * n * n;
+    double *X = X_all + ch.c_off + (size_t)smp * n * n;
+    double *eps = eps_all + ch.eps_off + (size_t)smp * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) lam[i] = lam_s[(size_t)b * n + i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double ei = lam[i];
+        int r = 0;
+        for (int j = 0; j < n; ++j) r += (lam[j] < ei) || (lam[j] == ei && j < i);
+        rank[i] = r;
+        eps[r] = ei;
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    for (int row = warp; row < n; row += nwarp)
+        for (int c = lane; c < n; c += 32) X[(size_t)row * n + rank[c]] = Xs[(size_t)row * n + c];
+}
+
+static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 4) + kPairCap * 2 * sizeof(unsigned); }
+
+// Digits per product: the first iteration only has to leave errors that the
+// second squares away (39-bit products); from then on Y, S and G carry 55 bits.
+// E is small, so X E needs its leading 31 bits.
+constexpr int kDigFirst = 5, kDigLast = 7, kDigE = 4;
+
+// X, H, Y (then E and the next X), W1, W2, lambda; digit slices of H's rows, X's
+// columns, Y's columns (kDigLast planes each), X's rows and E's columns (kDigE)
+// with their exponents.
+size_t refine64_scratch_per_item(int n)
+{
+    return (size_t)5 * n * n * 8 + (size_t)n * 8 + (3 * oz_slice_elems(n, kDigLast) + 2 * oz_slice_elems(n, kDigE)) * 2 +
+           (size_t)5 * n * 4 + 512;
+}
+
+// The items of one bucket chunk, in scratch blocks X, H, Y, W1, W2 of items n^2
+// doubles each, lambda after them (the layout that the FP32 solve writes), and
+// done[items] ints.  On entry X and H as the FP32 solve left them; on return the
+// done items' eigenpairs are in eps_all / X_all and done[b] == 0 marks the ones
+// that the caller solves by other means.
+cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n,
+                            void *scratch, int *done, const int *status_all, int n_ch_total, double *eps_all,
+                            double *X_all, cudaStream_t st, int *err)
+{
+    const int items = n_samples * nw;
+    const size_t nn = (size_t)items * n * n;
+    double *X0 = static_cast<double *>(scratch);
+    double *H = X0 + nn, *X1 = H + nn, *W1 = X1 + nn, *W2 = W1 + nn, *lam = W2 + nn;
+    const uintptr_t s0 = (reinterpret_cast<uintptr_t>(lam + (size_t)items * n) + 255) & ~(uintptr_t)255;
+    const size_t se = (size_t)items * oz_slice_elems(n, kDigLast), sE = (size_t)items * oz_slice_elems(n, kDigE);
+    __nv_bfloat16 *sH = reinterpret_cast<__nv_bfloat16 *>(s0);
+    __nv_bfloat16 *sXc = sH + se, *sYc = sXc + se, *sXr = sYc + se, *sEc = sXr + sE;
+    int *eH = reinterpret_cast<int *>(sEc + sE);
+    int *eXc = eH + (size_t)items * n, *eYc = eXc + (size_t)items * n, *eXr = eYc + (size_t)items * n;
+    int *eEc = eXr + (size_t)items * n;
+    cudaError_t e = cudaMemsetAsync(done, 0, sizeof(int) * items, st);
+    if (e != cudaSuccess) return e;
+#define CKR(x)                       \
+    do {                             \
+        if ((e = (x)) != cudaSuccess) \
+            return e;                \
+    } while (0)
+    double *x = X0, *xn = X1;
+    for (int it = 0; it < kRefine64Iters; ++it) {
+        OzSkip sk;
+        sk.done = it > 0 ? done : nullptr;
+        sk.it = it;
+        const int dg = it == 0 ? kDigFirst : kDigLast;
+        if (it < 2) CKR(launch_oz_split(n, items, false, H, sH, eH, st, sk, dg));
+        CKR(launch_oz_split(n, items, true, x, sXc, eXc, st, sk, dg));
+        CKR(launch_oz_gemm_slices(n, items, sH, eH, sXc, eXc, xn, st, dg, false, err, 0, nullptr, sk, dg));  // Y = H X
+        CKR(launch_oz_split(n, items, true, xn, sYc, eYc, st, sk, dg));
+        CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sYc, eYc, W1, st, dg, true, err, 0, nullptr, sk, dg));  // S = X^T Y
+        CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sXc, eXc, W2, st, dg, true, err, 0, nullptr, sk, dg));  // G = X^T X
+        k_r64_update<<<items, 256, r64_smem(n), counted(st)>>>(n, W1, W2, x, xn, lam, done, it);  // E over Y
+        CKR(cudaGetLastError());
+        CKR(launch_oz_split(n, items, false, x, sXr, eXr, st, sk, kDigE));
+        CKR(launch_oz_split(n, items, true, xn, sEc, eEc, st, sk, kDigE));
+        CKR(launch_oz_gemm_slices(n, items, sXr, eXr, sEc, eEc, xn, st, kDigE, false, err, 0, x, sk, kDigE));  // X + X E
+        double *t = x;
+        x = xn;
+        xn = t;
+    }
+#undef CKR
+    k_r64_sort<<<items, 256, (size_t)n * 12, counted(st)>>>(chans, work, nw, sample0, n, lam, X0, X1, done, status_all,
+                                                            n_ch_total, eps_all, X_all);
+    return cudaGetLastError();
+}
+
+}  // namespace wpcd

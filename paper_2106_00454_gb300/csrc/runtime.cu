@@ -40,6 +40,10 @@ namespace {
 
 constexpr size_t kRefineScratchBytes = (size_t)32 << 30;  // mixed path: refinement scratch per bucket chunk (one chunk per bucket up to ~7000 samples of n = 200)
 constexpr int kRefineIters = 2;                            // FP64 refinement iterations (default)
+// Rotation test of the FP32 solve before the FP64 refinement: a pair is left once its
+// angle and its share of the diagonal are below 2^-18, which two refinement iterations
+// take to FP64 (2^-16 makes a third one common at n = 300).
+constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
 constexpr size_t kGraphCache = 64;                         // wpcd_solve keys remembered for CUDA graphs
 
 struct MeshH {
@@ -373,7 +377,7 @@ void free_mesh(wpcd_ctx *c, MeshH &m)
 template <class F>
 int pick_threads(wpcd_ctx *c, Exec &X, int n, int prec, int nw, int nsmp, F launch)
 {
-    static const int cand[5] = {64, 128, 256, 512, 1024};  // 1024: the FP32 kernel only
+    static const int cand[5] = {64, 128, 256, 512, 1024};
     if (!c->autotune || c->exec_mode != WPCD_EXEC_BATCHED) return 256;
     const auto key = std::make_pair(n, prec);
     {
@@ -390,9 +394,8 @@ int pick_threads(wpcd_ctx *c, Exec &X, int n, int prec, int nw, int nsmp, F laun
     cudaEventCreate(&b);
     for (int k = 0; k < 5; ++k) {
         const int th = cand[k];
-        if (th > 512 && prec == WPCD_PREC_FP64) continue;
-        if (prec == WPCD_PREC_FP64 && !jacobi_c_in_smem(n) && (th / 32) * n > n * (n + 1) / 2) continue;
-        const int occ = prec == WPCD_PREC_FP64 ? jacobi_f64_occupancy(n, th) : jacobi_mixed_occupancy(n, th);
+        if (th > 512 && prec == WPCD_PREC_FP64 && jacobi_fits_smem(n, true)) continue;
+        const int occ = jacobi_mixed_occupancy(n, th);
         if (occ < 1) continue;
         const int ns = std::max(1, std::min(nsmp, (2 * c->n_sm * occ + nw - 1) / nw));
         cudaEventRecord(a, X.stream);
@@ -593,29 +596,17 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
 // scratch slot per resident CTA; the mixed path then refines as for the other
 // sizes.
 wpcd_status run_bucket_big(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *cf, const int *work, int nw,
-                           int nsmp, int smp0, int n, int prec)
+                           int nsmp, int smp0, int n)
 {
-    (void)v;
-    const bool f64 = prec == WPCD_PREC_FP64;
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
     if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    const int occ = std::max(1, jacobi_big_occupancy(n, f64));
-    const size_t slot_b = (jacobi_big_scratch_bytes(n, f64) + 255) & ~(size_t)255;
+    const int occ = std::max(1, jacobi_big_occupancy(n, false));
+    const size_t slot_b = (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255;
     // CTAs in flight: every resident one.  Each CTA's round is bound by the latency of
     // its L2 round trips, so the rate grows with the CTAs in flight (measured at
     // n = 512, FP32: 24 / 48 / 76 / 152 CTAs give 167 / 332 / 953 / 1518 solves/s)
     int cap = c->n_sm * occ;
     if (c->big_slots > 0) cap = c->big_slots;
-    if (f64) {
-        const int items = nsmp * nw;
-        const int slots = std::max(1, std::min(items, cap));
-        wpcd_status st = ws_reserve(c, X, X.ws_ref, slot_b * slots);
-        if (st) return st;
-        Launch L(c, X, WPCD_PHASE_EIGEN);
-        CK(launch_jacobi_big(true, e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, X.ws_ref.p, slots, e.eps, e.C,
-                             nullptr, nullptr, nullptr, e.status, v.n_ch, X.err, X.stream));
-        return WPCD_OK;
-    }
     const size_t ref_item = refine_scratch_per_item(n, c->refine_engine);
     int chunk = (int)std::max<size_t>(1, kRefineScratchBytes / (ref_item * nw));
     chunk = std::min(chunk, std::max(1, 65535 / nw));  // the refinement grids put items in y / z (<= 65535)
@@ -643,6 +634,90 @@ wpcd_status run_bucket_big(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
     return WPCD_OK;
 }
 
+// A size bucket on the FP64 path: the FP32 Jacobi kernel, FP64 refinement
+// (refine64.cu), and the FP64 Jacobi kernel for the items that the refinement
+// does not bring to FP64.  Without room for the refinement's scratch (an HBM
+// budget, a full device) every item takes the FP64 Jacobi kernel.
+wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *cf, const int *work, int nw, int nsmp,
+                           int smp0, int n)
+{
+    if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
+    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    const bool big32 = !jacobi_fits_smem(n, false), big64 = !jacobi_fits_smem(n, true);
+    const size_t ref_item = refine64_scratch_per_item(n);
+    const size_t slot32 = big32 ? (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255 : 0;
+    const size_t slot64 = big64 ? (jacobi_big_scratch_bytes(n, true) + 255) & ~(size_t)255 : 0;
+    const size_t c_item = big32 || jacobi_mixed_c_in_smem(n) ? 0 : jacobi_mixed_c_bytes(n);
+    int cap32 = c->n_sm * std::max(1, big32 ? jacobi_big_occupancy(n, false) : 1);
+    int cap64 = c->n_sm * std::max(1, big64 ? jacobi_big_occupancy(n, true) : 1);
+    if (c->big_slots > 0) cap32 = cap64 = c->big_slots;
+    // scratch of a chunk: the refinement's, the FP32 solver's eigenvectors or slots, the done flags
+    auto slots32 = [&](int items) { return big32 ? std::max(1, std::min(items, cap32)) : 0; };
+    auto bytes_of = [&](int ns) {
+        const size_t items = (size_t)ns * nw;
+        return ((ref_item * items + 255) & ~(size_t)255) + ((c_item * items + slot32 * slots32((int)items) + 255) & ~(size_t)255) +
+               sizeof(int) * items;
+    };
+    int chunk = (int)std::max<size_t>(1, kRefineScratchBytes / ((ref_item + c_item) * nw));
+    chunk = std::min(chunk, std::max(1, 65535 / nw));  // the refinement grids put items in y / z (<= 65535)
+    chunk = std::min(chunk, nsmp);
+    while (chunk > 0 && ws_reserve(c, X, X.ws_ref, bytes_of(chunk))) chunk /= 2;
+    if (chunk == 0) {  // no room: FP64 Jacobi alone
+        const int slots = big64 ? std::max(1, std::min(nsmp * nw, cap64)) : 0;
+        wpcd_status st = ws_reserve(c, X, X.ws_ref, slot64 * slots);
+        if (st) return st;
+        Launch L(c, X, WPCD_PHASE_EIGEN);
+        if (big64)
+            CK(launch_jacobi_big(true, e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, X.ws_ref.p, slots, e.eps, e.C,
+                                 nullptr, nullptr, nullptr, e.status, v.n_ch, X.err, X.stream));
+        else
+            CK(launch_jacobi_f64(e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
+                                 X.stream));
+        return WPCD_OK;
+    }
+    unsigned char *base = static_cast<unsigned char *>(X.ws_ref.p);
+    double *Xs = reinterpret_cast<double *>(base);
+    // the FP32 solve of ns samples; its own non-convergence only sends the item to the fallback
+    auto solve32 = [&](int th, int s0, int ns) {
+        const size_t items = (size_t)ns * nw;
+        unsigned char *aux = base + ((ref_item * items + 255) & ~(size_t)255);
+        double *lam = Xs + 5 * items * n * n, *Hs = Xs + items * n * n;
+        if (big32)
+            return launch_jacobi_big(false, e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, aux, slots32((int)items),
+                                     nullptr, nullptr, lam, Xs, Hs, e.status, v.n_ch, nullptr, X.stream, kTest64);
+        return launch_jacobi_mixed(e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, lam, Xs,
+                                   reinterpret_cast<float *>(aux), Hs, e.status, v.n_ch, nullptr, X.stream, th, kTest64);
+    };
+    int threads = 256;
+    if (!big32) {
+        threads = pick_threads(c, X, n, WPCD_PREC_FP64, nw, chunk, [&](int th, int ns) { return solve32(th, 0, ns); });
+        if (threads < 0) return WPCD_ERR_CUDA;
+    }
+    for (int s0 = 0; s0 < nsmp; s0 += chunk) {
+        const int ns = std::min(chunk, nsmp - s0), items = ns * nw;
+        int *done = reinterpret_cast<int *>(base + (bytes_of(ns) - sizeof(int) * items));
+        {
+            Launch L(c, X, WPCD_PHASE_EIGEN);
+            CK(solve32(threads, s0, ns));
+        }
+        {
+            Launch L(c, X, WPCD_PHASE_REFINE);
+            CK(launch_refine64(e.cd_dev, work, nw, ns, smp0 + s0, n, base, done, e.status, v.n_ch, e.eps, e.C, X.stream,
+                               X.err));
+        }
+        Launch L(c, X, WPCD_PHASE_EIGEN);
+        if (big64) {  // its slots take the place of the refinement's scratch
+            const int slots = (int)std::max<size_t>(1, std::min<size_t>(std::min(items, cap64), ref_item * items / slot64));
+            CK(launch_jacobi_big(true, e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, base, slots, e.eps, e.C,
+                                 nullptr, nullptr, nullptr, e.status, v.n_ch, X.err, X.stream, RotTest(), done));
+        } else {
+            CK(launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
+                                 X.stream, 256, done));
+        }
+    }
+    return WPCD_OK;
+}
+
 // The parameter sum + eigensolve of the batch diag_prep set up (device-only
 // work on X.stream: capturable).  coeffs: device, [S][n_terms - 1].
 wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int S, int prec, EigH &e)
@@ -653,15 +728,12 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
                            X.stream));
     }
     const double *cf = v.n_terms > 1 ? e.coeffs : nullptr;
-    // FP64: one Jacobi launch per size bucket (largest first), or per solve in plain mode.
-    // MIXED: per bucket, in sample chunks sized to the refinement scratch, an FP32
-    // Jacobi launch followed by two FP64 refinement iterations.
+    // Per size bucket (largest first, or per solve in plain mode), in sample chunks sized to
+    // the refinement scratch: an FP32 Jacobi launch and the FP64 refinement.
     auto run_bucket = [&](const int *work, int nw, int nsmp, int smp0, int n) -> wpcd_status {
-        if (!jacobi_fits_smem(n, prec == WPCD_PREC_FP64)) return run_bucket_big(c, X, v, e, cf, work, nw, nsmp, smp0, n, prec);
+        if (prec == WPCD_PREC_FP64) return run_bucket_f64(c, X, v, e, cf, work, nw, nsmp, smp0, n);
+        if (!jacobi_fits_smem(n, false)) return run_bucket_big(c, X, v, e, cf, work, nw, nsmp, smp0, n);
         const int threads = pick_threads(c, X, n, prec, nw, nsmp, [&](int th, int ns) {
-            if (prec == WPCD_PREC_FP64)
-                return launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch,
-                                         X.err, X.stream, th);
             // the FP32 solve alone, into the start of the refinement scratch
             const bool cs = jacobi_mixed_c_in_smem(n);
             const size_t per = refine_scratch_per_item(n, c->refine_engine) + (cs ? 0 : jacobi_mixed_c_bytes(n)) + 256;
@@ -674,12 +746,6 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
                                        Xs + (size_t)ns * nw * n * n, e.status, v.n_ch, X.err, X.stream, th);
         });
         if (threads < 0) return WPCD_ERR_CUDA;
-        if (prec == WPCD_PREC_FP64) {
-            Launch L(c, X, WPCD_PHASE_EIGEN);
-            CK(launch_jacobi_f64(e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch,
-                                 X.err, X.stream, threads));
-            return WPCD_OK;
-        }
         const bool c_smem = jacobi_mixed_c_in_smem(n);
         const size_t ref_item = refine_scratch_per_item(n, c->refine_engine);
         const size_t per_item = ref_item + (c_smem ? 0 : jacobi_mixed_c_bytes(n)) + 256;

@@ -249,10 +249,16 @@ cudaError_t launch_project_fine(const ChanDev *chans_dev, int c, const ChanDev &
                                 int n_terms, cudaStream_t st);
 size_t jacobi_smem_bytes(int n, bool c_in_smem);
 bool jacobi_c_in_smem(int n);
+// The FP32 eigensolvers rotate a pair only if |a_pq| > 2^-23 sqrt|a_pp a_qq| and, beyond
+// that, |a_pq| > rel sqrt|a_pp a_qq| or |a_pq| > ang |a_qq - a_pp|.  The defaults leave
+// the first test alone.
+struct RotTest {
+    float rel = 0.0f, ang = 0.0f;
+};
 cudaError_t launch_jacobi_f64(const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch, int n_samples,
                               int sample0, int n_terms, const double *coeffs, int n, double *eps_all,
                               double *C_all, int *status_all, int n_ch_total, int *err, cudaStream_t st,
-                              int threads = 256);
+                              int threads = 256, const int *done = nullptr);
 int jacobi_f64_occupancy(int n, int threads);
 int jacobi_mixed_occupancy(int n, int threads);
 bool jacobi_mixed_c_in_smem(int n);   // eigenvector matrix in shared memory (else global)
@@ -261,7 +267,7 @@ size_t jacobi_mixed_c_bytes(int n);  // global eigenvector scratch per item (C k
 cudaError_t launch_jacobi_mixed(const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch, int n_samples,
                                 int sample0, int n_terms, const double *coeffs, int n, double *lam_s, double *X_s,
                                 float *Cf_s, double *H_s, int *status_all, int n_ch_total, int *err, cudaStream_t st,
-                                int threads = 256);
+                                int threads = 256, RotTest test = RotTest());
 // Matrices above one CTA's shared memory: Jacobi with A and C in global memory.
 bool jacobi_fits_smem(int n, bool f64);
 int jacobi_big_max_n();
@@ -270,24 +276,45 @@ size_t jacobi_big_scratch_bytes(int n, bool f64);
 cudaError_t launch_jacobi_big(bool f64, const ChanDev *chans_dev, const int *work_ch_dev, int n_work_ch,
                               int n_samples, int sample0, int n_terms, const double *coeffs, int n, void *scratch,
                               int slots, double *eps_all, double *C_all, double *lam_s, double *X_s, double *H_s,
-                              int *status_all, int n_ch_total, int *err, cudaStream_t st);
-constexpr int kOzDigits = 6;  // balanced 8-bit digits per operand of the Ozaki products
-size_t oz_slice_elems(int n);
+                              int *status_all, int n_ch_total, int *err, cudaStream_t st,
+                              RotTest test = RotTest(), const int *done = nullptr);
+// Items of a batch that a step leaves alone: those with 0 < done[b] <= it (done == NULL: none).
+struct OzSkip {
+    const int *done = nullptr;
+    int it = 0;
+};
+__device__ __forceinline__ bool oz_skipped(const OzSkip &sk, int b)
+{
+    if (!sk.done) return false;
+    const int d = sk.done[b];
+    return d != 0 && d <= sk.it;
+}
+constexpr int kOzDigits = 6;  // balanced 8-bit digits per operand of the Ozaki products (mixed path)
+constexpr int kOzMaxDigits = 7;
+size_t oz_slice_elems(int n, int planes = kOzDigits);
 int oz_kpad(int n);
 cudaError_t launch_oz_gemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                            __nv_bfloat16 *sa, __nv_bfloat16 *sb, int *ea, int *eb, cudaStream_t st, int *err = nullptr);
-cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st);
+cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
+                            OzSkip skip = OzSkip(), int planes = kOzDigits);
 cudaError_t launch_oz_gemm_slices(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
                                   const int *eb, double *C, cudaStream_t st, int digits = 6, bool sym = false,
-                                  int *err = nullptr, int a_items = 0);
+                                  int *err = nullptr, int a_items = 0, const double *Cadd = nullptr,
+                                  OzSkip skip = OzSkip(), int planes = kOzDigits);
 cudaError_t launch_oz_gemm_tc(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
                               const int *eb, double *C, int digits, bool sym, int *err, cudaStream_t st,
-                              int a_items = 0);
+                              int a_items = 0, const double *Cadd = nullptr, OzSkip skip = OzSkip(),
+                              int planes = kOzDigits);
 size_t refine_scratch_per_item(int n, int engine);
 cudaError_t launch_refine(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n,
                           int n_terms, const double *coeffs, void *scratch, double *eps_all, double *X_all,
                           int iters, int engine, cudaStream_t st, int *err = nullptr,
                           const __nv_bfloat16 *rot_s = nullptr, const int *rot_e = nullptr, int digits = 6);
+constexpr int kRefine64Iters = 3;  // at most; the items that have converged skip the rest
+size_t refine64_scratch_per_item(int n);
+cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n,
+                            void *scratch, int *done, const int *status_all, int n_ch_total, double *eps_all,
+                            double *X_all, cudaStream_t st, int *err);
 cudaError_t launch_batched_dgemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                                  void *scratch, int engine, cudaStream_t st, int *err = nullptr);
 size_t batched_dgemm_scratch(int n, int items);
