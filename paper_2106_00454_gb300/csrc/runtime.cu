@@ -1595,7 +1595,13 @@ double cg_racah(int j1, int m1, int j2, int m2, int J, int M)
     if (m1 + m2 != M || std::abs(m1) > j1 || std::abs(m2) > j2 || std::abs(M) > J || J < std::abs(j1 - j2) ||
         J > j1 + j2)
         return 0.0;
-    auto lf = [](int n) { return std::lgamma((double)n + 1.0); };
+    // ln n! for every argument that J <= kMaxJ gives (J + j1 + j2 + 1 <= 3 kMaxJ)
+    static const std::vector<double> tab = [] {
+        std::vector<double> t(4 * kMaxJ + 8);
+        for (size_t n = 0; n < t.size(); ++n) t[n] = std::lgamma((double)n + 1.0);
+        return t;
+    }();
+    auto lf = [](int n) { return tab[(size_t)n]; };
     const double pre = 0.5 * (std::log(2.0 * J + 1.0) + lf(J + j1 - j2) + lf(J - j1 + j2) + lf(j1 + j2 - J) -
                               lf(j1 + j2 + J + 1) + lf(J + M) + lf(J - M) + lf(j1 - m1) + lf(j1 + m1) + lf(j2 - m2) +
                               lf(j2 + m2));
@@ -1617,6 +1623,7 @@ wpcd_status wpcd_saclay(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, con
         (!abcde && !dsig))
         return WPCD_ERR_ARG;
     std::vector<SacChanDev> tab(n_ch);
+    int Lmax = 0;
     for (int k = 0; k < n_ch; ++k) {
         const wpcd_channel &ch = channels[k];
         if (ch.J < 0 || ch.J > kMaxJ || (ch.s != 0 && ch.s != 1)) return WPCD_ERR_ARG;
@@ -1630,15 +1637,21 @@ wpcd_status wpcd_saclay(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, con
         d.K = ch.coupled ? 2 : 1;
         d.l[0] = ch.coupled ? ch.J - 1 : ch.l;
         d.l[1] = ch.coupled ? ch.J + 1 : ch.l;
+        if (ch.tz != 0) continue;  // not part of the np sum
+        bool any = false;
+        // (m', m) of M_ss | M_11, M_1-1, M_10, M_01, M_00
+        static const int mm[6][2] = {{0, 0}, {1, 1}, {1, -1}, {1, 0}, {0, 1}, {0, 0}};
         for (int ip = 0; ip < d.K; ++ip)
             for (int il = 0; il < d.K; ++il)
-                for (int mp = -ch.s; mp <= ch.s; ++mp)
-                    for (int m = -ch.s; m <= ch.s; ++m) {
-                        const int lp = d.l[ip], l = d.l[il];
-                        d.tab[((ip * 2 + il) * 3 + mp + 1) * 3 + m + 1] =
-                            std::sqrt(4.0 * kPi) * std::sqrt(2.0 * l + 1.0) *
-                            cg_racah(lp, m - mp, ch.s, mp, ch.J, m) * cg_racah(l, 0, ch.s, m, ch.J, m);
-                    }
+                for (int f = ch.s; f < (ch.s ? 6 : 1); ++f) {
+                    const int lp = d.l[ip], l = d.l[il], mp = mm[f][0], m = mm[f][1];
+                    const double w = std::sqrt(4.0 * kPi) * std::sqrt(2.0 * l + 1.0) *
+                                     cg_racah(lp, m - mp, ch.s, mp, ch.J, m) * cg_racah(l, 0, ch.s, m, ch.J, m);
+                    d.w[ip * 2 + il][f] = m - mp == -1 ? -w : w;
+                    any |= w != 0.0;
+                }
+        if (any) Lmax = std::max(Lmax, d.l[d.K - 1]);
+        else d.tz = 1;  // an l that J and s do not couple to: no contribution
     }
     std::lock_guard<std::mutex> lk(c->mu);
     CK(cudaSetDevice(c->device));
@@ -1648,7 +1661,7 @@ wpcd_status wpcd_saclay(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, con
     CK(cudaMemcpyAsync(X.ws_in.p, tab.data(), sizeof(SacChanDev) * n_ch, cudaMemcpyHostToDevice, X.stream));
     Launch L(c, X, WPCD_PHASE_OBSERVABLES);
     CK(launch_saclay(static_cast<SacChanDev *>(X.ws_in.p), n_ch, S, n_E, e_lab, delta, n_theta, theta, abcde, dsig,
-                     X.stream));
+                     Lmax, X.stream));
     CK(cudaStreamSynchronize(X.stream));  // the channel table lives in a reusable workspace
     return WPCD_OK;
 }

@@ -61,13 +61,14 @@ struct MiChanDev {
     long long vg_off, von_off;
 };
 
-// Channel of the spin-observable kernel: spin, J, T_z, K, its l values and the
-// coupling products sqrt(4 pi) sqrt(2l+1) C(l' (m-m') s m' | J m) C(l 0 s m | J m)
-// at tab[((l' block * 2 + l block) * 3 + m' + 1) * 3 + m + 1].
+// Channel of the spin-observable kernel: spin, J, T_z, K, its l values and, per
+// (l' block, l block), the coupling product sqrt(4 pi) sqrt(2l+1) C(l' (m-m') s m' | J m)
+// C(l 0 s m | J m) of each of the six functions M_ss, M_11, M_1-1, M_10, M_01, M_00
+// (those with m - m' < 0 with the sign of Y_l^{-mu} = (-1)^mu Y_l^mu).
 struct SacChanDev {
     int s, J, tz, K;
     int l[2];
-    double tab[36];
+    double w[4][6];
 };
 
 struct ChanDev {
@@ -324,7 +325,7 @@ cudaError_t launch_tbin(const ChanDev *chans_dev, int n_ch, int n_samples, int n
                         const double *eps_all, const double *C_all, PlanDev plan, int maxN, int n_E, double *tout,
                         double *phout, int *err, cudaStream_t st, bool vc_identity, int mode);
 cudaError_t launch_saclay(const SacChanDev *chans_dev, int n_ch, int n_samples, int n_E, const double *e_lab,
-                          const double *delta, int n_th, const double *theta, double *abcde, double *dsig,
+                          const double *delta, int n_th, const double *theta, double *abcde, double *dsig, int Lmax,
                           cudaStream_t st);
 constexpr int kMiMaxNQ = 100;  // MI grid points per l-block: 2 (N_Q + 1) rows fit one CTA's shared memory in FP32
 cudaError_t launch_mi_grid(int NQ, double cmap, const double *glx, const double *glw, double *k, double *w,
