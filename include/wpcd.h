@@ -342,9 +342,11 @@ wpcd_status wpcd_mi_prepare(wpcd_ctx *ctx, const wpcd_channel *channels, int n_c
  * channel, then interpolate the phase shifts linearly in T_lab to the requested
  * energies e_lab_dev [n_E] (the end segments extended; delta moved by
  * multiples of 180 deg to within 90 deg of the segment start) and form the np
- * total cross section as wpcd_observables does.  Each system is factorised in
- * FP32 (partial pivoting) and its solution refined with FP64 residuals until
- * it converges (below).  Outputs (device, any may be
+ * total cross section as wpcd_observables does.  Each system is solved in FP32
+ * -- by its own factorisation (partial pivoting), or, for many systems at four
+ * energies and more, through one eigendecomposition of the grid problem per
+ * (sample, channel) that inverts every energy -- and the solution refined with
+ * FP64 residuals until it converges (below).  Outputs (device, any may be
  * NULL but not all): k_out_dev [n_samples][n_ch][n_I][2][2] the on-shell K
  * (fm^2, uncoupled channels in [0][0]); delta_dev [n_samples][n_ch][n_E][3]
  * degrees; sigma_dev [n_samples][n_E] mb; status_dev (may be NULL)

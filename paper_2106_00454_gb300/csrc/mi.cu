@@ -15,9 +15,11 @@
 //
 // GB300 layout: the potential terms on the grid are computed once per channel
 // set (k_mi_pot_grid) and the on-shell rows once per energy list
-// (k_mi_pot_onshell); k_mi_solve runs persistent CTAs, each owning a slot of
+// (k_mi_pot_onshell).  Many systems go through one eigendecomposition per
+// (sample, channel) (k_mi_energies below).  Few of them, and those it leaves,
+// are solved by elimination: k_mi_solve runs persistent CTAs, each owning a slot of
 // FP64 scratch for one (sample, channel) matrix V = V0 + sum_a c_a V_a, and for
-// every energy inverts 1 - V D in FP32 in shared memory (Gauss-Jordan, partial
+// every energy of its chunk inverts 1 - V D in FP32 in shared memory (Gauss-Jordan, partial
 // pivoting; FP32 issues at 58x the FP64 rate) and refines the solution to FP64
 // accuracy with FP64 residuals r = b - (x - V (D x)) (classical iterative
 // refinement: every step is two matrix-vector products).
@@ -201,8 +203,62 @@ __device__ __forceinline__ double mi_block_sum(double v, double *red)
     return t;
 }
 
-// Items (sample, work channel) of one block size; CTA blockIdx.x owns scratch
-// slot Vs + blockIdx.x n^2 and walks the items item = blockIdx.x, + gridDim.x, ...
+// T = (1 + i pi mu p K)^-1 K of the on-shell K (2 x 2 frame) and the phases of S.
+__device__ __forceinline__ void mi_phases(int K, double p, const double *Km, double *po)
+{
+    const double g = kPi * kMu * p;
+    double T[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (K == 1) {
+        const double dre = 1.0, dim = g * Km[0], dd = dre * dre + dim * dim;
+        T[0] = Km[0] * dre / dd;
+        T[1] = -Km[0] * dim / dd;
+    } else {
+        // M = 1 + i g K (complex 2 x 2); T = M^-1 K
+        const double m00r = 1.0, m00i = g * Km[0], m01i = g * Km[1], m10i = g * Km[2], m11r = 1.0,
+                     m11i = g * Km[3];
+        // det = m00 m11 - m01 m10
+        const double detr = m00r * m11r - m00i * m11i + m01i * m10i;
+        const double deti = m00r * m11i + m00i * m11r;
+        const double dd = detr * detr + deti * deti;
+        // inverse = [[m11, -m01], [-m10, m00]] / det
+        const double ir = detr / dd, ii = -deti / dd;
+        const double inv[8] = {m11r * ir - m11i * ii, m11r * ii + m11i * ir,  // (0,0)
+                               m01i * ii, -m01i * ir,                          // (0,1) = -i m01i / det
+                               m10i * ii, -m10i * ir,                          // (1,0)
+                               m00r * ir - m00i * ii, m00r * ii + m00i * ir};  // (1,1)
+        for (int a = 0; a < 2; ++a)
+            for (int bb = 0; bb < 2; ++bb) {
+                double re = 0.0, im = 0.0;
+                for (int k = 0; k < 2; ++k) {
+                    re += inv[(a * 2 + k) * 2] * Km[k * 2 + bb];
+                    im += inv[(a * 2 + k) * 2 + 1] * Km[k * 2 + bb];
+                }
+                T[(a * 2 + bb) * 2] = re;
+                T[(a * 2 + bb) * 2 + 1] = im;
+            }
+    }
+    phases_of_T(K, p, T, po);
+}
+
+// The most refinement steps of a (sample, channel), -1 (a failed system) sticking.
+__device__ __forceinline__ void mi_worst(int *status, int worst)
+{
+    if (worst < 0) {
+        atomicExch(status, -1);
+        return;
+    }
+    int old = atomicAdd(status, 0);
+    while (old >= 0 && old < worst) {
+        const int was = atomicCAS(status, old, worst);
+        if (was == old) break;
+        old = was;
+    }
+}
+
+// Items (sample, work channel, chunk of ne energies) of one block size; CTA
+// blockIdx.x owns scratch slot Vs + blockIdx.x n^2 and walks the items item =
+// blockIdx.x, + gridDim.x, ...  redo (may be NULL; with ne = 1): only the systems
+// with redo[(smp n_ch_total + channel) n_I + energy] != 0.  status is zero on entry.
 // Outputs per (sample, channel, energy): phases ph [S][n_ch][n_I][3] (degrees)
 // and, if k_out, the on-shell K [S][n_ch][n_I][2][2].
 __global__ void __launch_bounds__(kMiThreads) k_mi_solve(const MiChanDev *chans, const int *work_ch, int n_work,
@@ -210,7 +266,8 @@ __global__ void __launch_bounds__(kMiThreads) k_mi_solve(const MiChanDev *chans,
                                                          const double *wg, int n_terms, const double *coeffs,
                                                          const double *Vg, const double *Von, int n_I,
                                                          const double *e_int, double *Vs_all, double *ph,
-                                                         double *k_out, int *status, int *err)
+                                                         double *k_out, int *status, int *err, int ne, int n_chunk,
+                                                         const int *redo)
 {
     const int M = NQ + 1;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
@@ -231,8 +288,10 @@ __global__ void __launch_bounds__(kMiThreads) k_mi_solve(const MiChanDev *chans,
     double *red = reinterpret_cast<double *>(perm + n0 + (n0 & 1));
     double *Vs = Vs_all + (size_t)blockIdx.x * 2 * n0 * n0;  // V, then the FP64 fallback matrix
 
-    for (int item = blockIdx.x; item < n_samples * n_work; item += gridDim.x) {
-        const int smp = item / n_work, cidx = work_ch[item - smp * n_work];
+    for (long long item = blockIdx.x; item < (long long)n_samples * n_work * n_chunk; item += gridDim.x) {
+        const int sw = (int)(item / n_chunk), chunk = (int)(item - (long long)sw * n_chunk);
+        const int smp = sw / n_work, cidx = work_ch[sw - smp * n_work];
+        if (redo && redo[((size_t)smp * n_ch_total + cidx) * n_I + chunk] == 0) continue;
         const MiChanDev ch = chans[cidx];
         const int n = ch.n, K = ch.K;
         const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
@@ -246,7 +305,8 @@ __global__ void __launch_bounds__(kMiThreads) k_mi_solve(const MiChanDev *chans,
             Vs[e] = v;
         }
         int worst = 0;
-        for (int ie = 0; ie < n_I; ++ie) {
+        const int ie1 = min(n_I, (chunk + 1) * ne);
+        for (int ie = chunk * ne; ie < ie1; ++ie) {
             const double p = sqrt(kMn * e_int[ie] / 2.0) / kHbarc, p2 = p * p;
             // D and the on-shell rows and columns of V at this energy
             double part = 0.0;
@@ -456,66 +516,37 @@ __global__ void __launch_bounds__(kMiThreads) k_mi_solve(const MiChanDev *chans,
             if (!conv) worst = -1;
             else if (worst >= 0 && steps > worst) worst = steps;
             if (tid == 0) {
-                // on-shell K, T = (1 + i pi mu p K)^-1 K, phases
+                // on-shell K and its phases
                 double Km[4] = {0, 0, 0, 0};
                 for (int a = 0; a < K; ++a)
                     for (int bb = 0; bb < K; ++bb) Km[a * 2 + bb] = xv[bb * n0 + a * M + NQ];
-                const double g = kPi * kMu * p;
-                double T[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                if (K == 1) {
-                    const double dre = 1.0, dim = g * Km[0], dd = dre * dre + dim * dim;
-                    T[0] = Km[0] * dre / dd;
-                    T[1] = -Km[0] * dim / dd;
-                } else {
-                    // M = 1 + i g K (complex 2 x 2); T = M^-1 K
-                    const double m00r = 1.0, m00i = g * Km[0], m01i = g * Km[1], m10i = g * Km[2], m11r = 1.0,
-                                 m11i = g * Km[3];
-                    // det = m00 m11 - m01 m10
-                    const double detr = m00r * m11r - m00i * m11i + m01i * m10i;
-                    const double deti = m00r * m11i + m00i * m11r;
-                    const double dd = detr * detr + deti * deti;
-                    // inverse = [[m11, -m01], [-m10, m00]] / det
-                    const double ir = detr / dd, ii = -deti / dd;
-                    const double inv[8] = {m11r * ir - m11i * ii, m11r * ii + m11i * ir,  // (0,0)
-                                           m01i * ii, -m01i * ir,                          // (0,1) = -i m01i / det
-                                           m10i * ii, -m10i * ir,                          // (1,0)
-                                           m00r * ir - m00i * ii, m00r * ii + m00i * ir};  // (1,1)
-                    for (int a = 0; a < 2; ++a)
-                        for (int bb = 0; bb < 2; ++bb) {
-                            double re = 0.0, im = 0.0;
-                            for (int k = 0; k < 2; ++k) {
-                                re += inv[(a * 2 + k) * 2] * Km[k * 2 + bb];
-                                im += inv[(a * 2 + k) * 2 + 1] * Km[k * 2 + bb];
-                            }
-                            T[(a * 2 + bb) * 2] = re;
-                            T[(a * 2 + bb) * 2 + 1] = im;
-                        }
-                }
                 const size_t o = ((size_t)smp * n_ch_total + cidx) * n_I + ie;
-                phases_of_T(K, p, T, ph + o * 3);
+                mi_phases(K, p, Km, ph + o * 3);
                 if (k_out)
                     for (int k = 0; k < 4; ++k) k_out[o * 4 + k] = Km[k];
             }
             __syncthreads();
         }
         if (tid == 0) {
-            status[(size_t)smp * n_ch_total + cidx] = worst;
+            mi_worst(&status[(size_t)smp * n_ch_total + cidx], worst);
             if (worst < 0) record_error(err, kDevNoConverge);
         }
     }
 }
 
+// status zeroed by the caller; n_chunk chunks of ne energies per (sample, channel).
 cudaError_t launch_mi_solve(const MiChanDev *chans_dev, const int *work_dev, int n_work, int n, int n_ch_total,
                             int n_samples, int NQ, const double *kg, const double *wg, int n_terms,
                             const double *coeffs, const double *Vg, const double *Von, int n_I, const double *e_int,
-                            double *Vs, int slots, double *ph, double *k_out, int *status, int *err,
-                            cudaStream_t st)
+                            double *Vs, int slots, double *ph, double *k_out, int *status, int *err, cudaStream_t st,
+                            int ne, const int *redo)
 {
     const size_t smem = mi_smem(n, NQ + 1);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (smem > 227 * 1024 || ne < 1 || (redo && ne != 1)) return cudaErrorInvalidValue;
     raise_smem_limit((const void *)k_mi_solve, smem);
     k_mi_solve<<<slots, kMiThreads, smem, counted(st)>>>(chans_dev, work_dev, n_work, n_ch_total, n_samples, NQ, kg, wg, n_terms,
-                                                coeffs, Vg, Von, n_I, e_int, Vs, ph, k_out, status, err);
+                                                coeffs, Vg, Von, n_I, e_int, Vs, ph, k_out, status, err, ne,
+                                                (n_I + ne - 1) / ne, redo);
     return cudaGetLastError();
 }
 
@@ -526,6 +557,393 @@ int mi_slots_per_sm(int n, int NQ)
     int blocks = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_mi_solve, kMiThreads, smem);
     return blocks;
+}
+
+// ------------------------------------------------------------------------------------- solve, all energies at once
+// With w = D y, (1 - V D) y = r reads (D^-1 - V) w = r, and on the grid
+//     D_j^-1 = (p^2 - k_j^2) / (2 mu w_j k_j^2)
+// is affine in p^2: V - D^-1 = S^-1 (Ht - p^2) S^-1 with S_j = sqrt(2 mu w_j) k_j and
+// Ht = diag(k^2) + S V S, the same for every energy.  One eigendecomposition
+// Ht = Q diag(lambda) Q^T per (sample, channel) thus inverts the grid part at every
+// energy, M^-1 = S Q (lambda - p^2)^-1 Q^T S, and the on-shell point is a K x K border:
+//     w_p = (1/D_N - R)^-1 (r_p - v^T M^-1 r_g),  w_g = -M^-1 (r_g + v w_p),
+//     R = V_pp - v^T M^-1 v,  v = V(grid, p).
+// Q is held in FP32 and lambda - p^2 formed in FP64, so every direction is
+// inverted to FP32's relative accuracy, close poles included; FP64 residuals
+// of the original system then refine the solution to FP64 as for the FP32
+// inverse of k_mi_solve (which takes the systems that do not converge here).
+// Per energy this costs K n^2 FP64 multiply-adds a residual (the bound: two or
+// three of them) instead of an n^3 elimination whose n steps wait for each other:
+// 64 samples x 15 channels x 32 energies, N_Q = 96: 134.4 -> 22.0 ms, errors against
+// 64 bits unchanged (the eigendecompositions are 15 ms of it).
+
+// S V_t S over the grid and k^2, from the grid terms of every channel.
+__global__ void __launch_bounds__(256) k_mi_scale(const MiChanDev *chans, int n_ch, int NQ, const double *kg,
+                                                  const double *wg, int n_terms, const double *Vg, double *Vt,
+                                                  const long long *vt_off, double *k2)
+{
+    const int c = blockIdx.y;
+    const MiChanDev ch = chans[c];
+    const int M = NQ + 1, ng = ch.K * NQ;
+    if (c == 0)
+        for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < NQ; j += (long long)gridDim.x * blockDim.x)
+            k2[j] = kg[j] * kg[j];
+    const long long total = (long long)n_terms * ng * ng;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (long long)gridDim.x * blockDim.x) {
+        const int t = (int)(e / ((long long)ng * ng)), rc = (int)(e - (long long)t * ng * ng), r = rc / ng, q = rc - r * ng;
+        const int i = r % NQ, j = q % NQ;
+        const double v = Vg[ch.vg_off + ((size_t)t * ch.n + (r / NQ) * M + i) * ch.n + (q / NQ) * M + j];
+        const double si = sqrt(2.0 * kMu * wg[i]) * kg[i], sj = sqrt(2.0 * kMu * wg[j]) * kg[j];
+        Vt[vt_off[c] + e] = v * (si * sj);
+    }
+}
+
+cudaError_t launch_mi_scale(const MiChanDev *chans_dev, int n_ch, int NQ, const double *kg, const double *wg, int n_terms,
+                            const double *Vg, double *Vt, const long long *vt_off, double *k2, cudaStream_t st)
+{
+    k_mi_scale<<<dim3(64, n_ch), 256, 0, counted(st)>>>(chans_dev, n_ch, NQ, kg, wg, n_terms, Vg, Vt, vt_off, k2);
+    return cudaGetLastError();
+}
+
+constexpr int kMeCols = 8;      // right-hand sides a pass carries: 8 / K energies
+// 16 warps for coupled channels (14 row-block tasks of the residual), 8 for uncoupled ones (7 to 8),
+// two or three of which share an SM
+__host__ __device__ inline int me_threads(int K) { return K == 2 ? 512 : 256; }
+constexpr int kMeMaxRefine = 10;
+
+__host__ __device__ inline int me_ldq(int ng) { return ng | 1; }  // odd row pitch of Q: conflict-free along both indices
+
+// Q float [ng][ldq] | z, x, b double [ng][8] | T = M^-1 v, u, h float [ng][8] | lambda, S double [ng] |
+// D double [NQ][8 / K] | per column: p^2, D_N, x_p, r_p, y_p ... double [8 x 16] | maxima double [16][16]
+__host__ __device__ inline size_t me_smem(int ng, int NQ, int K)
+{
+    size_t b = ((size_t)ng * me_ldq(ng) * 4 + 15) & ~(size_t)15;
+    b += (size_t)3 * ng * kMeCols * 8 + (size_t)3 * ng * kMeCols * 4 + (size_t)2 * ng * 8;
+    b += (size_t)NQ * (kMeCols / K) * 8 + (size_t)8 * 16 * 8 + (size_t)32 * kMeCols * 8;
+    return b;
+}
+
+// u = Q^T (S o rhs) in FP32, divided by lambda - p^2, then h = S o (Q u): h = M^-1 rhs
+// for the pass's columns (rhs FP64 [ng][8], h float [ng][8]).
+__device__ __forceinline__ void me_apply(int ng, int NQ, int ldq, const float *Q, const double *lam, const double *Sg,
+                                         const double *p2c, const double *rhs, float *u, float *h)
+{
+    const int tid = threadIdx.x, nt = blockDim.x;
+    // h as the FP32 copy of S o rhs first
+    for (int e = tid; e < ng * kMeCols; e += nt) h[e] = (float)(rhs[e] * Sg[e / kMeCols]);
+    __syncthreads();
+    for (int task = tid; task < ng * 2; task += nt) {  // (eigenvector i, four columns)
+        const int q = task / ng, i = task - q * ng;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r = 0; r < ng; ++r) {
+            const float v = Q[r * ldq + i];
+            const float4 b = *reinterpret_cast<const float4 *>(h + r * kMeCols + 4 * q);
+            a.x = fmaf(v, b.x, a.x);
+            a.y = fmaf(v, b.y, a.y);
+            a.z = fmaf(v, b.z, a.z);
+            a.w = fmaf(v, b.w, a.w);
+        }
+        const double l = lam[i], *p = p2c + 4 * q;
+        a.x *= 1.0f / (float)(l - p[0]);
+        a.y *= 1.0f / (float)(l - p[1]);
+        a.z *= 1.0f / (float)(l - p[2]);
+        a.w *= 1.0f / (float)(l - p[3]);
+        *reinterpret_cast<float4 *>(u + i * kMeCols + 4 * q) = a;
+    }
+    __syncthreads();
+    for (int task = tid; task < ng * 2; task += nt) {  // (grid point r, four columns)
+        const int q = task / ng, r = task - q * ng;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < ng; ++i) {
+            const float v = Q[r * ldq + i];
+            const float4 b = *reinterpret_cast<const float4 *>(u + i * kMeCols + 4 * q);
+            a.x = fmaf(v, b.x, a.x);
+            a.y = fmaf(v, b.y, a.y);
+            a.z = fmaf(v, b.z, a.z);
+            a.w = fmaf(v, b.w, a.w);
+        }
+        const float s = (float)Sg[r];
+        *reinterpret_cast<float4 *>(h + r * kMeCols + 4 * q) = make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
+    }
+    __syncthreads();
+}
+
+// One CTA per (sample, work channel), slot Vs + blockIdx.x ng^2 for its V on the grid.
+__global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, const ChanDev *eig_ch, const int *work_ch, int n_work,
+                                                            int n_ch_total, int sample0, int n_samples, int NQ,
+                                                            const double *kg, const double *wg, int n_terms,
+                                                            const double *coeffs, const double *Vg, const double *Von,
+                                                            int n_I, const double *e_int, const double *eps_all,
+                                                            const double *Q_all, double *Vs_all, double *ph,
+                                                            double *k_out, int *status, int *redo, int *err)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int K = chans[work_ch[0]].K, M = NQ + 1, ng = K * NQ, ldq = me_ldq(ng), EC = kMeCols / K;
+    if ((size_t)dyn_smem_bytes() < me_smem(ng, NQ, K)) {
+        if (tid == 0) record_error(err, kDevBadSize);
+        return;
+    }
+    extern __shared__ __align__(16) unsigned char me_sm[];
+    float *Q = reinterpret_cast<float *>(me_sm);
+    double *z = reinterpret_cast<double *>(me_sm + (((size_t)ng * ldq * 4 + 15) & ~(size_t)15));  // D x, or a right-hand side
+    double *x = z + (size_t)ng * kMeCols, *b = x + (size_t)ng * kMeCols;
+    double *lam = b + (size_t)ng * kMeCols, *Sg = lam + ng;
+    double *D = Sg + ng;                                   // [NQ][EC]
+    double *p2c = D + (size_t)NQ * EC;                     // per column: p^2
+    double *DNc = p2c + 8, *xp = DNc + 8, *rp = xp + 16, *Rm = rp + 16, *Vpp = Rm + 16, *wp = Vpp + 16;  // [8][K] each
+    double *ymx = wp + 16, *ypr = ymx + 8;                 // maxima of the correction, this step's and the last one's
+    int *nst = reinterpret_cast<int *>(ypr + 8);           // per column: 0, or the step it converged at
+    double *red = p2c + 8 * 16;                            // [32][8]
+    float *T = reinterpret_cast<float *>(red + 32 * kMeCols), *u = T + (size_t)ng * kMeCols, *h = u + (size_t)ng * kMeCols;
+    double *V = Vs_all + (size_t)blockIdx.x * ng * ng;
+
+    for (int item = blockIdx.x; item < n_samples * n_work; item += gridDim.x) {
+        const int smp = sample0 + item / n_work, cidx = work_ch[item % n_work];
+        const MiChanDev ch = chans[cidx];
+        const ChanDev ec = eig_ch[cidx];
+        const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
+        const double *Vgc = Vg + ch.vg_off;
+        const double *Qg = Q_all + ec.c_off + (size_t)(smp - sample0) * ng * ng;
+        const double *lg = eps_all + ec.eps_off + (size_t)(smp - sample0) * ng;
+        __syncthreads();  // the last item is done with shared memory
+        for (int e = tid; e < ng * ng; e += nt) {
+            const int r = e / ng, c = e - r * ng;
+            const size_t o = (size_t)((r / NQ) * M + r % NQ) * ch.n + (c / NQ) * M + c % NQ;
+            double v = Vgc[o];
+            for (int t = 1; t < n_terms; ++t) v = fma(cf[t - 1], Vgc[(size_t)t * ch.n * ch.n + o], v);
+            V[e] = v;
+            Q[r * ldq + c] = (float)Qg[e];
+        }
+        for (int i = tid; i < ng; i += nt) {
+            lam[i] = lg[i];
+            Sg[i] = sqrt(2.0 * kMu * wg[i % NQ]) * kg[i % NQ];
+        }
+        int worst = 0;
+        for (int e0 = 0; e0 < n_I; e0 += EC) {
+            // columns c = (energy el = c / K, right-hand side bb = c % K); past the last energy the last one again
+            __syncthreads();
+            for (int el = warp; el < EC; el += nw) {
+                const int ie = min(e0 + el, n_I - 1);
+                const double p = sqrt(kMn * e_int[ie] / 2.0) / kHbarc, p2 = p * p;
+                double part = 0.0;
+                for (int j = lane; j < NQ; j += 32) {
+                    const double den = p2 - kg[j] * kg[j];
+                    D[j * EC + el] = wg[j] * kg[j] * kg[j] * 2.0 * kMu / den;
+                    part += wg[j] / den;
+                }
+                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+                if (lane < K) {
+                    p2c[el * K + lane] = p2;
+                    DNc[el * K + lane] = -2.0 * kMu * p2 * part;
+                }
+            }
+            // v_{(a, i), bb} at the column's energy, V_pp, and the first right-hand side b = v
+            for (int e = tid; e < (ng + K) * kMeCols; e += nt) {
+                const int r = e / kMeCols, c = e - r * kMeCols, el = c / K, bb = c - el * K;
+                const int ie = min(e0 + el, n_I - 1);
+                const int a = r < ng ? r / NQ : r - ng, i = r < ng ? r % NQ : NQ;
+                const double *Vo = Von + ch.von_off + (size_t)ie * n_terms * K * K * M + (size_t)(a * K + bb) * M + i;
+                double v = Vo[0];
+                for (int t = 1; t < n_terms; ++t) v = fma(cf[t - 1], Vo[(size_t)t * K * K * M], v);
+                if (r < ng) {
+                    b[r * kMeCols + c] = v;
+                    x[r * kMeCols + c] = 0.0;
+                } else {
+                    Vpp[c * 2 + a] = v;
+                    rp[c * 2 + a] = v;
+                    xp[c * 2 + a] = 0.0;
+                }
+            }
+            if (tid < kMeCols) nst[tid] = 0;
+            __syncthreads();
+            me_apply(ng, NQ, ldq, Q, lam, Sg, p2c, b, u, h);
+            for (int e = tid; e < ng * kMeCols; e += nt) T[e] = h[e];
+            __syncthreads();
+            // R = V_pp - v^T T, one warp per (column, row block)
+            for (int w = warp; w < kMeCols * K; w += nw) {
+                const int c = w / K, a = w - c * K, ca = (c / K) * K + a;  // v of block a at this energy: column ca
+                double s = 0.0;
+                for (int r = lane; r < ng; r += 32) s = fma(b[r * kMeCols + ca], (double)T[r * kMeCols + c], s);
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) Rm[c * 2 + a] = Vpp[c * 2 + a] - s;
+            }
+            __syncthreads();
+            int it = 0;
+            bool done = false;
+            for (; it < kMeMaxRefine && !done; ++it) {
+                if (it > 0) {
+                    // h = M^-1 r for the residual in z
+                    me_apply(ng, NQ, ldq, Q, lam, Sg, p2c, z, u, h);
+                }
+                // r_p - v^T h (the first step: h = T, so this is R), then w_p and the correction of x_p
+                for (int w = warp; w < kMeCols * K; w += nw) {
+                    const int c = w / K, a = w - c * K, ca = (c / K) * K + a;
+                    double s = 0.0;
+                    for (int r = lane; r < ng; r += 32) s = fma(b[r * kMeCols + ca], (double)h[r * kMeCols + c], s);
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if (lane == 0) wp[c * 2 + a] = rp[c * 2 + a] - s;
+                }
+                __syncthreads();
+                if (tid < kMeCols) {
+                    const int c = tid, k0 = (c / K) * K;
+                    const double DN = DNc[c];
+                    if (K == 1) {
+                        wp[c * 2] = DN * wp[c * 2] / (1.0 - DN * Rm[c * 2]);
+                    } else {  // (1 - D_N R) w = D_N s, R[a][b] = Rm of column b, block a
+                        const double a00 = 1.0 - DN * Rm[k0 * 2], a01 = -DN * Rm[(k0 + 1) * 2], a10 = -DN * Rm[k0 * 2 + 1],
+                                     a11 = 1.0 - DN * Rm[(k0 + 1) * 2 + 1];
+                        const double det = a00 * a11 - a01 * a10, s0 = DN * wp[c * 2], s1 = DN * wp[c * 2 + 1];
+                        wp[c * 2] = (a11 * s0 - a01 * s1) / det;
+                        wp[c * 2 + 1] = (a00 * s1 - a10 * s0) / det;
+                    }
+                }
+                __syncthreads();
+                // y_g = -(h + T w_p) / D, y_p = w_p / D_N; x += y, z = D x, the maxima of |y| and |x|
+                double ym[kMeCols / 4], xm[kMeCols / 4];  // this thread's columns are tid % 4, + 4
+                for (int q = 0; q < kMeCols / 4; ++q) ym[q] = xm[q] = 0.0;
+                for (int e = tid; e < ng * 4; e += nt) {
+                    const int r = e >> 2;
+#pragma unroll
+                    for (int q = 0; q < kMeCols / 4; ++q) {
+                        const int c = (e & 3) + 4 * q, k0 = (c / K) * K;
+                        float w = h[r * kMeCols + c];
+                        double t = (double)w;
+                        for (int a = 0; a < K; ++a) t = fma((double)T[r * kMeCols + k0 + a], wp[c * 2 + a], t);
+                        const double d = D[(r % NQ) * EC + c / K];
+                        const double y = -t / d, xn = x[r * kMeCols + c] + y;
+                        x[r * kMeCols + c] = xn;
+                        z[r * kMeCols + c] = d * xn;
+                        ym[q] = nan_max(ym[q], fabs(y));
+                        xm[q] = nan_max(xm[q], fabs(xn));
+                    }
+                }
+                // lanes with the same tid % 4 hold the same columns
+#pragma unroll
+                for (int q = 0; q < kMeCols / 4; ++q) {
+                    for (int o = 16; o >= 4; o >>= 1) {
+                        ym[q] = nan_max(ym[q], __shfl_xor_sync(0xffffffffu, ym[q], o));
+                        xm[q] = nan_max(xm[q], __shfl_xor_sync(0xffffffffu, xm[q], o));
+                    }
+                    if (lane < 4) {
+                        red[warp * kMeCols + lane + 4 * q] = ym[q];
+                        red[(16 + warp) * kMeCols + lane + 4 * q] = xm[q];
+                    }
+                }
+                __syncthreads();
+                if (tid < kMeCols) {
+                    const int c = tid;
+                    double y = 0.0, xx = 0.0;
+                    for (int w = 0; w < nw; ++w) {
+                        y = nan_max(y, red[w * kMeCols + c]);
+                        xx = nan_max(xx, red[(16 + w) * kMeCols + c]);
+                    }
+                    for (int a = 0; a < K; ++a) {
+                        const double yp = wp[c * 2 + a] / DNc[c];
+                        xp[c * 2 + a] += yp;
+                        y = nan_max(y, fabs(yp));
+                        xx = nan_max(xx, fabs(xp[c * 2 + a]));
+                    }
+                    const double pr = ypr[c];
+                    ypr[c] = y;
+                    ymx[c] = y;
+                    // done when the correction is negligible, when the next one will be (it shrinks by the
+                    // same factor y / pr again, to below the rounding of x), or when it has stopped shrinking at
+                    // the accuracy floor of the FP64 residual
+                    const bool conv = y <= 1e-14 * xx || (it > 0 && y <= 1e-3 * pr && y * y <= 2e-15 * xx * pr) ||
+                                      (it > 0 && y > 0.25 * pr && y <= 1e-9 * xx);
+                    if (conv && nst[c] == 0) nst[c] = it + 1;
+                    if (!conv) nst[c] = 0;
+                }
+                __syncthreads();
+                done = true;
+                for (int c = 0; c < kMeCols; ++c) done &= nst[c] != 0;
+                if (done) break;
+                // z <- r = b - x + V (D x), grid part: lanes along the rows (V is symmetric: row c of V is
+                // its column), four columns per thread; the results wait for everyone's reads of z
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                const int rq = warp & 1, rr = (warp >> 1) * 32 + lane;  // one task a warp (the launch checks)
+                if (rr < ng) {
+                    const double *Vr = V + rr;
+#pragma unroll 4
+                    for (int c = 0; c < ng; ++c) {
+                        const double v = Vr[(size_t)c * ng];
+                        const double2 z0 = *reinterpret_cast<const double2 *>(z + c * kMeCols + 4 * rq);
+                        const double2 z1 = *reinterpret_cast<const double2 *>(z + c * kMeCols + 4 * rq + 2);
+                        acc[0] = fma(v, z0.x, acc[0]);
+                        acc[1] = fma(v, z0.y, acc[1]);
+                        acc[2] = fma(v, z1.x, acc[2]);
+                        acc[3] = fma(v, z1.y, acc[3]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = 4 * rq + j, k0 = (c / K) * K;
+                        // the on-shell column: v_a D_N x_p[a]
+                        for (int bb = 0; bb < K; ++bb) acc[j] = fma(b[rr * kMeCols + k0 + bb], DNc[c] * xp[c * 2 + bb], acc[j]);
+                        acc[j] = b[rr * kMeCols + c] - x[rr * kMeCols + c] + acc[j];
+                    }
+                }
+                // r_p = V_pp - x_p + v^T (D x_g) + V_pp D_N x_p
+                for (int w = warp; w < kMeCols * K; w += nw) {
+                    const int c = w / K, a = w - c * K, k0 = (c / K) * K;
+                    double s = 0.0;
+                    for (int r = lane; r < ng; r += 32) s = fma(b[r * kMeCols + k0 + a], z[r * kMeCols + c], s);
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if (lane == 0) {
+                        for (int bb = 0; bb < K; ++bb) s = fma(Vpp[(k0 + bb) * 2 + a], DNc[c] * xp[c * 2 + bb], s);
+                        rp[c * 2 + a] = Vpp[c * 2 + a] - xp[c * 2 + a] + s;
+                    }
+                }
+                __syncthreads();
+                if (rr < ng)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) z[rr * kMeCols + 4 * rq + j] = acc[j];
+                __syncthreads();
+            }
+            for (int c = 0; c < kMeCols; ++c) worst = max(worst, nst[c]);
+            if (tid < EC && e0 + tid < n_I) {
+                const int ie = e0 + tid;
+                bool ok = true;
+                for (int bb = 0; bb < K; ++bb) ok &= nst[tid * K + bb] != 0;
+                redo[((size_t)smp * n_ch_total + cidx) * n_I + ie] = ok ? 0 : 1;
+                double Km[4] = {0, 0, 0, 0};
+                for (int a = 0; a < K; ++a)
+                    for (int bb = 0; bb < K; ++bb) Km[a * 2 + bb] = xp[(tid * K + bb) * 2 + a];
+                const size_t o = ((size_t)smp * n_ch_total + cidx) * n_I + ie;
+                mi_phases(K, sqrt(kMn * e_int[ie] / 2.0) / kHbarc, Km, ph + o * 3);
+                if (k_out)
+                    for (int k = 0; k < 4; ++k) k_out[o * 4 + k] = Km[k];
+            }
+        }
+        if (tid == 0) status[(size_t)smp * n_ch_total + cidx] = worst;  // the elimination kernel adds what it redoes
+    }
+}
+
+bool mi_energies_fit(int NQ, int K) { return me_smem(K * NQ, NQ, K) <= 227 * 1024 && (K * NQ + 31) / 32 * 2 <= me_threads(K) / 32; }
+
+int mi_energies_per_sm(int NQ, int K)
+{
+    const size_t smem = me_smem(K * NQ, NQ, K);
+    raise_smem_limit((const void *)k_mi_energies, smem);
+    int blocks = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_mi_energies, me_threads(K), smem);
+    return blocks;
+}
+
+// n_samples samples from sample0; eps / Q: the eigenpairs of this range (eig_ch offsets).
+cudaError_t launch_mi_energies(const MiChanDev *chans_dev, const ChanDev *eig_ch, const int *work_dev, int n_work, int K,
+                               int n_ch_total, int sample0, int n_samples, int NQ, const double *kg, const double *wg,
+                               int n_terms, const double *coeffs, const double *Vg, const double *Von, int n_I,
+                               const double *e_int, const double *eps, const double *Q, double *Vs, int slots, double *ph,
+                               double *k_out, int *status, int *redo, int *err, cudaStream_t st)
+{
+    const size_t smem = me_smem(K * NQ, NQ, K);
+    if (!mi_energies_fit(NQ, K)) return cudaErrorInvalidValue;
+    raise_smem_limit((const void *)k_mi_energies, smem);
+    k_mi_energies<<<slots, me_threads(K), smem, counted(st)>>>(chans_dev, eig_ch, work_dev, n_work, n_ch_total, sample0,
+                                                            n_samples, NQ, kg, wg, n_terms, coeffs, Vg, Von, n_I, e_int,
+                                                            eps, Q, Vs, ph, k_out, status, redo, err);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------- observables

@@ -114,6 +114,11 @@ struct MiH {
     double *kg = nullptr, *wg = nullptr, *gp = nullptr, *Vg = nullptr;
     int *work_dev[2] = {nullptr, nullptr};  // channels with K = 1, 2
     int n_work[2] = {0, 0};
+    // diag(k^2) + S V S of every channel in the form of a projected set (mi.cu), for the
+    // eigendecomposition that serves all energies; empty when there was no room for it
+    VSetH set;
+    double *k2 = nullptr;
+    bool has_set = false;
 };
 
 enum Kind { kMesh = 1, kVSet = 2, kEig = 3, kMi = 4 };
@@ -359,6 +364,8 @@ void free_mi(wpcd_ctx *c, MiH &m)
     dfree(c, m.Vg);
     dfree(c, m.work_dev[0]);
     dfree(c, m.work_dev[1]);
+    free_vset(c, m.set);
+    dfree(c, m.k2);
 }
 
 void free_mesh(wpcd_ctx *c, MeshH &m)
@@ -1667,6 +1674,66 @@ wpcd_status wpcd_saclay(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, con
 }
 
 // ---- MI comparison method (Sec. 2.1, Sec. 6) ---------------------------------------------------
+namespace {
+// The set of diag(k^2) + S V S; without room for it the MI set works without.
+wpcd_status mi_eigen_set(wpcd_ctx *c, MiH &m)
+{
+    VSetH &v = m.set;
+    std::vector<long long> off;
+    size_t len = 0;
+    for (auto &d : m.ch) {
+        const size_t ng = (size_t)d.K * m.NQ;
+        off.push_back((long long)len);
+        len += (size_t)m.n_terms * ng * ng;
+    }
+    long long *off_dev = nullptr;
+    bool ok = dalloc(c, &v.V, len) == WPCD_OK && dalloc(c, &m.k2, (size_t)m.NQ) == WPCD_OK &&
+              dalloc(c, &off_dev, off.size()) == WPCD_OK;
+    v.n_ch = m.n_ch;
+    v.n_terms = m.n_terms;
+    v.maxN = m.NQ;
+    for (int k = 0; k < m.n_ch && ok; ++k) {
+        ChanDev d;
+        memset(&d, 0, sizeof(d));
+        d.coupled = m.ch[k].coupled;
+        d.N = m.NQ;
+        d.K = m.ch[k].K;
+        d.n = d.K * m.NQ;
+        d.h0 = m.k2;
+        d.V = v.V + off[k];
+        v.cd.push_back(d);
+        v.buckets[d.n].push_back(k);
+    }
+    if (ok) {
+        CK(cudaMemcpyAsync(off_dev, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice, c->main.stream));
+        Launch L(c, c->main, WPCD_PHASE_MI);
+        CK(launch_mi_scale(m.ch_dev, m.n_ch, m.NQ, m.kg, m.wg, m.n_terms, m.Vg, v.V, off_dev, m.k2, c->main.stream));
+        CK(cudaStreamSynchronize(c->main.stream));
+    } else {
+        dfree(c, v.V);
+        v.V = nullptr;
+        dfree(c, m.k2);
+        m.k2 = nullptr;
+    }
+    dfree(c, off_dev);
+    m.has_set = ok;
+    return WPCD_OK;
+}
+
+// Eigenpairs of S samples of one block size of an MI set into X.eig, on the FP64
+// path; a solve that fails shows in the energies (their refinement does not converge).
+wpcd_status mi_eigen(wpcd_ctx *c, Exec &X, MiH &m, const double *cf, int S, int K)
+{
+    wpcd_status st = diag_prep(c, X, m.set, -1, S, WPCD_PREC_FP64, X.eig);
+    if (st) return st;
+    int *err = X.err;
+    X.err = nullptr;
+    st = run_bucket_f64(c, X, m.set, X.eig, cf, m.work_dev[K - 1], m.n_work[K - 1], S, 0, K * m.NQ);
+    X.err = err;
+    return st;
+}
+}  // namespace
+
 wpcd_status wpcd_mi_prepare(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, int generator_id,
                             const double *gp_host, int n_gp, int n_terms, int n_quad, double c_map_fm, int *mi_id)
 {
@@ -1744,6 +1811,10 @@ wpcd_status wpcd_mi_prepare(wpcd_ctx *c, const wpcd_channel *channels, int n_ch,
         CK(launch_mi_pot(gen, m->ch_dev, n_ch, n_quad, m->kg, m->Lmax, m->gp, angx, angw, n_terms, m->Vg,
                          c->main.stream));
     }
+    if ((st = mi_eigen_set(c, *m))) {
+        free_mi(c, *m);
+        return st;
+    }
     CK(cudaStreamSynchronize(c->main.stream));
     const int id = c->next_id++;
     Handle h;
@@ -1776,10 +1847,12 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
     wpcd_status st;
     const size_t ph_len = (size_t)S * m.n_ch * n_I * 3;
     if ((st = ws_reserve(c, X, X.ws_tbin, (von_len + ph_len) * sizeof(double)))) return st;
-    if ((st = ws_reserve(c, X, X.ws_plan_i, (size_t)S * m.n_ch * sizeof(int)))) return st;
+    if ((st = ws_reserve(c, X, X.ws_plan_i, (size_t)S * m.n_ch * (1 + n_I) * sizeof(int)))) return st;
     double *Von = static_cast<double *>(X.ws_tbin.p), *ph = Von + von_len;
     int *status = status_dev ? status_dev : static_cast<int *>(X.ws_plan_i.p);
+    int *redo = static_cast<int *>(X.ws_plan_i.p) + (size_t)S * m.n_ch;
     CK(cudaMemcpyAsync(m.ch_dev, m.ch.data(), sizeof(MiChanDev) * m.n_ch, cudaMemcpyHostToDevice, X.stream));
+    CK(cudaMemsetAsync(status, 0, sizeof(int) * S * m.n_ch, X.stream));
     double *angx = nullptr, *angw = nullptr;
     if (m.gen == WPCD_GEN_YUKAWA && (st = gl_rule(c, kAngleQ, &angx, &angw))) return st;
     {
@@ -1788,19 +1861,51 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
                              X.stream));
     }
     const double *cf = m.n_terms > 1 ? coeffs : nullptr;
-    for (int K = 1; K <= 2; ++K) {
+    for (int K = 2; K >= 1; --K) {
         const int nw = m.n_work[K - 1];
         if (!nw) continue;
-        const int n = K * M;
+        const int n = K * M, ng = K * m.NQ;
+        // One eigendecomposition costs three to four systems by elimination, and its latency more where
+        // the chip is not full: measured at 15 channels, N_Q = 24 / 48 / 96, the two meet at ~1900
+        // systems (4 samples x 32 energies: 2.35 against 2.46 ms, 3.8 / 4.4, 10.1 / 9.6; 1 sample 2.3 / 1.0,
+        // 3.7 / 1.5, 9.5 / 3.1; 64 samples 5.0 / 30.9, 7.6 / 56.9, 21.9 / 134.6; at 8 energies and 64
+        // samples still 3.6 / 8.5, 5.0 / 14.8, 15.2 / 33.7)
+        bool eig = m.has_set && mi_energies_fit(m.NQ, K) && n_I >= 4 && (long long)S * m.n_ch * n_I >= 12ll * c->n_sm;
+        if (eig) {
+            const int slots = std::max(1, std::min(S * nw, std::max(1, mi_energies_per_sm(m.NQ, K)) * c->n_sm));
+            // eigenpairs of a few GB of samples at a time
+            size_t per = 0;
+            for (auto &d : m.set.cd) per += (size_t)d.n * d.n * 8;
+            const int Sc = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, ((size_t)4 << 30) / per));
+            for (int s0 = 0; s0 < S && eig; s0 += Sc) {
+                const int ns = std::min(Sc, S - s0);
+                const double *cfs = cf ? cf + (size_t)s0 * (m.n_terms - 1) : nullptr;
+                if (mi_eigen(c, X, m, cfs, ns, K) || ws_reserve(c, X, X.ws_ref, (size_t)slots * ng * ng * sizeof(double))) {
+                    eig = false;  // no room: by elimination, from the first sample on
+                    CK(cudaMemsetAsync(status, 0, sizeof(int) * S * m.n_ch, X.stream));
+                    break;
+                }
+                Launch L(c, X, WPCD_PHASE_MI);
+                CK(launch_mi_energies(m.ch_dev, X.eig.cd_dev, m.work_dev[K - 1], nw, K, m.n_ch, s0, ns, m.NQ, m.kg, m.wg,
+                                      m.n_terms, cf, m.Vg, Von, n_I, e_int, X.eig.eps, X.eig.C,
+                                      static_cast<double *>(X.ws_ref.p), slots, ph, k_out, status, redo, X.err, X.stream));
+            }
+        }
         const int per_sm = mi_slots_per_sm(n, m.NQ);
         if (per_sm < 1) return WPCD_ERR_ARG;
-        const int items = S * nw;
-        const int slots = std::max(1, std::min(items, per_sm * c->n_sm));
+        // by elimination (after the eigendecomposition only the systems that did not converge, one
+        // by one), the energies of a (sample, channel) split over as many CTAs as the chip holds
+        const long long items = (long long)S * nw;
+        const int cap = per_sm * c->n_sm;
+        const int chunks = eig ? n_I : (int)std::max<long long>(1, std::min<long long>(n_I, cap / items));
+        const int ne = (n_I + chunks - 1) / chunks, nck = (n_I + ne - 1) / ne;
+        const int slots = (int)std::max<long long>(1, std::min<long long>(items * nck, cap));
         // two FP64 n x n matrices per slot: V, and the rarely used FP64 elimination fallback
         if ((st = ws_reserve(c, X, X.ws_ref, (size_t)slots * 2 * n * n * sizeof(double)))) return st;
         Launch L(c, X, WPCD_PHASE_MI);
         CK(launch_mi_solve(m.ch_dev, m.work_dev[K - 1], nw, n, m.n_ch, S, m.NQ, m.kg, m.wg, m.n_terms, cf, m.Vg, Von,
-                           n_I, e_int, static_cast<double *>(X.ws_ref.p), slots, ph, k_out, status, X.err, X.stream));
+                           n_I, e_int, static_cast<double *>(X.ws_ref.p), slots, ph, k_out, status, X.err, X.stream, ne,
+                           eig ? redo : nullptr));
     }
     if (delta || sigma) {
         Launch L(c, X, WPCD_PHASE_MI);

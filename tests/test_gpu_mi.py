@@ -98,3 +98,23 @@ def test_mi_refuses_bad_arguments(ctx):
         ctx.mi_prepare([(0, 0, 0, 0, 0, 0)], W.GEN_YAMAGUCHI, W.YAMAGUCHI_PARAMS, 1, n_quad=101)
     with pytest.raises(api.WpcdError):
         ctx.mi_prepare([(1, 1, 0, 2, 1, 0)], W.GEN_YAMAGUCHI, W.YAMAGUCHI_PARAMS, 1)
+
+
+@pytest.mark.parametrize("nq,jmax,S,n_I", [(33, 1, 20, 25), (64, 2, 12, 23), (96, 1, 96, 4), (100, 1, 40, 13)])
+def test_mi_many_systems(ctx, orc, nq, jmax, S, n_I):
+    """Enough systems for the eigendecomposition that serves all energies: energies
+    that do not fill the last pass, one and two l-blocks, the largest grid; some
+    samples against the oracle, and every phase against the few-systems route
+    (elimination, one sample a call)."""
+    chs = [c.astuple() for c in W.np_channels(jmax)]
+    coeffs, e_lab = W.coefficient_samples(S, 5), W.lab_energies(19)
+    e_int = W.chebyshev_energies(n_I)
+    assert S * len(chs) * n_I >= 12 * 152 and len(chs) * n_I < 12 * 152
+    gpu = _gpu(ctx, chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, coeffs, e_int, e_lab, nq)
+    pick = [0, S // 2, S - 1]
+    ora = orc.mi_batch(chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, coeffs[pick], e_int, e_lab, NQ=nq)
+    assert ora[3] == 0
+    _compare(chs, tuple(x[pick] for x in gpu), ora[:3])
+    for s in pick:
+        one = _gpu(ctx, chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, coeffs[s:s + 1], e_int, e_lab, nq)
+        assert np.max(np.abs(dphase(one[1][0], gpu[1][s]))) <= 1e-8
