@@ -377,7 +377,7 @@ static size_t big_smem(int n)
 bool jacobi_fits_smem(int n, bool f64)
 {
     const size_t cap = 227 * 1024;
-    return f64 ? jacobi_smem_bytes(n, false) <= cap : jacobi_mixed_smem_bytes(n, false) <= cap;
+    return f64 ? jacobi_smem_bytes(n, false) <= cap : jacobi_mixed_fits(n);
 }
 
 size_t jacobi_big_scratch_bytes(int n, bool f64) { return big_slot_elems<double>(n) * (f64 ? 8 : 4); }
