@@ -44,6 +44,8 @@ constexpr int kRefineIters = 2;                            // FP64 refinement it
 // angle and its share of the diagonal are below 2^-18, which two refinement iterations
 // take to FP64 (2^-16 makes a third one common at n = 300).
 constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
+// Batches up to this many solves per SM run their size buckets side by side.
+constexpr int kForkItems = 8;
 constexpr size_t kGraphCache = 64;                         // wpcd_solve keys remembered for CUDA graphs
 
 struct MeshH {
@@ -93,16 +95,20 @@ struct EigH {
 struct Buf {
     void *p = nullptr;
     size_t n = 0;
+    bool part = false;  // a share of another buffer: never reallocated
 };
 
 // One executor: a stream, its device status word and its workspaces.  The
 // synchronous API runs on the context's own executor; each serving slot has
 // one of its own so that batches overlap on the device.
+constexpr int kSides = 3;  // streams beside the executor's own for the size buckets of a small batch
 struct Exec {
     cudaStream_t stream = nullptr;
     int *err = nullptr;
     Buf ws_plan_i, ws_plan_d, ws_tbin, ws_phbin, ws_ref, ws_in, ws_out;
     EigH eig;
+    cudaStream_t side[kSides] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
 };
 
 // MI set: the momentum grid, the channels and their grid potential terms.
@@ -284,6 +290,7 @@ bool capturing(cudaStream_t st)
 wpcd_status ws_reserve(wpcd_ctx *c, const Exec &X, Buf &b, size_t bytes)
 {
     if (b.n >= bytes) return WPCD_OK;
+    if (b.part) return WPCD_ERR_NOMEM;
     if (capturing(X.stream)) return WPCD_ERR_CUDA;  // a graph cannot hold a reallocation
     if (b.p) {
         cudaStreamSynchronize(X.stream);
@@ -294,6 +301,37 @@ wpcd_status ws_reserve(wpcd_ctx *c, const Exec &X, Buf &b, size_t bytes)
     wpcd_status st = dmalloc(c, &b.p, bytes);
     if (st == WPCD_OK) b.n = bytes;
     return st;
+}
+
+// The side streams of an executor (never made inside a capture); false: go without.
+bool side_streams(Exec &X)
+{
+    if (X.ev_fork) return true;
+    if (capturing(X.stream)) return false;
+    for (int k = 0; k < kSides; ++k)
+        if ((!X.side[k] && cudaStreamCreateWithFlags(&X.side[k], cudaStreamNonBlocking) != cudaSuccess) ||
+            (!X.ev_join[k] && cudaEventCreateWithFlags(&X.ev_join[k], cudaEventDisableTiming) != cudaSuccess)) {
+            cudaGetLastError();
+            return false;
+        }
+    if (cudaEventCreateWithFlags(&X.ev_fork, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        X.ev_fork = nullptr;
+        return false;
+    }
+    return true;
+}
+
+void free_side_streams(Exec &X)
+{
+    for (int k = 0; k < kSides; ++k) {
+        if (X.side[k]) cudaStreamDestroy(X.side[k]);
+        if (X.ev_join[k]) cudaEventDestroy(X.ev_join[k]);
+        X.side[k] = nullptr;
+        X.ev_join[k] = nullptr;
+    }
+    if (X.ev_fork) cudaEventDestroy(X.ev_fork);
+    X.ev_fork = nullptr;
 }
 
 wpcd_status gl_rule(wpcd_ctx *c, int n, double **x, double **w)
@@ -560,6 +598,8 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
     }
     const size_t coeff_len = (size_t)S * std::max(v.n_terms - 1, 1);
     wpcd_status st = WPCD_OK;
+    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    if (v.buckets.size() > 1 && (long long)S * v.n_ch <= (long long)kForkItems * c->n_sm) side_streams(X);
     // grow-only storage: a smaller batch or another set with as many channels reuses it
     if (e.eps_len < eps_len || e.c_len < c_len || e.coeff_len < coeff_len || e.status_len < (size_t)S * v.n_ch ||
         e.cd_len < (size_t)v.n_ch) {
@@ -641,6 +681,35 @@ wpcd_status run_bucket_big(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
     return WPCD_OK;
 }
 
+// Scratch of a size bucket on the FP64 path, for chunks of samples: the refinement's,
+// the FP32 solver's eigenvectors or slots, the done flags.
+struct F64Scratch {
+    int nw;
+    bool big32, big64;
+    size_t ref_item, slot32, slot64, c_item;
+    int cap32, cap64;
+    F64Scratch(wpcd_ctx *c, int n, int nw_) : nw(nw_)
+    {
+        if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+        big32 = !jacobi_fits_smem(n, false);
+        big64 = !jacobi_fits_smem(n, true);
+        ref_item = refine64_scratch_per_item(n);
+        slot32 = big32 ? (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255 : 0;
+        slot64 = big64 ? (jacobi_big_scratch_bytes(n, true) + 255) & ~(size_t)255 : 0;
+        c_item = big32 || jacobi_mixed_c_in_smem(n) ? 0 : jacobi_mixed_c_bytes(n);
+        cap32 = c->n_sm * std::max(1, big32 ? jacobi_big_occupancy(n, false) : 1);
+        cap64 = c->n_sm * std::max(1, big64 ? jacobi_big_occupancy(n, true) : 1);
+        if (c->big_slots > 0) cap32 = cap64 = c->big_slots;
+    }
+    int slots32(int items) const { return big32 ? std::max(1, std::min(items, cap32)) : 0; }
+    size_t bytes(int ns) const
+    {
+        const size_t items = (size_t)ns * nw;
+        return ((ref_item * items + 255) & ~(size_t)255) +
+               ((c_item * items + slot32 * slots32((int)items) + 255) & ~(size_t)255) + sizeof(int) * items;
+    }
+};
+
 // A size bucket on the FP64 path: the FP32 Jacobi kernel, FP64 refinement
 // (refine64.cu), and the FP64 Jacobi kernel for the items that the refinement
 // does not bring to FP64.  Without room for the refinement's scratch (an HBM
@@ -650,21 +719,12 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
 {
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
     if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    const bool big32 = !jacobi_fits_smem(n, false), big64 = !jacobi_fits_smem(n, true);
-    const size_t ref_item = refine64_scratch_per_item(n);
-    const size_t slot32 = big32 ? (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255 : 0;
-    const size_t slot64 = big64 ? (jacobi_big_scratch_bytes(n, true) + 255) & ~(size_t)255 : 0;
-    const size_t c_item = big32 || jacobi_mixed_c_in_smem(n) ? 0 : jacobi_mixed_c_bytes(n);
-    int cap32 = c->n_sm * std::max(1, big32 ? jacobi_big_occupancy(n, false) : 1);
-    int cap64 = c->n_sm * std::max(1, big64 ? jacobi_big_occupancy(n, true) : 1);
-    if (c->big_slots > 0) cap32 = cap64 = c->big_slots;
-    // scratch of a chunk: the refinement's, the FP32 solver's eigenvectors or slots, the done flags
-    auto slots32 = [&](int items) { return big32 ? std::max(1, std::min(items, cap32)) : 0; };
-    auto bytes_of = [&](int ns) {
-        const size_t items = (size_t)ns * nw;
-        return ((ref_item * items + 255) & ~(size_t)255) + ((c_item * items + slot32 * slots32((int)items) + 255) & ~(size_t)255) +
-               sizeof(int) * items;
-    };
+    const F64Scratch sc(c, n, nw);
+    const size_t ref_item = sc.ref_item, c_item = sc.c_item, slot64 = sc.slot64;
+    const bool big32 = sc.big32, big64 = sc.big64;
+    const int cap64 = sc.cap64;
+    auto slots32 = [&](int items) { return sc.slots32(items); };
+    auto bytes_of = [&](int ns) { return sc.bytes(ns); };
     int chunk = (int)std::max<size_t>(1, kRefineScratchBytes / ((ref_item + c_item) * nw));
     chunk = std::min(chunk, std::max(1, 65535 / nw));  // the refinement grids put items in y / z (<= 65535)
     chunk = std::min(chunk, nsmp);
@@ -725,6 +785,61 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
     return WPCD_OK;
 }
 
+// Scratch that the whole of a size bucket takes in one chunk.
+size_t bucket_scratch(wpcd_ctx *c, int n, int nw, int S, int prec)
+{
+    if (prec == WPCD_PREC_FP64) return F64Scratch(c, n, nw).bytes(S);
+    const size_t ref_item = refine_scratch_per_item(n, c->refine_engine);
+    if (jacobi_fits_smem(n, false))
+        return (ref_item + (jacobi_mixed_c_in_smem(n) ? 0 : jacobi_mixed_c_bytes(n)) + 256) * nw * S;
+    const size_t slot_b = (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255;
+    int cap = c->n_sm * std::max(1, jacobi_big_occupancy(n, false));
+    if (c->big_slots > 0) cap = c->big_slots;
+    return ((ref_item * nw * S + 255) & ~(size_t)255) + slot_b * std::max(1, std::min(S * nw, cap));
+}
+
+// The size buckets of a small batch side by side on the executor's streams, each in its
+// own share of the scratch (false: the caller runs them one after another).  A bucket
+// of few matrices is one chain of latencies on few SMs, so the buckets' times add up to
+// the longest instead of their sum: see kForkItems for what it measured.
+template <class F>
+bool fork_buckets(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_bucket, std::vector<wpcd_status> &sts)
+{
+    if (c->prof || v.buckets.size() < 2 || (long long)S * v.n_ch > (long long)kForkItems * c->n_sm) return false;
+    if (c->autotune) {  // the autotuner times its candidates alone
+        std::lock_guard<std::mutex> lk(c->tmu);
+        for (auto &kv : v.buckets)
+            if (jacobi_fits_smem(kv.first, false) && !c->tuned.count(std::make_pair(kv.first, prec))) return false;
+    }
+    std::vector<size_t> off;
+    size_t total = 0;
+    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
+        off.push_back(total);
+        total += (bucket_scratch(c, it->first, (int)it->second.size(), S, prec) + 255) & ~(size_t)255;
+    }
+    off.push_back(total);
+    if (total > kRefineScratchBytes || !side_streams(X) || ws_reserve(c, X, X.ws_ref, total)) return false;
+    if (cudaEventRecord(X.ev_fork, X.stream) != cudaSuccess) return false;
+    const int sides = std::min<int>(kSides, (int)v.buckets.size() - 1);
+    for (int k = 0; k < sides; ++k) cudaStreamWaitEvent(X.side[k], X.ev_fork, 0);
+    int b = 0;
+    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it, ++b) {
+        Exec Y;
+        Y.stream = b == 0 ? X.stream : X.side[(b - 1) % sides];
+        Y.err = X.err;
+        Y.ws_ref.p = static_cast<unsigned char *>(X.ws_ref.p) + off[b];
+        Y.ws_ref.n = off[b + 1] - off[b];
+        Y.ws_ref.part = true;
+        sts.push_back(run_bucket(Y, v.bucket_dev[it->first], (int)it->second.size(), S, 0, it->first));
+    }
+    for (int k = 0; k < sides; ++k) {  // joined whatever the buckets returned
+        const bool ok = cudaEventRecord(X.ev_join[k], X.side[k]) == cudaSuccess &&
+                        cudaStreamWaitEvent(X.stream, X.ev_join[k], 0) == cudaSuccess;
+        sts.push_back(ok ? WPCD_OK : WPCD_ERR_CUDA);
+    }
+    return true;
+}
+
 // The parameter sum + eigensolve of the batch diag_prep set up (device-only
 // work on X.stream: capturable).  coeffs: device, [S][n_terms - 1].
 wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int S, int prec, EigH &e)
@@ -737,7 +852,7 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
     const double *cf = v.n_terms > 1 ? e.coeffs : nullptr;
     // Per size bucket (largest first, or per solve in plain mode), in sample chunks sized to
     // the refinement scratch: an FP32 Jacobi launch and the FP64 refinement.
-    auto run_bucket = [&](const int *work, int nw, int nsmp, int smp0, int n) -> wpcd_status {
+    auto run_bucket = [&](Exec &X, const int *work, int nw, int nsmp, int smp0, int n) -> wpcd_status {
         if (prec == WPCD_PREC_FP64) return run_bucket_f64(c, X, v, e, cf, work, nw, nsmp, smp0, n);
         if (!jacobi_fits_smem(n, false)) return run_bucket_big(c, X, v, e, cf, work, nw, nsmp, smp0, n);
         const int threads = pick_threads(c, X, n, prec, nw, nsmp, [&](int th, int ns) {
@@ -784,10 +899,14 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
         // one solve per launch: the baseline execution on the same GPU
         for (int s = 0; s < S; ++s)
             for (int k = 0; k < v.n_ch; ++k)
-                if ((st = run_bucket(v.ident_dev + k, 1, 1, s, v.cd[k].n))) return st;
+                if ((st = run_bucket(X, v.ident_dev + k, 1, 1, s, v.cd[k].n))) return st;
     } else {
-        for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it)
-            if ((st = run_bucket(v.bucket_dev[it->first], (int)it->second.size(), S, 0, it->first))) return st;
+        std::vector<wpcd_status> sts;
+        if (!fork_buckets(c, X, v, S, prec, run_bucket, sts))
+            for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it)
+                if ((st = run_bucket(X, v.bucket_dev[it->first], (int)it->second.size(), S, 0, it->first))) return st;
+        for (wpcd_status f : sts)
+            if (f) return f;
     }
     return WPCD_OK;
 }
@@ -938,6 +1057,7 @@ void wpcd_destroy(wpcd_ctx *c)
         dfree(c, kv.second.second);
     }
     Exec &M = c->main;
+    free_side_streams(M);
     for (auto *b : {&M.ws_plan_i, &M.ws_plan_d, &M.ws_tbin, &M.ws_phbin, &M.ws_in, &M.ws_out, &M.ws_ref}) dfree(c, b->p);
     dfree(c, c->err_dev);
     delete c;
@@ -2186,6 +2306,7 @@ void serve_shutdown(wpcd_ctx *c)
         dfree(c, sl.X.err);
         if (sl.pin_in) cudaFreeHost(sl.pin_in);
         if (sl.pin_out) cudaFreeHost(sl.pin_out);
+        free_side_streams(sl.X);
         cudaStreamDestroy(sl.X.stream);
     }
     c->server = nullptr;
