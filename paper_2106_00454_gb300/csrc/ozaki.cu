@@ -165,6 +165,82 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(int n, int Kp, const doub
     }
 }
 
+// Matrix b of a batch: back to back, or where an eigen buffer holds it.
+__device__ __forceinline__ const double *oz_item(const OzItems &src, const double *M_all, int b, int n)
+{
+    if (!src.chans) return M_all + (size_t)b * n * n;
+    return M_all + src.chans[src.work[b % src.nw]].c_off + (size_t)(src.sample0 + b / src.nw) * n * n;
+}
+
+// Row slices (seven digits) of V = V0 + sum_a c_a V_a for the bins that the energy
+// plan needs (row v belongs to bin v mod N; the other rows keep whatever the buffer
+// holds: a product's rows do not mix).  One warp per row, the sum in FP64 as the
+// eigensolvers form it.
+template <int PAIRS>
+__global__ void __launch_bounds__(256) k_oz_vsum(const ChanDev *chans, const int *work, int nw, int sample0, int n, int Kp,
+                                                 int n_terms, const double *coeffs, PlanDev plan, int n_ch, int maxN,
+                                                 int *e_all, __nv_bfloat16 *S_all)
+{
+    constexpr int P = kOzMaxDigits;
+    const int b = blockIdx.y, v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (v >= n) return;
+    const int c = work[b % nw], smp = sample0 + b / nw;
+    const ChanDev ch = chans[c];
+    const size_t pc = (size_t)plan_of(plan, smp) * n_ch + c;
+    const int *list = plan.list + pc * maxN, bin = v % ch.N;
+    int lo = 0, hi = plan.cnt[pc] - 1;  // ascending
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] < bin) lo = mid + 1;
+        else hi = mid;
+    }
+    if (hi < 0 || list[lo] != bin) {
+        if (lane == 0) e_all[(size_t)b * n + v] = 0;
+        return;
+    }
+    const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
+    const double *row = ch.V + (size_t)v * n;
+    double x0[PAIRS], x1[PAIRS];
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) {
+        const int k = 2 * lane + 64 * j;
+        x0[j] = k < n ? row[k] : 0.0;
+        x1[j] = k + 1 < n ? row[k + 1] : 0.0;
+    }
+    for (int t = 1; t < n_terms; ++t) {
+        const double ct = cf[t - 1], *rt = row + (size_t)t * n * n;
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {
+            const int k = 2 * lane + 64 * j;
+            if (k < n) x0[j] = fma(ct, rt[k], x0[j]);
+            if (k + 1 < n) x1[j] = fma(ct, rt[k + 1], x1[j]);
+        }
+    }
+    unsigned long long m = 0;
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) m = max(m, max(oz_mag(x0[j]), oz_mag(x1[j])));
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int ex = oz_exp_of(m);
+    if (lane == 0) e_all[(size_t)b * n + v] = ex;
+    __nv_bfloat16 *S = S_all + (size_t)b * P * n * Kp + (size_t)v * Kp;
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) {
+        const int k = 2 * lane + 64 * j;
+        if (k < Kp) oz_digits2<P>(x0[j], x1[j], ex, S + k, (size_t)n * Kp);
+    }
+}
+
+cudaError_t launch_oz_vsum(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, const PlanDev &plan, int n_ch, int maxN, __nv_bfloat16 *S, int *e,
+                           cudaStream_t st)
+{
+    const int Kp = oz_kpad(n);
+    const dim3 g((n + 7) / 8, n_samples * nw);
+    auto *k = Kp <= 256 ? k_oz_vsum<4> : Kp <= 512 ? k_oz_vsum<8> : k_oz_vsum<16>;
+    k<<<g, 256, 0, counted(st)>>>(chans, work, nw, sample0, n, Kp, n_terms, coeffs, plan, n_ch, maxN, e, S);
+    return cudaGetLastError();
+}
+
 // Column slices for Kp <= kOzColBlockKp: one CTA (32 x 8) per 32 columns reads
 // its Kp x 32 block once into shared memory (pitch 33 doubles; v fastest,
 // coalesced), takes the column maxima while loading, and writes the digits
@@ -172,7 +248,7 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(int n, int Kp, const doub
 constexpr int kOzColBlockKp = 384;  // 101 KB of shared memory at most
 template <int P>
 __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, const double *M_all, int *e_all,
-                                                             __nv_bfloat16 *S_all, OzSkip skip)
+                                                             __nv_bfloat16 *S_all, OzSkip skip, OzItems src)
 {
     if (oz_skipped(skip, blockIdx.y)) return;
     extern __shared__ double blk[];  // [Kp][33]
@@ -180,7 +256,7 @@ __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, cons
     __shared__ int ecol[32];
     const int b = blockIdx.y;
     const int v0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y, v = v0 + tx;
-    const double *M = M_all + (size_t)b * n * n;
+    const double *M = oz_item(src, M_all, b, n);
     unsigned long long m = 0;
 #pragma unroll 8
     for (int k = ty; k < Kp; k += 8) {
@@ -209,7 +285,7 @@ __global__ void __launch_bounds__(256) k_oz_split_cols_block(int n, int Kp, cons
 // writes (k fastest, two per thread) are coalesced.
 template <int P>
 __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const double *M_all, int *e_all,
-                                                       __nv_bfloat16 *S_all, OzSkip skip)
+                                                       __nv_bfloat16 *S_all, OzSkip skip, OzItems src)
 {
     if (oz_skipped(skip, blockIdx.y)) return;
     __shared__ double tile[64][33];
@@ -217,7 +293,7 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const doub
     __shared__ int ecol[32];
     const int b = blockIdx.y;
     const int v0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
-    const double *M = M_all + (size_t)b * n * n;
+    const double *M = oz_item(src, M_all, b, n);
     unsigned long long m = 0;
     if (v0 + tx < n)
         for (int k = ty; k < n; k += 8) m = max(m, oz_mag(M[(size_t)k * n + v0 + tx]));
@@ -248,7 +324,7 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(int n, int Kp, const doub
 // n x n matrices: S [items][P][n][Kp] bf16, e [items][n], P = planes digits.
 template <int P>
 static cudaError_t oz_split_p(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
-                              OzSkip skip)
+                              OzSkip skip, OzItems src)
 {
     const int Kp = oz_kpad(n);
     if (!cols) {
@@ -261,21 +337,22 @@ static cudaError_t oz_split_p(int n, int items, bool cols, const double *M, __nv
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_oz_split_cols_block<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kOzColBlockKp * 33 * (int)sizeof(double));
-        k_oz_split_cols_block<P><<<dim3((n + 31) / 32, items), dim3(32, 8), smem, counted(st)>>>(n, Kp, M, e, S, skip);
+        k_oz_split_cols_block<P><<<dim3((n + 31) / 32, items), dim3(32, 8), smem, counted(st)>>>(n, Kp, M, e, S, skip, src);
     } else {
-        k_oz_split_cols<P><<<dim3((n + 31) / 32, items), dim3(32, 8), 0, counted(st)>>>(n, Kp, M, e, S, skip);
+        k_oz_split_cols<P><<<dim3((n + 31) / 32, items), dim3(32, 8), 0, counted(st)>>>(n, Kp, M, e, S, skip, src);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
-                            OzSkip skip, int planes)
+                            OzSkip skip, int planes, OzItems src)
 {
+    if (src.chans && !cols) return cudaErrorInvalidValue;
     switch (planes) {
-    case 4: return oz_split_p<4>(n, items, cols, M, S, e, st, skip);
-    case 5: return oz_split_p<5>(n, items, cols, M, S, e, st, skip);
-    case 6: return oz_split_p<6>(n, items, cols, M, S, e, st, skip);
-    case 7: return oz_split_p<7>(n, items, cols, M, S, e, st, skip);
+    case 4: return oz_split_p<4>(n, items, cols, M, S, e, st, skip, src);
+    case 5: return oz_split_p<5>(n, items, cols, M, S, e, st, skip, src);
+    case 6: return oz_split_p<6>(n, items, cols, M, S, e, st, skip, src);
+    case 7: return oz_split_p<7>(n, items, cols, M, S, e, st, skip, src);
     }
     return cudaErrorInvalidValue;
 }
@@ -299,6 +376,37 @@ cudaError_t launch_oz_gemm(int n, int items, bool ta, const double *A, const dou
     if ((e = launch_oz_split(n, items, ta, A, sa, ea, st))) return e;
     if ((e = launch_oz_split(n, items, true, B, sb, eb, st))) return e;
     return launch_oz_gemm_slices(n, items, sa, ea, sb, eb, C, st, kOzDigits, false, err);
+}
+
+// The rows of V C that the energy plan needs, for a bucket's items: 55-bit products of
+// V's rows and the columns of the eigenvectors in C_all, in `scratch`
+// (vc_rows_scratch_per_item bytes an item).
+size_t vc_rows_scratch_per_item(int n)
+{
+    return (size_t)n * n * 8 + 2 * (oz_slice_elems(n, kOzMaxDigits) * 2 + (size_t)n * 4) + 512;
+}
+
+cudaError_t launch_vc_rows(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, const double *C_all, const PlanDev &plan, int n_ch, int maxN,
+                           void *scratch, const double **rows, int *err, cudaStream_t st)
+{
+    constexpr int P = kOzMaxDigits;
+    const int items = n_samples * nw;
+    double *R = static_cast<double *>(scratch);
+    const uintptr_t s0 = (reinterpret_cast<uintptr_t>(R + (size_t)items * n * n) + 255) & ~(uintptr_t)255;
+    __nv_bfloat16 *sV = reinterpret_cast<__nv_bfloat16 *>(s0), *sC = sV + (size_t)items * oz_slice_elems(n, P);
+    int *eV = reinterpret_cast<int *>(sC + (size_t)items * oz_slice_elems(n, P)), *eC = eV + (size_t)items * n;
+    cudaError_t e = launch_oz_vsum(chans, work, nw, n_samples, sample0, n, n_terms, coeffs, plan, n_ch, maxN, sV, eV, st);
+    if (e != cudaSuccess) return e;
+    OzItems src;
+    src.chans = chans;
+    src.work = work;
+    src.nw = nw;
+    src.sample0 = sample0;
+    e = launch_oz_split(n, items, true, C_all, sC, eC, st, OzSkip(), P, src);
+    if (e != cudaSuccess) return e;
+    *rows = R;
+    return launch_oz_gemm_slices(n, items, sV, eV, sC, eC, R, st, P, false, err, 0, nullptr, OzSkip(), P);
 }
 
 }  // namespace wpcd

@@ -44,6 +44,8 @@ constexpr int kRefineIters = 2;                            // FP64 refinement it
 // angle and its share of the diagonal are below 2^-18, which two refinement iterations
 // take to FP64 (2^-16 makes a third one common at n = 300).
 constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
+constexpr size_t kVcScratchBytes = (size_t)8 << 30;  // FP64 T: scratch of the rows of V C, per chunk
+constexpr int kVcRowsN = 48;                         // ... for matrices from this size on
 // Batches up to this many solves per SM run their size buckets side by side.
 constexpr int kForkItems = 8;
 constexpr size_t kGraphCache = 64;                         // wpcd_solve keys remembered for CUDA graphs
@@ -948,8 +950,39 @@ wpcd_status run_tbin(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *e_la
     Launch L(c, X, WPCD_PHASE_TMATRIX);
     const double *cf = v.n_terms > 1 ? e.coeffs : nullptr;
     double *tb = static_cast<double *>(X.ws_tbin.p), *pb = static_cast<double *>(X.ws_phbin.p);
-    CK(launch_tbin(e.cd_dev, nch, S, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream,
-                   e.prec == WPCD_PREC_MIXED, res));
+    if (e.prec == WPCD_PREC_MIXED) {
+        CK(launch_tbin(e.cd_dev, nch, S, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, true, res));
+        return WPCD_OK;
+    }
+    // FP64: per size bucket, in sample chunks, the needed rows of V C from the tensor cores, then T;
+    // a bucket of small matrices, or without room for the rows, forms them in the T kernel
+    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
+        const int n = it->first, nw = (int)it->second.size();
+        const size_t per = vc_rows_scratch_per_item(n);
+        int chunk = 0;
+        if (n >= kVcRowsN) {
+            chunk = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, kVcScratchBytes / (per * nw)));
+            chunk = std::min(chunk, std::max(1, 65535 / nw));  // items in the grid's y
+            while (chunk > 0 && ws_reserve(c, X, X.ws_ref, per * nw * chunk)) chunk /= 2;
+        }
+        TWork tw;
+        tw.work = v.bucket_dev[n];
+        tw.n_work = nw;
+        tw.n = n;
+        if (chunk == 0) {
+            CK(launch_tbin(e.cd_dev, nch, S, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, false,
+                           res, tw));
+            continue;
+        }
+        for (int s0 = 0; s0 < S; s0 += chunk) {
+            const int ns = std::min(chunk, S - s0);
+            tw.sample0 = s0;
+            CK(launch_vc_rows(e.cd_dev, tw.work, nw, ns, s0, n, v.n_terms, cf, e.C, plan, nch, maxN, X.ws_ref.p, &tw.rows,
+                              X.err, X.stream));
+            CK(launch_tbin(e.cd_dev, nch, ns, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, false,
+                           res, tw));
+        }
+    }
     return WPCD_OK;
 }
 

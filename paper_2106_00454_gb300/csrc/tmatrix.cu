@@ -136,22 +136,34 @@ __device__ __forceinline__ double xlogabs(double d) { return d == 0.0 ? 0.0 : d 
 //    channels).
 // Averaged modes visit the needed bins in ascending order, so the X(E_{i+1}, B)
 // of one bin are the X(E_i, B) of the next whenever the bins are adjacent.
-// VCID: the VC rows from the eigen-equation.  H0 is diagonal in the free
+// VC = kVcIdentity: the VC rows from the eigen-equation.  H0 is diagonal in the free
 // packet basis, so V C = H C - H0 C = C diag(e) - H0 C, i.e.
 //     R_as = C_(a,i),s (e_s - h0_i),
 // exact for exact eigenpairs; its error is the eigen residual (~u ||H||
 // absolute).  Used on the mixed path, whose eigenpairs are refined to FP64
-// residuals; the FP64 path keeps the explicit products (their error scales with
-// ||V|| rather than ||H||, which holds the relative accuracy of small T).
+// residuals; the FP64 path keeps the product V C (its error scales with ||V||
+// rather than ||H||, which holds the relative accuracy of small T): kVcRows takes its
+// rows from memory, where the tensor cores left them as 55-bit products of V's rows
+// and C's columns (launch_vc_rows), kVcExplicit forms them here, K n^2 multiply-adds a
+// bin on the FP64 pipe, for callers without room for the rows.  T phase, explicit and one
+// CTA a solve -> rows and shares: 20 channels at N_WP = 150, 8 samples 5.68 -> 0.68 ms; at
+// N_WP = 100, one sample 1.35 -> 0.15 ms; 15 channels N_WP 40/64/100, 256 samples 5.9 -> 3.7 ms.
+// The CTAs of a (sample, channel) (gridDim.y) take consecutive shares of its items: one
+// CTA walks them one after another, which leaves the chip idle for a few solves.
 // Output, 8 doubles (complex 2 x 2) and 3 phases per item: modes 0, 1 at
 // [S][n_ch][stride = maxN][bin], mode 2 at [S][n_ch][stride = n_E][energy].
 // ---------------------------------------------------------------------------------------------
-template <bool VCID, int MODE>
+enum { kVcExplicit = 0, kVcIdentity = 1, kVcRows = 2 };
+
+template <int VC, int MODE>
 __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int n_ch, int n_terms, const double *coeffs,
                                                     const double *eps_all, const double *C_all, PlanDev plan,
-                                                    int n_E, int stride, double *tout, double *phout, int *err)
+                                                    int n_E, int stride, double *tout, double *phout, int *err,
+                                                    const TWork tw)
 {
-    const int c = blockIdx.x % n_ch, smp = blockIdx.x / n_ch;
+    constexpr bool VCID = VC == kVcIdentity;
+    const int nwk = tw.work ? tw.n_work : n_ch;
+    const int c = tw.work ? tw.work[blockIdx.x % nwk] : blockIdx.x % nwk, smp = tw.sample0 + blockIdx.x / nwk;
     const ChanDev ch = chans[c];
     const int n = ch.n, N = ch.N, K = ch.K;
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -184,7 +196,9 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
     const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
     const int ps = plan_of(plan, smp);
     const size_t pc = (size_t)ps * n_ch + c;
-    const int cnt = MODE == 2 ? plan_nE(plan, ps, n_E) : plan.cnt[pc];
+    const int cnt_all = MODE == 2 ? plan_nE(plan, ps, n_E) : plan.cnt[pc];
+    const int share = (cnt_all + gridDim.y - 1) / gridDim.y;  // this CTA's items [ii0, cnt)
+    const int ii0 = blockIdx.y * share, cnt = min(cnt_all, ii0 + share);
     const size_t obase = ((size_t)smp * n_ch + c) * stride;
 
     if (tid == 0) { s_nb = 0; s_bad = 0; }
@@ -195,7 +209,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
     __syncthreads();
     const int nb = s_nb, P = n - nb;
     if (MODE == 1 && (K != 1 || nb != 0)) {  // SWP-bin averaging is defined for these only
-        for (int ii = tid; ii < cnt; ii += nt) {
+        for (int ii = ii0 + tid; ii < cnt; ii += nt) {
             const int i = plan.list[pc * stride + ii];
             for (int k = 0; k < 8; ++k) tout[(obase + i) * 8 + k] = __longlong_as_double(0x7ff8000000000000ll);
             for (int k = 0; k < 3; ++k) phout[(obase + i) * 3 + k] = __longlong_as_double(0x7ff8000000000000ll);
@@ -246,7 +260,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
     __syncthreads();
 
     if (MODE != 2) {
-        for (int ii = tid; ii < cnt; ii += nt) {
+        for (int ii = ii0 + tid; ii < cnt; ii += nt) {
             const int i = plan.list[pc * stride + ii];
             double a, b;
             if (MODE == 1) {
@@ -271,7 +285,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
 
     const int dstride = (K == 2) ? (n >> 1) + 2 : n + 1;  // boundary slots per branch (K * dstride <= n + 4)
     int prev = -2;                                          // bin whose upper-edge X values sit in XB
-    for (int ii = 0; ii < cnt; ++ii) {
+    for (int ii = ii0; ii < cnt; ++ii) {
         int i;
         double Ea = 0.0, Ebn = 0.0, E = 0.0, p = 0.0;
         if (MODE == 2) {
@@ -285,9 +299,10 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
         }
         // this bin's eigenvector rows, first element per thread issued early so
         // that the load overlaps the logarithms below
-        const double *C0 = C + (size_t)i * n, *C1 = C + (size_t)(N + i) * n;
+        const double *Cv = VC == kVcRows ? tw.rows + (size_t)blockIdx.x * n * n : C;
+        const double *C0 = Cv + (size_t)i * n, *C1 = Cv + (size_t)(N + i) * n;
         double c0pre = 0.0, c1pre = 0.0;
-        if (VCID && tid < n) {
+        if (VC != kVcExplicit && tid < n) {
             c0pre = C0[tid];
             if (K == 2) c1pre = C1[tid];
         }
@@ -295,7 +310,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
         // forms entry w, lane l its terms l, l + 32, ... (loads in flight during the
         // logarithms below, summed with a butterfly after them)
         double vterm = 0.0;
-        if (VCID && (tid >> 5) < K * K) {
+        if (VC != kVcExplicit && (tid >> 5) < K * K) {
             const int w = tid >> 5, a = w / K, bb = w - a * K;
             const size_t off = (size_t)(a * N + i) * n + bb * N + i;
             for (int t = tid & 31; t < n_terms; t += 32) {
@@ -322,7 +337,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
                 }
             }
         }
-        if (VCID) {
+        if (VC != kVcExplicit) {
             if ((tid >> 5) < K * K) {  // warp-uniform
                 for (int o = 16; o > 0; o >>= 1) vterm += __shfl_xor_sync(0xffffffffu, vterm, o);
                 if ((tid & 31) == 0) vd[tid >> 5] = vterm;
@@ -349,7 +364,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
         // thread 0 keeps the diagonal V entries in registers: the next item rewrites them
         double v00 = 0.0, v01 = 0.0, v10 = 0.0, v11 = 0.0;
         if (tid == 0) {
-            if (VCID) {
+            if (VC != kVcExplicit) {
                 v00 = vd[0];
                 if (K == 2) { v01 = vd[1]; v10 = vd[2]; v11 = vd[3]; }
             } else {
@@ -383,6 +398,9 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
                 const double de = eps[s] - h0i;
                 r0 = (s == tid ? c0pre : C0[s]) * de;
                 if (K == 2) r1 = (s == tid ? c1pre : C1[s]) * de;
+            } else if (VC == kVcRows) {
+                r0 = s == tid ? c0pre : C0[s];
+                if (K == 2) r1 = s == tid ? c1pre : C1[s];
             } else {
                 r0 = R[s];
                 if (K == 2) r1 = R[n + s];
@@ -452,7 +470,7 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
     // S and the phases of every item, one item per thread (their T were
     // written above by thread 0 of this CTA)
     __syncthreads();
-    for (int ii = tid; ii < cnt; ii += nt) {
+    for (int ii = ii0 + tid; ii < cnt; ii += nt) {
         const int slot = MODE == 2 ? ii : plan.list[pc * stride + ii];
         const int i = MODE == 2 ? plan.bin[pc * n_E + ii] : slot;
         const double q = MODE == 2 ? plan.pE[(size_t)ps * n_E + ii] : ip_point(ch.kb, i, plan.ip_frac);
@@ -462,34 +480,49 @@ __global__ void __launch_bounds__(kTThreads, 5) k_tmat(const ChanDev *chans, int
 
 size_t tbin_smem_bytes(int nmax) { return tbin_smem_doubles(nmax) * sizeof(double); }
 
-template <bool VCID, int MODE>
+template <int VC, int MODE>
 static void launch_tmat_t(const ChanDev *chans_dev, int n_ch, int n_samples, int n_terms, const double *coeffs,
                           const double *eps_all, const double *C_all, PlanDev plan, int n_E, int stride,
-                          size_t smem, double *tout, double *phout, int *err, cudaStream_t st)
+                          size_t smem, double *tout, double *phout, int *err, cudaStream_t st, TWork tw)
 {
-    raise_smem_limit((const void *)k_tmat<VCID, MODE>, smem);
-    k_tmat<VCID, MODE><<<(unsigned)(n_samples * n_ch), kTThreads, smem, counted(st)>>>(chans_dev, n_ch, n_terms, coeffs, eps_all,
-                                                                              C_all, plan, n_E, stride, tout, phout,
-                                                                              err);
+    raise_smem_limit((const void *)k_tmat<VC, MODE>, smem);
+    // shares per solve: the chip holds five CTAs an SM; a share below four items costs more in the
+    // boundaries that each CTA forms than it gains
+    static int sms = 0;
+    if (sms == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms <= 0) sms = 1;
+    }
+    const long long solves = (long long)n_samples * (tw.work ? tw.n_work : n_ch);
+    const int most = (MODE == 2 ? n_E : min(stride, 2 * n_E + 2)) / 4;
+    const int shares = (int)max(1ll, min((long long)most, 5ll * sms / solves));
+    k_tmat<VC, MODE><<<dim3((unsigned)solves, shares), kTThreads, smem, counted(st)>>>(
+        chans_dev, n_ch, n_terms, coeffs, eps_all, C_all, plan, n_E, stride, tout, phout, err, tw);
 }
 
 cudaError_t launch_tbin(const ChanDev *chans_dev, int n_ch, int n_samples, int n_terms, const double *coeffs,
                         const double *eps_all, const double *C_all, PlanDev plan, int maxN, int n_E, double *tout,
-                        double *phout, int *err, cudaStream_t st, bool vc_identity, int mode)
+                        double *phout, int *err, cudaStream_t st, bool vc_identity, int mode, TWork tw)
 {
-    if (mode < 0 || mode > 2) return cudaErrorInvalidValue;
-    const size_t smem = tbin_smem_bytes(2 * maxN);
+    if (mode < 0 || mode > 2 || (vc_identity && tw.rows) || (tw.work && tw.n < 1)) return cudaErrorInvalidValue;
+    const size_t smem = tbin_smem_bytes(tw.work ? tw.n : 2 * maxN);
     const int stride = mode == 2 ? n_E : maxN;
 #define WPCD_TMAT(V, M) \
-    launch_tmat_t<V, M>(chans_dev, n_ch, n_samples, n_terms, coeffs, eps_all, C_all, plan, n_E, stride, smem, tout, phout, err, st)
+    launch_tmat_t<V, M>(chans_dev, n_ch, n_samples, n_terms, coeffs, eps_all, C_all, plan, n_E, stride, smem, tout, phout, err, st, tw)
     if (vc_identity) {
-        if (mode == 0) WPCD_TMAT(true, 0);
-        else if (mode == 1) WPCD_TMAT(true, 1);
-        else WPCD_TMAT(true, 2);
+        if (mode == 0) WPCD_TMAT(kVcIdentity, 0);
+        else if (mode == 1) WPCD_TMAT(kVcIdentity, 1);
+        else WPCD_TMAT(kVcIdentity, 2);
+    } else if (tw.rows) {
+        if (mode == 0) WPCD_TMAT(kVcRows, 0);
+        else if (mode == 1) WPCD_TMAT(kVcRows, 1);
+        else WPCD_TMAT(kVcRows, 2);
     } else {
-        if (mode == 0) WPCD_TMAT(false, 0);
-        else if (mode == 1) WPCD_TMAT(false, 1);
-        else WPCD_TMAT(false, 2);
+        if (mode == 0) WPCD_TMAT(kVcExplicit, 0);
+        else if (mode == 1) WPCD_TMAT(kVcExplicit, 1);
+        else WPCD_TMAT(kVcExplicit, 2);
     }
 #undef WPCD_TMAT
     return cudaGetLastError();

@@ -291,6 +291,12 @@ __device__ __forceinline__ bool oz_skipped(const OzSkip &sk, int b)
     const int d = sk.done[b];
     return d != 0 && d <= sk.it;
 }
+// The eigenvector matrices of a bucket's items inside an eigen buffer.
+struct OzItems {
+    const ChanDev *chans = nullptr;
+    const int *work = nullptr;
+    int nw = 0, sample0 = 0;
+};
 constexpr int kOzDigits = 6;  // balanced 8-bit digits per operand of the Ozaki products (mixed path)
 constexpr int kOzMaxDigits = 7;
 size_t oz_slice_elems(int n, int planes = kOzDigits);
@@ -298,7 +304,10 @@ int oz_kpad(int n);
 cudaError_t launch_oz_gemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                            __nv_bfloat16 *sa, __nv_bfloat16 *sb, int *ea, int *eb, cudaStream_t st, int *err = nullptr);
 cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_bfloat16 *S, int *e, cudaStream_t st,
-                            OzSkip skip = OzSkip(), int planes = kOzDigits);
+                            OzSkip skip = OzSkip(), int planes = kOzDigits, OzItems src = OzItems());
+cudaError_t launch_oz_vsum(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, const PlanDev &plan, int n_ch, int maxN, __nv_bfloat16 *S, int *e,
+                           cudaStream_t st);
 cudaError_t launch_oz_gemm_slices(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
                                   const int *eb, double *C, cudaStream_t st, int digits = 6, bool sym = false,
                                   int *err = nullptr, int a_items = 0, const double *Cadd = nullptr,
@@ -320,11 +329,23 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
 cudaError_t launch_batched_dgemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                                  void *scratch, int engine, cudaStream_t st, int *err = nullptr);
 size_t batched_dgemm_scratch(int n, int items);
+// A T launch over the channels of a work list from sample0 on (work == NULL: every channel),
+// with the rows of V C [item][n][n] where they are there, items channel-fastest.
+struct TWork {
+    const int *work = nullptr;
+    int n_work = 0, sample0 = 0;
+    int n = 0;  // their matrix size (sizes the shared memory)
+    const double *rows = nullptr;
+};
+size_t vc_rows_scratch_per_item(int n);
+cudaError_t launch_vc_rows(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, const double *C_all, const PlanDev &plan, int n_ch, int maxN,
+                           void *scratch, const double **rows, int *err, cudaStream_t st);
 cudaError_t launch_plan(const ChanDev *chans_dev, int n_ch, int maxN, const double *e_lab, int n_E, PlanDev plan,
                         int *err, cudaStream_t st, int n_plans = 1);
 cudaError_t launch_tbin(const ChanDev *chans_dev, int n_ch, int n_samples, int n_terms, const double *coeffs,
                         const double *eps_all, const double *C_all, PlanDev plan, int maxN, int n_E, double *tout,
-                        double *phout, int *err, cudaStream_t st, bool vc_identity, int mode);
+                        double *phout, int *err, cudaStream_t st, bool vc_identity, int mode, TWork tw = TWork());
 cudaError_t launch_saclay(const SacChanDev *chans_dev, int n_ch, int n_samples, int n_E, const double *e_lab,
                           const double *delta, int n_th, const double *theta, double *abcde, double *dsig, int Lmax,
                           cudaStream_t st);
