@@ -375,11 +375,15 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
 // 51.5 -> 44.5, n = 200 (512 threads) 19.9 -> 18.6, n = 180 16.5 -> 14.3; n = 150 14.5 -> 18.8 and
 // n = 128 6.2 -> 6.4, where several smaller CTAs share an SM and already overlap.
 // The slot-pair table of k_jacobi_mixed gives way to the lists.
+//
+// Sparse rounds (few slots rotate: half of a solve's time at n = 300) deal the 32-slot
+// pieces of the rotating slots' rows out over all matrix warps, and a block whose other
+// slot stays put takes only the row rotation: its slot's c and s' are not even read.
 
-// A float [mix_a_floats] | slot records uint4 [h] {c, s', a | b << 16, mcol(a) | mcol(b) << 16} |
-// the rotations of two rounds for the eigenvectors uint4 [2][h] {c, s', a | b << 16, -} |
-// a_aa', a_bb' float [h] each | flags int [12] | rank of each slot among the round's rotating
-// slots int [h] | rotating slots ushort [h, even]
+// A float [mix_a_floats] | the rotations of two rounds for the eigenvectors uint4 [2][h] {c, s',
+// a | b << 16, -} | slots uint2 [h] {a | b << 16, mcol(a) | mcol(b) << 16} | their rotations float2 [h]
+// {c, s'} | a_aa', a_bb' float [h] each | flags int [12] | rank of each slot among the round's
+// rotating slots int [h] | rotating slots ushort [h, even]
 __host__ __device__ inline size_t teams_smem(int n)
 {
     const int h = mpad(n) / 2;
@@ -460,13 +464,13 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
     extern __shared__ float4 smem_f4[];
     unsigned char *sb = reinterpret_cast<unsigned char *>(smem_f4);
     float *A = reinterpret_cast<float *>(sb);
-    // one 16-byte record a slot (one shared-memory load): the rotation of the pair (a, b) in
-    // tournament order, J = [[c, s'], [-s', c]] on (a, b), s' = s when a < b and -s otherwise
-    // (the rotation of the sorted pair (p, q) seen with its indices swapped), then a | b << 16
-    // and the column starts mcol(a) | mcol(b) << 16 (A has fewer than 2^16 floats)
-    uint4 *rec = reinterpret_cast<uint4 *>(A + mix_a_floats(n));
-    uint4 *list = rec + h;  // [2][h]
-    float *daa = reinterpret_cast<float *>(list + 2 * h), *dbb = daa + h;
+    // slot k's pair (a, b) in tournament order with its column starts (A has fewer than 2^16
+    // floats), and its rotation J = [[c, s'], [-s', c]] on (a, b), s' = s when a < b and -s
+    // otherwise (the rotation of the sorted pair (p, q) seen with its indices swapped)
+    uint4 *list = reinterpret_cast<uint4 *>(A + mix_a_floats(n));  // [2][h]
+    uint2 *geo = reinterpret_cast<uint2 *>(list + 2 * h);
+    float2 *cs = reinterpret_cast<float2 *>(geo + h);
+    float *daa = reinterpret_cast<float *>(cs + h), *dbb = daa + h;
     // flags: [0] rotation in this sweep; [4..6] the round's count of rotating slots, cycled over
     // three rounds; [8..9] the number of rotations in each list (-1: no more)
     int *flags = reinterpret_cast<int *>(dbb + h);
@@ -532,21 +536,25 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
                 P2 = P + (h >> 1);
             }
         };
-        // 2 x 2 block B of A in rows (a, b) of the slot of record r1 and columns (a, b) of the slot
-        // of record r2: J_1^T B J_2
-        auto quad_update = [&](const uint4 r1, const uint4 r2) {
-            const int ua = (int)(r1.z & 0xFFFFu), ub = (int)(r1.z >> 16), va = (int)(r2.z & 0xFFFFu), vb = (int)(r2.z >> 16);
-            const int sua = (int)(r1.w & 0xFFFFu), sub = (int)(r1.w >> 16), sva = (int)(r2.w & 0xFFFFu), svb = (int)(r2.w >> 16);
+        // 2 x 2 block B of A in rows (a, b) of slot P and columns (a, b) of slot P2: J_P^T B J_P2, J_P2
+        // the identity unless `both`
+        auto quad_update = [&](const uint2 g1, const float2 j1, const uint2 g2, const float2 j2, bool both) {
+            const int ua = (int)(g1.x & 0xFFFFu), ub = (int)(g1.x >> 16), va = (int)(g2.x & 0xFFFFu), vb = (int)(g2.x >> 16);
+            const int sua = (int)(g1.y & 0xFFFFu), sub = (int)(g1.y >> 16), sva = (int)(g2.y & 0xFFFFu), svb = (int)(g2.y >> 16);
             // element (x, y) at mcol(max) + min
             const int i00 = ua <= va ? sva + ua : sua + va;
             const int i01 = ua <= vb ? svb + ua : sua + vb;
             const int i10 = ub <= va ? sva + ub : sub + va;
             const int i11 = ub <= vb ? svb + ub : sub + vb;
             const float b00 = A[i00], b01 = A[i01], b10 = A[i10], b11 = A[i11];
-            const float c = __uint_as_float(r1.x), s = __uint_as_float(r1.y);
-            const float c2 = __uint_as_float(r2.x), s2 = __uint_as_float(r2.y);
-            const float x00 = c2 * b00 - s2 * b01, x01 = s2 * b00 + c2 * b01;
-            const float x10 = c2 * b10 - s2 * b11, x11 = s2 * b10 + c2 * b11;
+            const float c = j1.x, s = j1.y, c2 = j2.x, s2 = j2.y;
+            float x00 = b00, x01 = b01, x10 = b10, x11 = b11;
+            if (both) {
+                x00 = c2 * b00 - s2 * b01;
+                x01 = s2 * b00 + c2 * b01;
+                x10 = c2 * b10 - s2 * b11;
+                x11 = s2 * b10 + c2 * b11;
+            }
             A[i00] = c * x00 - s * x10;
             A[i01] = c * x01 - s * x11;
             A[i10] = s * x00 + c * x10;
@@ -611,8 +619,8 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
                     } else {
                         rank[k] = -1;
                     }
-                    rec[k] = make_uint4(__float_as_uint(c), __float_as_uint(ab ? s : -s), (unsigned)a | ((unsigned)b << 16),
-                                        (unsigned)ca | ((unsigned)cb << 16));
+                    geo[k] = make_uint2((unsigned)a | ((unsigned)b << 16), (unsigned)ca | ((unsigned)cb << 16));
+                    cs[k] = make_float2(c, ab ? s : -s);
                     daa[k] = ab ? app : aqq;
                     dbb[k] = ab ? aqq : app;
                 }
@@ -626,33 +634,44 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
                         for (int e = tid; e < nq; e += nta) {
                             int P, P2;
                             slot_pair(e, P, P2);
-                            const uint4 r1 = rec[P], r2 = rec[P2];
+                            const float2 j1 = cs[P], j2 = cs[P2];
                             // both rotations the identity (s' = +-0)
-                            if (__uint_as_float(r1.y) == 0.0f && __uint_as_float(r2.y) == 0.0f) continue;
-                            quad_update(r1, r2);
+                            if (j1.y == 0.0f && j2.y == 0.0f) continue;
+                            quad_update(geo[P], j1, geo[P2], j2, true);
                         }
                     } else {
-                        // few slots rotate (late sweeps, threshold sweeps): only the pairs that
-                        // hold a rotating slot, one warp per rotating slot P, lanes over the
-                        // others, rows from P's pair; a pair of two rotating slots is done
-                        // once, by the lower one's warp.  A pair with a non-rotating slot
-                        // gives the same bits in either orientation (the identity's c = 1,
-                        // s' = +-0 leave its side exact), so the result does not depend on
-                        // the order of the rotating list.
-                        for (int i = warp; i < na; i += nwarps) {
-                            const int P = act[i];
-                            const uint4 r1 = rec[P];
-                            for (int P2 = lane; P2 < h; P2 += 32) {
-                                if (P2 == P || (P2 < P && rank[P2] >= 0)) continue;
-                                quad_update(r1, rec[P2]);
+                        // few slots rotate (late sweeps, threshold sweeps): only the pairs that hold a
+                        // rotating slot P, rows from P's pair, a piece of 32 other slots a warp; a pair
+                        // of two rotating slots is done once, from the lower one.  A pair with a
+                        // non-rotating slot gives the same bits in either orientation, so the result
+                        // does not depend on the order of the rotating list.
+                        const int np = (h + 31) >> 5, di = nwarps / np, dq = nwarps - di * np;
+                        int i = warp / np, q = warp - i * np;
+                        while (i < na) {
+                            const int P = act[i], P2 = q * 32 + lane;
+                            const uint2 g1 = geo[P];
+                            const float2 j1 = cs[P];
+                            if (P2 < h && P2 != P) {
+                                const bool both = rank[P2] >= 0;
+                                if (!both || P2 > P) {
+                                    float2 j2 = make_float2(1.0f, 0.0f);
+                                    if (both) j2 = cs[P2];
+                                    quad_update(g1, j1, geo[P2], j2, both);
+                                }
+                            }
+                            i += di;
+                            q += dq;
+                            if (q >= np) {
+                                q -= np;
+                                ++i;
                             }
                         }
                     }
                     for (int i = tid; i < na; i += nta) {
                         const int k = act[i];
-                        const uint4 rk = rec[k];
-                        const int a = (int)(rk.z & 0xFFFFu), b = (int)(rk.z >> 16);
-                        const int ca = (int)(rk.w & 0xFFFFu), cb = (int)(rk.w >> 16);
+                        const uint2 g = geo[k];
+                        const int a = (int)(g.x & 0xFFFFu), b = (int)(g.x >> 16);
+                        const int ca = (int)(g.y & 0xFFFFu), cb = (int)(g.y >> 16);
                         A[ca + a] = daa[k];
                         A[cb + b] = dbb[k];
                         A[a < b ? cb + a : ca + b] = 0.0f;
