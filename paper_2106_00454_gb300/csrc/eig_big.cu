@@ -25,6 +25,14 @@
 //      (a_pp', 0; 0, a_qq').  The same phase rotates columns p, q of Cc.
 // Different row pairs touch disjoint rows, so phase 2 needs no atomics.
 //
+// A round is bound by what one SM can move to and from the L2 (A and Cc are read and
+// written whole in a dense round, 4 MB at n = 512 in FP32, ~65 bytes a clock), so
+// where the items leave SMs idle a cluster of 2, 4 or 8 CTAs shares one matrix: every
+// CTA finds the round's rotations for itself, and the row pairs are dealt out over the
+// cluster's warps.  A and Cc then pass through the L2 (loads that skip the L1) and
+// cluster barriers stand around phase 2.  Same operations, same bits.  16 samples x
+// 15 channels at N_WP = 256 (64 matrices of n = 512: clusters of two): a call 125.5 -> 73.0 ms.
+//
 // FP64 (T = double): a pair rotates whenever a_pq != 0; sweeps stop when
 // off(A) <= 1e-15 ||H||_F (as the shared-memory FP64 kernel).  Eigenvalues
 // leave sorted ascending, eigenvectors permuted alike, in the eigen-buffer
@@ -34,6 +42,7 @@
 // |a_pq| > 2^-23 sqrt|a_pp a_qq| (plus a threshold in the first two sweeps);
 // sweeps stop after a sweep without rotations.  Eigenpairs leave unsorted as
 // FP64 in the refinement's layout.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "wpcd_internal.cuh"
@@ -100,7 +109,23 @@ __device__ __forceinline__ void big_rot(double c, double s, double u, double v, 
     o2 = fma(s, u, __dmul_rn(c, v));
 }
 
-template <class T, bool TEST>
+// Reads of A and Cc: from the L2 where another CTA of the cluster may have written them.
+template <bool CL, class T>
+__device__ __forceinline__ T big_ld(const T *p)
+{
+    return CL ? __ldcg(p) : *p;
+}
+
+// Barrier over the matrix's CTAs, their global writes included.
+template <bool CL>
+__device__ __forceinline__ void big_sync()
+{
+    if (CL) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+}
+
+// CL: the grid runs in clusters, one matrix each; otherwise one CTA a matrix.
+template <class T, bool TEST, bool CL>
 __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *chans, const int *work_ch, int n_work_ch,
                                                           int n_items, int sample0, int n_terms, const double *coeffs,
                                                           T *scratch, double *eps_all, double *C_all, double *lam_s,
@@ -111,7 +136,10 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
     constexpr int kBigUnroll = BigUnroll<T>::v;
     extern __shared__ double smem_big[];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const int cr = CL ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+    const int cn = CL ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
+    const int team = blockIdx.x / cn, teams = gridDim.x / cn;
+    for (int item = team; item < n_items; item += teams) {
         if (done && done[item] != 0) continue;  // already solved (CTA-uniform)
         const int wc = item % n_work_ch;
         const int smp = sample0 + item / n_work_ch;
@@ -135,14 +163,14 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
             }
             continue;
         }
-        T *A = scratch + (size_t)blockIdx.x * big_slot_elems<T>(n);
+        T *A = scratch + (size_t)team * big_slot_elems<T>(n);
         T *Cc = A + (size_t)np * np;
         const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
         double *Hg = (!F64 && H_s) ? H_s + (size_t)item * n * n : nullptr;
 
         // ---- (a2) H = diag(H0) + V0 + sum_a c_a V_a (full matrix), and Cc = I
         double fro2 = 0.0;
-        for (int e = tid; e < np * np; e += nt) {
+        for (int e = tid + cr * nt; e < np * np; e += nt * cn) {
             const int i = e / np, j = e - i * np;
             double v = 0.0;
             if (i < n && j < n) {
@@ -159,7 +187,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
         }
         fro2 = cta_sum64(fro2, red);
         if (tid < 4) flag[tid] = 0;
-        __syncthreads();
+        big_sync<CL>();
         const double tol2 = 1e-30 * fro2;  // FP64 stop: (1e-15 ||H||_F)^2
 
         int sweeps = 0, g3 = 0;
@@ -171,7 +199,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                 double o2 = 0.0;
                 for (int i = warp; i < n; i += nwarp)
                     for (int j = i + 1 + lane; j < n; j += 32) {
-                        const double x = (double)A[(size_t)i * np + j];
+                        const double x = (double)big_ld<CL>(&A[(size_t)i * np + j]);
                         o2 = fma(x, x, o2);
                     }
                 o2 = cta_sum64(o2, red);
@@ -195,8 +223,8 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                     int a, b;
                     big_pair(r, k, M, a, b);
                     const int p = a < b ? a : b, q = a < b ? b : a;
-                    T c = T(1), s = T(0), app = A[(size_t)p * np + p], aqq = A[(size_t)q * np + q];
-                    const T apq = A[(size_t)p * np + q];
+                    T c = T(1), s = T(0), app = big_ld<CL>(&A[(size_t)p * np + p]), aqq = big_ld<CL>(&A[(size_t)q * np + q]);
+                    const T apq = big_ld<CL>(&A[(size_t)p * np + q]);
                     bool rotate;
                     if (F64) rotate = apq != T(0);
                     else {
@@ -222,12 +250,13 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                 __syncthreads();
                 const int na = flag[1 + g3];  // rotating slots this round
                 if (na > 0) {
+                    if (CL) big_sync<CL>();  // no CTA writes A before all have read the pairs
                     // phase 2: rows p, q of every row pair, and columns p, q of Cc.  Each lane
                     // issues the loads of kBigUnroll column slots (or rows of Cc) before any
                     // store: the accesses are L2 round trips, and a store may alias a later
                     // load for all the compiler knows, so batching them is what keeps
                     // enough requests in flight
-                    for (int P = warp; P < h; P += nwarp) {
+                    for (int P = warp + cr * nwarp; P < h; P += nwarp * cn) {
                         const int4 u = sl[P];
                         const BigRot<T> r1 = rot[P];
                         T *Rp = A + (size_t)u.x * np, *Rq = A + (size_t)u.y * np;
@@ -249,10 +278,10 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                                     const int4 v = sl[k];
                                     ca[t] = v.z;
                                     cb[t] = v.w;
-                                    pa[t] = Rp[v.z];
-                                    pb[t] = Rp[v.w];
-                                    qa[t] = Rq[v.z];
-                                    qb[t] = Rq[v.w];
+                                    pa[t] = big_ld<CL>(&Rp[v.z]);
+                                    pb[t] = big_ld<CL>(&Rp[v.w]);
+                                    qa[t] = big_ld<CL>(&Rq[v.z]);
+                                    qb[t] = big_ld<CL>(&Rq[v.w]);
                                 }
                             }
 #pragma unroll
@@ -301,8 +330,8 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                                 for (int t = 0; t < kBigUnroll; ++t) {
                                     const int row = r0 + 32 * t;
                                     if (row < np) {
-                                        a[t] = Cp[row];
-                                        b[t] = Cq[row];
+                                        a[t] = big_ld<CL>(&Cp[row]);
+                                        b[t] = big_ld<CL>(&Cq[row]);
                                     }
                                 }
 #pragma unroll
@@ -318,7 +347,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
                             }
                         }
                     }
-                    __syncthreads();
+                    big_sync<CL>();
                 }
                 g3 = nx3;
             }
@@ -352,15 +381,16 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_jacobi_big(const ChanDev *ch
             }
         } else {
             double *X = X_s + (size_t)item * n * n;  // row-major, unsorted
-            for (int s = warp; s < n; s += nwarp)
-                for (int row = lane; row < n; row += 32) X[(size_t)row * n + s] = (double)Cc[(size_t)s * np + row];
-            for (int i = tid; i < n; i += nt) lam_s[(size_t)item * n + i] = (double)A[(size_t)i * np + i];
+            for (int s = warp + cr * nwarp; s < n; s += nwarp * cn)
+                for (int row = lane; row < n; row += 32) X[(size_t)row * n + s] = (double)big_ld<CL>(&Cc[(size_t)s * np + row]);
+            if (cr == 0)
+                for (int i = tid; i < n; i += nt) lam_s[(size_t)item * n + i] = (double)big_ld<CL>(&A[(size_t)i * np + i]);
         }
-        if (tid == 0) {
+        if (tid == 0 && cr == 0) {
             status_all[(size_t)smp * n_ch_total + cidx] = converged ? sweeps : -1;
             if (!converged) record_error(err, kDevNoConverge);
         }
-        __syncthreads();  // the slot's scratch and tables are reused by the next item
+        big_sync<CL>();  // the slot's scratch and tables are reused by the next item
     }
 }
 
@@ -388,9 +418,39 @@ int jacobi_big_max_n() { return kBigMaxN; }
 int jacobi_big_occupancy(int n, bool f64)
 {
     int blocks = 0;
-    if (f64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<double, false>, kBigThreads, big_smem<double>(n));
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<float, false>, kBigThreads, big_smem<float>(n));
+    if (f64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<double, false, false>, kBigThreads, big_smem<double>(n));
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_jacobi_big<float, false, false>, kBigThreads, big_smem<float>(n));
     return blocks;
+}
+
+// Clusters of cl CTAs (2, 4, 8) of the FP32 kernel that the chip holds at once; 0 if it
+// cannot say.
+static int big_clusters(int cl)
+{
+    struct Held {
+        int n[3] = {0, 0, 0};
+        Held()
+        {
+            for (int k = 0; k < 3; ++k) {
+                cudaLaunchConfig_t cfg{};
+                const int c = 2 << k;
+                cfg.gridDim = dim3((unsigned)(c * 64));
+                cfg.blockDim = dim3(kBigThreads);
+                cfg.dynamicSmemBytes = big_smem<float>(kBigMaxN);
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = (unsigned)c;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                int m = 0;
+                if (cudaOccupancyMaxActiveClusters(&m, k_jacobi_big<float, false, true>, &cfg) == cudaSuccess) n[k] = m;
+                else cudaGetLastError();
+            }
+        }
+    };
+    static const Held held;
+    return held.n[cl == 2 ? 0 : cl == 4 ? 1 : 2];
 }
 
 // FP64: eigenpairs into the eigen buffer (eps_all / C_all at the channel offsets).
@@ -408,17 +468,35 @@ cudaError_t launch_jacobi_big(bool f64, const ChanDev *chans_dev, const int *wor
     const int grid = items < slots ? items : slots;
     if (f64) {
         const size_t sm = big_smem<double>(n);
-        raise_smem_limit((const void *)k_jacobi_big<double, false>, sm);
-        k_jacobi_big<double, false><<<grid, kBigThreads, sm, counted(st)>>>(
+        raise_smem_limit((const void *)k_jacobi_big<double, false, false>, sm);
+        k_jacobi_big<double, false, false><<<grid, kBigThreads, sm, counted(st)>>>(
             chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs, static_cast<double *>(scratch), eps_all,
             C_all, nullptr, nullptr, nullptr, status_all, n_ch_total, err, test, done);
     } else {
         const size_t sm = big_smem<float>(n);
-        auto *k = test.rel > 0.0f || test.ang > 0.0f ? k_jacobi_big<float, true> : k_jacobi_big<float, false>;
+        int cl = 8;  // CTAs a matrix: the most with which all `grid` matrices are resident at once
+        while (cl > 1 && big_clusters(cl) < grid) cl /= 2;
+        const bool loose = test.rel > 0.0f || test.ang > 0.0f;
+        auto *k = cl > 1 ? (loose ? k_jacobi_big<float, true, true> : k_jacobi_big<float, false, true>)
+                         : (loose ? k_jacobi_big<float, true, false> : k_jacobi_big<float, false, false>);
         raise_smem_limit((const void *)k, sm);
-        k<<<grid, kBigThreads, sm, counted(st)>>>(chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs,
-                                                  static_cast<float *>(scratch), nullptr, nullptr, lam_s, X_s, H_s,
-                                                  status_all, n_ch_total, err, test, nullptr);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(grid * cl));
+        cfg.blockDim = dim3(kBigThreads);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = counted(st);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = cl > 1 ? 1 : 0;
+        double *none = nullptr;
+        const int *no_done = nullptr;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, k, chans_dev, work_ch_dev, n_work_ch, items, sample0, n_terms, coeffs,
+                                           static_cast<float *>(scratch), none, none, lam_s, X_s, H_s, status_all,
+                                           n_ch_total, err, test, no_done);
+        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }

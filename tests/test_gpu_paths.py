@@ -1,0 +1,88 @@
+"""Sizes and batch shapes at which a solve changes its route.
+
+* FP64 T: V C rows from the tensor cores from n = 48 on, explicit below, shares of
+  the bins over several CTAs: around that size and the products' tiles (64, 128),
+  with energies that fill one share or leave the last one ragged, both kinds of
+  resolvent, against the oracle at the FP64 tolerances.
+* FP32 Jacobi: one team of warps below n = 160, two from there to n = 304, global
+  memory above: mixed solves around both limits against the oracle at the mixed ones.
+* Small batches run their size buckets on several streams, and a large matrix on
+  a cluster of as many CTAs as are free: the same samples one after another
+  (profiling), alone and in a larger batch give the same bits."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2106_00454_gb300 import inputs as W
+
+from parity_util import compare, compare_mixed, gpu_run, oracle_run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_00454_gb300 import api, build
+    build.build()
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+def _wl(channels, n_wp, S, n_e, lo=2.0, hi=300.0, wp_kind=W.WP_MOMENTUM):
+    return W.Workload("paths", channels, [n_wp] * len(channels), W.GEN_YUKAWA, W.YUKAWA_PARAMS.copy(), W.N_TERMS_YUKAWA,
+                      W.coefficient_samples(S, 11), np.linspace(lo, hi, n_e), wp_kind=wp_kind)
+
+
+UNC, CPL = W.Channel(0, 0, 0, 0, 0), W.Channel(1, 1, 0, 2, 1)
+
+
+@pytest.mark.parametrize("ch,n_wp", [(UNC, 47), (UNC, 48), (CPL, 24), (CPL, 25), (UNC, 64), (UNC, 65), (CPL, 64), (CPL, 65)],
+                         ids=lambda x: x if isinstance(x, int) else x.name)
+@pytest.mark.parametrize("n_e,res", [(1, 0), (50, 0), (2, 2), (33, 2)])
+def test_fp64_t_routes(ctx, orc, ch, n_wp, n_e, res):
+    from paper_2106_00454_gb300 import api
+    wl = _wl([ch], n_wp, 2, n_e, wp_kind=W.WP_ENERGY if res else W.WP_MOMENTUM)
+    md = api.Model(ctx, wl)
+    compare(wl, gpu_run(ctx, md, wl, res=res), oracle_run(orc, wl, mode=res))
+
+
+@pytest.mark.parametrize("ch,n_wp", [(UNC, 159), (UNC, 160), (UNC, 161), (CPL, 80), (CPL, 152), (CPL, 153)],
+                         ids=lambda x: x if isinstance(x, int) else x.name)
+def test_mixed_kernel_limits(ctx, orc, ch, n_wp):
+    from paper_2106_00454_gb300 import api
+    wl = _wl([ch], n_wp, 2, 9)
+    md = api.Model(ctx, wl)
+    compare_mixed(wl, gpu_run(ctx, md, wl, prec=1), oracle_run(orc, wl))
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
+def test_buckets_on_streams_same_bits(ctx, prec):
+    from paper_2106_00454_gb300 import api
+    wl = W.workload_batched(n_samples=5, n_e=21, nwp_choices=(21, 30, 41, 52))
+    md = api.Model(ctx, wl)
+    gpu_run(ctx, md, wl, prec=prec)  # the autotuner's calls
+    a = [gpu_run(ctx, md, wl, prec=prec) for _ in range(2)]
+    ctx.profile(True)
+    try:
+        b = gpu_run(ctx, md, wl, prec=prec)
+    finally:
+        ctx.profile(False)
+    for r in a:
+        for x, y in zip(r, b):
+            assert np.array_equal(x, y)
+
+
+def test_large_matrices_same_bits_alone_and_in_a_batch(ctx):
+    from paper_2106_00454_gb300 import api
+    wl = _wl([CPL], 160, 80, 7)
+    md = api.Model(ctx, wl)
+    whole = gpu_run(ctx, md, wl, prec=1)
+    for s, k in ((3, 1), (0, 20), (10, 40)):  # clusters of 8, 4 or less, 2 or less
+        part = gpu_run(ctx, md, dataclasses.replace(wl, coeffs=wl.coeffs[s:s + k]), prec=1)
+        for x, y in zip(part, whole):
+            assert np.array_equal(x, y[s:s + k])
