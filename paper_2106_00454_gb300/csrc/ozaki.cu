@@ -172,31 +172,36 @@ __device__ __forceinline__ const double *oz_item(const OzItems &src, const doubl
     return M_all + src.chans[src.work[b % src.nw]].c_off + (size_t)(src.sample0 + b / src.nw) * n * n;
 }
 
-// Row slices (seven digits) of V = V0 + sum_a c_a V_a for the bins that the energy
-// plan needs (row v belongs to bin v mod N; the other rows keep whatever the buffer
-// holds: a product's rows do not mix).  One warp per row, the sum in FP64 as the
-// eigensolvers form it.
-template <int PAIRS>
+// Row slices of a sample's matrix, summed in FP64 from the potential terms as the
+// eigensolvers form it, one warp per row:
+//   HSUM = false: seven digits of V = V0 + sum_a c_a V_a for the bins that the energy
+//     plan needs (row v belongs to bin v mod N; the other rows keep whatever the buffer
+//     holds: a product's rows do not mix);
+//   HSUM = true: five and seven digits (S5, S7, one exponent) of every row of
+//     H = diag(H0) + V, with H's rows never in memory.
+template <int PAIRS, bool HSUM>
 __global__ void __launch_bounds__(256) k_oz_vsum(const ChanDev *chans, const int *work, int nw, int sample0, int n, int Kp,
                                                  int n_terms, const double *coeffs, PlanDev plan, int n_ch, int maxN,
-                                                 int *e_all, __nv_bfloat16 *S_all)
+                                                 int *e_all, __nv_bfloat16 *S_all, __nv_bfloat16 *S5_all)
 {
     constexpr int P = kOzMaxDigits;
     const int b = blockIdx.y, v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (v >= n) return;
     const int c = work[b % nw], smp = sample0 + b / nw;
     const ChanDev ch = chans[c];
-    const size_t pc = (size_t)plan_of(plan, smp) * n_ch + c;
-    const int *list = plan.list + pc * maxN, bin = v % ch.N;
-    int lo = 0, hi = plan.cnt[pc] - 1;  // ascending
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (list[mid] < bin) lo = mid + 1;
-        else hi = mid;
-    }
-    if (hi < 0 || list[lo] != bin) {
-        if (lane == 0) e_all[(size_t)b * n + v] = 0;
-        return;
+    if (!HSUM) {
+        const size_t pc = (size_t)plan_of(plan, smp) * n_ch + c;
+        const int *list = plan.list + pc * maxN, bin = v % ch.N;
+        int lo = 0, hi = plan.cnt[pc] - 1;  // ascending
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (list[mid] < bin) lo = mid + 1;
+            else hi = mid;
+        }
+        if (hi < 0 || list[lo] != bin) {
+            if (lane == 0) e_all[(size_t)b * n + v] = 0;
+            return;
+        }
     }
     const double *cf = coeffs ? coeffs + (size_t)smp * (n_terms - 1) : nullptr;
     const double *row = ch.V + (size_t)v * n;
@@ -216,6 +221,15 @@ __global__ void __launch_bounds__(256) k_oz_vsum(const ChanDev *chans, const int
             if (k + 1 < n) x1[j] = fma(ct, rt[k + 1], x1[j]);
         }
     }
+    if (HSUM) {
+        const double d = ch.h0[v % ch.N];
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {
+            const int k = 2 * lane + 64 * j;
+            if (k == v) x0[j] += d;
+            if (k + 1 == v) x1[j] += d;
+        }
+    }
     unsigned long long m = 0;
 #pragma unroll
     for (int j = 0; j < PAIRS; ++j) m = max(m, max(oz_mag(x0[j]), oz_mag(x1[j])));
@@ -223,10 +237,13 @@ __global__ void __launch_bounds__(256) k_oz_vsum(const ChanDev *chans, const int
     const int ex = oz_exp_of(m);
     if (lane == 0) e_all[(size_t)b * n + v] = ex;
     __nv_bfloat16 *S = S_all + (size_t)b * P * n * Kp + (size_t)v * Kp;
+    __nv_bfloat16 *S5 = HSUM ? S5_all + (size_t)b * 5 * n * Kp + (size_t)v * Kp : nullptr;
 #pragma unroll
     for (int j = 0; j < PAIRS; ++j) {
         const int k = 2 * lane + 64 * j;
-        if (k < Kp) oz_digits2<P>(x0[j], x1[j], ex, S + k, (size_t)n * Kp);
+        if (k >= Kp) continue;
+        oz_digits2<P>(x0[j], x1[j], ex, S + k, (size_t)n * Kp);
+        if (HSUM) oz_digits2<5>(x0[j], x1[j], ex, S5 + k, (size_t)n * Kp);
     }
 }
 
@@ -236,8 +253,18 @@ cudaError_t launch_oz_vsum(const ChanDev *chans, const int *work, int nw, int n_
 {
     const int Kp = oz_kpad(n);
     const dim3 g((n + 7) / 8, n_samples * nw);
-    auto *k = Kp <= 256 ? k_oz_vsum<4> : Kp <= 512 ? k_oz_vsum<8> : k_oz_vsum<16>;
-    k<<<g, 256, 0, counted(st)>>>(chans, work, nw, sample0, n, Kp, n_terms, coeffs, plan, n_ch, maxN, e, S);
+    auto *k = Kp <= 256 ? k_oz_vsum<4, false> : Kp <= 512 ? k_oz_vsum<8, false> : k_oz_vsum<16, false>;
+    k<<<g, 256, 0, counted(st)>>>(chans, work, nw, sample0, n, Kp, n_terms, coeffs, plan, n_ch, maxN, e, S, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_oz_hsum(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, __nv_bfloat16 *S5, __nv_bfloat16 *S7, int *e, cudaStream_t st)
+{
+    const int Kp = oz_kpad(n);
+    const dim3 g((n + 7) / 8, n_samples * nw);
+    auto *k = Kp <= 256 ? k_oz_vsum<4, true> : Kp <= 512 ? k_oz_vsum<8, true> : k_oz_vsum<16, true>;
+    k<<<g, 256, 0, counted(st)>>>(chans, work, nw, sample0, n, Kp, n_terms, coeffs, PlanDev{}, 0, 0, e, S7, S5);
     return cudaGetLastError();
 }
 

@@ -18,16 +18,25 @@
 // |s_ij| below the rounding of the products is left alone: its quotient is noise,
 // and the FP64 Jacobi kernel's stopping test would leave it too.
 //
-// An item is done once, after the first iteration, an update's ||E||_F^2 <= kDoneE2: what is left of the off-diagonal is second order in E, below the
+// An item is done once, after the first iteration, an update's ||E||_F^2 <= kDoneE2:
+// what is left of the off-diagonal is second order in E, below the
 // FP64 Jacobi kernel's own test off(A) <= 1e-15 ||H||_F.  Two iterations
 // usually do it, the third runs only for the items that need it, and an item
-// that is not done after that (or whose values do not fit FP32) is solved again
+// that is not done after that (or whose eigenvalues do not fit FP32) is solved again
 // by the FP64 Jacobi kernel (the caller's fallback over done[b] == 0).
 //
+// The FP32 solve may start from C0^T H C0, C0 the eigenvectors of diag(H0) + V0 (built
+// once per set): nearly diagonal, about half the sweeps, and the longest chains (a
+// channel with a bound state, 12 sweeps) shorten most.  It only supplies the start: H
+// itself is never rotated here.  Against the start from H: 20 channels at N_WP = 100, one
+// sample, 5.6 -> 4.0 ms a solve, 20 channels at N_WP = 150, 8 samples, 16.3 -> 11.7; where
+// the chip is full the change of basis costs what the sweeps give (15 channels of N_WP
+// 40/64/100, 256 samples, 24.0 -> 25.1).
+//
 // Measured against FP64 Jacobi alone (its rotations are bound by the FP64 pipe):
-// 20 channels at N_WP = 100, one sample, 161 -> 9.0 ms a solve; 15 channels of
-// N_WP 40/64/100, 256 samples, 339 -> 28 ms; 20 channels at N_WP = 150, 8 samples,
-// 850 -> 29 ms; 1S0 at N_WP = 32, 0.69 -> 0.36 ms; errors against 64-bit LAPACK
+// 20 channels at N_WP = 100, one sample, 145 -> 4.0 ms a solve; 15 channels of
+// N_WP 40/64/100, 256 samples, 337 -> 25 ms; 20 channels at N_WP = 150, 8 samples,
+// 850 -> 11.7 ms; 1S0 at N_WP = 32, 0.69 -> 0.29 ms; errors against 64-bit LAPACK
 // unchanged (T 2e-13 to 9e-13 in both).
 //
 // The update is X + X E with E small: the digit product's rounding, relative
@@ -71,12 +80,18 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
     const size_t off = (size_t)b * n * n;
     double *S = S_all + off, *G = G_all + off, *X = X_all + off, *E = E_all + off;
     const float round = it == 0 ? 2.910383e-11f : 8.881784e-16f;  // 2^-35 (39-bit products), 2^-50 (55-bit)
+    bool above = false, enough = false;
     for (int i = tid; i < n; i += nt) {
         const double l = S[(size_t)i * n + i] / G[(size_t)i * n + i];
+        const float lf = fabsf(f32_trunc(l));
         lam[i] = l;
         hl[i] = 0.5 * l;
-        al[i] = round * fabsf(f32_trunc(l));
+        al[i] = round * lf;
+        above |= !(lf < 1.2676506e30f);  // 2^100
+        enough |= lf > 8.6736174e-19f;   // 2^-60
     }
+    // the tests below are in FP32: H's scale has to leave them room on both sides
+    if (__syncthreads_or(above) || !__syncthreads_or(enough)) return;
     float ang = it == 0 ? kFirstAngle : kLaterAngle;
     float e2 = 0.0f;
     bool plain = true;  // S holds S (not yet s)
@@ -235,35 +250,51 @@ static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 4) + kPairCap * 2 * 
 
 // Digits per product: the first iteration only has to leave errors that the
 // second squares away (39-bit products); from then on Y, S and G carry 55 bits.
-// E is small, so X E needs its leading 31 bits.
-constexpr int kDigFirst = 5, kDigLast = 7, kDigE = 4;
+// E is small, so X E needs its leading 31 bits (kDigE), and so does the change of
+// basis X = C0 X' of a start in the mean-potential eigenbasis, which the
+// iterations refine.
+constexpr int kDigFirst = 5, kDigLast = 7;
 
-// X, H, Y (then E and the next X), W1, W2, lambda; digit slices of H's rows, X's
-// columns, Y's columns (kDigLast planes each), X's rows and E's columns (kDigE)
-// with their exponents.
+// X, Y (then E and the next X), W1, W2, lambda; digit slices of H's rows (kDigFirst and
+// kDigLast planes), X's columns and Y's columns (kDigLast each), X's rows and E's columns
+// (kDigE) with their exponents.
 size_t refine64_scratch_per_item(int n)
 {
-    return (size_t)5 * n * n * 8 + (size_t)n * 8 + (3 * oz_slice_elems(n, kDigLast) + 2 * oz_slice_elems(n, kDigE)) * 2 +
+    return (size_t)4 * n * n * 8 + (size_t)n * 8 +
+           (oz_slice_elems(n, kDigFirst) + 3 * oz_slice_elems(n, kDigLast) + 2 * oz_slice_elems(n, kDigE)) * 2 +
            (size_t)5 * n * 4 + 512;
 }
 
-// The items of one bucket chunk, in scratch blocks X, H, Y, W1, W2 of items n^2
-// doubles each, lambda after them (the layout that the FP32 solve writes), and
-// done[items] ints.  On entry X and H as the FP32 solve left them; on return the
-// done items' eigenpairs are in eps_all / X_all and done[b] == 0 marks the ones
-// that the caller solves by other means.
-cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n,
-                            void *scratch, int *done, const int *status_all, int n_ch_total, double *eps_all,
-                            double *X_all, cudaStream_t st, int *err)
+// Where the FP32 solve leaves its vectors (rotated: in the mean-potential basis), and its eigenvalues.
+double *refine64_start(void *scratch, int items, int n, bool rotated)
+{
+    return static_cast<double *>(scratch) + (rotated ? (size_t)items * n * n : 0);
+}
+double *refine64_lambda(void *scratch, int items, int n)
+{
+    return static_cast<double *>(scratch) + (size_t)4 * items * n * n;
+}
+
+// The items of one bucket chunk, in scratch blocks X, Y, W1, W2 of items n^2 doubles
+// each, lambda after them, and done[items] ints.  On entry the FP32 solve's vectors at
+// refine64_start; on return the done items' eigenpairs are in eps_all / X_all and
+// done[b] == 0 marks the ones that the caller solves by other means.  chans, coeffs: H is
+// summed from its terms, never from the FP32 solve's basis.  rot_s, rot_e: kDigE digit
+// slices of the rows of the nw channels' C0 when the vectors are given in that basis.
+cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                            const double *coeffs, void *scratch, int *done, const int *status_all, int n_ch_total,
+                            double *eps_all, double *X_all, cudaStream_t st, int *err, const __nv_bfloat16 *rot_s,
+                            const int *rot_e)
 {
     const int items = n_samples * nw;
     const size_t nn = (size_t)items * n * n;
     double *X0 = static_cast<double *>(scratch);
-    double *H = X0 + nn, *X1 = H + nn, *W1 = X1 + nn, *W2 = W1 + nn, *lam = W2 + nn;
+    double *X1 = X0 + nn, *W1 = X1 + nn, *W2 = W1 + nn, *lam = W2 + nn;
     const uintptr_t s0 = (reinterpret_cast<uintptr_t>(lam + (size_t)items * n) + 255) & ~(uintptr_t)255;
-    const size_t se = (size_t)items * oz_slice_elems(n, kDigLast), sE = (size_t)items * oz_slice_elems(n, kDigE);
-    __nv_bfloat16 *sH = reinterpret_cast<__nv_bfloat16 *>(s0);
-    __nv_bfloat16 *sXc = sH + se, *sYc = sXc + se, *sXr = sYc + se, *sEc = sXr + sE;
+    const size_t s5 = (size_t)items * oz_slice_elems(n, kDigFirst), se = (size_t)items * oz_slice_elems(n, kDigLast),
+                 sE = (size_t)items * oz_slice_elems(n, kDigE);
+    __nv_bfloat16 *sH5 = reinterpret_cast<__nv_bfloat16 *>(s0);
+    __nv_bfloat16 *sH7 = sH5 + s5, *sXc = sH7 + se, *sYc = sXc + se, *sXr = sYc + se, *sEc = sXr + sE;
     int *eH = reinterpret_cast<int *>(sEc + sE);
     int *eXc = eH + (size_t)items * n, *eYc = eXc + (size_t)items * n, *eXr = eYc + (size_t)items * n;
     int *eEc = eXr + (size_t)items * n;
@@ -274,15 +305,19 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
         if ((e = (x)) != cudaSuccess) \
             return e;                \
     } while (0)
+    if (rot_s) {  // X = C0 X'
+        CKR(launch_oz_split(n, items, true, X1, sEc, eEc, st, OzSkip(), kDigE));
+        CKR(launch_oz_gemm_slices(n, items, rot_s, rot_e, sEc, eEc, X0, st, kDigE, false, err, nw, nullptr, OzSkip(), kDigE));
+    }
+    CKR(launch_oz_hsum(chans, work, nw, n_samples, sample0, n, n_terms, coeffs, sH5, sH7, eH, st));
     double *x = X0, *xn = X1;
     for (int it = 0; it < kRefine64Iters; ++it) {
         OzSkip sk;
         sk.done = it > 0 ? done : nullptr;
         sk.it = it;
         const int dg = it == 0 ? kDigFirst : kDigLast;
-        if (it < 2) CKR(launch_oz_split(n, items, false, H, sH, eH, st, sk, dg));
         CKR(launch_oz_split(n, items, true, x, sXc, eXc, st, sk, dg));
-        CKR(launch_oz_gemm_slices(n, items, sH, eH, sXc, eXc, xn, st, dg, false, err, 0, nullptr, sk, dg));  // Y = H X
+        CKR(launch_oz_gemm_slices(n, items, it == 0 ? sH5 : sH7, eH, sXc, eXc, xn, st, dg, false, err, 0, nullptr, sk, dg));  // Y = H X
         CKR(launch_oz_split(n, items, true, xn, sYc, eYc, st, sk, dg));
         CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sYc, eYc, W1, st, dg, true, err, 0, nullptr, sk, dg));  // S = X^T Y
         CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sXc, eXc, W2, st, dg, true, err, 0, nullptr, sk, dg));  // G = X^T X

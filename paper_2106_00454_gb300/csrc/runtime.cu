@@ -80,6 +80,12 @@ struct VSetH {
     double *Vr = nullptr, *eps0 = nullptr, *C0 = nullptr;
     std::vector<ChanDev> cd_rot;  // host copy: V -> W_a, d0 -> eps0 (offsets zero)
     std::map<int, RotB> rotb;
+    // The same for the FP64 path's FP32 start, from its own eigenpairs of diag(H0) + V0 and
+    // with the C0 slices in kDigE digits (the start is refined against H itself).
+    int start_state = 0;
+    double *Vs = nullptr, *eps_s = nullptr;
+    std::vector<ChanDev> cd_start;
+    std::map<int, RotB> startb;
 };
 
 struct EigH {
@@ -109,6 +115,7 @@ struct Exec {
     int *err = nullptr;
     Buf ws_plan_i, ws_plan_d, ws_tbin, ws_phbin, ws_ref, ws_in, ws_out;
     EigH eig;
+    bool quiet = false;  // launches that belong to no call (neither counted nor timed)
     cudaStream_t side[kSides] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
 };
@@ -247,7 +254,9 @@ struct Launch {
     wpcd_ctx::Rec r{};
     bool on;
     unsigned long long k0;
-    Launch(wpcd_ctx *cc, const Exec &X, int phase) : c(cc), st(X.stream), on(cc->prof), k0(g_thread_kernels)
+    bool quiet;
+    Launch(wpcd_ctx *cc, const Exec &X, int phase)
+        : c(cc), st(X.stream), on(cc->prof && !X.quiet), k0(g_thread_kernels), quiet(X.quiet)
     {
         r.phase = phase;
         if (on) {
@@ -258,7 +267,7 @@ struct Launch {
     }
     ~Launch()
     {
-        c->launches += g_thread_kernels - k0;
+        if (!quiet) c->launches += g_thread_kernels - k0;
         if (on) {
             cudaEventRecord(r.b, st);
             std::lock_guard<std::mutex> lk(c->pmu);
@@ -289,7 +298,15 @@ bool capturing(cudaStream_t st)
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
-wpcd_status ws_reserve(wpcd_ctx *c, const Exec &X, Buf &b, size_t bytes)
+// Give the executor's solver scratch back (it only lives within a phase).
+void drop_scratch(wpcd_ctx *c, Exec &X)
+{
+    cudaStreamSynchronize(X.stream);
+    dfree(c, X.ws_ref.p);
+    X.ws_ref = Buf();
+}
+
+wpcd_status ws_reserve(wpcd_ctx *c, Exec &X, Buf &b, size_t bytes)
 {
     if (b.n >= bytes) return WPCD_OK;
     if (b.part) return WPCD_ERR_NOMEM;
@@ -301,6 +318,10 @@ wpcd_status ws_reserve(wpcd_ctx *c, const Exec &X, Buf &b, size_t bytes)
         b.n = 0;
     }
     wpcd_status st = dmalloc(c, &b.p, bytes);
+    if (st != WPCD_OK && &b != &X.ws_ref && X.ws_ref.p && !X.ws_ref.part) {
+        drop_scratch(c, X);
+        st = dmalloc(c, &b.p, bytes);
+    }
     if (st == WPCD_OK) b.n = bytes;
     return st;
 }
@@ -390,6 +411,12 @@ void free_vset(wpcd_ctx *c, VSetH &v)
     dfree(c, v.eps0);
     dfree(c, v.C0);
     for (auto &kv : v.rotb) {
+        dfree(c, kv.second.sC);
+        dfree(c, kv.second.eC);
+    }
+    dfree(c, v.Vs);
+    dfree(c, v.eps_s);
+    for (auto &kv : v.startb) {
         dfree(c, kv.second.sC);
         dfree(c, kv.second.eC);
     }
@@ -588,7 +615,9 @@ wpcd_status ensure_rotation(wpcd_ctx *c, Exec &X, VSetH &v)
 // Allocate (or reuse) eigenpair storage for `S` samples of vset v and upload
 // the channel table with this batch's offsets (a pageable host copy, so it
 // stays outside CUDA graphs).
-wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int prec, EigH &e)
+bool ensure_start(wpcd_ctx *c, Exec &X, VSetH &v);
+
+wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int prec, EigH &e, bool with_start = true)
 {
     size_t eps_len = 0, c_len = 0;
     std::vector<ChanDev> cd = v.cd;
@@ -607,12 +636,19 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
         e.cd_len < (size_t)v.n_ch) {
         cudaStreamSynchronize(X.stream);
         free_eig(c, e);
-        if ((st = dalloc(c, &e.eps, eps_len))) return st;
-        if ((st = dalloc(c, &e.C, c_len))) return st;
-        if ((st = dalloc(c, &e.coeffs, coeff_len))) return st;
-        if ((st = dalloc(c, &e.status, (size_t)S * v.n_ch))) return st;
-        if ((st = dalloc(c, &e.cd_dev, (size_t)v.n_ch))) return st;
-        if ((st = dalloc(c, &e.cd_rot_dev, (size_t)v.n_ch))) return st;
+        auto get = [&]() -> wpcd_status {
+            wpcd_status g;
+            if ((g = dalloc(c, &e.eps, eps_len)) || (g = dalloc(c, &e.C, c_len)) || (g = dalloc(c, &e.coeffs, coeff_len)) ||
+                (g = dalloc(c, &e.status, (size_t)S * v.n_ch)) || (g = dalloc(c, &e.cd_dev, (size_t)v.n_ch)) ||
+                (g = dalloc(c, &e.cd_rot_dev, (size_t)v.n_ch)))
+                free_eig(c, e);
+            return g;
+        };
+        if ((st = get()) && X.ws_ref.p && !X.ws_ref.part) {  // the solver's scratch yields to the results
+            drop_scratch(c, X);
+            st = get();
+        }
+        if (st) return st;
         e.eps_len = eps_len;
         e.c_len = c_len;
         e.coeff_len = coeff_len;
@@ -624,6 +660,15 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
     e.prec = prec;
     CK(cudaMemcpyAsync(e.cd_dev, cd.data(), sizeof(ChanDev) * v.n_ch, cudaMemcpyHostToDevice, X.stream));
     e.rot = false;
+    if (prec == WPCD_PREC_FP64 && c->rotate && with_start && ensure_start(c, X, v)) {
+        std::vector<ChanDev> cr = v.cd_start;
+        for (int k = 0; k < v.n_ch; ++k) {
+            cr[k].eps_off = cd[k].eps_off;
+            cr[k].c_off = cd[k].c_off;
+        }
+        CK(cudaMemcpyAsync(e.cd_rot_dev, cr.data(), sizeof(ChanDev) * v.n_ch, cudaMemcpyHostToDevice, X.stream));
+        e.rot = true;
+    }
     if (prec == WPCD_PREC_MIXED && c->rotate && c->refine_engine == WPCD_REFINE_TENSOR) {
         if ((st = ensure_rotation(c, X, v))) return st;
         if (v.rot_state == 1) {
@@ -745,17 +790,18 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         return WPCD_OK;
     }
     unsigned char *base = static_cast<unsigned char *>(X.ws_ref.p);
-    double *Xs = reinterpret_cast<double *>(base);
+    const VSetH::RotB *sb = e.rot ? &v.startb.at(n) : nullptr;
     // the FP32 solve of ns samples; its own non-convergence only sends the item to the fallback
     auto solve32 = [&](int th, int s0, int ns) {
         const size_t items = (size_t)ns * nw;
         unsigned char *aux = base + ((ref_item * items + 255) & ~(size_t)255);
-        double *lam = Xs + 5 * items * n * n, *Hs = Xs + items * n * n;
+        double *x = refine64_start(base, (int)items, n, e.rot), *lam = refine64_lambda(base, (int)items, n);
+        const ChanDev *cd = e.rot ? e.cd_rot_dev : e.cd_dev;
         if (big32)
-            return launch_jacobi_big(false, e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, aux, slots32((int)items),
-                                     nullptr, nullptr, lam, Xs, Hs, e.status, v.n_ch, nullptr, X.stream, kTest64);
-        return launch_jacobi_mixed(e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, lam, Xs,
-                                   reinterpret_cast<float *>(aux), Hs, e.status, v.n_ch, nullptr, X.stream, th, kTest64);
+            return launch_jacobi_big(false, cd, work, nw, ns, smp0 + s0, v.n_terms, cf, n, aux, slots32((int)items), nullptr,
+                                     nullptr, lam, x, nullptr, e.status, v.n_ch, nullptr, X.stream, kTest64);
+        return launch_jacobi_mixed(cd, work, nw, ns, smp0 + s0, v.n_terms, cf, n, lam, x, reinterpret_cast<float *>(aux),
+                                   nullptr, e.status, v.n_ch, nullptr, X.stream, th, kTest64);
     };
     int threads = 256;
     if (!big32) {
@@ -771,8 +817,8 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         }
         {
             Launch L(c, X, WPCD_PHASE_REFINE);
-            CK(launch_refine64(e.cd_dev, work, nw, ns, smp0 + s0, n, base, done, e.status, v.n_ch, e.eps, e.C, X.stream,
-                               X.err));
+            CK(launch_refine64(e.cd_dev, work, nw, ns, smp0 + s0, n, v.n_terms, cf, base, done, e.status, v.n_ch, e.eps, e.C,
+                               X.stream, X.err, sb ? sb->sC : nullptr, sb ? sb->eC : nullptr));
         }
         Launch L(c, X, WPCD_PHASE_EIGEN);
         if (big64) {  // its slots take the place of the refinement's scratch
@@ -785,6 +831,109 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         }
     }
     return WPCD_OK;
+}
+
+// The mean-potential eigenbasis of a set for the FP64 path's FP32 start (built once, on
+// the executor's stream; concurrent callers wait on the set's lock): C0, eps0 by that path
+// itself, W_a = C0^T V_a C0 by tensor-core products (T_a = C0^T V_a, then C0^T T_a^T, which
+// is W_a as W_a is symmetric).  false: none, the start is H itself -- without sample terms
+// (the basis would be the answer), without memory, or when a solve failed.
+bool ensure_start(wpcd_ctx *c, Exec &X, VSetH &v)
+{
+    if (v.n_terms < 2 || c->budget) return false;  // (a budget's room is the caller's)
+    std::lock_guard<std::mutex> lk(*v.rot_mu);
+    if (v.start_state != 0) return v.start_state == 1;
+    if (capturing(X.stream)) return false;
+    v.start_state = -1;
+    const int na = v.n_terms - 1;
+    EigH m;
+    double *T = nullptr;
+    void *scratch = nullptr;
+    int *err = X.err;
+    X.quiet = true;
+    auto build = [&]() -> wpcd_status {
+        size_t ne = 0, vlen = 0;
+        int nmax = 0;
+        for (auto &d : v.cd) {
+            ne += (size_t)d.n;
+            vlen += (size_t)v.n_terms * d.n * d.n;
+            nmax = std::max(nmax, d.n);
+        }
+        wpcd_status st;
+        if ((st = dalloc(c, &v.eps_s, ne)) || (st = dalloc(c, &v.Vs, vlen))) return st;
+        if ((st = diag_prep(c, X, v, -1, 1, WPCD_PREC_FP64, m, false))) return st;
+        CK(cudaMemsetAsync(m.coeffs, 0, sizeof(double) * na, X.stream));
+        X.err = nullptr;  // a failed solve only leaves the set without the basis
+        for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it)
+            if ((st = run_bucket_f64(c, X, v, m, m.coeffs, v.bucket_dev[it->first], (int)it->second.size(), 1, 0, it->first)))
+                return st;
+        CK(cudaMemcpyAsync(v.eps_s, m.eps, sizeof(double) * ne, cudaMemcpyDeviceToDevice, X.stream));
+        const size_t se = oz_slice_elems(nmax, kDigE);
+        const size_t bytes = ((size_t)na + 1) * (se * 2 + (size_t)nmax * 4) + 1024;
+        if ((st = dalloc(c, &T, (size_t)na * nmax * nmax)) || (st = dmalloc(c, &scratch, bytes))) return st;
+        __nv_bfloat16 *sC = static_cast<__nv_bfloat16 *>(scratch), *sM = sC + se;
+        int *eC = reinterpret_cast<int *>(sM + (size_t)na * se), *eM = eC + nmax;
+        size_t co = 0;
+        for (int k = 0; k < v.n_ch; ++k) {
+            const int n = v.cd[k].n;
+            const size_t nn = (size_t)n * n;
+            const double *C0 = m.C + co;
+            double *W = v.Vs + (v.cd[k].V - v.V);
+            co += nn;
+            CK(cudaMemsetAsync(W, 0, nn * sizeof(double), X.stream));  // W_0 = 0
+            CK(launch_oz_split(n, 1, true, C0, sC, eC, X.stream, OzSkip(), kDigE));
+            CK(launch_oz_split(n, na, true, v.cd[k].V + nn, sM, eM, X.stream, OzSkip(), kDigE));
+            CK(launch_oz_gemm_slices(n, na, sC, eC, sM, eM, T, X.stream, kDigE, false, err, 1, nullptr, OzSkip(), kDigE));
+            CK(launch_oz_split(n, na, false, T, sM, eM, X.stream, OzSkip(), kDigE));
+            CK(launch_oz_gemm_slices(n, na, sC, eC, sM, eM, W + nn, X.stream, kDigE, false, err, 1, nullptr, OzSkip(), kDigE));
+        }
+        for (auto &kv : v.buckets) {  // the rows of C0, the bucket's channels in bucket order
+            const int n = kv.first, nw = (int)kv.second.size();
+            VSetH::RotB &rb = v.startb[n];
+            if ((st = dalloc(c, &rb.sC, (size_t)nw * oz_slice_elems(n, kDigE))) || (st = dalloc(c, &rb.eC, (size_t)nw * n)))
+                return st;
+            for (int i = 0; i < nw; ++i) {
+                size_t at = 0;
+                for (int k = 0; k < kv.second[i]; ++k) at += (size_t)v.cd[k].n * v.cd[k].n;
+                CK(launch_oz_split(n, 1, false, m.C + at, rb.sC + (size_t)i * oz_slice_elems(n, kDigE), rb.eC + (size_t)i * n,
+                                   X.stream, OzSkip(), kDigE));
+            }
+        }
+        std::vector<int> hs(v.n_ch);
+        CK(cudaMemcpyAsync(hs.data(), m.status, sizeof(int) * v.n_ch, cudaMemcpyDeviceToHost, X.stream));
+        CK(cudaStreamSynchronize(X.stream));
+        for (int k = 0; k < v.n_ch; ++k)
+            if (hs[k] < 0) return WPCD_ERR_NOCONVERGE;
+        return WPCD_OK;
+    };
+    const wpcd_status st = build();
+    X.err = err;
+    X.quiet = false;
+    cudaStreamSynchronize(X.stream);
+    dfree(c, T);
+    dfree(c, scratch);
+    free_eig(c, m);
+    if (st != WPCD_OK) {
+        cudaGetLastError();
+        dfree(c, v.Vs);
+        dfree(c, v.eps_s);
+        v.Vs = v.eps_s = nullptr;
+        for (auto &kv : v.startb) {
+            dfree(c, kv.second.sC);
+            dfree(c, kv.second.eC);
+        }
+        v.startb.clear();
+        return false;
+    }
+    v.cd_start = v.cd;
+    size_t eo = 0;
+    for (int k = 0; k < v.n_ch; ++k) {
+        v.cd_start[k].V = v.Vs + (v.cd[k].V - v.V);
+        v.cd_start[k].d0 = v.eps_s + eo;
+        eo += v.cd[k].n;
+    }
+    v.start_state = 1;
+    return true;
 }
 
 // Scratch that the whole of a size bucket takes in one chunk.
@@ -1861,8 +2010,17 @@ wpcd_status mi_eigen_set(wpcd_ctx *c, MiH &m)
         CK(cudaMemcpyAsync(off_dev, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice, c->main.stream));
         Launch L(c, c->main, WPCD_PHASE_MI);
         CK(launch_mi_scale(m.ch_dev, m.n_ch, m.NQ, m.kg, m.wg, m.n_terms, m.Vg, v.V, off_dev, m.k2, c->main.stream));
+        for (auto &kv : v.buckets) {
+            int *list = nullptr;
+            ok = ok && dalloc(c, &list, kv.second.size()) == WPCD_OK;
+            if (!ok) break;
+            v.bucket_dev[kv.first] = list;
+            CK(cudaMemcpyAsync(list, kv.second.data(), sizeof(int) * kv.second.size(), cudaMemcpyHostToDevice,
+                               c->main.stream));
+        }
         CK(cudaStreamSynchronize(c->main.stream));
-    } else {
+    }
+    if (!ok) {
         dfree(c, v.V);
         v.V = nullptr;
         dfree(c, m.k2);

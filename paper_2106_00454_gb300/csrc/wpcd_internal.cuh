@@ -308,6 +308,8 @@ cudaError_t launch_oz_split(int n, int items, bool cols, const double *M, __nv_b
 cudaError_t launch_oz_vsum(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
                            const double *coeffs, const PlanDev &plan, int n_ch, int maxN, __nv_bfloat16 *S, int *e,
                            cudaStream_t st);
+cudaError_t launch_oz_hsum(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                           const double *coeffs, __nv_bfloat16 *S5, __nv_bfloat16 *S7, int *e, cudaStream_t st);
 cudaError_t launch_oz_gemm_slices(int n, int items, const __nv_bfloat16 *sa, const int *ea, const __nv_bfloat16 *sb,
                                   const int *eb, double *C, cudaStream_t st, int digits = 6, bool sym = false,
                                   int *err = nullptr, int a_items = 0, const double *Cadd = nullptr,
@@ -323,9 +325,13 @@ cudaError_t launch_refine(const ChanDev *chans, const int *work, int nw, int n_s
                           const __nv_bfloat16 *rot_s = nullptr, const int *rot_e = nullptr, int digits = 6);
 constexpr int kRefine64Iters = 3;  // at most; the items that have converged skip the rest
 size_t refine64_scratch_per_item(int n);
-cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n,
-                            void *scratch, int *done, const int *status_all, int n_ch_total, double *eps_all,
-                            double *X_all, cudaStream_t st, int *err);
+constexpr int kDigE = 4;  // digits of the FP64 path's updates and of the basis change of its start
+double *refine64_start(void *scratch, int items, int n, bool rotated);
+double *refine64_lambda(void *scratch, int items, int n);
+cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
+                            const double *coeffs, void *scratch, int *done, const int *status_all, int n_ch_total,
+                            double *eps_all, double *X_all, cudaStream_t st, int *err, const __nv_bfloat16 *rot_s,
+                            const int *rot_e);
 cudaError_t launch_batched_dgemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                                  void *scratch, int engine, cudaStream_t st, int *err = nullptr);
 size_t batched_dgemm_scratch(int n, int items);
