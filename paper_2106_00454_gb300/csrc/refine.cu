@@ -197,7 +197,7 @@ size_t sort_eig_smem(int n) { return (size_t)n * 8 + (size_t)n * 4; }
 
 size_t refine_scratch_per_item(int n, int engine)
 {
-    size_t b = (size_t)5 * n * n * 8 + (size_t)n * 8;  // X, H, Y, W1, W2, lambda
+    size_t b = (size_t)5 * n * n * 8 + (size_t)n * 8;  // X, H, Y, G, S, lambda
     if (engine == 0) b += 5 * oz_slice_elems(n) * 2 + (size_t)5 * n * 4 + 512;  // 5 digit-slice sets
     return b;
 }
@@ -224,7 +224,7 @@ cudaError_t launch_refine(const ChanDev *chans, const int *work, int nw, int n_s
     const int items = n_samples * nw;
     const size_t nn = (size_t)items * n * n;
     double *Xs = static_cast<double *>(scratch);
-    double *H = Xs + nn, *Y = H + nn, *W1 = Y + nn, *W2 = W1 + nn, *lam = W2 + nn;
+    double *H = Xs + nn, *Y = H + nn, *G = Y + nn, *S = G + nn, *lam = S + nn;
     // digit slices start on a 256-byte boundary (16-byte vector loads)
     const uintptr_t s0 = (reinterpret_cast<uintptr_t>(lam + (size_t)items * n) + 255) & ~(uintptr_t)255;
     const size_t se = (size_t)items * oz_slice_elems(n);
@@ -252,21 +252,21 @@ cudaError_t launch_refine(const ChanDev *chans, const int *work, int nw, int n_s
             CKR(launch_oz_split(n, items, true, x, sXc, eXc, st));                   // columns of X
             CKR(launch_oz_gemm_slices(n, items, sH, eH, sXc, eXc, xn, st, dg, false, err));       // Y = H X
             CKR(launch_oz_split(n, items, true, xn, sYc, eYc, st));                  // columns of Y
-            // S = X^T H X and G = X^T X are symmetric: upper tiles, mirrored
-            CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sYc, eYc, W1, st, dg, true, err));  // S = X^T Y
-            CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sXc, eXc, W2, st, dg, true, err));  // G = X^T X
+            // G = X^T X and S = X^T H X = X^T Y are symmetric: upper tiles, mirrored; in one
+            // launch, as the column slices of Y follow those of X and S follows G
+            CKR(launch_oz_gemm_slices(n, 2 * items, sXc, eXc, sXc, eXc, G, st, dg, true, err, items));
         } else {
             k_bgemm64<false><<<gg, 256, 0, counted(st)>>>(n, H, x, xn);
-            k_bgemm64<true><<<gg, 256, 0, counted(st)>>>(n, x, xn, W1);
-            k_bgemm64<true><<<gg, 256, 0, counted(st)>>>(n, x, x, W2);
+            k_bgemm64<true><<<gg, 256, 0, counted(st)>>>(n, x, xn, S);
+            k_bgemm64<true><<<gg, 256, 0, counted(st)>>>(n, x, x, G);
         }
-        k_oa_update<<<items, 256, (size_t)n * 8, counted(st)>>>(n, W1, W2, lam);
+        k_oa_update<<<items, 256, (size_t)n * 8, counted(st)>>>(n, S, G, lam);
         if (engine == 0) {
             CKR(launch_oz_split(n, items, false, x, sXr, eXr, st));              // rows of X
-            CKR(launch_oz_split(n, items, true, W2, sEc, eEc, st));              // columns of I + E
+            CKR(launch_oz_split(n, items, true, G, sEc, eEc, st));              // columns of I + E
             CKR(launch_oz_gemm_slices(n, items, sXr, eXr, sEc, eEc, xn, st, dg, false, err)); // X (I + E)
         } else {
-            k_bgemm64<false><<<gg, 256, 0, counted(st)>>>(n, x, W2, xn);
+            k_bgemm64<false><<<gg, 256, 0, counted(st)>>>(n, x, G, xn);
         }
         double *t = x;
         x = xn;

@@ -255,7 +255,7 @@ static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 4) + kPairCap * 2 * 
 // iterations refine.
 constexpr int kDigFirst = 5, kDigLast = 7;
 
-// X, Y (then E and the next X), W1, W2, lambda; digit slices of H's rows (kDigFirst and
+// X, Y (then E and the next X), G, S, lambda; digit slices of H's rows (kDigFirst and
 // kDigLast planes), X's columns and Y's columns (kDigLast each), X's rows and E's columns
 // (kDigE) with their exponents.
 size_t refine64_scratch_per_item(int n)
@@ -275,7 +275,7 @@ double *refine64_lambda(void *scratch, int items, int n)
     return static_cast<double *>(scratch) + (size_t)4 * items * n * n;
 }
 
-// The items of one bucket chunk, in scratch blocks X, Y, W1, W2 of items n^2 doubles
+// The items of one bucket chunk, in scratch blocks X, Y, G, S of items n^2 doubles
 // each, lambda after them, and done[items] ints.  On entry the FP32 solve's vectors at
 // refine64_start; on return the done items' eigenpairs are in eps_all / X_all and
 // done[b] == 0 marks the ones that the caller solves by other means.  chans, coeffs: H is
@@ -289,12 +289,12 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
     const int items = n_samples * nw;
     const size_t nn = (size_t)items * n * n;
     double *X0 = static_cast<double *>(scratch);
-    double *X1 = X0 + nn, *W1 = X1 + nn, *W2 = W1 + nn, *lam = W2 + nn;
+    double *X1 = X0 + nn, *G = X1 + nn, *S = G + nn, *lam = S + nn;
     const uintptr_t s0 = (reinterpret_cast<uintptr_t>(lam + (size_t)items * n) + 255) & ~(uintptr_t)255;
     const size_t s5 = (size_t)items * oz_slice_elems(n, kDigFirst), se = (size_t)items * oz_slice_elems(n, kDigLast),
                  sE = (size_t)items * oz_slice_elems(n, kDigE);
     __nv_bfloat16 *sH5 = reinterpret_cast<__nv_bfloat16 *>(s0);
-    __nv_bfloat16 *sH7 = sH5 + s5, *sXc = sH7 + se, *sYc = sXc + se, *sXr = sYc + se, *sEc = sXr + sE;
+    __nv_bfloat16 *sH7 = sH5 + s5, *sXc = sH7 + se, *sXr = sXc + 2 * se, *sEc = sXr + sE;
     int *eH = reinterpret_cast<int *>(sEc + sE);
     int *eXc = eH + (size_t)items * n, *eYc = eXc + (size_t)items * n, *eXr = eYc + (size_t)items * n;
     int *eEc = eXr + (size_t)items * n;
@@ -318,10 +318,13 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
         const int dg = it == 0 ? kDigFirst : kDigLast;
         CKR(launch_oz_split(n, items, true, x, sXc, eXc, st, sk, dg));
         CKR(launch_oz_gemm_slices(n, items, it == 0 ? sH5 : sH7, eH, sXc, eXc, xn, st, dg, false, err, 0, nullptr, sk, dg));  // Y = H X
+        // G = X^T X and S = X^T Y in one launch: the column slices of Y follow those of X
+        __nv_bfloat16 *sYc = sXc + (size_t)items * oz_slice_elems(n, dg);
+        OzSkip two = sk;
+        two.mod = items;
         CKR(launch_oz_split(n, items, true, xn, sYc, eYc, st, sk, dg));
-        CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sYc, eYc, W1, st, dg, true, err, 0, nullptr, sk, dg));  // S = X^T Y
-        CKR(launch_oz_gemm_slices(n, items, sXc, eXc, sXc, eXc, W2, st, dg, true, err, 0, nullptr, sk, dg));  // G = X^T X
-        k_r64_update<<<items, 256, r64_smem(n), counted(st)>>>(n, W1, W2, x, xn, lam, done, it);  // E over Y
+        CKR(launch_oz_gemm_slices(n, 2 * items, sXc, eXc, sXc, eXc, G, st, dg, true, err, items, nullptr, two, dg));
+        k_r64_update<<<items, 256, r64_smem(n), counted(st)>>>(n, S, G, x, xn, lam, done, it);  // E over Y
         CKR(cudaGetLastError());
         CKR(launch_oz_split(n, items, false, x, sXr, eXr, st, sk, kDigE));
         CKR(launch_oz_split(n, items, true, xn, sEc, eEc, st, sk, kDigE));

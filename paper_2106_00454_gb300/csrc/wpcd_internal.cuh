@@ -281,14 +281,15 @@ cudaError_t launch_jacobi_big(bool f64, const ChanDev *chans_dev, const int *wor
                               int *status_all, int n_ch_total, int *err, cudaStream_t st,
                               RotTest test = RotTest(), const int *done = nullptr);
 // Items of a batch that a step leaves alone: those with 0 < done[b] <= it (done == NULL: none).
+// Products of two kinds in one launch (b and b + mod of one item) share the item's flag.
 struct OzSkip {
     const int *done = nullptr;
-    int it = 0;
+    int it = 0, mod = 0x7fffffff;
 };
 __device__ __forceinline__ bool oz_skipped(const OzSkip &sk, int b)
 {
     if (!sk.done) return false;
-    const int d = sk.done[b];
+    const int d = sk.done[b % sk.mod];
     return d != 0 && d <= sk.it;
 }
 // The eigenvector matrices of a bucket's items inside an eigen buffer.
