@@ -685,6 +685,15 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
     return WPCD_OK;
 }
 
+// Position in its size bucket of a work list's first channel: the whole bucket, or one
+// channel of it (plain execution).
+size_t bucket_pos(const VSetH &v, const int *work, int n)
+{
+    if (!v.ident_dev || work < v.ident_dev || work >= v.ident_dev + v.n_ch) return 0;
+    const std::vector<int> &b = v.buckets.at(n);
+    return (size_t)(std::find(b.begin(), b.end(), (int)(work - v.ident_dev)) - b.begin());
+}
+
 // A size bucket whose matrices exceed one CTA's shared memory: the Jacobi
 // kernel with the matrix and eigenvectors in global memory (eig_big.cu), one
 // scratch slot per resident CTA; the mixed path then refines as for the other
@@ -722,8 +731,10 @@ wpcd_status run_bucket_big(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         }
         Launch L(c, X, WPCD_PHASE_REFINE);
         const VSetH::RotB *rb = e.rot ? &v.rotb.at(n) : nullptr;
+        const size_t pos = bucket_pos(v, work, n);
         CK(launch_refine(e.cd_dev, work, nw, ns, smp0 + s0, n, v.n_terms, cf, base, e.eps, e.C, c->refine_iters,
-                         c->refine_engine, X.stream, X.err, rb ? rb->sC : nullptr, rb ? rb->eC : nullptr, c->refine_digits));
+                         c->refine_engine, X.stream, X.err, rb ? rb->sC + pos * oz_slice_elems(n) : nullptr,
+                             rb ? rb->eC + pos * n : nullptr, c->refine_digits));
     }
     return WPCD_OK;
 }
@@ -791,6 +802,7 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
     }
     unsigned char *base = static_cast<unsigned char *>(X.ws_ref.p);
     const VSetH::RotB *sb = e.rot ? &v.startb.at(n) : nullptr;
+    const size_t pos = bucket_pos(v, work, n);
     // the FP32 solve of ns samples; its own non-convergence only sends the item to the fallback
     auto solve32 = [&](int th, int s0, int ns) {
         const size_t items = (size_t)ns * nw;
@@ -818,7 +830,8 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         {
             Launch L(c, X, WPCD_PHASE_REFINE);
             CK(launch_refine64(e.cd_dev, work, nw, ns, smp0 + s0, n, v.n_terms, cf, base, done, e.status, v.n_ch, e.eps, e.C,
-                               X.stream, X.err, sb ? sb->sC : nullptr, sb ? sb->eC : nullptr));
+                               X.stream, X.err, sb ? sb->sC + pos * oz_slice_elems(n, kDigE) : nullptr,
+                               sb ? sb->eC + pos * n : nullptr));
         }
         Launch L(c, X, WPCD_PHASE_EIGEN);
         if (big64) {  // its slots take the place of the refinement's scratch
@@ -1041,8 +1054,10 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
             }
             Launch L(c, X, WPCD_PHASE_REFINE);
             const VSetH::RotB *rb = e.rot ? &v.rotb.at(n) : nullptr;
+            const size_t pos = bucket_pos(v, work, n);
             CK(launch_refine(e.cd_dev, work, nw, ns, smp0 + s0, n, v.n_terms, cf, base, e.eps, e.C, c->refine_iters,
-                             c->refine_engine, X.stream, X.err, rb ? rb->sC : nullptr, rb ? rb->eC : nullptr, c->refine_digits));
+                             c->refine_engine, X.stream, X.err, rb ? rb->sC + pos * oz_slice_elems(n) : nullptr,
+                             rb ? rb->eC + pos * n : nullptr, c->refine_digits));
         }
         return WPCD_OK;
     };

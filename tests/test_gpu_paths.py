@@ -86,3 +86,19 @@ def test_large_matrices_same_bits_alone_and_in_a_batch(ctx):
         part = gpu_run(ctx, md, dataclasses.replace(wl, coeffs=wl.coeffs[s:s + k]), prec=1)
         for x, y in zip(part, whole):
             assert np.array_equal(x, y[s:s + k])
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
+def test_one_solve_per_launch_same_bits(ctx, prec):
+    """Plain execution of several channels of one size (each its own mean-potential basis)."""
+    from paper_2106_00454_gb300 import api
+    wl = _wl([UNC, W.Channel(1, 1, 1, 1, 0), CPL, W.Channel(1, 2, 1, 3, 1)], 32, 2, 9)
+    md = api.Model(ctx, wl)
+    a = gpu_run(ctx, md, wl, prec=prec)
+    ctx.set_exec(api.EXEC_PLAIN)
+    try:
+        b = gpu_run(ctx, md, wl, prec=prec)
+    finally:
+        ctx.set_exec(api.EXEC_BATCHED)
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
