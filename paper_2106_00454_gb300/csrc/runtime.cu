@@ -10,6 +10,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -46,8 +47,6 @@ constexpr int kRefineIters = 2;                            // FP64 refinement it
 constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
 constexpr size_t kVcScratchBytes = (size_t)8 << 30;  // FP64 T: scratch of the rows of V C, per chunk
 constexpr int kVcRowsN = 48;                         // ... for matrices from this size on
-// Batches up to this many solves per SM run their size buckets side by side.
-constexpr int kForkItems = 8;
 constexpr size_t kGraphCache = 64;                         // wpcd_solve keys remembered for CUDA graphs
 
 struct MeshH {
@@ -109,13 +108,14 @@ struct Buf {
 // One executor: a stream, its device status word and its workspaces.  The
 // synchronous API runs on the context's own executor; each serving slot has
 // one of its own so that batches overlap on the device.
-constexpr int kSides = 3;  // streams beside the executor's own for the size buckets of a small batch
+constexpr int kSides = 3;  // streams beside the executor's own for the size buckets of a batch
 struct Exec {
     cudaStream_t stream = nullptr;
     int *err = nullptr;
     Buf ws_plan_i, ws_plan_d, ws_tbin, ws_phbin, ws_ref, ws_in, ws_out;
     EigH eig;
     bool quiet = false;  // launches that belong to no call (neither counted nor timed)
+    size_t no_fork = ~(size_t)0;  // scratch of the streams' shares that found no room
     cudaStream_t side[kSides] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
 };
@@ -630,7 +630,7 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
     const size_t coeff_len = (size_t)S * std::max(v.n_terms - 1, 1);
     wpcd_status st = WPCD_OK;
     if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    if (v.buckets.size() > 1 && (long long)S * v.n_ch <= (long long)kForkItems * c->n_sm) side_streams(X);
+    if ((long long)S * v.n_ch > 1) side_streams(X);
     // grow-only storage: a smaller batch or another set with as many channels reuses it
     if (e.eps_len < eps_len || e.c_len < c_len || e.coeff_len < coeff_len || e.status_len < (size_t)S * v.n_ch ||
         e.cd_len < (size_t)v.n_ch) {
@@ -962,43 +962,73 @@ size_t bucket_scratch(wpcd_ctx *c, int n, int nw, int S, int prec)
     return ((ref_item * nw * S + 255) & ~(size_t)255) + slot_b * std::max(1, std::min(S * nw, cap));
 }
 
-// The size buckets of a small batch side by side on the executor's streams, each in its
-// own share of the scratch (false: the caller runs them one after another).  A bucket
-// of few matrices is one chain of latencies on few SMs, so the buckets' times add up to
-// the longest instead of their sum: see kForkItems for what it measured.
+// The size buckets side by side on the executor's streams, each stream in its own share
+// of the scratch, the next unit on the stream with the least work (n^3) so far; a bucket
+// whose scratch exceeds a share goes in sample ranges (false: the caller runs the buckets
+// one after another).  A bucket of few matrices is a chain of latencies on few SMs, and
+// then the buckets take the time of the longest instead of their sum: 20 channels at
+// N_WP = 100, one sample, 5.0 -> 3.7 ms.  Full ones gain too: a bucket's last wave and its
+// refinement (HBM, FP64) run beside the next one's Jacobi rounds (shared memory, latency),
+// and T (FP64) beside both: 15 channels of N_WP 40/64/100, 256 samples FP64 25.1 -> 19.3 ms,
+// 1024 samples mixed 60.0 -> 51.9, 20 channels of N_WP = 150, 1024 samples mixed 381 -> 365.
+// Finer ranges lose it again: each is a chain with its own last wave (8 solves per SM and
+// range: 53.4 and 382 ms in the last two); two streams 22.4, 59.4 and 397.
 template <class F>
-bool fork_buckets(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_bucket, std::vector<wpcd_status> &sts)
+bool fork_units(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_unit, std::vector<wpcd_status> &sts)
 {
-    if (c->prof || v.buckets.size() < 2 || (long long)S * v.n_ch > (long long)kForkItems * c->n_sm) return false;
+    if (c->prof || (long long)S * v.n_ch < 2) return false;
+    struct Unit {
+        int n, nw, s0, ns, lane;
+    };
+    std::vector<Unit> units;
+    const int lanes = kSides + 1;
+    const size_t cap = kRefineScratchBytes / lanes;
+    double load[kSides + 1] = {};
+    size_t share[kSides + 1] = {}, off[kSides + 2] = {};
+    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
+        const int n = it->first, nw = (int)it->second.size();
+        auto bytes = [&](int ns) { return (bucket_scratch(c, n, nw, ns, prec) + 255) & ~(size_t)255; };
+        if (bytes(1) > cap) return false;
+        int pieces = (int)std::min<size_t>(S, (bytes(S) + cap - 1) / cap);
+        while (bytes((S + pieces - 1) / pieces) > cap) ++pieces;
+        for (int q = 0; q < pieces; ++q) {
+            const int s0 = (int)((long long)S * q / pieces), ns = (int)((long long)S * (q + 1) / pieces) - s0;
+            int lane = 0;
+            for (int k = 1; k < lanes; ++k)
+                if (load[k] < load[lane]) lane = k;
+            load[lane] += (double)n * n * n * nw * ns;
+            share[lane] = std::max(share[lane], bytes(ns));
+            units.push_back({n, nw, s0, ns, lane});
+        }
+    }
+    for (int k = 0; k < lanes; ++k) off[k + 1] = off[k] + share[k];
+    const size_t total = off[lanes];
+    if (units.size() < 2 || total >= X.no_fork || !side_streams(X)) return false;
+    if (ws_reserve(c, X, X.ws_ref, total)) {
+        if (!capturing(X.stream)) X.no_fork = total;
+        return false;
+    }
     if (c->autotune) {  // the autotuner times its candidates alone
         std::lock_guard<std::mutex> lk(c->tmu);
         for (auto &kv : v.buckets)
             if (jacobi_fits_smem(kv.first, false) && !c->tuned.count(std::make_pair(kv.first, prec))) return false;
     }
-    std::vector<size_t> off;
-    size_t total = 0;
-    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
-        off.push_back(total);
-        total += (bucket_scratch(c, it->first, (int)it->second.size(), S, prec) + 255) & ~(size_t)255;
-    }
-    off.push_back(total);
-    if (total > kRefineScratchBytes || !side_streams(X) || ws_reserve(c, X, X.ws_ref, total)) return false;
     if (cudaEventRecord(X.ev_fork, X.stream) != cudaSuccess) return false;
-    const int sides = std::min<int>(kSides, (int)v.buckets.size() - 1);
-    for (int k = 0; k < sides; ++k) cudaStreamWaitEvent(X.side[k], X.ev_fork, 0);
-    int b = 0;
-    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it, ++b) {
+    for (int k = 1; k < lanes; ++k)
+        if (share[k]) cudaStreamWaitEvent(X.side[k - 1], X.ev_fork, 0);
+    for (const Unit &u : units) {
         Exec Y;
-        Y.stream = b == 0 ? X.stream : X.side[(b - 1) % sides];
+        Y.stream = u.lane == 0 ? X.stream : X.side[u.lane - 1];
         Y.err = X.err;
-        Y.ws_ref.p = static_cast<unsigned char *>(X.ws_ref.p) + off[b];
-        Y.ws_ref.n = off[b + 1] - off[b];
+        Y.ws_ref.p = static_cast<unsigned char *>(X.ws_ref.p) + off[u.lane];
+        Y.ws_ref.n = share[u.lane];
         Y.ws_ref.part = true;
-        sts.push_back(run_bucket(Y, v.bucket_dev[it->first], (int)it->second.size(), S, 0, it->first));
+        sts.push_back(run_unit(Y, v.bucket_dev[u.n], u.nw, u.ns, u.s0, u.n));
     }
-    for (int k = 0; k < sides; ++k) {  // joined whatever the buckets returned
-        const bool ok = cudaEventRecord(X.ev_join[k], X.side[k]) == cudaSuccess &&
-                        cudaStreamWaitEvent(X.stream, X.ev_join[k], 0) == cudaSuccess;
+    for (int k = 1; k < lanes; ++k) {  // joined whatever the units returned
+        if (!share[k]) continue;
+        const bool ok = cudaEventRecord(X.ev_join[k - 1], X.side[k - 1]) == cudaSuccess &&
+                        cudaStreamWaitEvent(X.stream, X.ev_join[k - 1], 0) == cudaSuccess;
         sts.push_back(ok ? WPCD_OK : WPCD_ERR_CUDA);
     }
     return true;
@@ -1006,7 +1036,11 @@ bool fork_buckets(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_bucket,
 
 // The parameter sum + eigensolve of the batch diag_prep set up (device-only
 // work on X.stream: capturable).  coeffs: device, [S][n_terms - 1].
-wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int S, int prec, EigH &e)
+// then(Y, work, nw, nsmp, smp0, n): launches on Y.stream for the solves of one unit, where
+// the units run side by side (*ran: it was called for all of them).
+using UnitStep = std::function<wpcd_status(Exec &, const int *, int, int, int, int)>;
+wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int S, int prec, EigH &e,
+                      const UnitStep &then = UnitStep(), bool *ran = nullptr)
 {
     wpcd_status st = WPCD_OK;
     if (v.n_terms > 1) {
@@ -1068,7 +1102,13 @@ wpcd_status diag_body(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int 
                 if ((st = run_bucket(X, v.ident_dev + k, 1, 1, s, v.cd[k].n))) return st;
     } else {
         std::vector<wpcd_status> sts;
-        if (!fork_buckets(c, X, v, S, prec, run_bucket, sts))
+        auto run_unit = [&](Exec &Y, const int *work, int nw, int nsmp, int smp0, int n) {
+            const wpcd_status u = run_bucket(Y, work, nw, nsmp, smp0, n);
+            return u || !then ? u : then(Y, work, nw, nsmp, smp0, n);
+        };
+        if (fork_units(c, X, v, S, prec, run_unit, sts)) {
+            if (ran) *ran = (bool)then;
+        } else
             for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it)
                 if ((st = run_bucket(X, v.bucket_dev[it->first], (int)it->second.size(), S, 0, it->first))) return st;
         for (wpcd_status f : sts)
@@ -1083,11 +1123,11 @@ wpcd_status run_diag(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, const double *
     return st ? st : diag_body(c, X, v, coeffs, S, prec, e);
 }
 
-// Energy plan + T at the needed bins into the executor's workspaces.  With
+// Energy plan and the room for T at the needed bins in the executor's workspaces.  With
 // n_E_s (device, per-sample list lengths) every sample has its own energy
 // list at e_lab + s * n_E; otherwise one list serves all samples.
-wpcd_status run_tbin(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *e_lab, int n_E, const int *n_E_s,
-                     PlanDev &plan, int res = WPCD_AVG_FREE_BIN)
+wpcd_status plan_tbin(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *e_lab, int n_E, const int *n_E_s,
+                      PlanDev &plan, int res = WPCD_AVG_FREE_BIN)
 {
     const int nch = v.n_ch, maxN = v.maxN, S = e.n_samples;
     const int P = n_E_s ? S : 1;
@@ -1107,47 +1147,75 @@ wpcd_status run_tbin(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *e_la
     plan.per_sample = n_E_s ? 1 : 0;
     plan.n_E_s = n_E_s;
     plan.ip_frac = c->ip_frac;
-    {
-        Launch L(c, X, WPCD_PHASE_PLAN);
-        CK(launch_plan(e.cd_dev, nch, maxN, e_lab, n_E, plan, X.err, X.stream, P));
-    }
-    Launch L(c, X, WPCD_PHASE_TMATRIX);
+    Launch L(c, X, WPCD_PHASE_PLAN);
+    CK(launch_plan(e.cd_dev, nch, maxN, e_lab, n_E, plan, X.err, X.stream, P));
+    return WPCD_OK;
+}
+
+// T at the needed bins of nsmp samples from smp0 on of nw channels of size n, on Y.stream (X
+// holds the results, Y the scratch).  FP64: in sample chunks, the needed rows of V C from the
+// tensor cores, then T; small matrices, or without room for the rows, form them in the T kernel.
+wpcd_status tbin_unit(wpcd_ctx *c, Exec &X, Exec &Y, VSetH &v, EigH &e, int n_E, const PlanDev &plan, int res,
+                      const int *work, int nw, int nsmp, int smp0, int n)
+{
+    const int nch = v.n_ch, maxN = v.maxN;
     const double *cf = v.n_terms > 1 ? e.coeffs : nullptr;
     double *tb = static_cast<double *>(X.ws_tbin.p), *pb = static_cast<double *>(X.ws_phbin.p);
-    if (e.prec == WPCD_PREC_MIXED) {
-        CK(launch_tbin(e.cd_dev, nch, S, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, true, res));
-        return WPCD_OK;
+    const size_t per = vc_rows_scratch_per_item(n);
+    const bool mixed = e.prec == WPCD_PREC_MIXED;
+    int chunk = 0;
+    if (!mixed && n >= kVcRowsN) {
+        chunk = (int)std::min<size_t>((size_t)nsmp, std::max<size_t>(1, kVcScratchBytes / (per * nw)));
+        chunk = std::min(chunk, std::max(1, 65535 / nw));  // items in the grid's y
+        while (chunk > 0 && ws_reserve(c, Y, Y.ws_ref, per * nw * chunk)) chunk /= 2;
     }
-    // FP64: per size bucket, in sample chunks, the needed rows of V C from the tensor cores, then T;
-    // a bucket of small matrices, or without room for the rows, forms them in the T kernel
-    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
-        const int n = it->first, nw = (int)it->second.size();
-        const size_t per = vc_rows_scratch_per_item(n);
-        int chunk = 0;
-        if (n >= kVcRowsN) {
-            chunk = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, kVcScratchBytes / (per * nw)));
-            chunk = std::min(chunk, std::max(1, 65535 / nw));  // items in the grid's y
-            while (chunk > 0 && ws_reserve(c, X, X.ws_ref, per * nw * chunk)) chunk /= 2;
-        }
-        TWork tw;
-        tw.work = v.bucket_dev[n];
-        tw.n_work = nw;
-        tw.n = n;
-        if (chunk == 0) {
-            CK(launch_tbin(e.cd_dev, nch, S, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, false,
-                           res, tw));
-            continue;
-        }
-        for (int s0 = 0; s0 < S; s0 += chunk) {
-            const int ns = std::min(chunk, S - s0);
-            tw.sample0 = s0;
-            CK(launch_vc_rows(e.cd_dev, tw.work, nw, ns, s0, n, v.n_terms, cf, e.C, plan, nch, maxN, X.ws_ref.p, &tw.rows,
-                              X.err, X.stream));
-            CK(launch_tbin(e.cd_dev, nch, ns, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, X.stream, false,
-                           res, tw));
-        }
+    TWork tw;
+    tw.work = work;
+    tw.n_work = nw;
+    tw.n = n;
+    for (int s0 = 0; s0 < nsmp; s0 += chunk ? chunk : nsmp) {
+        const int ns = chunk ? std::min(chunk, nsmp - s0) : nsmp;
+        tw.sample0 = smp0 + s0;
+        if (chunk)
+            CK(launch_vc_rows(e.cd_dev, work, nw, ns, tw.sample0, n, v.n_terms, cf, e.C, plan, nch, maxN, Y.ws_ref.p,
+                              &tw.rows, X.err, Y.stream));
+        CK(launch_tbin(e.cd_dev, nch, ns, v.n_terms, cf, e.eps, e.C, plan, maxN, n_E, tb, pb, X.err, Y.stream, mixed, res, tw));
     }
     return WPCD_OK;
+}
+
+// T at the needed bins of the whole batch.
+wpcd_status run_tbin(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, int n_E, const PlanDev &plan, int res = WPCD_AVG_FREE_BIN)
+{
+    Launch L(c, X, WPCD_PHASE_TMATRIX);
+    if (e.prec == WPCD_PREC_MIXED) {
+        CK(launch_tbin(e.cd_dev, v.n_ch, e.n_samples, v.n_terms, v.n_terms > 1 ? e.coeffs : nullptr, e.eps, e.C, plan, v.maxN,
+                       n_E, static_cast<double *>(X.ws_tbin.p), static_cast<double *>(X.ws_phbin.p), X.err, X.stream, true,
+                       res));
+        return WPCD_OK;
+    }
+    for (auto it = v.buckets.rbegin(); it != v.buckets.rend(); ++it) {
+        wpcd_status st = tbin_unit(c, X, X, v, e, n_E, plan, res, v.bucket_dev[it->first], (int)it->second.size(),
+                                   e.n_samples, 0, it->first);
+        if (st) return st;
+    }
+    return WPCD_OK;
+}
+
+// The eigensolve that diag_prep set up and T from it: T of a unit right behind its eigenpairs
+// where the units run side by side.
+wpcd_status diag_tbin(wpcd_ctx *c, Exec &X, VSetH &v, const double *coeffs, int S, int prec, EigH &e, const double *e_lab,
+                      int n_E, const int *n_E_s, PlanDev &plan, int res = WPCD_AVG_FREE_BIN)
+{
+    wpcd_status st = plan_tbin(c, X, v, e, e_lab, n_E, n_E_s, plan, res);
+    if (st) return st;
+    bool ran = false;
+    auto then = [&](Exec &Y, const int *work, int nw, int nsmp, int smp0, int n) {
+        Launch L(c, Y, WPCD_PHASE_TMATRIX);
+        return tbin_unit(c, X, Y, v, e, n_E, plan, res, work, nw, nsmp, smp0, n);
+    };
+    if ((st = diag_body(c, X, v, coeffs, S, prec, e, then, &ran))) return st;
+    return ran ? WPCD_OK : run_tbin(c, X, v, e, n_E, plan, res);
 }
 
 // T at the energies and/or phases + cross sections, after run_tbin.
@@ -1634,8 +1702,8 @@ static wpcd_status tmatrix_impl(wpcd_ctx *c, VSetH &v, EigH &e, const double *e_
 {
     if (!resolvent_ok(v, res)) return WPCD_ERR_ARG;
     PlanDev plan{};
-    wpcd_status st = run_tbin(c, c->main, v, e, e_lab, n_E, nullptr, plan, res);
-    if (st) return st;
+    wpcd_status st = plan_tbin(c, c->main, v, e, e_lab, n_E, nullptr, plan, res);
+    if (st || (st = run_tbin(c, c->main, v, e, n_E, plan, res))) return st;
     return run_outputs(c, c->main, v, e, n_E, plan, t_out, delta, sigma, res);
 }
 
@@ -1680,8 +1748,9 @@ static wpcd_status solve_graph(wpcd_ctx *c, VSetH &v, int vset_id, const double 
     Exec &X = c->main;
     EigH &e = X.eig;
     auto body = [&]() -> wpcd_status {
-        wpcd_status st = diag_body(c, X, v, coeffs, S, prec, e);
-        return st ? st : tmatrix_impl(c, v, e, e_lab, n_E, res, t_out, delta, sigma);
+        PlanDev plan{};
+        wpcd_status st = diag_tbin(c, X, v, coeffs, S, prec, e, e_lab, n_E, nullptr, plan, res);
+        return st ? st : run_outputs(c, X, v, e, n_E, plan, t_out, delta, sigma, res);
     };
     typedef unsigned long long u64;
     const std::array<u64, 12> key = {(u64)vset_id, (u64)S, (u64)n_E, (u64)prec, (u64)res, (u64)c->refine_engine,
@@ -1763,9 +1832,11 @@ wpcd_status wpcd_solve(wpcd_ctx *c, int vset_id, const double *coeffs, int S, co
     CK(cudaSetDevice(c->device));
     if (c->use_graphs && c->exec_mode == WPCD_EXEC_BATCHED && !c->prof)
         return solve_graph(c, v, vset_id, coeffs, S, e_lab, n_E, prec, res, t_out, delta, sigma);
-    wpcd_status st = run_diag(c, c->main, v, vset_id, coeffs, S, prec, c->main.eig);
-    if (st) return st;
-    return tmatrix_impl(c, v, c->main.eig, e_lab, n_E, res, t_out, delta, sigma);
+    Exec &X = c->main;
+    PlanDev plan{};
+    wpcd_status st = diag_prep(c, X, v, vset_id, S, prec, X.eig);
+    if (st || (st = diag_tbin(c, X, v, coeffs, S, prec, X.eig, e_lab, n_E, nullptr, plan, res))) return st;
+    return run_outputs(c, X, v, X.eig, n_E, plan, t_out, delta, sigma, res);
 }
 
 wpcd_status wpcd_solve_host(wpcd_ctx *c, int vset_id, const double *coeffs_h, int S, const double *e_lab_h, int n_E,
@@ -2369,9 +2440,9 @@ wpcd_status launch_batch(Server *sv, Slot &sl)
     int *dn = reinterpret_cast<int *>(de + (size_t)S * nE);
     double *dout = static_cast<double *>(X.ws_out.p);
     CK(cudaMemcpyAsync(dc, hc, in_bytes, cudaMemcpyHostToDevice, X.stream));
-    if ((st = run_diag(c, X, v, m.vset_id, v.n_terms > 1 ? dc : nullptr, S, r0.prec, X.eig))) return st;
     PlanDev plan{};
-    if ((st = run_tbin(c, X, v, X.eig, de, nE, dn, plan))) return st;
+    if ((st = diag_prep(c, X, v, m.vset_id, S, r0.prec, X.eig))) return st;
+    if ((st = diag_tbin(c, X, v, v.n_terms > 1 ? dc : nullptr, S, r0.prec, X.eig, de, nE, dn, plan))) return st;
     if ((st = run_outputs(c, X, v, X.eig, nE, plan, dout, dout + sl.nt, dout + sl.nt + sl.nd))) return st;
     CK(cudaMemcpyAsync(dout + sl.nt + sl.nd + sl.ns, X.err, sizeof(int), cudaMemcpyDeviceToDevice, X.stream));
     CK(cudaMemcpyAsync(dout + sl.nt + sl.nd + sl.ns + 1, X.eig.status, sizeof(int) * S * v.n_ch,

@@ -102,3 +102,45 @@ def test_one_solve_per_launch_same_bits(ctx, prec):
         ctx.set_exec(api.EXEC_BATCHED)
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+def test_sample_ranges_same_bits(ctx):
+    """One size bucket above a stream's share of the scratch goes in sample ranges."""
+    from paper_2106_00454_gb300 import api
+    wl = _wl([CPL], 100, 2500, 3)
+    md = api.Model(ctx, wl)
+    gpu_run(ctx, md, dataclasses.replace(wl, coeffs=wl.coeffs[:2]), prec=1)
+    whole = gpu_run(ctx, md, wl, prec=1)
+    for s in (0, 1240, 1250, 2490):
+        part = gpu_run(ctx, md, dataclasses.replace(wl, coeffs=wl.coeffs[s:s + 10]), prec=1)
+        for x, y in zip(part, whole):
+            assert np.array_equal(x, y[s:s + 10])
+
+
+def test_no_room_for_the_streams_same_bits(ctx):
+    """A budget that holds one bucket's scratch at a time, not a share for each stream."""
+    import torch
+    from paper_2106_00454_gb300 import api
+    wl = W.workload_batched(n_samples=40, n_e=9, nwp_choices=(30, 31, 32, 33))
+    S, nch = 40, len(wl.channels)
+
+    def phases(c, md, n):
+        cf = torch.tensor(wl.coeffs, dtype=torch.float64, device="cuda:0")
+        e = torch.tensor(wl.e_lab, dtype=torch.float64, device="cuda:0")
+        d = torch.zeros((S, nch, 9, 3), dtype=torch.float64, device="cuda:0")
+        for _ in range(n):
+            c.solve(md.vset, cf, S, e, None, d, None, prec=1)
+            c.sync()
+        return d.cpu().numpy()
+
+    probe = api.Context(0)
+    md = api.Model(probe, wl)
+    probe.profile(True)  # one bucket after another
+    phases(probe, md, 2)
+    room = probe.bytes_in_use() + (1 << 20)
+    probe.close()
+    tight = api.Context(0, hbm_budget_bytes=room)
+    a = phases(tight, api.Model(tight, wl), 4)
+    assert tight.bytes_in_use() <= room
+    tight.close()
+    assert np.array_equal(a, phases(ctx, api.Model(ctx, wl), 3))
