@@ -574,8 +574,10 @@ int mi_slots_per_sm(int n, int NQ)
 // inverse of k_mi_solve (which takes the systems that do not converge here).
 // Per energy this costs K n^2 FP64 multiply-adds a residual (the bound: two or
 // three of them) instead of an n^3 elimination whose n steps wait for each other:
-// 64 samples x 15 channels x 32 energies, N_Q = 96: 134.4 -> 22.0 ms, errors against
-// 64 bits unchanged (the eigendecompositions are 15 ms of it).
+// 64 samples x 15 channels x 32 energies, N_Q = 96: 134.4 -> 20.1 ms, errors against
+// 64 bits unchanged (the eigendecompositions are 10 ms of it).  The rest of the pass is
+// kept off the FP64 pipe where it can be: -w / D as a product with (k^2 - p^2) / (2 mu w
+// k^2), one reciprocal for D and the sum in D_N, V summed over one triangle (20.9 -> 20.1).
 
 // S V_t S over the grid and k^2, from the grid terms of every channel.
 __global__ void __launch_bounds__(256) k_mi_scale(const MiChanDev *chans, int n_ch, int NQ, const double *kg,
@@ -615,12 +617,12 @@ constexpr int kMeMaxRefine = 10;
 __host__ __device__ inline int me_ldq(int ng) { return ng | 1; }  // odd row pitch of Q: conflict-free along both indices
 
 // Q float [ng][ldq] | z, x, b double [ng][8] | T = M^-1 v, u, h float [ng][8] | lambda, S double [ng] |
-// D double [NQ][8 / K] | per column: p^2, D_N, x_p, r_p, y_p ... double [8 x 16] | maxima double [16][16]
+// 1 / (2 mu w k^2) double [NQ] | D double [NQ][8 / K] | per column: p^2, D_N, x_p, r_p, y_p ... double [8 x 16] | maxima double [16][16]
 __host__ __device__ inline size_t me_smem(int ng, int NQ, int K)
 {
     size_t b = ((size_t)ng * me_ldq(ng) * 4 + 15) & ~(size_t)15;
     b += (size_t)3 * ng * kMeCols * 8 + (size_t)3 * ng * kMeCols * 4 + (size_t)2 * ng * 8;
-    b += (size_t)NQ * (kMeCols / K) * 8 + (size_t)8 * 16 * 8 + (size_t)32 * kMeCols * 8;
+    b += (size_t)(NQ + (NQ & 1)) * 8 + (size_t)NQ * (kMeCols / K) * 8 + (size_t)8 * 16 * 8 + (size_t)32 * kMeCols * 8;
     return b;
 }
 
@@ -689,7 +691,8 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
     double *z = reinterpret_cast<double *>(me_sm + (((size_t)ng * ldq * 4 + 15) & ~(size_t)15));  // D x, or a right-hand side
     double *x = z + (size_t)ng * kMeCols, *b = x + (size_t)ng * kMeCols;
     double *lam = b + (size_t)ng * kMeCols, *Sg = lam + ng;
-    double *D = Sg + ng;                                   // [NQ][EC]
+    double *iw = Sg + ng;                                  // [NQ]: 1 / (2 mu w k^2)
+    double *D = iw + NQ + (NQ & 1);                        // [NQ][EC] (T, u, h further on need 16 bytes)
     double *p2c = D + (size_t)NQ * EC;                     // per column: p^2
     double *DNc = p2c + 8, *xp = DNc + 8, *rp = xp + 16, *Rm = rp + 16, *Vpp = Rm + 16, *wp = Vpp + 16;  // [8][K] each
     double *ymx = wp + 16, *ypr = ymx + 8;                 // maxima of the correction, this step's and the last one's
@@ -707,17 +710,22 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
         const double *Qg = Q_all + ec.c_off + (size_t)(smp - sample0) * ng * ng;
         const double *lg = eps_all + ec.eps_off + (size_t)(smp - sample0) * ng;
         __syncthreads();  // the last item is done with shared memory
-        for (int e = tid; e < ng * ng; e += nt) {
-            const int r = e / ng, c = e - r * ng;
-            const size_t o = (size_t)((r / NQ) * M + r % NQ) * ch.n + (c / NQ) * M + c % NQ;
-            double v = Vgc[o];
-            for (int t = 1; t < n_terms; ++t) v = fma(cf[t - 1], Vgc[(size_t)t * ch.n * ch.n + o], v);
-            V[e] = v;
-            Q[r * ldq + c] = (float)Qg[e];
+        for (int r = warp; r < ng; r += nw) {  // V is symmetric: the upper triangle, mirrored
+            const size_t orow = (size_t)((r / NQ) * M + r % NQ) * ch.n;
+            for (int c = lane; c < ng; c += 32) {
+                Q[r * ldq + c] = (float)Qg[(size_t)r * ng + c];
+                if (c < r) continue;
+                const size_t o = orow + (c / NQ) * M + c % NQ;
+                double v = Vgc[o];
+                for (int t = 1; t < n_terms; ++t) v = fma(cf[t - 1], Vgc[(size_t)t * ch.n * ch.n + o], v);
+                V[(size_t)r * ng + c] = v;
+                V[(size_t)c * ng + r] = v;
+            }
         }
         for (int i = tid; i < ng; i += nt) {
             lam[i] = lg[i];
             Sg[i] = sqrt(2.0 * kMu * wg[i % NQ]) * kg[i % NQ];
+            if (i < NQ) iw[i] = 1.0 / (wg[i] * kg[i] * kg[i] * 2.0 * kMu);
         }
         int worst = 0;
         for (int e0 = 0; e0 < n_I; e0 += EC) {
@@ -728,9 +736,9 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
                 const double p = sqrt(kMn * e_int[ie] / 2.0) / kHbarc, p2 = p * p;
                 double part = 0.0;
                 for (int j = lane; j < NQ; j += 32) {
-                    const double den = p2 - kg[j] * kg[j];
-                    D[j * EC + el] = wg[j] * kg[j] * kg[j] * 2.0 * kMu / den;
-                    part += wg[j] / den;
+                    const double rden = 1.0 / (p2 - kg[j] * kg[j]);
+                    D[j * EC + el] = wg[j] * kg[j] * kg[j] * 2.0 * kMu * rden;
+                    part = fma(wg[j], rden, part);
                 }
                 for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
                 if (lane < K) {
@@ -803,17 +811,17 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
                 double ym[kMeCols / 4], xm[kMeCols / 4];  // this thread's columns are tid % 4, + 4
                 for (int q = 0; q < kMeCols / 4; ++q) ym[q] = xm[q] = 0.0;
                 for (int e = tid; e < ng * 4; e += nt) {
-                    const int r = e >> 2;
+                    const int r = e >> 2, j = r % NQ;
+                    const double k2 = kg[j] * kg[j], iwj = iw[j];
 #pragma unroll
                     for (int q = 0; q < kMeCols / 4; ++q) {
                         const int c = (e & 3) + 4 * q, k0 = (c / K) * K;
                         float w = h[r * kMeCols + c];
                         double t = (double)w;
                         for (int a = 0; a < K; ++a) t = fma((double)T[r * kMeCols + k0 + a], wp[c * 2 + a], t);
-                        const double d = D[(r % NQ) * EC + c / K];
-                        const double y = -t / d, xn = x[r * kMeCols + c] + y;
+                        const double y = t * ((k2 - p2c[c]) * iwj), xn = x[r * kMeCols + c] + y;  // -t / D
                         x[r * kMeCols + c] = xn;
-                        z[r * kMeCols + c] = d * xn;
+                        z[r * kMeCols + c] = D[j * EC + c / K] * xn;
                         ym[q] = nan_max(ym[q], fabs(y));
                         xm[q] = nan_max(xm[q], fabs(xn));
                     }
