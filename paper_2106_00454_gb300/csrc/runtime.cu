@@ -2117,16 +2117,14 @@ wpcd_status mi_eigen_set(wpcd_ctx *c, MiH &m)
     return WPCD_OK;
 }
 
-// Eigenpairs of S samples of one block size of an MI set into X.eig, on the FP64
-// path; a solve that fails shows in the energies (their refinement does not converge).
-wpcd_status mi_eigen(wpcd_ctx *c, Exec &X, MiH &m, const double *cf, int S, int K)
+// Eigenpairs of S samples of one block size of an MI set into e (as diag_prep left it), on the
+// FP64 path; a solve that fails shows in the energies (their refinement does not converge).
+wpcd_status mi_eigen(wpcd_ctx *c, Exec &Y, EigH &e, MiH &m, const double *cf, int S, int K)
 {
-    wpcd_status st = diag_prep(c, X, m.set, -1, S, WPCD_PREC_FP64, X.eig);
-    if (st) return st;
-    int *err = X.err;
-    X.err = nullptr;
-    st = run_bucket_f64(c, X, m.set, X.eig, cf, m.work_dev[K - 1], m.n_work[K - 1], S, 0, K * m.NQ);
-    X.err = err;
+    int *err = Y.err;
+    Y.err = nullptr;
+    const wpcd_status st = run_bucket_f64(c, Y, m.set, e, cf, m.work_dev[K - 1], m.n_work[K - 1], S, 0, K * m.NQ);
+    Y.err = err;
     return st;
 }
 }  // namespace
@@ -2258,52 +2256,109 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
                              X.stream));
     }
     const double *cf = m.n_terms > 1 ? coeffs : nullptr;
-    for (int K = 2; K >= 1; --K) {
-        const int nw = m.n_work[K - 1];
-        if (!nw) continue;
-        const int n = K * M, ng = K * m.NQ;
-        // One eigendecomposition costs three to four systems by elimination, and its latency more where
-        // the chip is not full: measured at 15 channels, N_Q = 24 / 48 / 96, the two meet at ~1900
-        // systems (4 samples x 32 energies: 2.35 against 2.46 ms, 3.8 / 4.4, 10.1 / 9.6; 1 sample 2.3 / 1.0,
-        // 3.7 / 1.5, 9.5 / 3.1; 64 samples 5.0 / 30.9, 7.6 / 56.9, 21.9 / 134.6; at 8 energies and 64
-        // samples still 3.6 / 8.5, 5.0 / 14.8, 15.2 / 33.7)
-        bool eig = m.has_set && mi_energies_fit(m.NQ, K) && n_I >= 4 && (long long)S * m.n_ch * n_I >= 12ll * c->n_sm;
-        if (eig) {
-            const int slots = std::max(1, std::min(S * nw, std::max(1, mi_energies_per_sm(m.NQ, K)) * c->n_sm));
-            // eigenpairs of a few GB of samples at a time
-            size_t per = 0;
-            for (auto &d : m.set.cd) per += (size_t)d.n * d.n * 8;
-            const int Sc = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, ((size_t)4 << 30) / per));
-            for (int s0 = 0; s0 < S && eig; s0 += Sc) {
-                const int ns = std::min(Sc, S - s0);
-                const double *cfs = cf ? cf + (size_t)s0 * (m.n_terms - 1) : nullptr;
-                if (mi_eigen(c, X, m, cfs, ns, K) || ws_reserve(c, X, X.ws_ref, (size_t)slots * ng * ng * sizeof(double))) {
-                    eig = false;  // no room: by elimination, from the first sample on
-                    CK(cudaMemsetAsync(status, 0, sizeof(int) * S * m.n_ch, X.stream));
-                    break;
-                }
-                Launch L(c, X, WPCD_PHASE_MI);
-                CK(launch_mi_energies(m.ch_dev, X.eig.cd_dev, m.work_dev[K - 1], nw, K, m.n_ch, s0, ns, m.NQ, m.kg, m.wg,
-                                      m.n_terms, cf, m.Vg, Von, n_I, e_int, X.eig.eps, X.eig.C,
-                                      static_cast<double *>(X.ws_ref.p), slots, ph, k_out, status, redo, X.err, X.stream));
-            }
-        }
-        const int per_sm = mi_slots_per_sm(n, m.NQ);
-        if (per_sm < 1) return WPCD_ERR_ARG;
-        // by elimination (after the eigendecomposition only the systems that did not converge, one
-        // by one), the energies of a (sample, channel) split over as many CTAs as the chip holds
-        const long long items = (long long)S * nw;
-        const int cap = per_sm * c->n_sm;
+    // One eigendecomposition costs three to four systems by elimination, and its latency more where
+    // the chip is not full: measured at 15 channels, N_Q = 24 / 48 / 96, the two meet at ~1900
+    // systems (4 samples x 32 energies: 2.35 against 2.46 ms, 3.8 / 4.4, 10.1 / 9.6; 1 sample 2.3 / 1.0,
+    // 3.7 / 1.5, 9.5 / 3.1; 64 samples 5.0 / 30.9, 7.6 / 56.9, 21.9 / 134.6; at 8 energies and 64
+    // samples still 3.6 / 8.5, 5.0 / 14.8, 15.2 / 33.7)
+    auto by_eigen = [&](int K) {
+        return m.has_set && mi_energies_fit(m.NQ, K) && n_I >= 4 && (long long)S * m.n_ch * n_I >= 12ll * c->n_sm;
+    };
+    auto eig_slots = [&](int K) {
+        return std::max(1, std::min(S * m.n_work[K - 1], std::max(1, mi_energies_per_sm(m.NQ, K)) * c->n_sm));
+    };
+    // eigenpairs of a few GB of samples at a time
+    size_t per = 1;
+    for (auto &d : m.set.cd) per += (size_t)d.n * d.n * 8;
+    const int Sc = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, ((size_t)4 << 30) / per));
+    // by elimination (after the eigendecomposition only the systems that did not converge, one
+    // by one), the energies of a (sample, channel) split over as many CTAs as the chip holds
+    struct Elim {
+        int ne, slots;
+        size_t bytes;
+    };
+    auto elim = [&](int K, bool eig) {
+        const long long items = (long long)S * m.n_work[K - 1];
+        const int n = K * M, cap = mi_slots_per_sm(n, m.NQ) * c->n_sm;
         const int chunks = eig ? n_I : (int)std::max<long long>(1, std::min<long long>(n_I, cap / items));
         const int ne = (n_I + chunks - 1) / chunks, nck = (n_I + ne - 1) / ne;
         const int slots = (int)std::max<long long>(1, std::min<long long>(items * nck, cap));
         // two FP64 n x n matrices per slot: V, and the rarely used FP64 elimination fallback
-        if ((st = ws_reserve(c, X, X.ws_ref, (size_t)slots * 2 * n * n * sizeof(double)))) return st;
-        Launch L(c, X, WPCD_PHASE_MI);
+        return Elim{ne, slots, (size_t)slots * 2 * n * n * sizeof(double)};
+    };
+    // the systems of one block size on Y.stream, in Y's scratch (prepared: X.eig is set up for all samples)
+    auto pass = [&](Exec &Y, int K, bool prepared) -> wpcd_status {
+        const int nw = m.n_work[K - 1], n = K * M, ng = K * m.NQ;
+        bool eig = by_eigen(K);
+        for (int s0 = 0; s0 < S && eig; s0 += Sc) {
+            const int ns = std::min(Sc, S - s0), slots = eig_slots(K);
+            const double *cfs = cf ? cf + (size_t)s0 * (m.n_terms - 1) : nullptr;
+            if ((!prepared && diag_prep(c, X, m.set, -1, ns, WPCD_PREC_FP64, X.eig)) ||
+                mi_eigen(c, Y, X.eig, m, cfs, ns, K) || ws_reserve(c, Y, Y.ws_ref, (size_t)slots * ng * ng * sizeof(double))) {
+                eig = false;  // no room: by elimination, from the first sample on
+                break;
+            }
+            Launch L(c, Y, WPCD_PHASE_MI);
+            CK(launch_mi_energies(m.ch_dev, X.eig.cd_dev, m.work_dev[K - 1], nw, K, m.n_ch, s0, ns, m.NQ, m.kg, m.wg,
+                                  m.n_terms, cf, m.Vg, Von, n_I, e_int, X.eig.eps, X.eig.C,
+                                  static_cast<double *>(Y.ws_ref.p), slots, ph, k_out, status, redo, X.err, Y.stream));
+        }
+        if (mi_slots_per_sm(n, m.NQ) < 1) return WPCD_ERR_ARG;
+        const Elim el = elim(K, eig);
+        wpcd_status es = ws_reserve(c, Y, Y.ws_ref, el.bytes);
+        if (es) return es;
+        Launch L(c, Y, WPCD_PHASE_MI);
         CK(launch_mi_solve(m.ch_dev, m.work_dev[K - 1], nw, n, m.n_ch, S, m.NQ, m.kg, m.wg, m.n_terms, cf, m.Vg, Von,
-                           n_I, e_int, static_cast<double *>(X.ws_ref.p), slots, ph, k_out, status, X.err, X.stream, ne,
+                           n_I, e_int, static_cast<double *>(Y.ws_ref.p), el.slots, ph, k_out, status, X.err, Y.stream, el.ne,
                            eig ? redo : nullptr));
-    }
+        return WPCD_OK;
+    };
+    // Both block sizes by eigendecomposition: side by side on two streams, as the size buckets of a solve
+    // (the last wave and the latencies of one beside the other: 64 samples x 15 channels x 32 energies,
+    // N_Q = 96, 20.1 -> 17.0 ms, same bits).
+    auto side_by_side = [&](wpcd_status *out) {
+        if (c->prof || !m.n_work[0] || !m.n_work[1] || !by_eigen(1) || !by_eigen(2) || Sc < S ||
+            mi_slots_per_sm(M, m.NQ) < 1 || mi_slots_per_sm(2 * M, m.NQ) < 1)
+            return false;
+        if (diag_prep(c, X, m.set, -1, S, WPCD_PREC_FP64, X.eig)) return false;
+        size_t share[2];
+        for (int K = 1; K <= 2; ++K)
+            share[K - 1] = (std::max(std::max(F64Scratch(c, K * m.NQ, m.n_work[K - 1]).bytes(S), elim(K, true).bytes),
+                                     (size_t)eig_slots(K) * K * m.NQ * K * m.NQ * sizeof(double)) + 255) & ~(size_t)255;
+        const size_t total = share[0] + share[1];
+        if (total > kRefineScratchBytes || total >= X.no_fork || !side_streams(X)) return false;
+        if (ws_reserve(c, X, X.ws_ref, total)) {
+            X.no_fork = total;
+            return false;
+        }
+        if (c->autotune) {  // the autotuner times its candidates alone
+            std::lock_guard<std::mutex> tl(c->tmu);
+            for (int K = 1; K <= 2; ++K)
+                if (jacobi_fits_smem(K * m.NQ, false) && !c->tuned.count(std::make_pair(K * m.NQ, (int)WPCD_PREC_FP64)))
+                    return false;
+        }
+        if (cudaEventRecord(X.ev_fork, X.stream) != cudaSuccess) return false;
+        cudaStreamWaitEvent(X.side[0], X.ev_fork, 0);
+        for (int K = 2; K >= 1; --K) {
+            Exec Y;
+            Y.stream = K == 2 ? X.stream : X.side[0];
+            Y.err = X.err;
+            Y.ws_ref.p = static_cast<unsigned char *>(X.ws_ref.p) + (K == 2 ? 0 : share[1]);
+            Y.ws_ref.n = share[K - 1];
+            Y.ws_ref.part = true;
+            const wpcd_status es = pass(Y, K, true);
+            if (es) *out = es;
+        }
+        if (cudaEventRecord(X.ev_join[0], X.side[0]) != cudaSuccess ||
+            cudaStreamWaitEvent(X.stream, X.ev_join[0], 0) != cudaSuccess)
+            *out = WPCD_ERR_CUDA;
+        return true;
+    };
+    st = WPCD_OK;
+    if (!side_by_side(&st))
+        for (int K = 2; K >= 1 && !st; --K)
+            if (m.n_work[K - 1]) st = pass(X, K, false);
+    if (st) return st;
     if (delta || sigma) {
         Launch L(c, X, WPCD_PHASE_MI);
         CK(launch_mi_observables(m.ch_dev, m.n_ch, S, n_I, e_int, ph, n_E, e_lab, delta, sigma, X.stream));

@@ -144,3 +144,23 @@ def test_no_room_for_the_streams_same_bits(ctx):
     assert tight.bytes_in_use() <= room
     tight.close()
     assert np.array_equal(a, phases(ctx, api.Model(ctx, wl), 3))
+
+
+@pytest.mark.parametrize("nq,S", [(24, 60), (33, 41)])
+def test_inversion_side_by_side_same_bits(ctx, nq, S):
+    """Both block sizes of an inversion on two streams (once their kernels are tuned),
+    against one after the other (profiling)."""
+    from test_gpu_mi import _gpu
+    chs = [c.astuple() for c in W.np_channels(2)]
+    coeffs, e_lab, e_int = W.coefficient_samples(S, 6), W.lab_energies(9), W.chebyshev_energies(14)
+    args = (chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, coeffs, e_int, e_lab, nq)
+    assert S * len(chs) * 14 >= 12 * 152
+    runs = [_gpu(ctx, *args) for _ in range(3)]
+    ctx.profile(True)
+    try:
+        runs.append(_gpu(ctx, *args))
+    finally:
+        ctx.profile(False)
+    for r in runs[1:]:
+        for x, y in zip(r, runs[0]):
+            assert np.array_equal(x, y)
