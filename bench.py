@@ -14,7 +14,7 @@ step end to end through wpcd_solve_host (host buffers, copies timed), the
 dominant kernel's roofline, the plain (one eigensolve per launch) and batched
 FP64 paths on the same GPU, the mixed path's error against the FP64 path and
 against the CPU oracle on a seeded subset, the 4096-sample x 15-channel
-batched workload (FP64 eigensolve as specified, and mixed), the MI comparison
+batched workload (FP64 and mixed), the MI comparison
 method, spin observables, a served Poisson request stream with N_WP in
 {32, 64, 128, 256} (latency, the FP64 per-request latency, a saturation
 sweep), and the oracle's CPU throughput.
@@ -694,12 +694,12 @@ def run_wpcd(args, ws, rank, lrank):
         eig_ms, eig_n = prof["eigen"]
         ref_ms, ref_n = prof["refine"]
         big = [n * (2 if c.coupled else 1) for n, c in zip(wl.nwp, wl.channels)]
-        jac = {"kernel": "k_jacobi_f64" if prec == api.PREC_FP64 else "k_jacobi_mixed", "bound": "alu",
+        jac = {"kernel": "k_jacobi_mixed (n < 160), k_jacobi_teams (160 <= n <= 304)", "bound": "alu",
                "flops_per_step": S * (8.0 / 3.0) * sum_n3,
                "flops_note": "(8/3) n^3 per channel-solve, the paper's symmetric-eigensolve count (Sec. 4.2.1)",
                "ms_per_step": eig_ms / kp, "launches_per_step": eig_n / kp, "matrix_sizes": sorted(set(big)),
-               "peak": FP64_PEAK_TFLOPS if prec == api.PREC_FP64 else FP32_PEAK_TFLOPS,
-               "peak_source": FP64_PEAK_NOTE if prec == api.PREC_FP64 else FP32_PEAK_NOTE,
+               "peak": FP32_PEAK_TFLOPS,
+               "peak_source": FP32_PEAK_NOTE,
                "timing": ("CUDA events around each eigensolver launch (one kernel per launch), over "
                           f"{kp} further steps launched kernel by kernel")}
         if args.exec == "batched" and args.sweep_samples > 0:

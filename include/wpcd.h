@@ -112,8 +112,9 @@ enum {
  * from C0^T H C0, C0 the FP64 eigenvectors of the projected set's diag(H0) + V0
  * (built once per set, on its first mixed solve), which is nearly diagonal for
  * samples near the mean and takes fewer Jacobi sweeps; the refined
- * eigenvectors are rotated back with FP64-accurate products.  0 = the FP32
- * eigensolve starts from H itself.  WPCD_OPT_REFINE_ITERS (1..4, default 2):
+ * eigenvectors are rotated back with FP64-accurate products.  The FP64 path's
+ * FP32 start takes the same kind of basis (on the set's first FP64 solve; not
+ * under an HBM budget).  0 = the FP32 eigensolve starts from H itself.  WPCD_OPT_REFINE_ITERS (1..4, default 2):
  * FP64 refinement iterations of the mixed path; each squares the eigenvector
  * error.  Measured on the 16384-sample N_WP = 150 workload against the FP64
  * path: two iterations leave phase errors below 1e-6 deg and cross-section
