@@ -46,7 +46,12 @@ constexpr int kRefineIters = 2;                            // FP64 refinement it
 // take to FP64 (2^-16 makes a third one common at n = 300).
 constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
 constexpr size_t kVcScratchBytes = (size_t)8 << 30;  // FP64 T: scratch of the rows of V C, per chunk
-constexpr int kVcRowsN = 48;                         // ... for matrices from this size on
+// ... for matrices from this size on.  T phase in us, formed in the T kernel / rows by products,
+// 4 channels of one size, 128 energies, 512 samples: n = 32 409 / 674, 48 752 / 948, 64 1113 / 1205,
+// 96 2395 / 1947, coupled n = 64 1093 / 1259; one sample: 33 / 55, 29 / 53, 31 / 55, 35 / 57 and, 20
+// channels at N_WP = 100 (coupled n = 200), 1350 / 150.  The size decides, not the batch: a solve's
+// bits are the same alone and in any batch.
+constexpr int kVcRowsN = 80;
 constexpr size_t kGraphCache = 64;                         // wpcd_solve keys remembered for CUDA graphs
 
 struct MeshH {

@@ -145,7 +145,7 @@ __device__ __forceinline__ double xlogabs(double d) { return d == 0.0 ? 0.0 : d 
 // rather than ||H||, which holds the relative accuracy of small T): kVcRows takes its
 // rows from memory, where the tensor cores left them as 55-bit products of V's rows
 // and C's columns (launch_vc_rows), kVcExplicit forms them here, K n^2 multiply-adds a
-// bin on the FP64 pipe, for callers without room for the rows.  T phase, explicit and one
+// bin on the FP64 pipe, for small matrices and callers without room for the rows.  T phase, explicit and one
 // CTA a solve -> rows and shares: 20 channels at N_WP = 150, 8 samples 5.68 -> 0.68 ms; at
 // N_WP = 100, one sample 1.35 -> 0.15 ms; 15 channels N_WP 40/64/100, 256 samples 5.9 -> 3.7 ms.
 // The CTAs of a (sample, channel) (gridDim.y) take consecutive shares of its items: one

@@ -1,6 +1,6 @@
 """Sizes and batch shapes at which a solve changes its route.
 
-* FP64 T: V C rows from the tensor cores from n = 48 on, explicit below, shares of
+* FP64 T: V C rows from the tensor cores from n = 80 on, explicit below, shares of
   the bins over several CTAs: around that size and the products' tiles (64, 128),
   with energies that fill one share or leave the last one ragged, both kinds of
   resolvent, against the oracle at the FP64 tolerances.
@@ -41,7 +41,7 @@ def _wl(channels, n_wp, S, n_e, lo=2.0, hi=300.0, wp_kind=W.WP_MOMENTUM):
 UNC, CPL = W.Channel(0, 0, 0, 0, 0), W.Channel(1, 1, 0, 2, 1)
 
 
-@pytest.mark.parametrize("ch,n_wp", [(UNC, 47), (UNC, 48), (CPL, 24), (CPL, 25), (UNC, 64), (UNC, 65), (CPL, 64), (CPL, 65)],
+@pytest.mark.parametrize("ch,n_wp", [(UNC, 79), (UNC, 80), (CPL, 39), (CPL, 40), (UNC, 64), (UNC, 65), (CPL, 64), (CPL, 65)],
                          ids=lambda x: x if isinstance(x, int) else x.name)
 @pytest.mark.parametrize("n_e,res", [(1, 0), (50, 0), (2, 2), (33, 2)])
 def test_fp64_t_routes(ctx, orc, ch, n_wp, n_e, res):
