@@ -34,13 +34,14 @@
 // 40/64/100, 256 samples, 24.0 -> 25.1).
 //
 // Measured against FP64 Jacobi alone (its rotations are bound by the FP64 pipe):
-// 20 channels at N_WP = 100, one sample, 145 -> 4.0 ms a solve; 15 channels of
-// N_WP 40/64/100, 256 samples, 337 -> 25 ms; 20 channels at N_WP = 150, 8 samples,
-// 850 -> 11.7 ms; 1S0 at N_WP = 32, 0.69 -> 0.29 ms; errors against 64-bit LAPACK
+// 20 channels at N_WP = 100, one sample, 145 -> 3.1 ms a solve; 15 channels of
+// N_WP 40/64/100, 256 samples, 337 -> 19.3 ms; 20 channels at N_WP = 150, 8 samples,
+// 850 -> 10.7 ms; 1S0 at N_WP = 32, 0.69 -> 0.29 ms; errors against 64-bit LAPACK
 // unchanged (T 2e-13 to 9e-13 in both).
 //
 // The update is X + X E with E small: the digit product's rounding, relative
 // to E's columns, then vanishes beside X, and X keeps its 53 bits.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -58,11 +59,19 @@ constexpr float kDoneE2 = 2e-14f;     // ||E||_F <= 1.4e-7: its square is below 
 constexpr int kPairCap = 64;          // pairs turned per scan
 constexpr int kPairScans = 6;
 
-// One CTA per item.  S, G and X change only where pairs are turned; E goes to
+// One CTA per item, or a cluster of them (CL) where the items are few: the CTAs take the
+// rows in turn, the pairs found and the rows' sums of E^2 meet in the first one's shared
+// memory, and what others may have written is read past the L1.  No result depends on how
+// many share an item (||E||^2 is summed by rows).  Bound by the FP64 pipe where the chip is
+// full, by the latency of S and G where it is not (64 matrices of n = 200, one CTA each, 0.40
+// and 0.64 ms for the two iterations, the sort 0.12).  One CTA an item -> up to eight, a whole
+// solve: 20 channels at N_WP = 100, one sample, 3.70 -> 3.11 ms; N_WP = 150, 8 samples, 11.9 ->
+// 10.7; 15 channels N_WP 40/64/100, 256 samples, unchanged.  S, G and X change only where pairs are turned; E goes to
 // E_all (the buffer of the next X, whose old content is dead).  FP64 where it
 // must be: the Rayleigh quotients, the differences and s (both cancel for close
 // eigenvalues) and the sums; the quotient s / d is formed in FP32, with one
 // correction step for the angles above 2^-26, so its error stays below 2^-50.
+template <bool CL>
 __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double *G_all, double *X_all,
                                                     double *E_all, double *lam_all, int *done, int it)
 {
@@ -72,17 +81,29 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
     unsigned *pr = reinterpret_cast<unsigned *>(hl + n);         // kPairCap: the scan's pairs, unordered
     unsigned *ps = pr + kPairCap;                                // kPairCap: the same in order
     float *al = reinterpret_cast<float *>(ps + kPairCap);        // n: |lambda| times the rounding of the products
+    float *rs = al + n;                                          // n: the rows' sums of E^2
     __shared__ double red[32];
     __shared__ int s_cnt;
-    const int b = blockIdx.x;
+    const int cr = CL ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+    const int cn = CL ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
+    const int b = blockIdx.x / cn;
     if (done[b] != 0) return;
     const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
+    auto sync = [&]() {
+        if (CL) cooperative_groups::this_cluster().sync();
+        else __syncthreads();
+    };
+    unsigned *pr0 = CL ? cooperative_groups::this_cluster().map_shared_rank(pr, 0) : pr;
+    float *rs0 = CL ? cooperative_groups::this_cluster().map_shared_rank(rs, 0) : rs;
+    int *cnt0 = CL ? cooperative_groups::this_cluster().map_shared_rank(&s_cnt, 0) : &s_cnt;
+    const int w0 = cr * nwarp + warp, ws = cn * nwarp, t0 = cr * nt + tid, ts = cn * nt;  // over the cluster
+    auto ld = [](const double *q) { return CL ? __ldcg(q) : *q; };
     const size_t off = (size_t)b * n * n;
     double *S = S_all + off, *G = G_all + off, *X = X_all + off, *E = E_all + off;
     const float round = it == 0 ? 2.910383e-11f : 8.881784e-16f;  // 2^-35 (39-bit products), 2^-50 (55-bit)
     bool above = false, enough = false;
     for (int i = tid; i < n; i += nt) {
-        const double l = S[(size_t)i * n + i] / G[(size_t)i * n + i];
+        const double l = ld(S + (size_t)i * n + i) / ld(G + (size_t)i * n + i);
         const float lf = fabsf(f32_trunc(l));
         lam[i] = l;
         hl[i] = 0.5 * l;
@@ -93,33 +114,37 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
     // the tests below are in FP32: H's scale has to leave them room on both sides
     if (__syncthreads_or(above) || !__syncthreads_or(enough)) return;
     float ang = it == 0 ? kFirstAngle : kLaterAngle;
-    float e2 = 0.0f;
     bool plain = true;  // S holds S (not yet s)
     bool clear = false, later = false;
     for (int scan = 0;; ++scan) {
-        if (tid == 0) s_cnt = 0;
-        __syncthreads();
-        e2 = 0.0f;
-        for (int i = warp; i < n; i += nwarp) {
+        if (cr == 0 && tid == 0) s_cnt = 0;
+        sync();
+        for (int i = w0; i < n; i += ws) {
             const double li = lam[i], hi = hl[i];
             const float ai = al[i];
             const double *Si = S + (size_t)i * n, *Gi = G + (size_t)i * n;
             double *Ei = E + (size_t)i * n;
+            float e2 = 0.0f;
+            double sj = lane < n ? ld(Si + lane) : 0.0, gj = lane < n ? ld(Gi + lane) : 0.0;
             for (int j = lane; j < n; j += 32) {
-                const double g = Gi[j];
+                const double g = gj, sv = sj;
+                if (j + 32 < n) {  // the next step's values on their way
+                    sj = ld(Si + j + 32);
+                    gj = ld(Gi + j + 32);
+                }
                 double ev;
                 if (j == i) {
                     ev = 0.5 * (1.0 - g);
                 } else {
-                    const double s = plain ? fma(-(hi + hl[j]), g, Si[j]) : Si[j];
+                    const double s = plain ? fma(-(hi + hl[j]), g, sv) : sv;
                     const double d = lam[j] - li;
                     const float sf = f32_trunc(s), df = f32_trunc(d);
                     double th = 0.0;
                     const float as = fabsf(sf), ad = fabsf(df);
                     if (as > fmaxf(ai, al[j])) {
                         if (as > ang * ad && i < j) {
-                            const int k = atomicAdd(&s_cnt, 1);
-                            if (k < kPairCap) pr[k] = ((unsigned)i << 16) | (unsigned)j;
+                            const int k = atomicAdd(cnt0, 1);
+                            if (k < kPairCap) pr0[k] = ((unsigned)i << 16) | (unsigned)j;
                         }
                         if (as <= kMaxAngle * ad) {
                             const float rd = __frcp_rn(df), t0 = sf * rd;
@@ -133,13 +158,15 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
                 const float ef = f32_trunc(ev);
                 e2 = fmaf(ef, ef, e2);
             }
+            for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+            if (lane == 0) rs0[i] = e2;
         }
-        __syncthreads();
-        const int m = s_cnt;
+        sync();
+        const int m = *cnt0;
         if (m > kPairCap && ang < kMaxAngle) {  // too many: turn only those beyond first order
             ang = kMaxAngle;
             later = true;
-            __syncthreads();  // every thread has read the count
+            sync();  // every thread has read the count
             continue;
         }
         if (m == 0 || m > kPairCap || scan >= kPairScans) {
@@ -147,6 +174,10 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
             break;
         }
         // ---- turn the scan's pairs, in index order (the order of the list does not matter)
+        if (cr != 0) {
+            for (int k = tid; k < m; k += nt) pr[k] = pr0[k];
+            __syncthreads();
+        }
         for (int k = tid; k < m; k += nt) {
             const unsigned v = pr[k];
             int r = 0;
@@ -154,55 +185,59 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
             ps[r] = v;
         }
         if (plain) {
-            for (int i = warp; i < n; i += nwarp)
+            for (int i = w0; i < n; i += ws)
                 for (int j = lane; j < n; j += 32) {
                     const size_t e = (size_t)i * n + j;
-                    S[e] = i == j ? lam[i] : fma(-(hl[i] + hl[j]), G[e], S[e]);
+                    S[e] = i == j ? lam[i] : fma(-(hl[i] + hl[j]), ld(G + e), ld(S + e));
                 }
             plain = false;
         }
-        __syncthreads();
+        sync();
         for (int k = 0; k < m; ++k) {
             const int i = (int)(ps[k] >> 16), j = (int)(ps[k] & 0xFFFFu);
-            const double s = S[(size_t)i * n + j], a = S[(size_t)i * n + i], q = S[(size_t)j * n + j];
+            const double s = ld(S + (size_t)i * n + j), a = ld(S + (size_t)i * n + i), q = ld(S + (size_t)j * n + j);
             double c = 1.0, sn = 0.0;
             if (s != 0.0) {
                 const double tau = (q - a) / (2.0 * s);
                 const double t = fabs(tau) > 1e150 ? 0.5 / tau
-                                                   : (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                c = 1.0 / sqrt(1.0 + t * t);
+                                                   : (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(fma(tau, tau, 1.0)));
+                c = 1.0 / sqrt(fma(t, t, 1.0));
                 sn = t * c;
             }
-            __syncthreads();  // every thread has read the pair's block
-            for (int r = tid; r < n; r += nt)  // columns i, j
+            sync();  // every thread has read the pair's block
+            for (int r = t0; r < n; r += ts)  // columns i, j
                 for (int w = 0; w < 3; ++w) {
                     double *M = w == 0 ? S : w == 1 ? G : X;
-                    const double x = M[(size_t)r * n + i], y = M[(size_t)r * n + j];
-                    M[(size_t)r * n + i] = c * x - sn * y;
-                    M[(size_t)r * n + j] = sn * x + c * y;
+                    const double x = ld(M + (size_t)r * n + i), y = ld(M + (size_t)r * n + j);
+                    M[(size_t)r * n + i] = fma(-sn, y, c * x);
+                    M[(size_t)r * n + j] = fma(sn, x, c * y);
                 }
-            __syncthreads();
-            for (int r = tid; r < n; r += nt)  // rows i, j
+            sync();
+            for (int r = t0; r < n; r += ts)  // rows i, j
                 for (int w = 0; w < 2; ++w) {
                     double *M = w == 0 ? S : G;
-                    const double x = M[(size_t)i * n + r], y = M[(size_t)j * n + r];
-                    M[(size_t)i * n + r] = c * x - sn * y;
-                    M[(size_t)j * n + r] = sn * x + c * y;
+                    const double x = ld(M + (size_t)i * n + r), y = ld(M + (size_t)j * n + r);
+                    M[(size_t)i * n + r] = fma(-sn, y, c * x);
+                    M[(size_t)j * n + r] = fma(sn, x, c * y);
                 }
-            __syncthreads();
+            sync();
             if (tid == 0) {
-                S[(size_t)i * n + j] = S[(size_t)j * n + i] = 0.0;
-                lam[i] = S[(size_t)i * n + i];
-                lam[j] = S[(size_t)j * n + j];
+                if (cr == 0) S[(size_t)i * n + j] = S[(size_t)j * n + i] = 0.0;
+                lam[i] = ld(S + (size_t)i * n + i);
+                lam[j] = ld(S + (size_t)j * n + j);
                 hl[i] = 0.5 * lam[i];
                 hl[j] = 0.5 * lam[j];
             }
-            __syncthreads();
+            sync();
         }
     }
+    sync();  // the first CTA's shared memory has been read
+    if (cr != 0) return;
     double *lo = lam_all + (size_t)b * n;
     for (int i = tid; i < n; i += nt) lo[i] = lam[i];
-    const double t2 = cta_sum64((double)e2, red);
+    double e2 = 0.0;
+    for (int i = tid; i < n; i += nt) e2 += (double)rs[i];
+    const double t2 = cta_sum64(e2, red);
     // (the first iteration's eigenvalues come from 39-bit products)
     if (tid == 0 && it > 0 && clear && t2 <= (double)kDoneE2) done[b] = it + 1;
 }
@@ -215,38 +250,73 @@ __global__ void __launch_bounds__(256) k_r64_sort(const ChanDev *chans, const in
                                                   const int *status_all, int n_ch_total, double *eps_all,
                                                   double *X_all)
 {
-    extern __shared__ double sm64s[];
-    double *lam = sm64s;                            // n
-    int *rank = reinterpret_cast<int *>(lam + n);   // n
-    const int b = blockIdx.x;
+    extern __shared__ long long sm64s[];
+    long long *key = sm64s;                         // n: the eigenvalues as integers in the same order
+    int *rank = reinterpret_cast<int *>(key + n);   // n
+    const int b = blockIdx.x, part = blockIdx.y, parts = gridDim.y;
     const int wc = b % nw, smp = sample0 + b / nw;
     const int d = done[b];
     if (d == 0) return;
     if (status_all[(size_t)smp * n_ch_total + work[wc]] <= 0) {
         __syncthreads();
-        if (threadIdx.x == 0) done[b] = 0;
+        if (threadIdx.x == 0 && part == 0) done[b] = 0;
         return;
     }
     const ChanDev ch = chans[work[wc]];
     const double *Xs = ((d & 1) ? X1 : X0) + (size_t)b * n * n;
     double *X = X_all + ch.c_off + (size_t)smp * n * n;
     double *eps = eps_all + ch.eps_off + (size_t)smp * n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) lam[i] = lam_s[(size_t)b * n + i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const long long v = __double_as_longlong(lam_s[(size_t)b * n + i] + 0.0);  // no negative zero
+        key[i] = v < 0 ? v ^ 0x7fffffffffffffffll : v;
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double ei = lam[i];
+        const long long ki = key[i];
         int r = 0;
-        for (int j = 0; j < n; ++j) r += (lam[j] < ei) || (lam[j] == ei && j < i);
+        for (int j = 0; j < n; ++j) r += (key[j] < ki) || (key[j] == ki && j < i);
         rank[i] = r;
-        eps[r] = ei;
+        if (part == 0) eps[r] = lam_s[(size_t)b * n + i];
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    for (int row = warp; row < n; row += nwarp)
+    for (int row = part * nwarp + warp; row < n; row += parts * nwarp)
         for (int c = lane; c < n; c += 32) X[(size_t)row * n + rank[c]] = Xs[(size_t)row * n + c];
 }
 
-static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 4) + kPairCap * 2 * sizeof(unsigned); }
+static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 2 * 4) + kPairCap * 2 * sizeof(unsigned); }
+
+// CTAs that share an item in k_r64_update and k_r64_sort: up to two of 256
+// threads on each of the 152 SMs (clusters wait for room beside other kernels, so a full chip
+// does better without: up to eight cost 19.2 -> 20.1 ms at 256 samples), two rows or more a warp.
+static int r64_share(int items, int n)
+{
+    int cl = 8;
+    while (cl > 1 && ((long long)items * cl > 2 * 152 || n < 16 * cl)) cl /= 2;
+    return cl;
+}
+
+static cudaError_t launch_r64_update(int items, int n, double *S, double *G, double *X, double *E, double *lam, int *done,
+                                     int it, cudaStream_t st)
+{
+    const int cl = r64_share(items, n);
+    if (cl == 1) {
+        k_r64_update<false><<<items, 256, r64_smem(n), counted(st)>>>(n, S, G, X, E, lam, done, it);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(items * cl));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = r64_smem(n);
+    cfg.stream = counted(st);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_r64_update<true>, n, S, G, X, E, lam, done, it);
+}
 
 // Digits per product: the first iteration only has to leave errors that the
 // second squares away (39-bit products); from then on Y, S and G carry 55 bits.
@@ -324,8 +394,7 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
         two.mod = items;
         CKR(launch_oz_split(n, items, true, xn, sYc, eYc, st, sk, dg));
         CKR(launch_oz_gemm_slices(n, 2 * items, sXc, eXc, sXc, eXc, G, st, dg, true, err, items, nullptr, two, dg));
-        k_r64_update<<<items, 256, r64_smem(n), counted(st)>>>(n, S, G, x, xn, lam, done, it);  // E over Y
-        CKR(cudaGetLastError());
+        CKR(launch_r64_update(items, n, S, G, x, xn, lam, done, it, st));  // E over Y
         CKR(launch_oz_split(n, items, false, x, sXr, eXr, st, sk, kDigE));
         CKR(launch_oz_split(n, items, true, xn, sEc, eEc, st, sk, kDigE));
         CKR(launch_oz_gemm_slices(n, items, sXr, eXr, sEc, eEc, xn, st, kDigE, false, err, 0, x, sk, kDigE));  // X + X E
@@ -334,7 +403,7 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
         xn = t;
     }
 #undef CKR
-    k_r64_sort<<<items, 256, (size_t)n * 12, counted(st)>>>(chans, work, nw, sample0, n, lam, X0, X1, done, status_all,
+    k_r64_sort<<<dim3(items, r64_share(items, n)), 256, (size_t)n * 12, counted(st)>>>(chans, work, nw, sample0, n, lam, X0, X1, done, status_all,
                                                             n_ch_total, eps_all, X_all);
     return cudaGetLastError();
 }

@@ -164,3 +164,16 @@ def test_inversion_side_by_side_same_bits(ctx, nq, S):
     for r in runs[1:]:
         for x, y in zip(r, runs[0]):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("ch,n_wp", [(UNC, 15), (UNC, 33), (CPL, 64)], ids=lambda x: x if isinstance(x, int) else x.name)
+def test_fp64_update_shared_by_ctas_same_bits(ctx, ch, n_wp):
+    """The refinement's update: one CTA a matrix in a large batch, up to eight in a small one."""
+    from paper_2106_00454_gb300 import api
+    wl = _wl([ch], n_wp, 1300, 5)
+    md = api.Model(ctx, wl)
+    whole = gpu_run(ctx, md, wl)
+    for s, k in ((7, 1), (100, 60), (300, 130)):
+        part = gpu_run(ctx, md, dataclasses.replace(wl, coeffs=wl.coeffs[s:s + k]))
+        for x, y in zip(part, whole):
+            assert np.array_equal(x, y[s:s + k])
