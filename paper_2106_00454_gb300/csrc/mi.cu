@@ -574,7 +574,7 @@ int mi_slots_per_sm(int n, int NQ)
 // inverse of k_mi_solve (which takes the systems that do not converge here).
 // Per energy this costs K n^2 FP64 multiply-adds a residual (the bound: two or
 // three of them) instead of an n^3 elimination whose n steps wait for each other:
-// 64 samples x 15 channels x 32 energies, N_Q = 96: 134.4 -> 17.0 ms, errors against
+// 64 samples x 15 channels x 32 energies, N_Q = 96: 134.4 -> 16.4 ms, errors against
 // 64 bits unchanged (the eigendecompositions are 10 ms of it).  The rest of the pass is
 // kept off the FP64 pipe where it can be: -w / D as a product with (k^2 - p^2) / (2 mu w
 // k^2), one reciprocal for D and the sum in D_N, V summed over one triangle (20.9 -> 20.1).
