@@ -820,8 +820,10 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         return launch_jacobi_mixed(cd, work, nw, ns, smp0 + s0, v.n_terms, cf, n, lam, x, reinterpret_cast<float *>(aux),
                                    nullptr, e.status, v.n_ch, nullptr, X.stream, th, kTest64);
     };
-    int threads = 256;
-    if (!big32) {
+    // a set's mean (quiet) is a handful of matrices on an empty chip: large CTAs, and the choice for
+    // real batches stays with the first of them
+    int threads = n < 96 ? 256 : 512;
+    if (!big32 && !X.quiet) {
         threads = pick_threads(c, X, n, WPCD_PREC_FP64, nw, chunk, [&](int th, int ns) { return solve32(th, 0, ns); });
         if (threads < 0) return WPCD_ERR_CUDA;
     }
