@@ -160,6 +160,13 @@ wpcd_status wpcd_set_option(wpcd_ctx *ctx, int key, int value);
  * recorded by device code since the last wpcd_sync, else WPCD_OK. */
 wpcd_status wpcd_sync(wpcd_ctx *ctx);
 
+/* FP64 solves since wpcd_create that the refinement of the FP32 eigenpairs did not
+ * bring to FP64 and the FP64 Jacobi kernel solved instead (synchronises the context
+ * stream; served batches count once they have finished).  Ordinary potentials leave
+ * none; a count that grows means slow solves, not inaccurate ones.  Solves that had
+ * no room for the refinement are not counted.  Errors: WPCD_ERR_ARG. */
+wpcd_status wpcd_fp64_unrefined(wpcd_ctx *ctx, unsigned long long *count);
+
 /* Device bytes currently held by the context. */
 size_t wpcd_bytes_in_use(const wpcd_ctx *ctx);
 

@@ -142,6 +142,12 @@ class Context:
     def bytes_in_use(self) -> int:
         return self.lib.wpcd_bytes_in_use(self.h)
 
+    def fp64_unrefined(self) -> int:
+        """FP64 solves so far that the refinement left to the FP64 Jacobi kernel."""
+        n = ctypes.c_ulonglong(0)
+        _ck(self.lib.wpcd_fp64_unrefined(self.h, ctypes.byref(n)), "wpcd_fp64_unrefined")
+        return n.value
+
     PHASES = ["mesh", "project", "eigen", "plan", "tmatrix", "gather", "observables", "refine", "mi"]
 
     def kernel_launches(self) -> int:

@@ -244,11 +244,12 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
 
 // Sorted eigenpairs of the items that are done, into the eigen-buffer layout;
 // the vectors of an item done at iteration k lie in X0 (k even) or X1 (k odd).
-// An item whose FP32 solve hit its sweep cap counts as not done.
+// An item whose FP32 solve hit its sweep cap counts as not done; left (may be NULL)
+// counts the items that are not.
 __global__ void __launch_bounds__(256) k_r64_sort(const ChanDev *chans, const int *work, int nw, int sample0, int n,
                                                   const double *lam_s, const double *X0, const double *X1, int *done,
                                                   const int *status_all, int n_ch_total, double *eps_all,
-                                                  double *X_all)
+                                                  double *X_all, unsigned long long *left)
 {
     extern __shared__ long long sm64s[];
     long long *key = sm64s;                         // n: the eigenvalues as integers in the same order
@@ -256,10 +257,13 @@ __global__ void __launch_bounds__(256) k_r64_sort(const ChanDev *chans, const in
     const int b = blockIdx.x, part = blockIdx.y, parts = gridDim.y;
     const int wc = b % nw, smp = sample0 + b / nw;
     const int d = done[b];
-    if (d == 0) return;
-    if (status_all[(size_t)smp * n_ch_total + work[wc]] <= 0) {
+    const bool failed = status_all[(size_t)smp * n_ch_total + work[wc]] <= 0;
+    if (d == 0 || failed) {
         __syncthreads();
-        if (threadIdx.x == 0 && part == 0) done[b] = 0;
+        if (threadIdx.x == 0 && part == 0) {
+            done[b] = 0;
+            if (left) atomicAdd(left, 1ull);
+        }
         return;
     }
     const ChanDev ch = chans[work[wc]];
@@ -354,7 +358,7 @@ double *refine64_lambda(void *scratch, int items, int n)
 cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
                             const double *coeffs, void *scratch, int *done, const int *status_all, int n_ch_total,
                             double *eps_all, double *X_all, cudaStream_t st, int *err, const __nv_bfloat16 *rot_s,
-                            const int *rot_e)
+                            const int *rot_e, unsigned long long *left)
 {
     const int items = n_samples * nw;
     const size_t nn = (size_t)items * n * n;
@@ -404,7 +408,7 @@ cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n
     }
 #undef CKR
     k_r64_sort<<<dim3(items, r64_share(items, n)), 256, (size_t)n * 12, counted(st)>>>(chans, work, nw, sample0, n, lam, X0, X1, done, status_all,
-                                                            n_ch_total, eps_all, X_all);
+                                                            n_ch_total, eps_all, X_all, left);
     return cudaGetLastError();
 }
 

@@ -175,6 +175,7 @@ struct wpcd_ctx {
     std::map<std::pair<int, int>, Tuned> tuned;  // (n, precision) -> eigensolver CTA size
     std::mutex tmu;
     int *err_dev = nullptr;
+    unsigned long long *left_dev = nullptr;  // solves that the FP64 refinement left to FP64 Jacobi
     std::mutex amu;  // device-memory accounting (shared with the serving thread)
     std::mutex pmu;  // profiling records
     // Gauss-Legendre rules cached on the device, keyed by order
@@ -838,7 +839,7 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
             Launch L(c, X, WPCD_PHASE_REFINE);
             CK(launch_refine64(e.cd_dev, work, nw, ns, smp0 + s0, n, v.n_terms, cf, base, done, e.status, v.n_ch, e.eps, e.C,
                                X.stream, X.err, sb ? sb->sC + pos * oz_slice_elems(n, kDigE) : nullptr,
-                               sb ? sb->eC + pos * n : nullptr));
+                               sb ? sb->eC + pos * n : nullptr, X.quiet ? nullptr : c->left_dev));
         }
         Launch L(c, X, WPCD_PHASE_EIGEN);
         if (big64) {  // its slots take the place of the refinement's scratch
@@ -1298,7 +1299,11 @@ wpcd_status wpcd_create(wpcd_ctx **out, int device, size_t hbm_budget_bytes, voi
     c->device = device;
     c->main.stream = static_cast<cudaStream_t>(cuda_stream);
     c->budget = hbm_budget_bytes;
-    if (dalloc(c, &c->err_dev, 1) != WPCD_OK || cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->main.stream) != cudaSuccess) {
+    if (dalloc(c, &c->err_dev, 1) != WPCD_OK || dalloc(c, &c->left_dev, 1) != WPCD_OK ||
+        cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->main.stream) != cudaSuccess ||
+        cudaMemsetAsync(c->left_dev, 0, sizeof(unsigned long long), c->main.stream) != cudaSuccess) {
+        dfree(c, c->left_dev);
+        dfree(c, c->err_dev);
         delete c;
         return WPCD_ERR_CUDA;
     }
@@ -1332,6 +1337,7 @@ void wpcd_destroy(wpcd_ctx *c)
     free_side_streams(M);
     for (auto *b : {&M.ws_plan_i, &M.ws_plan_d, &M.ws_tbin, &M.ws_phbin, &M.ws_in, &M.ws_out, &M.ws_ref}) dfree(c, b->p);
     dfree(c, c->err_dev);
+    dfree(c, c->left_dev);
     delete c;
 }
 
@@ -1405,6 +1411,16 @@ wpcd_status wpcd_sync(wpcd_ctx *c)
     case kDevBadSize: return WPCD_ERR_CUDA;
     default: return WPCD_ERR_ARG;
     }
+}
+
+wpcd_status wpcd_fp64_unrefined(wpcd_ctx *c, unsigned long long *count)
+{
+    if (!c || !count) return WPCD_ERR_ARG;
+    std::lock_guard<std::mutex> lk(c->mu);
+    CK(cudaSetDevice(c->device));
+    CK(cudaMemcpyAsync(count, c->left_dev, sizeof(*count), cudaMemcpyDeviceToHost, c->main.stream));
+    CK(cudaStreamSynchronize(c->main.stream));
+    return WPCD_OK;
 }
 
 size_t wpcd_bytes_in_use(const wpcd_ctx *c) { return c ? c->in_use : 0; }

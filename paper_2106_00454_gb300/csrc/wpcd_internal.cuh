@@ -332,7 +332,7 @@ double *refine64_lambda(void *scratch, int items, int n);
 cudaError_t launch_refine64(const ChanDev *chans, const int *work, int nw, int n_samples, int sample0, int n, int n_terms,
                             const double *coeffs, void *scratch, int *done, const int *status_all, int n_ch_total,
                             double *eps_all, double *X_all, cudaStream_t st, int *err, const __nv_bfloat16 *rot_s,
-                            const int *rot_e);
+                            const int *rot_e, unsigned long long *left = nullptr);
 cudaError_t launch_batched_dgemm(int n, int items, bool ta, const double *A, const double *B, double *C,
                                  void *scratch, int engine, cudaStream_t st, int *err = nullptr);
 size_t batched_dgemm_scratch(int n, int items);
