@@ -45,6 +45,13 @@ constexpr int kRefineIters = 2;                            // FP64 refinement it
 // angle and its share of the diagonal are below 2^-18, which two refinement iterations
 // take to FP64 (2^-16 makes a third one common at n = 300).
 constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
+// FP64 eigenpairs by refinement from this size on, below by the FP64 Jacobi kernel alone: there its
+// one launch costs less than the refinement's chain of some thirty.  A call in us, Jacobi / refinement,
+// 1S0, 1 and 4096 samples: n = 4 82 / 159 and 410 / 1817, n = 8 139 / 172 and 999 / 2137, n = 12 234 / 190
+// and 1794 / 2570, n = 16 300 / 207 and 2818 / 3001, n = 18 417 / 232 and 3754 / 3300, n = 24 559 / 278 and
+// 6285 / 4023; 7 channels J <= 2 of n = 8 and 16, 4096 samples, 8432 / 18011.  The size alone decides
+// (the same bits alone and in a batch), so the line lies where no batch loses.
+constexpr int kRefine64N = 17;
 constexpr size_t kVcScratchBytes = (size_t)8 << 30;  // FP64 T: scratch of the rows of V C, per chunk
 // ... for matrices from this size on.  T phase in us, formed in the T kernel / rows by products,
 // 4 channels of one size, 128 energies, 512 samples: n = 32 409 / 674, 48 752 / 948, 64 1113 / 1205,
@@ -475,7 +482,7 @@ int pick_threads(wpcd_ctx *c, Exec &X, int n, int prec, int nw, int nsmp, F laun
     for (int k = 0; k < 5; ++k) {
         const int th = cand[k];
         if (th > 512 && prec == WPCD_PREC_FP64 && jacobi_fits_smem(n, true)) continue;
-        const int occ = jacobi_mixed_occupancy(n, th);
+        const int occ = prec == WPCD_PREC_FP64 && n < kRefine64N ? jacobi_f64_occupancy(n, th) : jacobi_mixed_occupancy(n, th);
         if (occ < 1) continue;
         const int ns = std::max(1, std::min(nsmp, (2 * c->n_sm * occ + nw - 1) / nw));
         cudaEventRecord(a, X.stream);
@@ -783,6 +790,17 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
 {
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
     if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    if (n < kRefine64N) {
+        auto solve = [&](int th, int ns) {
+            return launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
+                                     X.stream, th);
+        };
+        const int threads = X.quiet ? 256 : pick_threads(c, X, n, WPCD_PREC_FP64, nw, nsmp, solve);
+        if (threads < 0) return WPCD_ERR_CUDA;
+        Launch L(c, X, WPCD_PHASE_EIGEN);
+        CK(solve(threads, nsmp));
+        return WPCD_OK;
+    }
     const F64Scratch sc(c, n, nw);
     const size_t ref_item = sc.ref_item, c_item = sc.c_item, slot64 = sc.slot64;
     const bool big32 = sc.big32, big64 = sc.big64;
@@ -861,7 +879,8 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
 // (the basis would be the answer), without memory, or when a solve failed.
 bool ensure_start(wpcd_ctx *c, Exec &X, VSetH &v)
 {
-    if (v.n_terms < 2 || c->budget) return false;  // (a budget's room is the caller's)
+    if (v.n_terms < 2 || v.buckets.rbegin()->first < kRefine64N) return false;
+    if (c->budget) return false;  // a budget's room is the caller's
     std::lock_guard<std::mutex> lk(*v.rot_mu);
     if (v.start_state != 0) return v.start_state == 1;
     if (capturing(X.stream)) return false;
@@ -960,7 +979,7 @@ bool ensure_start(wpcd_ctx *c, Exec &X, VSetH &v)
 // Scratch that the whole of a size bucket takes in one chunk.
 size_t bucket_scratch(wpcd_ctx *c, int n, int nw, int S, int prec)
 {
-    if (prec == WPCD_PREC_FP64) return F64Scratch(c, n, nw).bytes(S);
+    if (prec == WPCD_PREC_FP64) return n < kRefine64N ? 256 : F64Scratch(c, n, nw).bytes(S);  // (a share says: in use)
     const size_t ref_item = refine_scratch_per_item(n, c->refine_engine);
     if (jacobi_fits_smem(n, false))
         return (ref_item + (jacobi_mixed_c_in_smem(n) ? 0 : jacobi_mixed_c_bytes(n)) + 256) * nw * S;
