@@ -2105,9 +2105,11 @@ wpcd_status wpcd_saclay(wpcd_ctx *c, const wpcd_channel *channels, int n_ch, con
 
 // ---- MI comparison method (Sec. 2.1, Sec. 6) ---------------------------------------------------
 namespace {
-// The set of diag(k^2) + S V S; without room for it the MI set works without.
+// The set of diag(k^2) + S V S; without room for it the MI set works without (by elimination),
+// and so it does under an HBM budget, whose room is the caller's.
 wpcd_status mi_eigen_set(wpcd_ctx *c, MiH &m)
 {
+    if (c->budget) return WPCD_OK;
     VSetH &v = m.set;
     std::vector<long long> off;
     size_t len = 0;
@@ -2284,7 +2286,8 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
     wpcd_status st;
     const size_t ph_len = (size_t)S * m.n_ch * n_I * 3;
     if ((st = ws_reserve(c, X, X.ws_tbin, (von_len + ph_len) * sizeof(double)))) return st;
-    if ((st = ws_reserve(c, X, X.ws_plan_i, (size_t)S * m.n_ch * (1 + n_I) * sizeof(int)))) return st;
+    // status, and for the systems of an eigendecomposition whether they are left to elimination
+    if ((st = ws_reserve(c, X, X.ws_plan_i, (size_t)S * m.n_ch * (1 + (m.has_set ? n_I : 0)) * sizeof(int)))) return st;
     double *Von = static_cast<double *>(X.ws_tbin.p), *ph = Von + von_len;
     int *status = status_dev ? status_dev : static_cast<int *>(X.ws_plan_i.p);
     int *redo = static_cast<int *>(X.ws_plan_i.p) + (size_t)S * m.n_ch;
@@ -2346,8 +2349,28 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
                                   static_cast<double *>(Y.ws_ref.p), slots, ph, k_out, status, redo, X.err, Y.stream));
         }
         if (mi_slots_per_sm(n, m.NQ) < 1) return WPCD_ERR_ARG;
-        const Elim el = elim(K, eig);
+        Elim el = elim(K, eig);
         wpcd_status es = ws_reserve(c, Y, Y.ws_ref, el.bytes);
+        // no room: what only the eigendecompositions need yields to the elimination (their kernels
+        // have run by then), and then it makes do with fewer slots
+        if (es && !Y.ws_ref.part) {
+            cudaStreamSynchronize(Y.stream);
+            free_eig(c, X.eig);
+            es = ws_reserve(c, Y, Y.ws_ref, el.bytes);
+        }
+        if (es && !Y.ws_ref.part && m.has_set) {
+            free_vset(c, m.set);
+            m.set = VSetH();
+            dfree(c, m.k2);
+            m.k2 = nullptr;
+            m.has_set = false;
+            es = ws_reserve(c, Y, Y.ws_ref, el.bytes);
+        }
+        while (es && el.slots > 1) {
+            el.bytes = el.bytes / el.slots * (el.slots / 2);
+            el.slots /= 2;
+            es = ws_reserve(c, Y, Y.ws_ref, el.bytes);
+        }
         if (es) return es;
         Launch L(c, Y, WPCD_PHASE_MI);
         CK(launch_mi_solve(m.ch_dev, m.work_dev[K - 1], nw, n, m.n_ch, S, m.NQ, m.kg, m.wg, m.n_terms, cf, m.Vg, Von,
