@@ -135,6 +135,12 @@ enum { WPCD_OPT_EXEC = 1, WPCD_OPT_REFINE = 2, WPCD_OPT_AUTOTUNE = 3, WPCD_OPT_G
 /* Create a context on CUDA device `device`.  hbm_budget_bytes caps the device
  * memory the context may hold (0 = no cap).  cuda_stream: a cudaStream_t on
  * that device (NULL = the legacy default stream); the context does not own it.
+ * Solves keep their scratch for the next one, up to 32 GB for the context and for
+ * each serving slot.  Scratch that a solve is only faster with (the FP64 refinement's,
+ * the rows of V C, a share for each size bucket) shrinks to the room that there is,
+ * down to none, and is given back when another allocation of the context finds no
+ * room; admission of requests does not count it.  Memory of other users of the
+ * device is only left to them by a cap.
  * Errors: WPCD_ERR_ARG (null out pointer, bad device), WPCD_ERR_CUDA. */
 wpcd_status wpcd_create(wpcd_ctx **out, int device, size_t hbm_budget_bytes, void *cuda_stream);
 

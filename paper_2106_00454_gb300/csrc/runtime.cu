@@ -115,6 +115,7 @@ struct Buf {
     void *p = nullptr;
     size_t n = 0;
     bool part = false;  // a share of another buffer: never reallocated
+    bool spare = false;  // scratch that its calls would also do without: yields to other allocations (give_back)
 };
 
 // One executor: a stream, its device status word and its workspaces.  The
@@ -163,7 +164,7 @@ struct Handle {
 struct wpcd_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
-    size_t budget = 0, in_use = 0;
+    size_t budget = 0, in_use = 0, spare = 0;  // spare: the part of in_use that yields
     std::map<void *, size_t> sizes;
     std::map<int, Handle> handles;
     int next_id = 1;
@@ -225,19 +226,31 @@ namespace {
         if (e_ != cudaSuccess) return WPCD_ERR_CUDA; \
     } while (0)
 
-wpcd_status dmalloc(wpcd_ctx *c, void **p, size_t bytes)
+// Free the spare scratch that this thread may reach; true if there was some.  The caller holds
+// c->mu or is the serving thread (inside launch_batch).
+bool give_back(wpcd_ctx *c);
+
+// spare: without giving spare scratch back (the caller would do without the memory).
+wpcd_status dmalloc(wpcd_ctx *c, void **p, size_t bytes, bool spare = false)
 {
-    std::lock_guard<std::mutex> lk(c->amu);
     if (bytes == 0) bytes = 8;
-    if (c->budget && c->in_use + bytes > c->budget) return WPCD_ERR_BUDGET;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return WPCD_ERR_NOMEM;
+    for (;;) {
+        wpcd_status st = WPCD_ERR_BUDGET;
+        {
+            std::lock_guard<std::mutex> lk(c->amu);
+            if (!c->budget || c->in_use + bytes <= c->budget) {
+                if (cudaMalloc(p, bytes) == cudaSuccess) {
+                    c->in_use += bytes;
+                    c->sizes[*p] = bytes;
+                    ++c->graph_gen;
+                    return WPCD_OK;
+                }
+                cudaGetLastError();
+                st = WPCD_ERR_NOMEM;
+            }
+        }
+        if (spare || !give_back(c)) return st;
     }
-    c->in_use += bytes;
-    c->sizes[*p] = bytes;
-    ++c->graph_gen;
-    return WPCD_OK;
 }
 
 void dfree(wpcd_ctx *c, void *p)
@@ -311,31 +324,45 @@ bool capturing(cudaStream_t st)
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
+void ws_free(wpcd_ctx *c, Buf &b)
+{
+    if (b.spare) {
+        std::lock_guard<std::mutex> lk(c->amu);
+        c->spare -= b.n;
+    }
+    dfree(c, b.p);
+    b = Buf();
+}
+
 // Give the executor's solver scratch back (it only lives within a phase).
 void drop_scratch(wpcd_ctx *c, Exec &X)
 {
     cudaStreamSynchronize(X.stream);
-    dfree(c, X.ws_ref.p);
-    X.ws_ref = Buf();
+    ws_free(c, X.ws_ref);
 }
 
-wpcd_status ws_reserve(wpcd_ctx *c, Exec &X, Buf &b, size_t bytes)
+wpcd_status ws_reserve(wpcd_ctx *c, Exec &X, Buf &b, size_t bytes, bool spare = false)
 {
     if (b.n >= bytes) return WPCD_OK;
     if (b.part) return WPCD_ERR_NOMEM;
     if (capturing(X.stream)) return WPCD_ERR_CUDA;  // a graph cannot hold a reallocation
     if (b.p) {
         cudaStreamSynchronize(X.stream);
-        dfree(c, b.p);
-        b.p = nullptr;
-        b.n = 0;
+        ws_free(c, b);
     }
-    wpcd_status st = dmalloc(c, &b.p, bytes);
+    wpcd_status st = dmalloc(c, &b.p, bytes, spare);
     if (st != WPCD_OK && &b != &X.ws_ref && X.ws_ref.p && !X.ws_ref.part) {
         drop_scratch(c, X);
         st = dmalloc(c, &b.p, bytes);
     }
-    if (st == WPCD_OK) b.n = bytes;
+    if (st == WPCD_OK) {
+        b.n = bytes;
+        b.spare = spare;
+        if (spare) {
+            std::lock_guard<std::mutex> lk(c->amu);
+            c->spare += bytes;
+        }
+    }
     return st;
 }
 
@@ -810,7 +837,7 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
     int chunk = (int)std::max<size_t>(1, kRefineScratchBytes / ((ref_item + c_item) * nw));
     chunk = std::min(chunk, std::max(1, 65535 / nw));  // the refinement grids put items in y / z (<= 65535)
     chunk = std::min(chunk, nsmp);
-    while (chunk > 0 && ws_reserve(c, X, X.ws_ref, bytes_of(chunk))) chunk /= 2;
+    while (chunk > 0 && ws_reserve(c, X, X.ws_ref, bytes_of(chunk), true)) chunk /= 2;
     if (chunk == 0) {  // no room: FP64 Jacobi alone
         const int slots = big64 ? std::max(1, std::min(nsmp * nw, cap64)) : 0;
         wpcd_status st = ws_reserve(c, X, X.ws_ref, slot64 * slots);
@@ -1031,7 +1058,7 @@ bool fork_units(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_unit, std
     for (int k = 0; k < lanes; ++k) off[k + 1] = off[k] + share[k];
     const size_t total = off[lanes];
     if (units.size() < 2 || total >= X.no_fork || !side_streams(X)) return false;
-    if (ws_reserve(c, X, X.ws_ref, total)) {
+    if (ws_reserve(c, X, X.ws_ref, total, true)) {
         if (!capturing(X.stream)) X.no_fork = total;
         return false;
     }
@@ -1194,7 +1221,7 @@ wpcd_status tbin_unit(wpcd_ctx *c, Exec &X, Exec &Y, VSetH &v, EigH &e, int n_E,
     if (!mixed && n >= kVcRowsN) {
         chunk = (int)std::min<size_t>((size_t)nsmp, std::max<size_t>(1, kVcScratchBytes / (per * nw)));
         chunk = std::min(chunk, std::max(1, 65535 / nw));  // items in the grid's y
-        while (chunk > 0 && ws_reserve(c, Y, Y.ws_ref, per * nw * chunk)) chunk /= 2;
+        while (chunk > 0 && ws_reserve(c, Y, Y.ws_ref, per * nw * chunk, true)) chunk /= 2;
     }
     TWork tw;
     tw.work = work;
@@ -2339,7 +2366,7 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
             const int ns = std::min(Sc, S - s0), slots = eig_slots(K);
             const double *cfs = cf ? cf + (size_t)s0 * (m.n_terms - 1) : nullptr;
             if ((!prepared && diag_prep(c, X, m.set, -1, ns, WPCD_PREC_FP64, X.eig)) ||
-                mi_eigen(c, Y, X.eig, m, cfs, ns, K) || ws_reserve(c, Y, Y.ws_ref, (size_t)slots * ng * ng * sizeof(double))) {
+                mi_eigen(c, Y, X.eig, m, cfs, ns, K) || ws_reserve(c, Y, Y.ws_ref, (size_t)slots * ng * ng * sizeof(double), true)) {
                 eig = false;  // no room: by elimination, from the first sample on
                 break;
             }
@@ -2392,7 +2419,7 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
                                      (size_t)eig_slots(K) * K * m.NQ * K * m.NQ * sizeof(double)) + 255) & ~(size_t)255;
         const size_t total = share[0] + share[1];
         if (total > kRefineScratchBytes || total >= X.no_fork || !side_streams(X)) return false;
-        if (ws_reserve(c, X, X.ws_ref, total)) {
+        if (ws_reserve(c, X, X.ws_ref, total, true)) {
             X.no_fork = total;
             return false;
         }
@@ -2488,6 +2515,7 @@ struct Server {
     int n_ch = 0, n_terms = 0, max_batch = 64;
     size_t max_queue = 1 << 16;
     std::vector<std::unique_ptr<Slot>> slots;
+    std::mutex wmu;  // the serving thread is queueing a batch (the slots' buffers are in its hands)
     std::mutex mu;
     std::condition_variable cv;
     std::deque<std::shared_ptr<Req>> queue;
@@ -2507,6 +2535,30 @@ void CUDART_CB slot_done_cb(void *arg)
     sl->done.store(1);
 }
 
+thread_local bool g_serving = false;  // this is a context's serving thread
+
+bool give_back(wpcd_ctx *c)
+{
+    bool any = false;
+    auto drop = [&](Exec &X) {
+        if (!X.ws_ref.spare || capturing(X.stream)) return;
+        drop_scratch(c, X);
+        any = true;
+    };
+    if (!g_serving) drop(c->main);
+    if (Server *sv = c->server) {
+        std::unique_lock<std::mutex> lk(sv->wmu, std::defer_lock);
+        // a batch is queued in milliseconds; no waiting without end, since that thread may
+        // itself wait for a set that the caller is preparing
+        for (int k = 0; !g_serving && k < 1000 && !lk.try_lock(); ++k) std::this_thread::sleep_for(std::chrono::milliseconds(1));
+        if (g_serving || lk.owns_lock())
+            for (auto &sl : sv->slots) drop(sl->X);
+    }
+    return any;
+}
+
+// Admission counts what a request cannot do without: the FP64 solver's scratch shrinks to the
+// room that is there and yields to other allocations.
 size_t request_bytes(const ModelS &m, int prec)
 {
     size_t b = 0;
@@ -2629,6 +2681,11 @@ void fail_batch(Server *sv, Slot &sl, wpcd_status st)
 void serve_loop(Server *sv)
 {
     cudaSetDevice(sv->c->device);
+    g_serving = true;
+    auto launch = [&](Slot &sl) {
+        std::lock_guard<std::mutex> lk(sv->wmu);
+        return launch_batch(sv, sl);
+    };
     for (;;) {
         bool any_busy = false;
         for (auto &slp : sv->slots) {
@@ -2657,7 +2714,20 @@ void serve_loop(Server *sv)
             }
             sl.busy = true;
             any_busy = true;
-            wpcd_status st = launch_batch(sv, sl);
+            wpcd_status st = launch(sl);
+            if (st == WPCD_ERR_NOMEM || st == WPCD_ERR_BUDGET) {  // the synchronous calls' spare scratch yields, too
+                cudaStreamSynchronize(sl.X.stream);
+                bool again = false;
+                {
+                    wpcd_ctx *c = sv->c;
+                    std::lock_guard<std::mutex> lk(c->mu);
+                    if (c->main.ws_ref.spare && !capturing(c->main.stream)) {
+                        drop_scratch(c, c->main);
+                        again = true;
+                    }
+                }
+                if (again) st = launch(sl);
+            }
             if (st) {
                 cudaStreamSynchronize(sl.X.stream);
                 fail_batch(sv, sl, st);
@@ -2693,6 +2763,7 @@ void serve_shutdown(wpcd_ctx *c)
     }
     sv->cv.notify_all();
     if (sv->worker.joinable()) sv->worker.join();
+    std::lock_guard<std::mutex> lkc(c->mu);  // give_back looks at the server
     for (auto &slp : sv->slots) {
         Slot &sl = *slp;
         cudaStreamSynchronize(sl.X.stream);
@@ -2745,6 +2816,7 @@ wpcd_status wpcd_serve_start(wpcd_ctx *c, const wpcd_channel *channels, int n_ch
         sv->models.push_back(m);
     }
     CK(cudaSetDevice(c->device));
+    std::lock_guard<std::mutex> lkc(c->mu);
     for (int k = 0; k < n_slots; ++k) {
         auto sl = std::make_unique<Slot>();
         CK(cudaStreamCreateWithFlags(&sl->X.stream, cudaStreamNonBlocking));
@@ -2792,7 +2864,12 @@ wpcd_status wpcd_submit(wpcd_ctx *c, const wpcd_request *rq, uint64_t *ticket)
     r->bytes = request_bytes(sv->models[model], rq->prec);
     std::lock_guard<std::mutex> lk(sv->mu);
     if (sv->stop) return WPCD_ERR_ARG;
-    const size_t cap = c->budget ? (c->budget > c->in_use ? c->budget - c->in_use : 0) : (size_t)-1;
+    size_t held;  // by what does not yield
+    {
+        std::lock_guard<std::mutex> la(c->amu);
+        held = c->in_use - c->spare;
+    }
+    const size_t cap = c->budget ? (c->budget > held ? c->budget - held : 0) : (size_t)-1;
     if (sv->queue.size() >= sv->max_queue || (c->budget && sv->queued_bytes + r->bytes > cap))
         return WPCD_ERR_BUDGET;
     r->ticket = sv->next_ticket++;

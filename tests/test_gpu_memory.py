@@ -85,3 +85,123 @@ def test_inversion_on_a_nearly_full_device(api):
         torch.cuda.empty_cache()
         ctx.close()
     iv.same(got, want)
+
+
+def _wl(nwp, S, n_e=8, jmax=2):
+    chs = W.np_channels(jmax)
+    return W.Workload("memory", chs, [nwp[k % len(nwp)] for k in range(len(chs))], W.GEN_YUKAWA, W.YUKAWA_PARAMS.copy(),
+                      W.N_TERMS_YUKAWA, W.coefficient_samples(S, 2), np.linspace(2.0, 300.0, n_e))
+
+
+def _phases(ctx, md, wl, prec, n=3):
+    """Solved n times: one by one, captured, replayed."""
+    import torch
+    S, nE = wl.n_samples, len(wl.e_lab)
+    cf = torch.tensor(wl.coeffs, dtype=torch.float64, device="cuda:0")
+    e = torch.tensor(wl.e_lab, dtype=torch.float64, device="cuda:0")
+    d = torch.zeros((S, len(wl.channels), nE, 3), dtype=torch.float64, device="cuda:0")
+    for _ in range(n):
+        ctx.solve(md.vset, cf, S, e, None, d, None, prec=prec)
+        ctx.sync()
+    return d.cpu().numpy()
+
+
+def _close(a, b, tol):
+    assert np.max(np.abs(dphase(a[..., :2], b[..., :2]))) <= tol
+    assert np.max(np.abs(a[..., 2] - b[..., 2])) <= tol
+
+
+def _model_bytes(api, wl):
+    c = api.Context(0)
+    api.Model(c, wl)
+    c.sync()
+    n = c.bytes_in_use()
+    c.close()
+    return n
+
+
+def test_fp64_scratch_yields_to_a_second_set(api):
+    """A budget of two sets and one batch's eigenpairs and T: the refinement of the
+    first set's solves takes what is there, and the second set still finds its room."""
+    wl = _wl([64], 16)
+    n2 = sum((ch.K * 64) ** 2 for ch in wl.channels)
+    budget = 2 * _model_bytes(api, wl) + 8 * 16 * n2 + 3 * MB
+    free = api.Context(0)
+    want = _phases(free, api.Model(free, wl), wl, api.PREC_FP64)
+    free.close()
+    c = api.Context(0, hbm_budget_bytes=budget)
+    first = api.Model(c, wl)
+    a = _phases(c, first, wl, api.PREC_FP64)
+    second = api.Model(c, wl)
+    b = _phases(c, second, wl, api.PREC_FP64)
+    again = _phases(c, first, wl, api.PREC_FP64)
+    assert c.bytes_in_use() <= budget
+    c.close()
+    for x in (a, b, again):
+        _close(x, want, 1e-8)
+
+
+def test_shares_of_the_streams_yield_to_a_second_set(api):
+    """Mixed path, a budget of one size bucket's scratch at a time and a second set: the
+    shares for buckets side by side (5 MB more) may take the second set's room (7 MB), but
+    not keep it."""
+    wl = _wl([64], 2)
+    probe = api.Context(0)
+    probe.profile(True)  # one bucket after another
+    md = api.Model(probe, wl)
+    want = _phases(probe, md, wl, api.PREC_MIXED)
+    one = probe.bytes_in_use()
+    probe.close()
+    budget = one + _model_bytes(api, wl) + MB // 16
+    c = api.Context(0, hbm_budget_bytes=budget)
+    first = api.Model(c, wl)
+    a = _phases(c, first, wl, api.PREC_MIXED, 4)
+    api.Model(c, wl)
+    b = _phases(c, first, wl, api.PREC_MIXED)
+    assert c.bytes_in_use() <= budget
+    c.close()
+    assert np.array_equal(a, want) and np.array_equal(b, want)
+
+
+def test_served_fp64_under_a_budget(api):
+    """The scratch of a served FP64 batch is no part of what admission counts, yields to a
+    set that the program projects meanwhile, and the synchronous calls' scratch yields to
+    the server's batches."""
+    chs = W.np_channels(2)
+    rng = np.random.default_rng(8)
+    req = {n: (rng.standard_normal(14) * W.TERM_SCALE, np.sort(rng.uniform(1.0, 350.0, 20)), n) for n in (64, 96)}
+    args = (chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, [64, 96])
+
+    def ask(c, n):
+        r = c.wait(c.submit(*req[n], api.PREC_FP64))
+        assert r.status == 0
+        return r.delta
+
+    probe = api.Context(0)
+    probe.serve_start(*args, max_batch=4, n_slots=1)
+    want = {n: ask(probe, n) for n in (64, 96)}
+    probe.serve_stop()
+    probe.close()
+    probe = api.Context(0)
+    probe.serve_start(*args, max_batch=4, n_slots=1)
+    base = probe.bytes_in_use()
+    probe.serve_stop()
+    probe.close()
+    wl = _wl([64], 4)
+    need96 = 8 * sum((ch.K * 96) ** 2 for ch in chs)
+    # the server, a further set, and room for one request's eigenpairs and T (and little more)
+    budget = base + _model_bytes(api, wl) + need96 + 8 * 4 * sum((ch.K * 64) ** 2 for ch in chs) + MB
+    c = api.Context(0, hbm_budget_bytes=budget)
+    c.serve_start(*args, max_batch=4, n_slots=1)
+    try:
+        for _ in range(3):  # the first batch's scratch takes what is left
+            _close(ask(c, 64), want[64], 1e-8)
+        md = api.Model(c, wl)
+        _close(ask(c, 64), want[64], 1e-8)
+        _phases(c, md, wl, api.PREC_FP64)
+        _close(ask(c, 96), want[96], 1e-8)  # more eigenpairs than the slot holds
+        _close(ask(c, 64), want[64], 1e-8)
+        assert c.bytes_in_use() <= budget
+    finally:
+        c.serve_stop()
+        c.close()
