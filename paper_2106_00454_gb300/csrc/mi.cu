@@ -677,7 +677,8 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
                                                             const double *kg, const double *wg, int n_terms,
                                                             const double *coeffs, const double *Vg, const double *Von,
                                                             int n_I, const double *e_int, const double *eps_all,
-                                                            const double *Q_all, double *Vs_all, double *ph,
+                                                            const double *Q_all, const int *eig_status,
+                                                            const int *eig_err, double *Vs_all, double *ph,
                                                             double *k_out, int *status, int *redo, int *err)
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
@@ -709,6 +710,13 @@ __global__ void __launch_bounds__(512, 1) k_mi_energies(const MiChanDev *chans, 
         const double *Vgc = Vg + ch.vg_off;
         const double *Qg = Q_all + ec.c_off + (size_t)(smp - sample0) * ng * ng;
         const double *lg = eps_all + ec.eps_off + (size_t)(smp - sample0) * ng;
+        // eigenpairs that a solve did not converge to, or a product that timed out did not write, could
+        // pass for a solution (vectors of zeros give a correction of zero): all energies by elimination
+        if (*eig_err != 0 || eig_status[(size_t)(smp - sample0) * n_ch_total + cidx] < 0) {
+            for (int ie = tid; ie < n_I; ie += nt) redo[((size_t)smp * n_ch_total + cidx) * n_I + ie] = 1;
+            if (tid == 0) status[(size_t)smp * n_ch_total + cidx] = 0;
+            continue;
+        }
         __syncthreads();  // the last item is done with shared memory
         for (int r = warp; r < ng; r += nw) {  // V is symmetric: the upper triangle, mirrored
             const size_t orow = (size_t)((r / NQ) * M + r % NQ) * ch.n;
@@ -938,19 +946,21 @@ int mi_energies_per_sm(int NQ, int K)
     return blocks;
 }
 
-// n_samples samples from sample0; eps / Q: the eigenpairs of this range (eig_ch offsets).
+// n_samples samples from sample0; eps / Q: the eigenpairs of this range (eig_ch offsets), eig_status their
+// solves' status [sample][n_ch_total], eig_err their error word.
 cudaError_t launch_mi_energies(const MiChanDev *chans_dev, const ChanDev *eig_ch, const int *work_dev, int n_work, int K,
                                int n_ch_total, int sample0, int n_samples, int NQ, const double *kg, const double *wg,
                                int n_terms, const double *coeffs, const double *Vg, const double *Von, int n_I,
-                               const double *e_int, const double *eps, const double *Q, double *Vs, int slots, double *ph,
-                               double *k_out, int *status, int *redo, int *err, cudaStream_t st)
+                               const double *e_int, const double *eps, const double *Q, const int *eig_status,
+                               const int *eig_err, double *Vs, int slots, double *ph, double *k_out, int *status, int *redo,
+                               int *err, cudaStream_t st)
 {
     const size_t smem = me_smem(K * NQ, NQ, K);
     if (!mi_energies_fit(NQ, K)) return cudaErrorInvalidValue;
     raise_smem_limit((const void *)k_mi_energies, smem);
     k_mi_energies<<<slots, me_threads(K), smem, counted(st)>>>(chans_dev, eig_ch, work_dev, n_work, n_ch_total, sample0,
                                                             n_samples, NQ, kg, wg, n_terms, coeffs, Vg, Von, n_I, e_int,
-                                                            eps, Q, Vs, ph, k_out, status, redo, err);
+                                                            eps, Q, eig_status, eig_err, Vs, ph, k_out, status, redo, err);
     return cudaGetLastError();
 }
 

@@ -811,16 +811,18 @@ struct F64Scratch {
 // A size bucket on the FP64 path: the FP32 Jacobi kernel, FP64 refinement
 // (refine64.cu), and the FP64 Jacobi kernel for the items that the refinement
 // does not bring to FP64.  Without room for the refinement's scratch (an HBM
-// budget, a full device) every item takes the FP64 Jacobi kernel.
+// budget, a full device) every item takes the FP64 Jacobi kernel.  by_status: a solve that does
+// not converge shows in its status alone, not in the error word.
 wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double *cf, const int *work, int nw, int nsmp,
-                           int smp0, int n)
+                           int smp0, int n, bool by_status = false)
 {
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
     if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    int *jac_err = by_status ? nullptr : X.err;
     if (n < kRefine64N) {
         auto solve = [&](int th, int ns) {
-            return launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
-                                     X.stream, th);
+            return launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch,
+                                     jac_err, X.stream, th);
         };
         const int threads = X.quiet ? 256 : pick_threads(c, X, n, WPCD_PREC_FP64, nw, nsmp, solve);
         if (threads < 0) return WPCD_ERR_CUDA;
@@ -845,9 +847,9 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         Launch L(c, X, WPCD_PHASE_EIGEN);
         if (big64)
             CK(launch_jacobi_big(true, e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, X.ws_ref.p, slots, e.eps, e.C,
-                                 nullptr, nullptr, nullptr, e.status, v.n_ch, X.err, X.stream));
+                                 nullptr, nullptr, nullptr, e.status, v.n_ch, jac_err, X.stream));
         else
-            CK(launch_jacobi_f64(e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
+            CK(launch_jacobi_f64(e.cd_dev, work, nw, nsmp, smp0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, jac_err,
                                  X.stream));
         return WPCD_OK;
     }
@@ -890,9 +892,9 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
         if (big64) {  // its slots take the place of the refinement's scratch
             const int slots = (int)std::max<size_t>(1, std::min<size_t>(std::min(items, cap64), ref_item * items / slot64));
             CK(launch_jacobi_big(true, e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, base, slots, e.eps, e.C,
-                                 nullptr, nullptr, nullptr, e.status, v.n_ch, X.err, X.stream, RotTest(), done));
+                                 nullptr, nullptr, nullptr, e.status, v.n_ch, jac_err, X.stream, RotTest(), done));
         } else {
-            CK(launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, X.err,
+            CK(launch_jacobi_f64(e.cd_dev, work, nw, ns, smp0 + s0, v.n_terms, cf, n, e.eps, e.C, e.status, v.n_ch, jac_err,
                                  X.stream, 256, done));
         }
     }
@@ -2189,12 +2191,13 @@ wpcd_status mi_eigen_set(wpcd_ctx *c, MiH &m)
 }
 
 // Eigenpairs of S samples of one block size of an MI set into e (as diag_prep left it), on the
-// FP64 path; a solve that fails shows in the energies (their refinement does not converge).
-wpcd_status mi_eigen(wpcd_ctx *c, Exec &Y, EigH &e, MiH &m, const double *cf, int S, int K)
+// FP64 path.  What fails is left to elimination (k_mi_energies): a solve that does not converge
+// by its status, anything else by the error word eig_err.
+wpcd_status mi_eigen(wpcd_ctx *c, Exec &Y, EigH &e, MiH &m, const double *cf, int S, int K, int *eig_err)
 {
     int *err = Y.err;
-    Y.err = nullptr;
-    const wpcd_status st = run_bucket_f64(c, Y, m.set, e, cf, m.work_dev[K - 1], m.n_work[K - 1], S, 0, K * m.NQ);
+    Y.err = eig_err;
+    const wpcd_status st = run_bucket_f64(c, Y, m.set, e, cf, m.work_dev[K - 1], m.n_work[K - 1], S, 0, K * m.NQ, true);
     Y.err = err;
     return st;
 }
@@ -2313,11 +2316,14 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
     wpcd_status st;
     const size_t ph_len = (size_t)S * m.n_ch * n_I * 3;
     if ((st = ws_reserve(c, X, X.ws_tbin, (von_len + ph_len) * sizeof(double)))) return st;
-    // status, and for the systems of an eigendecomposition whether they are left to elimination
-    if ((st = ws_reserve(c, X, X.ws_plan_i, (size_t)S * m.n_ch * (1 + (m.has_set ? n_I : 0)) * sizeof(int)))) return st;
+    // status, and for the eigendecompositions their error words and which systems are left to elimination
+    const size_t plan_len = (size_t)S * m.n_ch + (m.has_set ? 2 + (size_t)S * m.n_ch * n_I : 0);
+    if ((st = ws_reserve(c, X, X.ws_plan_i, plan_len * sizeof(int)))) return st;
     double *Von = static_cast<double *>(X.ws_tbin.p), *ph = Von + von_len;
     int *status = status_dev ? status_dev : static_cast<int *>(X.ws_plan_i.p);
-    int *redo = static_cast<int *>(X.ws_plan_i.p) + (size_t)S * m.n_ch;
+    int *eig_err = static_cast<int *>(X.ws_plan_i.p) + (size_t)S * m.n_ch;  // one per block size
+    int *redo = eig_err + 2;
+    if (m.has_set) CK(cudaMemsetAsync(eig_err, 0, 2 * sizeof(int), X.stream));
     CK(cudaMemcpyAsync(m.ch_dev, m.ch.data(), sizeof(MiChanDev) * m.n_ch, cudaMemcpyHostToDevice, X.stream));
     CK(cudaMemsetAsync(status, 0, sizeof(int) * S * m.n_ch, X.stream));
     double *angx = nullptr, *angw = nullptr;
@@ -2366,13 +2372,13 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
             const int ns = std::min(Sc, S - s0), slots = eig_slots(K);
             const double *cfs = cf ? cf + (size_t)s0 * (m.n_terms - 1) : nullptr;
             if ((!prepared && diag_prep(c, X, m.set, -1, ns, WPCD_PREC_FP64, X.eig)) ||
-                mi_eigen(c, Y, X.eig, m, cfs, ns, K) || ws_reserve(c, Y, Y.ws_ref, (size_t)slots * ng * ng * sizeof(double), true)) {
+                mi_eigen(c, Y, X.eig, m, cfs, ns, K, eig_err + K - 1) || ws_reserve(c, Y, Y.ws_ref, (size_t)slots * ng * ng * sizeof(double), true)) {
                 eig = false;  // no room: by elimination, from the first sample on
                 break;
             }
             Launch L(c, Y, WPCD_PHASE_MI);
             CK(launch_mi_energies(m.ch_dev, X.eig.cd_dev, m.work_dev[K - 1], nw, K, m.n_ch, s0, ns, m.NQ, m.kg, m.wg,
-                                  m.n_terms, cf, m.Vg, Von, n_I, e_int, X.eig.eps, X.eig.C,
+                                  m.n_terms, cf, m.Vg, Von, n_I, e_int, X.eig.eps, X.eig.C, X.eig.status, eig_err + K - 1,
                                   static_cast<double *>(Y.ws_ref.p), slots, ph, k_out, status, redo, X.err, Y.stream));
         }
         if (mi_slots_per_sm(n, m.NQ) < 1) return WPCD_ERR_ARG;

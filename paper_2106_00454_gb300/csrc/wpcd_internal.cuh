@@ -378,8 +378,9 @@ int mi_energies_per_sm(int NQ, int K);
 cudaError_t launch_mi_energies(const MiChanDev *chans_dev, const ChanDev *eig_ch, const int *work_dev, int n_work, int K,
                                int n_ch_total, int sample0, int n_samples, int NQ, const double *kg, const double *wg,
                                int n_terms, const double *coeffs, const double *Vg, const double *Von, int n_I,
-                               const double *e_int, const double *eps, const double *Q, double *Vs, int slots, double *ph,
-                               double *k_out, int *status, int *redo, int *err, cudaStream_t st);
+                               const double *e_int, const double *eps, const double *Q, const int *eig_status,
+                               const int *eig_err, double *Vs, int slots, double *ph, double *k_out, int *status, int *redo,
+                               int *err, cudaStream_t st);
 cudaError_t launch_mi_observables(const MiChanDev *chans_dev, int n_ch, int n_samples, int n_I, const double *e_int,
                                   const double *ph, int n_E, const double *e_lab, double *delta, double *sigma,
                                   cudaStream_t st);
