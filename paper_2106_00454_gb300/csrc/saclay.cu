@@ -45,7 +45,8 @@ __host__ __device__ inline size_t sac_smem(int P, int L1, int TC)
     return ((size_t)P * L1 * 6 + (size_t)P * kSacChunk * 3) * 16 + ((size_t)3 * L1 * TC + 3 * L1 + 2 * TC) * 8;
 }
 
-// CTA (x, y): pairs x P .. + P - 1 of (sample, energy), angles y TC .. + TC - 1.
+// CTA (x, y, z): pairs x P .. + P - 1 of (sample, energy), angles tb TC .. + TC - 1, tb = y and, where
+// the angles need more rows than a grid has, z gridDim.y more.
 __global__ void __launch_bounds__(kSacThreads) k_saclay(const SacChanDev *chans, int n_ch, long long n_pairs, int n_E,
                                                         const double *e_lab, const double *delta, int n_th,
                                                         const double *theta, double *abcde, double *dsig, int P,
@@ -58,9 +59,10 @@ __global__ void __launch_bounds__(kSacThreads) k_saclay(const SacChanDev *chans,
     double *nrm = Y + (size_t)3 * L1 * TC;
     double *ct = nrm + 3 * L1, *st = ct + TC;
     const int tid = threadIdx.x, nt = blockDim.x;
-    const long long pair0 = (long long)blockIdx.x * P;
+    const long long pair0 = (long long)blockIdx.x * P, tb = (long long)blockIdx.z * gridDim.y + blockIdx.y;
+    if (tb * TC >= n_th) return;
     const int np = (int)min((long long)P, n_pairs - pair0);
-    const int th0 = blockIdx.y * TC, nth = min(TC, n_th - th0);
+    const int th0 = (int)tb * TC, nth = min(TC, n_th - th0);
 
     // ---- Y_l^mu(theta, 0), Condon-Shortley phase, mu = 0, 1, 2
     for (int e = tid; e < 3 * L1; e += nt) {  // sqrt((2l+1)/(4 pi) (l-mu)!/(l+mu)!), with (-1)^mu
@@ -218,7 +220,8 @@ cudaError_t launch_saclay(const SacChanDev *chans_dev, int n_ch, int n_samples, 
     const int L1 = Lmax + 1, TC = n_th < 32 ? n_th : 32;
     int P = 1024 / TC < 32 ? 1024 / TC : 32;
     while (P > 1 && sac_smem(P, L1, TC) > 48 * 1024) P /= 2;
-    const dim3 grid((unsigned)((n_pairs + P - 1) / P), (unsigned)((n_th + TC - 1) / TC));
+    const unsigned tbs = (unsigned)((n_th - 1) / TC + 1), rows = tbs < 65535u ? tbs : 65535u;
+    const dim3 grid((unsigned)((n_pairs + P - 1) / P), rows, (tbs + rows - 1) / rows);
     k_saclay<<<grid, kSacThreads, sac_smem(P, L1, TC), counted(st)>>>(chans_dev, n_ch, n_pairs, n_E, e_lab, delta,
                                                                       n_th, theta, abcde, dsig, P, L1, TC);
     return cudaGetLastError();
