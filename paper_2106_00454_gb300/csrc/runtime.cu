@@ -121,6 +121,7 @@ struct Buf {
 // One executor: a stream, its device status word and its workspaces.  The
 // synchronous API runs on the context's own executor; each serving slot has
 // one of its own so that batches overlap on the device.
+constexpr unsigned kForkRetry = 64;
 constexpr int kSides = 3;  // streams beside the executor's own for the size buckets of a batch
 struct Exec {
     cudaStream_t stream = nullptr;
@@ -128,7 +129,11 @@ struct Exec {
     Buf ws_plan_i, ws_plan_d, ws_tbin, ws_phbin, ws_ref, ws_in, ws_out;
     EigH eig;
     bool quiet = false;  // launches that belong to no call (neither counted nor timed)
-    size_t no_fork = ~(size_t)0;  // scratch of the streams' shares that found no room
+    // scratch of the streams' shares that found no room, and when: tried again after a wpcd_release
+    // or kForkRetry calls (a try that fails reallocates the scratch)
+    size_t no_fork = ~(size_t)0;
+    unsigned no_fork_calls = 0;
+    unsigned long long no_fork_gen = 0;
     cudaStream_t side[kSides] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
 };
@@ -207,6 +212,7 @@ struct wpcd_ctx {
     int big_slots = 0;     // CTAs of the global-memory eigensolver (0: automatic)
     int use_graphs = 1;
     std::atomic<unsigned long long> graph_gen{0};
+    std::atomic<unsigned long long> released{0};  // handles given back
     struct GraphE {
         unsigned long long gen = 0;  // generation when first seen / captured
         cudaGraphExec_t exec = nullptr;
@@ -383,6 +389,23 @@ bool side_streams(Exec &X)
         return false;
     }
     return true;
+}
+
+// Whether shares of `total` bytes are known to find no room.
+bool no_room_to_fork(wpcd_ctx *c, Exec &X, size_t total)
+{
+    if (total < X.no_fork) return false;
+    if (X.no_fork_gen == c->released.load() && ++X.no_fork_calls < kForkRetry) return true;
+    X.no_fork = ~(size_t)0;
+    return false;
+}
+
+void remember_no_room(wpcd_ctx *c, Exec &X, size_t total)
+{
+    if (capturing(X.stream)) return;
+    X.no_fork = total;
+    X.no_fork_calls = 0;
+    X.no_fork_gen = c->released.load();
 }
 
 void free_side_streams(Exec &X)
@@ -1059,9 +1082,9 @@ bool fork_units(wpcd_ctx *c, Exec &X, VSetH &v, int S, int prec, F run_unit, std
     }
     for (int k = 0; k < lanes; ++k) off[k + 1] = off[k] + share[k];
     const size_t total = off[lanes];
-    if (units.size() < 2 || total >= X.no_fork || !side_streams(X)) return false;
+    if (units.size() < 2 || no_room_to_fork(c, X, total) || !side_streams(X)) return false;
     if (ws_reserve(c, X, X.ws_ref, total, true)) {
-        if (!capturing(X.stream)) X.no_fork = total;
+        remember_no_room(c, X, total);
         return false;
     }
     if (c->autotune) {  // the autotuner times its candidates alone
@@ -2050,6 +2073,7 @@ wpcd_status wpcd_release(wpcd_ctx *c, int id)
     if (it->second.eig) free_eig(c, *it->second.eig);
     if (it->second.mi) free_mi(c, *it->second.mi);
     c->handles.erase(it);
+    ++c->released;
     return WPCD_OK;
 }
 
@@ -2424,9 +2448,9 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
             share[K - 1] = (std::max(std::max(F64Scratch(c, K * m.NQ, m.n_work[K - 1]).bytes(S), elim(K, true).bytes),
                                      (size_t)eig_slots(K) * K * m.NQ * K * m.NQ * sizeof(double)) + 255) & ~(size_t)255;
         const size_t total = share[0] + share[1];
-        if (total > kRefineScratchBytes || total >= X.no_fork || !side_streams(X)) return false;
+        if (total > kRefineScratchBytes || no_room_to_fork(c, X, total) || !side_streams(X)) return false;
         if (ws_reserve(c, X, X.ws_ref, total, true)) {
-            X.no_fork = total;
+            remember_no_room(c, X, total);
             return false;
         }
         if (c->autotune) {  // the autotuner times its candidates alone

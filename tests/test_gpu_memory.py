@@ -205,3 +205,25 @@ def test_served_fp64_under_a_budget(api):
     finally:
         c.serve_stop()
         c.close()
+
+
+def test_streams_are_taken_up_again_when_room_returns(api):
+    """Mixed path, two sets and one bucket's scratch at a time: no shares for the streams
+    (5 MB more); once the second set (7 MB) is released the next solves take them."""
+    wl = _wl([64], 2)
+    probe = api.Context(0)
+    probe.profile(True)  # one bucket after another
+    first = api.Model(probe, wl)
+    api.Model(probe, wl)
+    want = _phases(probe, first, wl, api.PREC_MIXED)
+    budget = probe.bytes_in_use() + MB
+    probe.close()
+    c = api.Context(0, hbm_budget_bytes=budget)
+    first, second = api.Model(c, wl), api.Model(c, wl)
+    a = _phases(c, first, wl, api.PREC_MIXED, 4)
+    second.release()
+    before = c.bytes_in_use()
+    b = _phases(c, first, wl, api.PREC_MIXED)
+    assert before + 4 * MB < c.bytes_in_use() <= budget
+    c.close()
+    assert np.array_equal(a, want) and np.array_equal(b, want)
