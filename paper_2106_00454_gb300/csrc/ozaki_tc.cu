@@ -591,13 +591,7 @@ static cudaError_t gemm_tc_p(int n, int items, const __nv_bfloat16 *sa, const in
     }
     const long long ntiles = (long long)per_item * items;
     if (ntiles > 0x7fffffffll) return cudaErrorInvalidValue;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
+    const int sms = device_sms();
     cudaError_t e = cudaFuncSetAttribute(k_oz_gemm_tc<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc<P>::kSmem);
     if (e != cudaSuccess) return e;
     const int grid = (int)(ntiles < sms ? ntiles : sms);

@@ -291,12 +291,13 @@ __global__ void __launch_bounds__(256) k_r64_sort(const ChanDev *chans, const in
 static size_t r64_smem(int n) { return (size_t)n * (2 * 8 + 2 * 4) + kPairCap * 2 * sizeof(unsigned); }
 
 // CTAs that share an item in k_r64_update and k_r64_sort: up to two of 256
-// threads on each of the 152 SMs (clusters wait for room beside other kernels, so a full chip
+// threads on each SM (clusters wait for room beside other kernels, so a full chip
 // does better without: up to eight cost 19.2 -> 20.1 ms at 256 samples), two rows or more a warp.
 static int r64_share(int items, int n)
 {
+    const long long room = 2ll * device_sms();
     int cl = 8;
-    while (cl > 1 && ((long long)items * cl > 2 * 152 || n < 16 * cl)) cl /= 2;
+    while (cl > 1 && ((long long)items * cl > room || n < 16 * cl)) cl /= 2;
     return cl;
 }
 

@@ -33,6 +33,17 @@ cudaError_t raise_smem_limit(const void *kernel, size_t bytes)
     if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+
+int device_sms()
+{
+    static std::atomic<int> of[64];  // by device, 0: not asked yet
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && (n = of[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+    if (dev >= 0 && dev < 64) of[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
 }
 
 using namespace wpcd;
@@ -523,7 +534,6 @@ int pick_threads(wpcd_ctx *c, Exec &X, int n, int prec, int nw, int nsmp, F laun
         if (it != c->tuned.end()) return it->second.threads;
     }
     if (capturing(X.stream)) return -1;  // tuning synchronises: never inside a capture
-    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     wpcd_ctx::Tuned t{256, {-1.f, -1.f, -1.f, -1.f, -1.f}};
     float best = 1e30f;
     cudaEvent_t a, b;
@@ -692,7 +702,6 @@ wpcd_status diag_prep(wpcd_ctx *c, Exec &X, VSetH &v, int vset_id, int S, int pr
     }
     const size_t coeff_len = (size_t)S * std::max(v.n_terms - 1, 1);
     wpcd_status st = WPCD_OK;
-    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     if ((long long)S * v.n_ch > 1) side_streams(X);
     // grow-only storage: a smaller batch or another set with as many channels reuses it
     if (e.eps_len < eps_len || e.c_len < c_len || e.coeff_len < coeff_len || e.status_len < (size_t)S * v.n_ch ||
@@ -765,7 +774,6 @@ wpcd_status run_bucket_big(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
                            int nsmp, int smp0, int n)
 {
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
-    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     const int occ = std::max(1, jacobi_big_occupancy(n, false));
     const size_t slot_b = (jacobi_big_scratch_bytes(n, false) + 255) & ~(size_t)255;
     // CTAs in flight: every resident one.  Each CTA's round is bound by the latency of
@@ -811,7 +819,6 @@ struct F64Scratch {
     int cap32, cap64;
     F64Scratch(wpcd_ctx *c, int n, int nw_) : nw(nw_)
     {
-        if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
         big32 = !jacobi_fits_smem(n, false);
         big64 = !jacobi_fits_smem(n, true);
         ref_item = refine64_scratch_per_item(n);
@@ -840,7 +847,6 @@ wpcd_status run_bucket_f64(wpcd_ctx *c, Exec &X, VSetH &v, EigH &e, const double
                            int smp0, int n, bool by_status = false)
 {
     if (n > jacobi_big_max_n()) return WPCD_ERR_ARG;
-    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     int *jac_err = by_status ? nullptr : X.err;
     if (n < kRefine64N) {
         auto solve = [&](int th, int ns) {
@@ -1378,6 +1384,7 @@ wpcd_status wpcd_create(wpcd_ctx **out, int device, size_t hbm_budget_bytes, voi
         delete c;
         return WPCD_ERR_CUDA;
     }
+    c->n_sm = device_sms();
     c->main.err = c->err_dev;
     *out = c;
     return WPCD_OK;
@@ -2328,7 +2335,6 @@ wpcd_status wpcd_mi_solve(wpcd_ctx *c, int mi_id, const double *coeffs, int S, c
     MiH &m = *h->mi;
     if (m.n_terms > 1 && !coeffs) return WPCD_ERR_ARG;
     CK(cudaSetDevice(c->device));
-    if (!c->n_sm) cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
     Exec &X = c->main;
     const int M = m.NQ + 1;
     // on-shell columns [ch][n_I][n_terms][K][K][M], phases [S][ch][n_I][3], status [S][ch]

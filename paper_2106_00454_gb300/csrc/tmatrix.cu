@@ -488,16 +488,9 @@ static void launch_tmat_t(const ChanDev *chans_dev, int n_ch, int n_samples, int
     raise_smem_limit((const void *)k_tmat<VC, MODE>, smem);
     // shares per solve: the chip holds five CTAs an SM; a share below four items costs more in the
     // boundaries that each CTA forms than it gains
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
     const long long solves = (long long)n_samples * (tw.work ? tw.n_work : n_ch);
     const int most = (MODE == 2 ? n_E : min(stride, 2 * n_E + 2)) / 4;
-    const int shares = (int)max(1ll, min((long long)most, 5ll * sms / solves));
+    const int shares = (int)max(1ll, min((long long)most, 5ll * device_sms() / solves));
     k_tmat<VC, MODE><<<dim3((unsigned)solves, shares), kTThreads, smem, counted(st)>>>(
         chans_dev, n_ch, n_terms, coeffs, eps_all, C_all, plan, n_E, stride, tout, phout, err, tw);
 }

@@ -52,6 +52,9 @@ inline cudaStream_t counted(cudaStream_t st)
 // launch needs, so the limit only grows (thread-safe).
 cudaError_t raise_smem_limit(const void *kernel, size_t bytes);
 
+// SMs of the calling thread's current device (thread-safe).
+int device_sms();
+
 // One channel of a projected potential set, as the kernels see it.
 // Channel of an MI set: its grid potential terms Vg [n_terms][n][n] start at
 // vg_off, its on-shell columns Von [n_I][n_terms][K][K][N_Q+1] at von_off;
