@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
     // and the column starts mcol(a) | mcol(b) << 16 (A has fewer than 2^16 floats)
     uint4 *rec = reinterpret_cast<uint4 *>(A + mix_a_floats(n));
     float *daa = reinterpret_cast<float *>(rec + h), *dbb = daa + h;
-    // flags: [0] rotation in this sweep; [1..3] rotation in this round and [4..6] the
-    // round's count of rotating slots, both cycled over three rounds
+    // flags: [0] rotation in this sweep; [4..6] the round's count of rotating slots, cycled
+    // over three rounds
     int *flags = reinterpret_cast<int *>(dbb + h);
     int *rank = flags + 8;                                            // [h]: index in act, or -1
     unsigned short *act = reinterpret_cast<unsigned short *>(rank + h);  // [h]: the rotating slots
@@ -206,6 +206,9 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
         if (tid == 0) flags[0] = 0;
         __syncthreads();
         float thr = 0.0f;
+        // (Never taken: sizes with threshold sweeps go to k_jacobi_teams.  Left out, the round's code
+        // comes out slower -- one set at N_WP = 64, mixed, 1327 -> 1344 us; 1024 samples x 15
+        // channels 53.8 -> 54.0 ms -- whichever way its rotation test and loops are written.)
         if (n >= kMixThreshN && sweeps < kMixThreshSweeps) {
             float o2 = 0.0f;  // columns j and n - 1 - j per thread: balanced lengths
             for (int j = tid; j < (n + 1) / 2; j += nt) {
@@ -225,10 +228,7 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
         ++sweeps;
         for (int r = 0; r < M; ++r) {
             const int nx3 = g3 == 2 ? 0 : g3 + 1;
-            if (tid == 0) {  // last read two rounds ago, before this round's barrier
-                flags[1 + nx3] = 0;
-                flags[4 + nx3] = 0;
-            }
+            if (tid == 0) flags[4 + nx3] = 0;  // last read two rounds ago, before this round's barrier
             for (int k = tid; k < h; k += nt) {
                 int a, b;
                 mix_pair(r, k, M, a, b);
@@ -249,7 +249,6 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
                     app -= t * apq;
                     aqq += t * apq;
                     flags[0] = 1;
-                    flags[1 + g3] = 1;
                     const int idx = atomicAdd(&flags[4 + g3], 1);
                     act[idx] = (unsigned short)k;
                     rank[k] = idx;
@@ -274,10 +273,10 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
                         quad_update(r1, r2);
                     }
                 } else {
-                    // few slots rotate (late sweeps, threshold sweeps): only the pairs that
-                    // hold a rotating slot, one warp per rotating slot P, lanes over the
-                    // others, rows from P's pair; a pair of two rotating slots is done
-                    // once, by the lower one's warp.  A pair with a non-rotating slot
+                    // few slots rotate (late sweeps): only the pairs that hold a rotating
+                    // slot, one warp per rotating slot P, lanes over the others, rows from
+                    // P's pair; a pair of two rotating slots is done once, by the lower
+                    // one's warp.  A pair with a non-rotating slot
                     // gives the same bits in either orientation (the identity's c = 1,
                     // s' = +-0 leave its side exact), so the result does not depend on
                     // the order of the rotating list.
@@ -308,12 +307,12 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
                     float4 *Cp = reinterpret_cast<float4 *>(C + (size_t)(rk.z & 0xFFFFu) * ldc);
                     float4 *Cq = reinterpret_cast<float4 *>(C + (size_t)(rk.z >> 16) * ldc);
                     const float c = __uint_as_float(rk.x), s = __uint_as_float(rk.y);
-                    if (!C_SMEM && nv <= 96) {
+                    if (!C_SMEM) {
                         // columns in global memory (L2): every load of the two columns is
                         // issued before the first store, one L2 round trip per rotation
-                        float4 a[3], b[3];
+                        float4 a[2], b[2];  // n < 160: at most 40 float4 a column
 #pragma unroll
-                        for (int t = 0; t < 3; ++t) {
+                        for (int t = 0; t < 2; ++t) {
                             const int v = lane + 32 * t;
                             if (v < nv) {
                                 a[t] = Cp[v];
@@ -321,7 +320,7 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
                             }
                         }
 #pragma unroll
-                        for (int t = 0; t < 3; ++t) {
+                        for (int t = 0; t < 2; ++t) {
                             const int v = lane + 32 * t;
                             if (v < nv) {
                                 Cp[v] = make_float4(c * a[t].x - s * b[t].x, c * a[t].y - s * b[t].y,
@@ -408,12 +407,12 @@ __device__ __forceinline__ void team_arrive(int id, int threads)
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// Rotate the pairs of columns that the list names, one warp per rotation, T float4 per lane and
+// Rotate the pairs of columns that the list names, one warp per rotation, up to three float4 per lane and
 // column; every load of the two columns is issued before the first store (one L2 round
 // trip).  C_a <- c C_a - s' C_b, C_b <- s' C_a + c C_b.
-template <int T>
 __device__ __forceinline__ void rotate_columns(const uint4 *list, int na, float *C, int ldc, int warp, int nwarps, int lane)
 {
+    constexpr int T = 3;  // n <= 304: at most 76 float4 a column
     const int nv = ldc >> 2;
     for (int i = warp; i < na; i += nwarps) {
         const uint4 rk = list[i];
@@ -514,7 +513,7 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
             const int na = flags[8 + b];
             if (na < 0) break;
             const uint4 *ls = list + b * h;
-            rotate_columns<3>(ls, na, C, ldc, w, nw, lane);
+            rotate_columns(ls, na, C, ldc, w, nw, lane);
             team_arrive(kBarEmpty + b, nt);
         }
     } else {
@@ -566,7 +565,7 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_teams(const Ch
             if (tid == 0) flags[0] = 0;
             team_sync(kBarA, nta);
             float thr = 0.0f;
-            if (n >= kMixThreshN && sweeps < kMixThreshSweeps) {
+            if (sweeps < kMixThreshSweeps) {
                 // columns j and n - 1 - j per lane (balanced lengths), 32 such pairs a warp and sum, whatever the CTA size
                 const int nj = (n + 1) / 2, ng = (nj + 31) >> 5;
                 for (int g = warp; g < ng; g += nwarps) {

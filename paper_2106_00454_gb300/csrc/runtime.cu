@@ -93,7 +93,6 @@ struct VSetH {
     // (W_0 = 0), so that C0^T H(c) C0 = diag(eps0) + sum_a c_a W_a; per size bucket
     // the digit slices of the rows of its channels' C0 for the back-rotation X = C0 X'.
     struct RotB {
-        double *C0 = nullptr;  // [nw][n][n], the bucket's channels in bucket order
         __nv_bfloat16 *sC = nullptr;
         int *eC = nullptr;
     };
@@ -661,12 +660,11 @@ wpcd_status ensure_rotation(wpcd_ctx *c, Exec &X, VSetH &v)
     for (auto &kv : v.buckets) {
         const int n = kv.first, nw = (int)kv.second.size();
         VSetH::RotB &rb = v.rotb[n];
-        rb.C0 = v.C0 + bstart[n];
         if ((st = dalloc(c, &rb.sC, (size_t)nw * oz_slice_elems(n))) || (st = dalloc(c, &rb.eC, (size_t)nw * n))) {
             cleanup();
             return st;
         }
-        CK(launch_oz_split(n, nw, false, rb.C0, rb.sC, rb.eC, X.stream));
+        CK(launch_oz_split(n, nw, false, v.C0 + bstart[n], rb.sC, rb.eC, X.stream));
     }
     std::vector<int> hs(v.n_ch);
     int herr = 0;
