@@ -498,7 +498,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
                 emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
             }
-            if (__all_sync(0xffffffffu, er - eshift + emin >= -1022 && er - eshift + emax <= 959)) {
+            // a vector with an infinity or a NaN (exponent 1025) has no digits: its seven-digit products,
+            // which stand for FP64 ones, are NaN
+            const bool finite = P < 7 || (er <= 1024 && emax <= 1024);
+            if (__all_sync(0xffffffffu, finite && er - eshift + emin >= -1022 && er - eshift + emax <= 959)) {
 #pragma unroll
                 for (int j = 0; j < kTcDrainCols; ++j) {
                     const long long e = er + __shfl_sync(0xffffffffu, ecl, j) - eshift;
@@ -507,8 +510,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             } else {
 #pragma unroll
                 for (int j = 0; j < kTcDrainCols; ++j) {
-                    const int e = er + __shfl_sync(0xffffffffu, ecl, j) - eshift;
-                    v[j] = f64_times_pow2_slow(__longlong_as_double((long long)u[j]), e);
+                    const int ec = __shfl_sync(0xffffffffu, ecl, j);
+                    v[j] = f64_times_pow2_slow(__longlong_as_double((long long)u[j]), er + ec - eshift);
+                    if (P >= 7 && (er > 1024 || ec > 1024)) v[j] = __longlong_as_double(0x7ff8000000000000ll);
                 }
             }
             if (sym) {
