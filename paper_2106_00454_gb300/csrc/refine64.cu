@@ -56,7 +56,12 @@ namespace wpcd {
 // first order cannot take is turned, and the item goes on to the next iteration.
 constexpr float kFirstAngle = 1.2207031e-4f, kLaterAngle = 1.4901161e-8f, kMaxAngle = 0.02f;
 constexpr float kDoneE2 = 2e-14f;     // ||E||_F <= 1.4e-7: its square is below the rounding of X^T X
-constexpr int kPairCap = 64;          // pairs turned per scan
+// Pairs turned per scan: 64 up to n = 512, 512 above.  Pairs that first order cannot take grow in
+// number with n, and a first iteration that leaves them is not made good by the other two: with
+// 64 everywhere, dense matrices above n = 512 and one in eight of the projected coupled ones at
+// N_WP = 512 went to FP64 Jacobi (3 matrices of n = 514 1980 -> 26 ms, 8 of n = 1024 31 s -> 180 ms;
+// those that finished before, n = 600, 62 -> 64 ms).
+constexpr int kPairCap = 512, kPairFew = 64;
 constexpr int kPairScans = 6;
 
 // One CTA per item, or a cluster of them (CL) where the items are few: the CTAs take the
@@ -114,6 +119,7 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
     // the tests below are in FP32: H's scale has to leave them room on both sides
     if (__syncthreads_or(above) || !__syncthreads_or(enough)) return;
     float ang = it == 0 ? kFirstAngle : kLaterAngle;
+    const int cap = n > 512 ? kPairCap : kPairFew;
     bool plain = true;  // S holds S (not yet s)
     bool clear = false, later = false;
     for (int scan = 0;; ++scan) {
@@ -163,13 +169,13 @@ __global__ void __launch_bounds__(256) k_r64_update(int n, double *S_all, double
         }
         sync();
         const int m = *cnt0;
-        if (m > kPairCap && ang < kMaxAngle) {  // too many: turn only those beyond first order
+        if (m > cap && ang < kMaxAngle) {  // too many: turn only those beyond first order
             ang = kMaxAngle;
             later = true;
             sync();  // every thread has read the count
             continue;
         }
-        if (m == 0 || m > kPairCap || scan >= kPairScans) {
+        if (m == 0 || m > cap || scan >= kPairScans) {
             clear = m == 0 && !later;
             break;
         }
