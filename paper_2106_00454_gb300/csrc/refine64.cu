@@ -18,9 +18,15 @@
 // |s_ij| below the rounding of the products is left alone: its quotient is noise,
 // and the FP64 Jacobi kernel's stopping test would leave it too.
 //
-// An item is done once, after the first iteration, an update's ||E||_F^2 <= kDoneE2:
-// what is left of the off-diagonal is second order in E, below the
-// FP64 Jacobi kernel's own test off(A) <= 1e-15 ||H||_F.  Two iterations
+// An item is done once, after the first iteration, an update's ||E||_F^2 <= kDoneE2 =
+// 2e-14: what is left of the off-diagonal, and the error of the eigenvalues, which come
+// from before the update, are second order in E and so below 2e-14 ||H||_F.  That bound is
+// seldom met: the second iteration's E is mostly the rounding of the products over small
+// gaps, whose second order is below the rounding of X.  Measured at 2e-14 and at 1e-15
+// alike: residual 3.9e-15 ||H||_F, eigenvalues 6e-16, orthogonality 2.6e-14 at n = 200 (FP64
+// Jacobi alone, which stops at off(A) <= 1e-15 ||H||_F: 3e-15, 1e-15, 1e-12), at 18.0 and
+// 20.1 ms for 128 samples x 15 channels at N_WP = 100, as the tighter one sends more items
+// through a third iteration; 2e-16 leaves items to FP64 Jacobi (85 ms).  Two iterations
 // usually do it, the third runs only for the items that need it, and an item
 // that is not done after that (or whose eigenvalues do not fit FP32) is solved again
 // by the FP64 Jacobi kernel (the caller's fallback over done[b] == 0).
@@ -55,7 +61,7 @@ namespace wpcd {
 // whose s only the second iteration's products resolve); where it is not, only what
 // first order cannot take is turned, and the item goes on to the next iteration.
 constexpr float kFirstAngle = 1.2207031e-4f, kLaterAngle = 1.4901161e-8f, kMaxAngle = 0.02f;
-constexpr float kDoneE2 = 2e-14f;     // ||E||_F <= 1.4e-7: its square is below the rounding of X^T X
+constexpr float kDoneE2 = 2e-14f;     // ||E||_F <= 1.4e-7; the bound on what its square leaves (above)
 // Pairs turned per scan: 64 up to n = 512, 512 above.  Pairs that first order cannot take grow in
 // number with n, and a first iteration that leaves them is not made good by the other two: with
 // 64 everywhere, dense matrices above n = 512 and one in eight of the projected coupled ones at
