@@ -227,3 +227,48 @@ def test_streams_are_taken_up_again_when_room_returns(api):
     assert before + 4 * MB < c.bytes_in_use() <= budget
     c.close()
     assert np.array_equal(a, want) and np.array_equal(b, want)
+
+
+def test_server_and_program_share_a_tight_budget(api):
+    """A program projects, solves and releases while the server works through FP64 and
+    mixed requests, under a budget in which each needs the other's spare scratch: every
+    call finishes, with the results that it has alone."""
+    import threading
+    chs = W.np_channels(2)
+    rng = np.random.default_rng(12)
+    reqs = [(rng.standard_normal(14) * W.TERM_SCALE, np.sort(rng.uniform(1.0, 350.0, 12)), (48, 64)[k % 2], k // 2 % 2)
+            for k in range(12)]
+    args = (chs, W.GEN_YUKAWA, W.YUKAWA_PARAMS, W.N_TERMS_YUKAWA, [48, 64])
+    wl = _wl([64], 6)
+    free = api.Context(0)
+    want_p = _phases(free, api.Model(free, wl), wl, api.PREC_FP64)
+    free.serve_start(*args, max_batch=2, n_slots=2)
+    want_r = [free.wait(free.submit(*r)).delta for r in reqs]
+    held = free.bytes_in_use()
+    free.close()
+    # what the server and the program need to keep, the mixed slots' scratch, a second set, and a little
+    c = api.Context(0, hbm_budget_bytes=held + _model_bytes(api, wl) - 44 * MB)
+    c.serve_start(*args, max_batch=2, n_slots=2)
+    bad = []
+
+    def serve():
+        try:
+            for k in range(60):
+                r = c.wait(c.submit(*reqs[k % len(reqs)]))
+                assert r.status == 0, r.status
+                _close(r.delta, want_r[k % len(reqs)], 1e-3 if reqs[k % len(reqs)][3] else 1e-8)
+        except Exception as ex:  # noqa: BLE001
+            bad.append(repr(ex))
+
+    th = threading.Thread(target=serve)
+    th.start()
+    try:
+        for _ in range(15):
+            md = api.Model(c, wl)
+            _close(_phases(c, md, wl, api.PREC_FP64, 2), want_p, 1e-8)
+            md.release()
+    finally:
+        th.join(120)
+    assert not th.is_alive() and not bad, bad
+    c.serve_stop()
+    c.close()
