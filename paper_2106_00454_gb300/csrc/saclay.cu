@@ -45,8 +45,8 @@ __host__ __device__ inline size_t sac_smem(int P, int L1, int TC)
     return ((size_t)P * L1 * 6 + (size_t)P * kSacChunk * 3) * 16 + ((size_t)3 * L1 * TC + 3 * L1 + 2 * TC) * 8;
 }
 
-// CTA (x, y, z): pairs x P .. + P - 1 of (sample, energy), angles tb TC .. + TC - 1, tb = y and, where
-// the angles need more rows than a grid has, z gridDim.y more.
+// CTA (x, y, z): pairs x P .. + P - 1 of (sample, energy), TC angles from y TC on and, where the angles
+// need more rows than a grid has, z gridDim.y TC further on.
 __global__ void __launch_bounds__(kSacThreads) k_saclay(const SacChanDev *chans, int n_ch, long long n_pairs, int n_E,
                                                         const double *e_lab, const double *delta, int n_th,
                                                         const double *theta, double *abcde, double *dsig, int P,
@@ -59,10 +59,11 @@ __global__ void __launch_bounds__(kSacThreads) k_saclay(const SacChanDev *chans,
     double *nrm = Y + (size_t)3 * L1 * TC;
     double *ct = nrm + 3 * L1, *st = ct + TC;
     const int tid = threadIdx.x, nt = blockDim.x;
-    const long long pair0 = (long long)blockIdx.x * P, tb = (long long)blockIdx.z * gridDim.y + blockIdx.y;
-    if (tb * TC >= n_th) return;
+    const long long pair0 = (long long)blockIdx.x * P;
+    const unsigned first = (blockIdx.z * gridDim.y + blockIdx.y) * (unsigned)TC;  // below 2^31 + 65535 TC
+    if (first >= (unsigned)n_th) return;
     const int np = (int)min((long long)P, n_pairs - pair0);
-    const int th0 = (int)tb * TC, nth = min(TC, n_th - th0);
+    const int th0 = (int)first, nth = min(TC, n_th - th0);
 
     // ---- Y_l^mu(theta, 0), Condon-Shortley phase, mu = 0, 1, 2
     for (int e = tid; e < 3 * L1; e += nt) {  // sqrt((2l+1)/(4 pi) (l-mu)!/(l+mu)!), with (-1)^mu
