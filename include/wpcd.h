@@ -59,9 +59,9 @@ typedef enum {
  * change less than 2e-14 ||H||_F (measured: residuals of 4e-15 at n = 200, 3e-14 at
  * n = 1024), and FP64 parallel Jacobi for any solve that the refinement does not
  * finish (values outside FP32's range, unresolved clusters; wpcd_fp64_unrefined
- * counts them), for matrices up to n = 16 and when there is no room for its scratch.  MIXED: H diagonalised in FP32 (Jacobi with a
- * relative rotation threshold), then two FP64 refinement iterations of the
- * eigenpairs (Ogita-Aishima: Y = HX, S = X^T Y, G = X^T X, X <- X(I + E)) as
+ * counts them), for matrices up to n = 16 and when there is no room for its scratch.
+ * MIXED: H diagonalised in FP32 (Jacobi with a relative rotation threshold), then two
+ * FP64 refinement iterations of the eigenpairs (Ogita-Aishima: Y = HX, S = X^T Y, G = X^T X, X <- X(I + E)) as
  * batched FP64 products; everything after the eigensolve (resolvent logs, T,
  * S, phases) is FP64 on both paths. */
 typedef enum { WPCD_PREC_FP64 = 0, WPCD_PREC_MIXED = 1 } wpcd_precision;
@@ -102,7 +102,9 @@ enum {
  * FP64 (FP64 CUDA cores).  WPCD_OPT_AUTOTUNE (1 = on, the default): on the first
  * batched eigensolve of each (matrix size, precision) the context times CTA
  * sizes of the FP32 kernel, 64/128/256/512/1024 (up to 512 on the FP64 path
- * below n ~ 230), on about two full waves of that bucket and keeps the fastest (wpcd_tuning reports the choices); 0 = fixed 256 threads.
+ * below n ~ 230; of the FP64 kernel up to n = 16), on about two full waves of that bucket, or
+ * on all of it where it is smaller, and keeps the fastest (wpcd_tuning reports the choices);
+ * 0 = fixed 256 threads.
  * WPCD_OPT_GRAPH (1 = on, the default): batched wpcd_solve / wpcd_solve_host
  * calls are replayed from CUDA graphs (see wpcd_solve); 0 = every call
  * launches its kernels one by one.  WPCD_OPT_BIG_SLOTS: CTAs (each with its

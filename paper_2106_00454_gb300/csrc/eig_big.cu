@@ -31,7 +31,8 @@
 // CTA finds the round's rotations for itself, and the row pairs are dealt out over the
 // cluster's warps.  A and Cc then pass through the L2 (loads that skip the L1) and
 // cluster barriers stand around phase 2.  Same operations, same bits.  16 samples x
-// 15 channels at N_WP = 256 (64 matrices of n = 512: clusters of two): a call 125.5 -> 73.0 ms.
+// 15 channels at N_WP = 256 (64 matrices of n = 512: clusters of two): a call 125.5 -> 73.0 ms on
+// one machine, 130 to 162 -> 89 to 99 on others.
 //
 // FP64 (T = double): a pair rotates whenever a_pq != 0; sweeps stop when
 // off(A) <= 1e-15 ||H||_F (as the shared-memory FP64 kernel).  Eigenvalues

@@ -368,7 +368,8 @@ __global__ void __launch_bounds__(2 * kMixMaxThreads, 1) k_jacobi_mixed(const Ch
 // through two lists.  A round of A is bound by shared memory and by the latency of its
 // warps, the columns by the L2, so the two overlap instead of following each other
 // (same operations on the same values as k_jacobi_mixed: the same bits).  A quarter of the
-// warps is enough for C, and A needs the rest: measured in us a solve, one team -> two,
+// warps is enough for C at 1024 threads, and A needs the rest (5/16 below, 3/8 at 256: not
+// swept there): measured in us a solve, one team -> two,
 // n = 300 (1024 threads, 8 warps for C) 85.2 -> 70.3 on 3S1-3D1 and 16.3 -> 13.7 on
 // 3F4-3H4 (6 / 7 / 10 / 16 warps for C: 73.1 / 70.3 / 71.4 / 79.1 on the first), n = 256
 // 51.5 -> 44.5, n = 200 (512 threads) 19.9 -> 18.6, n = 180 16.5 -> 14.3; n = 150 14.5 -> 18.8 and

@@ -34,16 +34,16 @@
 // The FP32 solve may start from C0^T H C0, C0 the eigenvectors of diag(H0) + V0 (built
 // once per set): nearly diagonal, about half the sweeps, and the longest chains (a
 // channel with a bound state, 12 sweeps) shorten most.  It only supplies the start: H
-// itself is never rotated here.  Against the start from H: 20 channels at N_WP = 100, one
-// sample, 5.6 -> 4.0 ms a solve, 20 channels at N_WP = 150, 8 samples, 16.3 -> 11.7; where
-// the chip is full the change of basis costs what the sweeps give (15 channels of N_WP
-// 40/64/100, 256 samples, 24.0 -> 25.1).
+// itself is never rotated here.  Start from H -> from the basis, ms a call: 20 channels at
+// N_WP = 100, one sample, 5.47 -> 3.20; at N_WP = 150, 8 samples, 14.8 -> 11.2; 15 channels of
+// N_WP 40/64/100, 32 samples 4.42 -> 3.96, 256 19.7 -> 18.4, 1024 74.1 -> 69.1.
 //
 // Measured against FP64 Jacobi alone (its rotations are bound by the FP64 pipe):
-// 20 channels at N_WP = 100, one sample, 145 -> 3.1 ms a solve; 15 channels of
-// N_WP 40/64/100, 256 samples, 337 -> 19.3 ms; 20 channels at N_WP = 150, 8 samples,
-// 850 -> 10.7 ms; 1S0 at N_WP = 32, 0.69 -> 0.29 ms; errors against 64-bit LAPACK
-// unchanged (T 2e-13 to 9e-13 in both).
+// 20 channels at N_WP = 100, one sample, 153 -> 3.2 to 4.0 ms a solve (by the sample); 15
+// channels of N_WP 40/64/100, 256 samples, 333 -> 18.7 ms; 20 channels at N_WP = 150, 8
+// samples, 843 to 918 -> 10.5 to 12.0 ms; 1S0 at N_WP = 32, 0.69 -> 0.29 ms; errors against
+// 64-bit LAPACK unchanged (T 3e-14 to 1.2e-12 in both).  Up to n = 16 FP64 Jacobi is faster
+// (runtime.cu).
 //
 // The update is X + X E with E small: the digit product's rounding, relative
 // to E's columns, then vanishes beside X, and X keeps its 53 bits.

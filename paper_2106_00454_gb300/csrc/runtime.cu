@@ -61,7 +61,7 @@ constexpr RotTest kTest64{3.8146973e-6f, 3.8146973e-6f};
 // 1S0, 1 and 4096 samples: n = 4 82 / 159 and 410 / 1817, n = 8 139 / 172 and 999 / 2137, n = 12 234 / 190
 // and 1794 / 2570, n = 16 300 / 207 and 2818 / 3001, n = 18 417 / 232 and 3754 / 3300, n = 24 559 / 278 and
 // 6285 / 4023; 7 channels J <= 2 of n = 8 and 16, 4096 samples, 8432 / 18011.  The size alone decides
-// (the same bits alone and in a batch), so the line lies where no batch loses.
+// (the same bits alone and in a batch): the line lies where the refinement wins at every batch.
 constexpr int kRefine64N = 17;
 constexpr size_t kVcScratchBytes = (size_t)8 << 30;  // FP64 T: scratch of the rows of V C, per chunk
 // ... for matrices from this size on.  T phase in us, formed in the T kernel / rows by products,
